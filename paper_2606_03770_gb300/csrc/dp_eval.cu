@@ -820,26 +820,47 @@ __device__ __forceinline__ void dp_eval_body(const Dims &dm, const Tables &tb, c
 }
 
 // ---------------------------------------------------------------------------
-// Blocks of several types (per-layer prefix sums): the plain-scan DP.
+// Blocks of several types (per-layer prefix sums).
 //
 // A stage's cost now depends on where it starts, and the best bottleneck of a
 // prefix is no longer monotone in its length (a heavy block can make fewer
-// blocks cost more), so the crossover bisection of dp_eval_body does not
-// apply.  Each cell takes the full minimum over its splits, as Eq. 1 writes
-// it, on the float64 times themselves (their bit patterns, which order like
-// the values), read from the per-layer cost table:
+// blocks cost more).  The columns are Eq. 1's, on the float64 times themselves
+// (their bit patterns, which order like the values), read from the per-layer
+// cost table:
 //   F_k[r] = min_s max(F_{k-1}[s], l_k(s+k-1 .. r+k-1), tau_k)     devices 1..k, no master
-//   G_k[b] = min_t max(l_k(first t+1 of its range), G_{k+1}[b-t], tau_{k+1})   devices k..m
+//   G_k[b] = min_u max(G_{k+1}[u], l_k(the b-u+1 blocks before them), tau_{k+1})   devices k..m
 //   V_mu   = min_{a,b} max(F_{mu-1}[a], l^head_mu(the W-a-b blocks between), G_{mu+1}[b], tau_mu, tau_mu+1)
-// mu* = the smallest mu with the least V_mu; its prefix columns (the head at
-// mu*) are recomputed from column mu* on, and the traceback takes the smallest
-// split attaining each cell's value.  Every value and tie is the oracle's.
+// The stage time falls as the split s rises (fewer blocks), so a split may be
+// charged the least F over all splits from s on without changing the minimum:
+// that range minimum rises with s, the stage time falls, and the cell is at
+// their crossover, found by bisection instead of a scan over the splits.
+// Range minima come from a sparse table of the previous column (minima over
+// 2^l entries), rebuilt per column.  A master's (a, b) search bisects over a
+// for each b in the same way.
+// mu* = the smallest mu with the least V_mu; masters are tried four at a time
+// until one reaches the master-free optimum F_m (the head only adds).  mu*'s
+// prefix columns are recomputed from column mu* on, and the traceback takes
+// the smallest split attaining each cell's value.  Every value and tie is the
+// oracle's.
+//
+// Bound by latency: about log2(W) dependent table reads (L2) per column.  The
+// scan it replaces made W / 2 reads per cell.
 // ---------------------------------------------------------------------------
+constexpr int kLayeredWarps = 4;
+
+// Levels above the column itself in the sparse table of W entries.
+__host__ __device__ __forceinline__ unsigned sparse_levels(unsigned W)
+{
+    unsigned l = 0;
+    while ((2u << l) <= W) ++l;
+    return l;
+}
+
 __host__ __device__ __forceinline__ unsigned dp_layered_item_bytes(int m, int N)
 {
     const unsigned W = (unsigned)(N - m + 1);
-    const unsigned bytes = 8u * (2u * (unsigned)m * W + 2u * (unsigned)m) + 4u * (unsigned)m + 2u * (unsigned)m;
-    return (bytes + 15u) & ~15u;
+    const unsigned keys = 2u * (unsigned)m * W + kLayeredWarps * sparse_levels(W) * W + 2u * (unsigned)m;
+    return (8u * keys + 4u * (unsigned)m + 2u * (unsigned)m + 15u) & ~15u;
 }
 
 size_t dp_layered_smem_bytes(int M, int N)
@@ -853,15 +874,53 @@ size_t dp_layered_smem_bytes(int M, int N)
     return best;
 }
 
-__global__ void __launch_bounds__(128) dp_layered_kernel(Dims dm, Tables tb, DevPop pop, EvalOut out, WorkList wl,
-                                                         SlotInfo si, SplitOut so)
+// The sparse table of a column by n threads (id 0..n-1), which `sync` joins:
+// sp[(l-1) W + i] = min col[i .. i + 2^l - 1].
+template <typename Sync>
+__device__ __forceinline__ void sparse_build(const uint64_t *col, uint64_t *sp, int W, int id, int n, Sync sync)
+{
+    const uint64_t *below = col;
+    for (int half = 1; 2 * half <= W; half *= 2) {
+        for (int i = id; i + 2 * half <= W; i += n) sp[i] = umin64(below[i], below[i + half]);
+        below = sp;
+        sp += W;
+        sync();
+    }
+}
+
+// min col[s .. r] (s <= r)
+__device__ __forceinline__ uint64_t range_min(const uint64_t *col, const uint64_t *sp, int W, int s, int r)
+{
+    const int l = 31 - __clz(r - s + 1);
+    const uint64_t *t = l ? sp + (size_t)(l - 1) * W : col;
+    return umin64(t[s], t[r - (1 << l) + 1]);
+}
+
+// min over s in [0, r] of max(col[s], cost(s)), cost non-increasing in s.
+template <typename Cost>
+__device__ __forceinline__ uint64_t crossover(const uint64_t *col, const uint64_t *sp, int W, int r, Cost cost)
+{
+    int lo = 0, hi = r + 1;
+    uint64_t left = kInfKey, right = kInfKey;     // cost just before the crossover, range minimum at it
+    while (lo < hi) {
+        const int mid = (lo + hi) >> 1;
+        const uint64_t c = cost(mid), q = range_min(col, sp, W, mid, r);
+        if (q >= c) { hi = mid; right = q; }
+        else { lo = mid + 1; left = c; }
+    }
+    return umin64(left, right);
+}
+
+__global__ void __launch_bounds__(32 * kLayeredWarps) dp_layered_kernel(Dims dm, Tables tb, DevPop pop, EvalOut out,
+                                                                        WorkList wl, SlotInfo si, SplitOut so)
 {
     extern __shared__ __align__(16) unsigned char lsm[];
     __shared__ unsigned s_item;
     __shared__ int s_done, s_mu;
+    __shared__ unsigned long long s_V0, s_V;
     __shared__ double s_T, s_L;
     const int K = dm.K, M = dm.M, N = dm.N;
-    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, NW = blockDim.x >> 5;
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const uint64_t INF = kInfKey;
     const unsigned n_items = wl.ctrl[kCtrlEnd];
     const size_t NN = (size_t)N * N;
@@ -882,165 +941,211 @@ __global__ void __launch_bounds__(128) dp_layered_kernel(Dims dm, Tables tb, Dev
         const int role = (int)((item >> 7) & 1u);
         const bool sweep = (item >> 6) & 1u;
         const int v = role ? code + 1 : 0;
+        const size_t sv = gk * dm.V + code;
         const int W = N - m + 1;
+        const size_t levels = sparse_levels((unsigned)W);
         uint64_t *F = reinterpret_cast<uint64_t *>(lsm);          // [m][W] prefix (then mu*'s) columns
         uint64_t *G = F + (size_t)m * W;                          // [m][W] suffix columns
-        uint64_t *Vmu = G + (size_t)m * W;                        // [m]
+        uint64_t *sp = G + (size_t)m * W;                         // [warps][levels][W] sparse tables
+        uint64_t *Vmu = sp + kLayeredWarps * levels * W;          // [m]
         uint64_t *tk = Vmu + m;                                   // [m] tk[k] = link k-1 -> k (0-based)
         int *nk = reinterpret_cast<int *>(tk + m);                // [m]
         uint16_t *devs = reinterpret_cast<uint16_t *>(nk + m);    // [m]
+        uint64_t *spw = sp + (size_t)wid * levels * W;            // this warp's table
         const double *lc = tb.lcost + (size_t)v * M * 2 * NN;
         for (int k = tid; k < m; k += blockDim.x) devs[k] = pop.perm[(size_t)g * M + off + k];
         __syncthreads();
         for (int k = tid; k < m; k += blockDim.x)
             tk[k] = k ? dkey(tb.tau[((size_t)v * M + devs[k - 1]) * M + devs[k]]) : 0ull;
-        // l_k(j .. j+n-1) (k 0-based), with the head when mf
-        auto cost = [&](int k, int j, int n, int mf) -> uint64_t {
-            return dkey(lc[((size_t)devs[k] * 2 + mf) * NN + (size_t)j * N + (n - 1)]);
-        };
-        __syncthreads();
+        // device k's (0-based) times: entry [j][n - 1] of blocks j .. j+n-1, with the head when mf
+        auto rows = [&](int k, int mf) -> const double * { return lc + ((size_t)devs[k] * 2 + mf) * NN; };
         unsigned long long probes = 0;
-        // ---- prefix columns F_1..F_m (no master)
-        for (int r = tid; r < W; r += blockDim.x) F[r] = cost(0, 0, r + 1, 0);
-        __syncthreads();
-        for (int k = 2; k <= m; ++k) {
-            const uint64_t *prev = F + (size_t)(k - 2) * W;
-            uint64_t *cur = F + (size_t)(k - 1) * W;
-            const uint64_t t = tk[k - 1];
-            for (int r = tid; r < W; r += blockDim.x) {
-                uint64_t best = INF;
-                for (int s2 = 0; s2 <= r; ++s2)
-                    best = umin64(best, umax64(umax64(prev[s2], cost(k - 1, s2 + k - 1, r - s2 + 1, 0)), t));
-                cur[r] = best;
-                probes += (unsigned long long)(r + 1);
-            }
-            __syncthreads();
+        for (int r = tid; r < W; r += blockDim.x) {
+            F[r] = dkey(rows(0, 0)[r]);
+            G[(size_t)(m - 1) * W + r] = dkey(rows(m - 1, 0)[(size_t)(N - 1 - r) * N + r]);
         }
-        // ---- suffix columns G_m..G_2: devices k..m hold the last b + m - k + 1 blocks
-        for (int b = tid; b < W; b += blockDim.x) G[(size_t)(m - 1) * W + b] = cost(m - 1, N - 1 - b, b + 1, 0);
         __syncthreads();
-        for (int k = m - 1; k >= 2; --k) {
-            const uint64_t *nxt = G + (size_t)k * W;
-            uint64_t *cur = G + (size_t)(k - 1) * W;
-            const uint64_t t = tk[k];
-            for (int b = tid; b < W; b += blockDim.x) {
-                const int j0 = N - (b + m - k + 1);
-                uint64_t best = INF;
-                for (int t2 = 0; t2 <= b; ++t2)
-                    best = umin64(best, umax64(umax64(cost(k - 1, j0, t2 + 1, 0), nxt[b - t2]), t));
-                cur[b] = best;
-                probes += (unsigned long long)(b + 1);
+        // cell r of device k's prefix column (0-based k >= 1), from column k - 1
+        auto prefix_cell = [&](const uint64_t *prev, const uint64_t *s_prev, int k, int mf, int r) -> uint64_t {
+            const double *t = rows(k, mf);
+            return umax64(crossover(prev, s_prev, W, r, [&](int s) {
+                              ++probes;
+                              return dkey(t[(size_t)(s + k) * N + (r - s)]);
+                          }), tk[k]);
+        };
+        // ---- prefix columns 1..m-2 on warps 0-1, suffix columns m-2..1 on warps 2-3
+        if (wid < 2) {
+            auto join = [] { bar_named(1, 64); };
+            for (int k = 1; k <= m - 2; ++k) {
+                const uint64_t *prev = F + (size_t)(k - 1) * W;
+                sparse_build(prev, sp, W, tid, 64, join);
+                for (int r = tid; r < W; r += 64) F[(size_t)k * W + r] = prefix_cell(prev, sp, k, 0, r);
+                join();
             }
-            __syncthreads();
-        }
-        // ---- masters: a warp per master, lanes over the (a, b) splits
-        for (int mu = wid + 1; mu <= m; mu += NW) {
-            const uint64_t *Fp = mu >= 2 ? F + (size_t)(mu - 2) * W : nullptr;
-            const uint64_t *Gs = mu <= m - 1 ? G + (size_t)mu * W : nullptr;
-            uint64_t lk = 0;
-            if (mu >= 2) lk = umax64(lk, tk[mu - 1]);
-            if (mu <= m - 1) lk = umax64(lk, tk[mu]);
-            uint64_t best = INF;
-            const int amax = mu >= 2 ? W - 1 : 0;
-            for (int a = 0; a <= amax; ++a) {
-                const uint64_t fa = Fp ? Fp[a] : 0ull;
-                if (fa >= best) continue;                       // cannot lower the minimum
-                const int bmax = mu <= m - 1 ? W - 1 - a : 0;
-                for (int b = lane; b <= bmax; b += 32) {
-                    const uint64_t gb = Gs ? Gs[b] : 0ull;
-                    const uint64_t h = cost(mu - 1, (mu - 1) + a, W - a - b, 1);
-                    best = umin64(best, umax64(umax64(fa, gb), umax64(h, lk)));
+        } else {
+            auto join = [] { bar_named(2, 64); };
+            uint64_t *s2 = sp + 2 * levels * W;
+            for (int k = m - 2; k >= 1; --k) {
+                const uint64_t *next = G + (size_t)(k + 1) * W;
+                sparse_build(next, s2, W, tid - 64, 64, join);
+                const double *t = rows(k, 0);
+                for (int b = tid - 64; b < W; b += 64) {
+                    const double *row = t + (size_t)(N - (b + m - k)) * N;   // its first block
+                    G[(size_t)k * W + b] = umax64(crossover(next, s2, W, b, [&](int u) {
+                                                      ++probes;
+                                                      return dkey(row[b - u]);
+                                                  }), tk[k + 1]);
                 }
-                probes += (unsigned long long)((bmax + 1 + 31 - lane) / 32);
+                join();
+            }
+        }
+        __syncthreads();
+        // ---- the master-free optimum F_m[W-1], over every split
+        if (wid == 0) {
+            uint64_t x = m == 1 ? dkey(rows(0, 0)[N - 1]) : INF;
+            if (m >= 2) {
+                const uint64_t *prev = F + (size_t)(m - 2) * W;
+                const double *t = rows(m - 1, 0);
+                for (int s = lane; s < W; s += 32) {
+                    x = umin64(x, umax64(prev[s], dkey(t[(size_t)(s + m - 1) * N + (W - 1 - s)])));
+                    ++probes;
+                }
+            }
+#pragma unroll
+            for (int o = 16; o; o >>= 1) x = umin64(x, __shfl_xor_sync(0xFFFFFFFFu, x, o));
+            if (lane == 0) {
+                s_V0 = umax64(x, tk[m - 1]);
+                s_V = INF;
+                s_mu = 0;
+            }
+        }
+        __syncthreads();
+        // ---- masters, four at a time in index order, a warp each, lanes over b
+        for (int mu0 = 1; mu0 <= m && s_V > s_V0; mu0 += kLayeredWarps) {   // (uniform: s_V changes below only)
+            const int mu = mu0 + wid;
+            uint64_t best = INF;
+            if (mu <= m) {
+                const uint64_t *Fp = F + (size_t)(mu >= 2 ? mu - 2 : 0) * W;
+                const uint64_t *Gs = G + (size_t)(mu <= m - 1 ? mu : m - 1) * W;
+                const double *h = rows(mu - 1, 1);
+                uint64_t lk = 0;
+                if (mu >= 2) lk = umax64(lk, tk[mu - 1]);
+                if (mu <= m - 1) lk = umax64(lk, tk[mu]);
+                if (mu >= 2) sparse_build(Fp, spw, W, lane, 32, [] { __syncwarp(); });
+                for (int b = lane; b < (mu <= m - 1 ? W : 1); b += 32) {
+                    const uint64_t gb = mu <= m - 1 ? Gs[b] : 0ull;
+                    if (gb >= best) continue;                     // cannot lower the minimum
+                    uint64_t x;
+                    if (mu == 1) {
+                        x = dkey(h[W - b - 1]);
+                        ++probes;
+                    } else {
+                        x = crossover(Fp, spw, W, W - 1 - b, [&](int a) {
+                            ++probes;
+                            return dkey(h[(size_t)(mu - 1 + a) * N + (W - a - b - 1)]);
+                        });
+                    }
+                    best = umin64(best, umax64(x, gb));
+                }
 #pragma unroll
                 for (int o = 16; o; o >>= 1) best = umin64(best, __shfl_xor_sync(0xFFFFFFFFu, best, o));
+                if (lane == 0) Vmu[mu - 1] = umax64(best, lk);
             }
-            if (lane == 0) Vmu[mu - 1] = best;
+            __syncthreads();
+            if (tid == 0)                                         // the smallest master with the least value
+                for (int q = mu0; q < mu0 + kLayeredWarps && q <= m; ++q)
+                    if (Vmu[q - 1] < s_V) { s_V = Vmu[q - 1]; s_mu = q; }
+            __syncthreads();
         }
-        __syncthreads();
-        if (tid == 0) {                                           // the smallest master with the least value
-            int mus = 1;
-            for (int mu = 2; mu <= m; ++mu)
-                if (Vmu[mu - 1] < Vmu[mus - 1]) mus = mu;
-            s_mu = mus;
-        }
-        __syncthreads();
         const int mus = s_mu;
-        const uint64_t V = Vmu[mus - 1];
+        const uint64_t V = s_V;
+        __syncthreads();                                          // (s_mu and s_V are the next run's)
         if (V == INF) {                                           // no partition (memory)
             if (tid == 0 && !role) {                              // a prefill result that does not exist
-                const size_t sv = gk * dm.V + code;
                 so.T[sv] = keyd(kInfKey);
                 so.L[sv] = keyd(kInfKey);
             }
-            if (lane == 0) atomicAdd(&out.stats[kStProbes], probes);
+            {                                                         // every thread's probes
+                unsigned p = (unsigned)probes;
+                p = __reduce_add_sync(0xFFFFFFFFu, p);
+                if (lane == 0) atomicAdd(&out.stats[kStProbes], (unsigned long long)p);
+            }
             if (tid == 0) atomicAdd(&out.stats[kStDpRuns], 1ull);
             __syncthreads();
             continue;
         }
         // ---- mu*'s prefix columns from column mu* on (the head at mu*)
-        for (int k = mus; k <= m; ++k) {
-            uint64_t *cur = F + (size_t)(k - 1) * W;
-            const int mf = k == mus;
-            if (k == 1) {
-                for (int r = tid; r < W; r += blockDim.x) cur[r] = cost(0, 0, r + 1, 1);
+        for (int k = mus - 1; k <= m - 2; ++k) {
+            uint64_t *cur = F + (size_t)k * W;
+            const int mf = k == mus - 1;
+            if (k == 0) {
+                for (int r = tid; r < W; r += blockDim.x) cur[r] = dkey(rows(0, 1)[r]);
             } else {
-                const uint64_t *prev = F + (size_t)(k - 2) * W;
-                const uint64_t t = tk[k - 1];
-                for (int r = tid; r < W; r += blockDim.x) {
-                    uint64_t best = INF;
-                    for (int s2 = 0; s2 <= r; ++s2)
-                        best = umin64(best, umax64(umax64(prev[s2], cost(k - 1, s2 + k - 1, r - s2 + 1, mf)), t));
-                    cur[r] = best;
-                    probes += (unsigned long long)(r + 1);
-                }
+                const uint64_t *prev = F + (size_t)(k - 1) * W;
+                sparse_build(prev, sp, W, tid, blockDim.x, [] { __syncthreads(); });
+                for (int r = tid; r < W; r += blockDim.x) cur[r] = prefix_cell(prev, sp, k, mf, r);
             }
             __syncthreads();
         }
         // ---- traceback (warp 0): the smallest split attaining each cell's value
         if (wid == 0) {
             int r = W - 1;
-            for (int k = m; k >= 2; --k) {
-                const uint64_t D = F[(size_t)(k - 1) * W + r];
-                const uint64_t *prev = F + (size_t)(k - 2) * W;
-                const uint64_t t = tk[k - 1];
-                const int mf = k == mus;
-                int sp = -1;
-                for (int base = 0; base <= r && sp < 0; base += 32) {
-                    const int s2 = base + lane;
-                    const bool hit = s2 <= r && umax64(umax64(prev[s2], cost(k - 1, s2 + k - 1, r - s2 + 1, mf)), t) == D;
+            uint64_t D = V;
+            for (int k = m - 1; k >= 1; --k) {
+                const uint64_t *prev = F + (size_t)(k - 1) * W;
+                const double *t = rows(k, k == mus - 1);
+                int split = -1;
+                for (int base = 0; base <= r && split < 0; base += 32) {
+                    const int s = base + lane;
+                    const bool hit = s <= r && umax64(umax64(prev[s], dkey(t[(size_t)(s + k) * N + (r - s)])), tk[k]) == D;
                     const unsigned bal = __ballot_sync(0xFFFFFFFFu, hit);
-                    if (bal) sp = base + __ffs(bal) - 1;
+                    if (bal) split = base + __ffs(bal) - 1;
                 }
-                if (sp < 0) {                                     // cannot happen: D is attained
-                    sp = 0;
+                if (split < 0) {                                  // cannot happen: D is attained
+                    split = 0;
                     if (lane == 0) atomicAdd(&out.stats[kStDeviceErrors], 1ull);
                 }
-                if (lane == 0) nk[k - 1] = r - sp + 1;
-                r = sp;
+                if (lane == 0) nk[k] = r - split + 1;
+                r = split;
+                D = prev[r];
             }
             if (lane == 0) nk[0] = r + 1;
             __syncwarp();
-            // stage and link times of the partition in pipeline order
-            if (lane == 0) {
-                double lam = 0.0;
-                uint64_t tmax = 0;
-                int j = 0;
-                for (int k = 0; k < m; ++k) {
-                    const double lk = keyd(cost(k, j, nk[k], k == mus - 1));
-                    const double tl = k ? keyd(tk[k]) : 0.0;
-                    if (k == 0) lam = lk;
-                    else { lam = lam + tl; lam = lam + lk; }
-                    tmax = umax64(tmax, umax64(dkey(lk), dkey(tl)));
-                    j += nk[k];
+            // stage and link times of the partition, lane k holds device k; Lambda in pipeline order
+            double lam = 0.0;
+            uint64_t tmax = 0;
+            int first = 0;                                        // first block of device `base`
+            for (int base = 0; base < m; base += 32) {
+                const int k = base + lane;
+                const int n = k < m ? nk[k] : 0;
+                int incl = n;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const int y = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+                    if (lane >= o) incl += y;
                 }
+                double l = 0.0, t = 0.0;
+                if (k < m) {
+                    l = rows(k, k == mus - 1)[(size_t)(first + incl - n) * N + n - 1];
+                    if (k) t = keyd(tk[k]);
+                    tmax = umax64(tmax, umax64(dkey(l), dkey(t)));
+                }
+                for (int q = 0; q < 32 && base + q < m; ++q) {
+                    const double lq = __shfl_sync(0xFFFFFFFFu, l, q), tq = __shfl_sync(0xFFFFFFFFu, t, q);
+                    if (base + q == 0) lam = lq;
+                    else { lam = lam + tq; lam = lam + lq; }
+                }
+                first += __shfl_sync(0xFFFFFFFFu, incl, 31);
+            }
+#pragma unroll
+            for (int o = 16; o; o >>= 1) tmax = umax64(tmax, __shfl_xor_sync(0xFFFFFFFFu, tmax, o));
+            if (lane == 0) {
                 s_L = lam;
                 s_T = keyd(tmax);
                 s_done = (!role) || lam <= dm.lam_max;            // 1.0 / lam >= Min_TPS
             }
         }
         __syncthreads();
-        const size_t sv = gk * dm.V + code;
         if (s_done) {
             int16_t *lay_out = so.layers + ((size_t)g * dm.V + code) * M + off;
             for (int k = tid; k < m; k += blockDim.x) lay_out[k] = (int16_t)nk[k];
@@ -1054,7 +1159,11 @@ __global__ void __launch_bounds__(128) dp_layered_kernel(Dims dm, Tables tb, Dev
         } else if (tid == 0 && !role) {
             so.T[sv] = keyd(kInfKey);
         }
-        if (lane == 0) atomicAdd(&out.stats[kStProbes], probes);
+        {                                                         // every thread's probes
+            unsigned p = (unsigned)probes;
+            p = __reduce_add_sync(0xFFFFFFFFu, p);
+            if (lane == 0) atomicAdd(&out.stats[kStProbes], (unsigned long long)p);
+        }
         if (tid == 0) {
             atomicAdd(&out.stats[kStDpRuns], 1ull);
             atomicAdd(&out.stats[kStCells], (unsigned long long)(2 * m + (m - mus + 1)) * W + m);
