@@ -13,9 +13,9 @@ CUDA events on the engine's stream, L2 flushed (256 MB write) between steps.
 e2e: the same metric through the C ABI with pinned host buffers: each step is
 one e2_run_generation_io call that uploads the population, evaluates, steps,
 and reads fitness and the next population back, synchronising once.
-roofline: the DP_Pipe kernel (both of its launches where the replica sizes
-form two shared-memory classes) against the integer issue rate of its own
-instruction mix, measured in the same run by e2_probe_int_rate.
+roofline: the DP_Pipe kernel (both of its launches where replicas of more than
+32 devices can occur) against the integer issue rate of a min / max / compare /
+select / add mix, measured in the same run by e2_probe_int_rate.
 configs: the other four workloads, device-timed the same way (the 256-device
 one over 200 back-to-back generations: generations per second).
 --impl reference times the CPU oracle on the host cores.  Under torchrun each
@@ -48,22 +48,20 @@ UNIT = "genomes/s"
 WORKLOAD = "c4"
 OTHER_CONFIGS = ("c1_tiny", "c2", "c3", "c5")
 L2_FLUSH_BYTES = 256 << 20
-# algorithmic int32 operations per unit of DP work, the rule of about five
-# integer operations per examined candidate: per crossover probe (of a
-# bisection, or the one-step advance to the next cell) two key loads, a
-# compare, a select or step and an index update; per DP cell a min, a max
-# with the link key, two guards and a store.  Probes and cells are the
-# kernel's own tallies (e2_get_stats).
+# algorithmic int32 operations per unit of DP work: per cost-row entry read (a
+# threshold compare, a count step, an index update, a min and a max of the
+# threshold's neighbours), and per stage settled (its cap, the prefix's excess,
+# its link, its count, a store).  Entries and stages are the kernel's own
+# tallies (e2_get_stats); the warp reductions and the estimate are not counted.
 OPS_PER_PROBE = 5
 OPS_PER_CELL = 5
 INT32_LANES_PER_SM = 128
 # dram__bytes_read.sum + dram__bytes_write.sum of the two DP launches of one
-# generation at the default workload (class 0: 30.21 + 9.29 MB, class 1:
-# 24.55 + 5.46 MB), from the ncu capture in profiles/; cold (ncu flushes the
-# caches before each launch), so it counts the L2-resident order-key rows
-# again
-DP_TRAFFIC_BYTES = 69_413_632
-DP_TRAFFIC_SOURCE = "profiles/dp_eval_c4_gen2.md (dram read+write, both DP launches of one generation, cold)"
+# evaluation at the default workload, from the ncu capture in profiles/; cold
+# (ncu flushes the caches before each launch), so it counts the L2-resident
+# tables again
+DP_TRAFFIC_BYTES = 48_986_688
+DP_TRAFFIC_SOURCE = "profiles/dp_order_c4.md (dram read+write, both DP launches of one evaluation, cold)"
 
 
 def parse():
@@ -513,14 +511,14 @@ def run_ours(args):
                                      sum(s["dp_runs_small"] for s in stats) / n]},
             "replicas_per_step": sum(s["replicas"] for s in stats) / n,
             "roofline": {"bound": "alu",
-                         "kernel": "dp_eval_kernel (DP_Pipe; both launches, timed by events around them)",
+                         "kernel": "dp_order_kernel (DP_Pipe; both launches, timed by events around them)",
                          "achieved": achieved / 1e12, "peak": peak_ops / 1e12 if peak_ops else None,
                          "unit": "Tops/s (int32)", "frac": achieved / peak_ops if peak_ops else None,
                          "traffic": DP_TRAFFIC_BYTES if args.config == WORKLOAD else None,
                          "traffic_source": DP_TRAFFIC_SOURCE,
-                         "per_unit": f"{OPS_PER_PROBE} int32 ops per crossover probe + {OPS_PER_CELL} per DP cell "
-                                     f"(about five per examined candidate); probes {m['probes']:.4g} and cells "
-                                     f"{m['cells']:.4g} per step, the kernel's own tallies",
+                         "per_unit": f"{OPS_PER_PROBE} int32 ops per cost-row entry read + {OPS_PER_CELL} per stage settled; "
+                                     f"entries {m['probes']:.4g} and stages {m['cells']:.4g} per step, the kernel's "
+                                     f"own tallies",
                          "peak_source": "measured in this run: e2_probe_int_rate kind 2 (min, max, compare, "
                                         "select, add on independent chains at full occupancy), best of 5",
                          "peak_nominal": nominal / 1e12,

@@ -104,9 +104,9 @@ typedef struct {
  * non-decreasing).  The stage of blocks j..i then costs PF[v][i+1]-PF[v][j]
  * flops (+ the head on the master), likewise bytes and memory.  A stage's cost
  * depends on where it starts, and the best bottleneck of a prefix is no longer
- * monotone in its length, so these contexts run the plain scan over every
- * split (Alg. 1's recurrence, with the masters factored through prefix and
- * suffix tables) instead of the identical-block kernel.  Needs
+ * monotone in its length, so these contexts run Alg. 1's recurrence column by
+ * column (a bisection per cell on range minima, the masters factored through
+ * prefix and suffix tables) instead of the identical-block kernel.  Needs
  * e2_workspace_bytes_ex(..., E2_WS_LAYERED), N <= E2_MAX_LAYERED_BLOCKS, and
  * no GPU-CPU offload (mem_cpu NULL or all zero).  blk_* must still hold valid
  * values (they bound the range checks; the largest block's work is a good
@@ -212,27 +212,27 @@ typedef struct {
     uint64_t genomes;           /* genomes evaluated                           */
     uint64_t replicas;          /* replicas evaluated (sum of R)                */
     uint64_t dp_runs;           /* DP_Pipe runs that reached the recurrence     */
-    uint64_t dp_cells;          /* DP cells D_mu(i,k) computed                  */
-    uint64_t dp_probes;         /* split-point probes made: a bisection for the
-                                   first cell of each thread's span of a column,
-                                   one probe for each further cell              */
+    uint64_t dp_cells;          /* stages settled: the devices of each run (per-layer
+                                   profiles: DP cells D_mu(i,k) computed)       */
+    uint64_t dp_probes;         /* cost-row entries read to find thresholds and
+                                   counts (per-layer profiles: by the bisections
+                                   of the cells)                                */
     uint64_t paper_candidates;  /* (mu,k,i,j) candidates Alg. 1 would examine   */
     uint64_t prechecked;        /* variants rejected by the memory count check
                                    (over each replica's whole sweep)            */
     uint64_t served;            /* replicas that can serve                      */
     uint64_t tps_pruned;        /* decode variants a latency lower bound proved
                                    to miss Min_TPS (their DP is skipped)        */
-    uint64_t dp_runs_small;     /* of dp_runs, those of the second DP launch:
-                                   the small replica sizes, run with
-                                   more runs in flight per SM, four warps per
-                                   run or one (0 where that raises no occupancy
-                                   and one launch runs them all)                */
+    uint64_t dp_runs_small;     /* of dp_runs, those of the second DP launch: the
+                                   replicas with several devices per lane (more
+                                   than 32), or on large populations of smaller
+                                   fleets those of more than 8 devices          */
     uint64_t dp_launches;       /* DP kernel launches per evaluation (1 or 2;
                                    fixed at e2_create)                          */
     uint64_t dp_ctas;           /* persistent CTAs of the first DP launch       */
     uint64_t dp_smem;           /* and its dynamic shared memory per CTA (B)    */
     uint64_t dp_ctas_small;     /* the same for the second launch (0: none)     */
-    uint64_t dp_smem_small;     /* (per run: per warp when a warp runs one)     */
+    uint64_t dp_smem_small;
     uint64_t launches;          /* kernels this context has launched since
                                    e2_create, cumulative (a recorded generation
                                    counts its kernel nodes per replay)          */
@@ -245,9 +245,8 @@ typedef struct {
                                    partition, or a traceback found no split
                                    attaining its cell); nonzero makes
                                    e2_get_stats return E2_EDEVICE               */
-    uint64_t dp_runs_per_cta_small; /* runs in flight per CTA of the second launch:
-                                   1 (four warps per run) or 4 (a warp each; 0:
-                                   no second launch)                            */
+    uint64_t dp_runs_per_cta_small; /* runs in flight per CTA of the second launch,
+                                   a warp each (0: no second launch)            */
 } e2_stats;
 
 typedef struct e2_ctx e2_ctx;
@@ -352,7 +351,7 @@ int e2_get_results(e2_ctx *ctx, double *fitness_out, const e2_partitions *parts)
  * use (one per population buffer, recorded on a private stream and again when
  * the timing events of e2_set_timing_events change) and afterwards replays it
  * on its stream, setting only the new seed and generation: one launch instead
- * of nine (two memsets and seven kernels).  If recording fails the calls are
+ * of ten or more.  If recording fails the calls are
  * issued one by one.
  * E2_EINVAL for a NULL context; E2_ECUDA on a CUDA failure. */
 int e2_run_generation(e2_ctx *ctx, uint64_t seed, uint32_t generation);

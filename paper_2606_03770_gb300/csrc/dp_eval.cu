@@ -1,48 +1,15 @@
-// dp_eval.cu -- population fitness: DP_Pipe per replica (Alg. 1, Eq. 1-2),
-// the decode batch sweep (Alg. 2), and the objective (Eq. 3-5).
+// dp_eval.cu -- population fitness around the DP: the pre-pass, the work list,
+// the DP of models with several block types, the objective (Eq. 3-5) and the
+// launch sequence of an evaluation.
 //
-// Work is split over four or five kernels per evaluation: a pre-pass that
-// decides, per (genome, replica slot, variant), whether a DP run can matter
-// (memory and latency bounds) and counts and orders the surviving runs; a
-// scatter that writes them into one work list; persistent DP CTAs that drain
-// the list (two launches where the replica sizes fall into two shared-memory
-// classes); and a warp per genome (a block per genome for a wide role search)
-// that picks each replica's answer and scores the genome.
-//
-// With identical blocks (Sec. 3.2: the premise that lets the paper fix the
-// node order) a stage's time depends only on its device, its block count n and
-// whether it is the master, so the replica's costs fit in two rows per device,
-// l_k(n) and l_k^head(n), staged in shared memory as 32-bit order keys (exact
-// ranks of the float64 times, built in ranks.cu).
-//
-// Band form of Eq. 1.  Device k can take at most W = N - m + 1 blocks.  Let
-// D_k[r] = DP(i = r + k - 1, k), r in [0, W).  Then
-//     D_1[r] = l_1(r + 1)                                         (Eq. 2)
-//     D_k[r] = min_{s in [0, r]} max(D_{k-1}[s], l_k(r - s + 1), tau_k)   (Eq. 1)
-// where s = j - (k - 1) indexes the split.  D_{k-1}[s] is non-decreasing in s
-// (one more block never lowers the best bottleneck when blocks are identical)
-// and l_k(r - s + 1) is non-increasing in s, so max(D_{k-1}[s], l_k(.)) falls
-// then rises: its minimum sits at the crossover s0 = first s with
-// D_{k-1}[s] >= l_k(r - s + 1) and equals min(l_k(r - s0 + 2), D_{k-1}[s0]).
-// A bisection over s finds s0, so a cell costs O(log W) probes instead of the
-// O(W) scan, with bit-identical values (min and max are exact); and the
-// crossover of cell r + 1 is that of cell r or one more, so a thread that owns
-// a span of cells bisects only for the first (dp_span).
-//
-// Tie rule.  The oracle keeps the smallest split j attaining the minimum.  The
-// set of minimisers is {s : D_{k-1}[s] <= D and l_k(r-s+1) <= D} (tau <= D
-// always), an interval whose first element is the first s with
-// l_k(r-s+1) <= D.  So the traceback needs only the cell value D and the cost
-// row: n_k = largest n <= r + 1 with l_k(n) <= D.
-//
-// Masters.  Alg. 1 reruns the whole table for every master mu.  Here the
-// master-free prefix columns F_k (devices 1..k) and suffix columns G_k
-// (devices k..m) are computed once per run, and each master's bottleneck
-// follows from F_{mu-1}, G_{mu+1} and the master's head row (dp_eval_body,
-// step 4).  mu* = the smallest mu with the least bottleneck (the oracle's
-// first-wins argmin); its columns are recomputed for the traceback.
+// An evaluation is a pre-pass that decides, per (genome, replica slot) and
+// role, which decode batches (or whether the prefill run) can matter (memory
+// and latency bounds); a count and a scatter that put the surviving work into
+// one list, by replica size; the DP (dp_order.cu for identical blocks,
+// dp_layered_kernel here for blocks of several types), persistent warps or
+// CTAs over the list; and a warp per genome (a block per genome for a wide
+// role search) that scores the genome.
 #include "e2ga_internal.cuh"
-#include "dp_span.cuh"
 
 namespace e2 {
 
@@ -58,32 +25,8 @@ __device__ __forceinline__ unsigned long long paper_candidates(int m, int N)
     return (unsigned long long)m * ((unsigned long long)N + s);
 }
 
-// Probes of one column of W cells split into contiguous spans over T = 32,
-// 64 or 128 threads (index 0, 1, 2): per span the bisection of its first cell
-// (floor(log2(r + 1)) + 1 probes for cell r), then one per further cell.
-__constant__ uint16_t c_span_probes[3][E2_MAX_BLOCKS + 1];
-
-}  // namespace
-
-// Shared-memory bytes for the largest replica the problem allows, with keys of
-// key_bytes bytes.
-size_t dp_smem_bytes(int M, int N, int threads, int key_bytes, bool spill)
-{
-    size_t best = 0;
-    const int mmax = M < N ? M : N;
-    for (int m = 1; m <= mmax; ++m) {
-        const size_t bytes = dp_item_bytes(m, N, threads / 32, key_bytes, spill);
-        if (bytes > best) best = bytes;
-    }
-    return best;
-}
-
-namespace {
-
-__device__ __forceinline__ void bar_named(int id, int nthreads)
-{
-    asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(nthreads) : "memory");
-}
+// A warp's sum, in every lane.
+__device__ __forceinline__ int warp_sum(int x) { return __reduce_add_sync(0xFFFFFFFFu, x); }
 
 }  // namespace
 
@@ -91,23 +34,18 @@ __device__ __forceinline__ void bar_named(int id, int nthreads)
 // up to 16 so that every warp's arrays start aligned).
 __host__ __device__ __forceinline__ size_t variant_stride(int mcap) { return ((size_t)mcap * 18 + 15) & ~(size_t)15; }
 
-// Per slot: slots with nothing to run get their outputs here (empty slots,
-// more devices than blocks, no variant left by the pre-pass).  Every other
-// slot contributes one work item per variant to run; items are ordered by
-// level (the variant's rank among its replica's variants, largest batch
-// first), then by work size (m * W, log scale), largest first.  A replica's
-// smaller batches thus come after every replica's larger ones, by which time
-// the larger batch has usually been decided: a variant below an accepted one
-// is skipped, as the sequential sweep of Alg. 2 would.  The items of DP class
-// 0 (size bit 4 clear) take the upper half of the bins, which the descending
-// scan places first; a replica's items all share its class.
-__device__ __forceinline__ int item_bin(int level, int size)
+// Bin of a replica of m devices in the work list: with two DP classes, the
+// sizes up to dp_split (class 0) take bins 0..31 and the larger ones bins
+// 32..63; larger first within a class.
+__device__ __forceinline__ uint32_t size_bin(const Dims &dm, int m)
 {
-    const int lv = level < 63 ? level : 63;
-    return ((size >> 4) ? 0 : kOrderBins) + (63 - lv) * kSizeBins + (size & (kSizeBins - 1));
+    constexpr int half = kListBins / 2;
+    if (!dm.dp_split) return (uint32_t)(kListBins - 1 - (m - 1) * kListBins / dm.dp_mmax);
+    if (m <= dm.dp_split) return (uint32_t)(half - 1 - (m - 1) * half / dm.dp_split);
+    return (uint32_t)(kListBins - 1 - (m - dm.dp_split - 1) * half / (dm.dp_mmax - dm.dp_split));
 }
 
-// Pre-pass and work count, one warp per (genome, replica slot).  For each
+// Pre-pass, one warp per (genome, replica slot).  For each
 // variant of the replica (prefill: v = 0; decode: v = 1..b_max, bit v-1) the
 // warp decides whether a DP run can matter:
 //  * memory: with identical blocks a partition with master mu exists iff every
@@ -132,14 +70,12 @@ __device__ __forceinline__ int item_bin(int level, int size)
 // too; rounding can only keep a variant the exact bound would drop, which
 // costs a DP run and changes no result.  Other profiles test every batch from
 // the largest down, and the first that passes keeps the smaller ones.
-// The surviving variants form the slot's mask.  A replica with nothing to run
-// (more devices than blocks, no variant left) gets its outputs here, and the
-// genome's last replica writes those of its empty slots (a warp on an empty
-// slot does nothing else); the others count their work items into the
-// ordering bins, which bins_kernel then scans into starting offsets, class 0
-// first and heaviest first within a class.
+// The verdicts go into the slot's info word (SlotBits), with the bin of its
+// size in the work list's order.  A replica with nothing to run (more devices
+// than blocks, no variant left) gets its outputs here, and the genome's last
+// replica writes those of its empty slots.
 __global__ void __launch_bounds__(64, 20) slot_kernel(Dims dm, Tables tb, DevPop pop, SlotInfo si, EvalOut out,
-                                                  unsigned *ctrl)
+                                                       SplitOut so, VariantOut vo)
 {
     // per warp: device ids, capacities and per-block times of up to mcap devices
     extern __shared__ __align__(16) unsigned char vsm[];
@@ -155,8 +91,7 @@ __global__ void __launch_bounds__(64, 20) slot_kernel(Dims dm, Tables tb, DevPop
         const int m_c = sz[c];
         const uint64_t roles = pop.roles[g];
         const int s_lo = lane < c ? sz[lane] : 0, s_hi = lane + 32 < c ? sz[lane + 32] : 0;
-        uint64_t mask = 0;
-        unsigned long long n_pre = 0, n_tps = 0;
+        uint32_t info = 0;
         int m = 0, off = 0, role = 0;
         if (c < R) {
             m = m_c;
@@ -229,8 +164,8 @@ __global__ void __launch_bounds__(64, 20) slot_kernel(Dims dm, Tables tb, DevPop
                 const int prole = dm.role_search ? (pass == 0) : role;
                 const int nvar = prole ? dm.b_max : 1;
                 if (dm.layered) {                           // per-layer profiles: every variant runs (the
-                    if (dm.role_search && !prole) mask |= 1ull << dm.b_max;   // tests assume identical blocks)
-                    else mask |= nvar >= 64 ? ~0ull : ((1ull << nvar) - 1ull);
+                    if (prole) info |= (uint32_t)nvar | (uint32_t)nvar << kSlotMemShift;   // tests assume
+                    else info |= kSlotPrefill;                                          // identical blocks)
                     continue;
                 }
                 const bool bound = prole && dm.min_tps > 0.0;
@@ -265,558 +200,129 @@ __global__ void __launch_bounds__(64, 20) slot_kernel(Dims dm, Tables tb, DevPop
                     next = !dm.grows ? hi - 1 : lo < 0 ? 0 : (lo + hi) >> 1;
                 }
                 const int bs = tps ? lo : bm;               // largest variant both tests keep
-                n_pre += (unsigned long long)(nvar - 1 - bm);
-                n_tps += (unsigned long long)(bm - bs);
-                if (bs >= 0) {
-                    if (dm.role_search && !prole) mask |= 1ull << dm.b_max;
-                    else mask |= (2ull << bs) - 1ull;       // this variant and every smaller batch
-                }
+                if (prole) info |= kSlotDecTested | (uint32_t)(bs + 1) | (uint32_t)(bm + 1) << kSlotMemShift;
+                else info |= kSlotPreTested | (bs >= 0 ? kSlotPrefill : 0u);
+            }
+            info |= size_bin(dm, m) << kSlotBinShift;
+        }
+        // ---- the slot's verdicts, and the outputs of a replica that cannot serve (the
+        //      genome's last replica also writes those of its slots past R)
+        if (lane == 0) {
+            si.info[slot] = info;
+            if (dm.layered) vo.best[slot] = -1;
+        }
+        const bool dec = (info & kSlotDecMask) != 0, pre = (info & kSlotPrefill) != 0;
+        if (dm.role_search) {
+            if (lane == 0 && c < R) {
+                if (!pre) so.code[slot * 2] = -1;
+                if (!dec) so.code[slot * 2 + 1] = -1;
+            }
+        } else if (c < R && !dec && !pre) {
+            for (int k = lane; k < m_c; k += 32) out.layers[(size_t)g * M + off + k] = -1;
+            if (lane == 0) {
+                out.master[slot] = -1; out.bsel[slot] = -1;
+                out.T[slot] = keyd(kInfKey); out.L[slot] = keyd(kInfKey);
             }
         }
-        // ---- the slot's outputs or its work count (the genome's last replica
-        //      also writes those of its slots past R)
-        if (c < R && !mask)                                          // a replica that cannot serve
-            for (int k = lane; k < m; k += 32) out.layers[(size_t)g * M + off + k] = -1;
         if (c == R - 1)
             for (int e = R + lane; e < K; e += 32) {
                 const size_t es = (size_t)g * K + e;
                 out.master[es] = -1; out.bsel[es] = -1;
                 out.T[es] = keyd(kInfKey); out.L[es] = keyd(kInfKey);
             }
-        if (lane == 0 && c < R) {
-            si.mask[slot] = mask;
-            si.best[slot] = -1;
-            if (n_pre) atomicAdd(&out.stats[kStPrecheck], n_pre);
-            if (n_tps) atomicAdd(&out.stats[kStTpsPruned], n_tps);
-            if (!mask) {
-                out.master[slot] = -1; out.bsel[slot] = -1;
-                out.T[slot] = keyd(kInfKey); out.L[slot] = keyd(kInfKey);
-                if (c < R) {
-                    atomicAdd(&out.stats[kStReplicas], 1ull);
-                    const int runs = dm.role_search ? dm.b_max + 1 : (role ? dm.b_max : 1);
-                    if (m <= N) atomicAdd(&out.stats[kStPaper], runs * paper_candidates(m, N));
-                }
-            } else {
-                const int W = N - m + 1;
-                const int lg = (int)(1.0f * __log2f(1.0f + (float)m * (float)W));
-                const int cls = dp_item_bytes(m, N, dm.dp_warps, 4, false) <= dm.dp_small;   // class 1 never spills
-                const int size = (lg < kSizeBins - 1 ? lg : kSizeBins - 1) | cls << 4;
-                si.size[slot] = (uint8_t)size;
-                const int nv = __popcll(mask);
-                for (int lv = 0; lv < nv; ++lv) atomicAdd(&ctrl[item_bin(lv, size)], 1u);
-            }
-        }
     }
 }
 
-// The ordering bins' scan, after the pre-pass: with nb bins in use (class
-// 1's only where that class exists), lane t owns positions [t nb/32,
-// (t+1) nb/32) of the descending bin order (class 0's bins, then class 1's),
-// read eight at a time.  One warp.
-__global__ void bins_kernel(Dims dm, unsigned *ctrl)
+// The work list's order: class 0 (the first DP launch) before class 1, larger
+// replicas first within a class, in kListBins bins of equal size ranges.  The
+// count (bins_kernel) and the scatter split the slots into the same chunks,
+// one per block; a block of the scatter gets its place in each bin from the
+// counts of the blocks before it, so neither takes a global atomic.
+// With per-layer profiles (long runs, few of them) each batch of a decode sweep
+// is an item of its own, all replicas' largest batches first: by the time the
+// smaller ones come up the larger one has usually been decided.
+__device__ __forceinline__ int items_of(uint32_t info)
 {
-    const int lane = threadIdx.x & 31;
-    const int per = (dm.dp_small ? kAllBins : kOrderBins) / 32;
-    unsigned *own = ctrl + kAllBins - 1 - lane * per;              // own[-j] = position per lane + j
-    unsigned sum = 0;
-    for (int j = 0; j < per; j += 8) {
-        unsigned v[8];
-#pragma unroll
-        for (int q = 0; q < 8; ++q) v[q] = __ldcg(own - j - q);
-#pragma unroll
-        for (int q = 0; q < 8; ++q) sum += v[q];
-    }
-    unsigned incl = sum;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const unsigned x = __shfl_up_sync(0xFFFFFFFFu, incl, o);
-        if (lane >= o) incl += x;
-    }
-    unsigned base = incl - sum;
-    if (dm.dp_small && lane == kOrderBins / per) {               // class 0 holds the first kOrderBins positions
-        ctrl[kCtrlEnd] = base;
-        ctrl[kCtrlNext + 1] = base;
-    }
-    for (int j = 0; j < per; j += 8) {
-        unsigned v[8];
-#pragma unroll
-        for (int q = 0; q < 8; ++q) v[q] = __ldcg(own - j - q);
-#pragma unroll
-        for (int q = 0; q < 8; ++q) {
-            own[-j - q] = base;
-            base += v[q];
-        }
-    }
-    if (lane == 31) {
-        ctrl[kCtrlEnd + 1] = base;
-        if (!dm.dp_small) ctrl[kCtrlEnd] = ctrl[kCtrlNext + 1] = base;   // one class: class 1 is empty
-    }
+    return ((info & kSlotDecMask) != 0) + ((info & kSlotPrefill) != 0);
 }
 
-// Item lv of a slot (its variants from the largest batch down) goes to bin
-// item_bin(lv, size) as (slot << 8) | role << 7 | sweep << 6 | bit: role 1 =
-// decode; sweep 1 = an accepted result stops the smaller batches (every item
-// but the prefill run of a searched role).  The lanes of a warp whose items
-// share a bin take their positions with one atomic.
-__global__ void order_scatter_kernel(Dims dm, DevPop pop, SlotInfo si, WorkList wl)
+__device__ __forceinline__ uint32_t layered_bin(uint32_t info, int level)
 {
-    const int total = dm.P * dm.K, lane = threadIdx.x & 31;
-    const unsigned below = (1u << lane) - 1u;
-    for (int base = blockIdx.x * blockDim.x + (threadIdx.x & ~31); base < total; base += gridDim.x * blockDim.x) {
-        const int slot = base + lane;
-        uint64_t mask = 0;
-        int size = 0, grole = 0;
-        if (slot < total) {
-            const int g = slot / dm.K, c = slot - g * dm.K;
-            if (c < pop.nclus[g]) mask = si.mask[slot];
-            if (mask) {
-                size = si.size[slot];
-                grole = (int)((pop.roles[g] >> c) & 1ull);
-            }
-        }
-        for (int lv = 0; __any_sync(0xFFFFFFFFu, mask != 0); ++lv) {
-            int bit = 0, bin = -1;
-            if (mask) {
-                bit = 63 - __clzll((long long)mask);
-                mask &= ~(1ull << bit);
-                bin = item_bin(lv, size);
-            }
-            const unsigned peers = __match_any_sync(0xFFFFFFFFu, bin);
-            if (bin >= 0) {
-                const int leader = __ffs(peers) - 1;
-                unsigned at = 0;
-                if (lane == leader) at = atomicAdd(&wl.ctrl[bin], (unsigned)__popc(peers));
-                at = __shfl_sync(peers, at, leader);
-                const bool pre = dm.role_search ? bit == dm.b_max : !grole;
-                const uint64_t flags = (pre ? 0u : 0x80u) | (dm.role_search && pre ? 0u : 0x40u);
-                wl.items[at + __popc(peers & below)] = ((uint64_t)slot << 8) | flags | (uint64_t)bit;
-            }
-        }
-    }
+    return (uint32_t)min(level, 7) * 8u + (info >> kSlotBinShift) / (kListBins / 8);
 }
 
-// Persistent CTAs; each work item is one (genome, replica slot, variant) the
-// pre-pass kept, skipped if a larger batch of its replica was already
-// accepted.  Per item:
-//  1. stage the master-free cost rows l_k(n) and the link times as 32-bit
-//     order keys (exact ranks, see ranks.cu);
-//  2. masters the memory allows;
-//  3. prefix columns F_k (no master, devices 1..k) on warps 0-1 and suffix
-//     columns G_k (no master, devices k..m) on warps 2-3, concurrently, each
-//     thread a span of a column:
-//        F_k[r] = min_s max(F_{k-1}[s], l_k(r-s+1), tau_k)
-//        G_k[r] = min_s max(G_{k+1}[s], l_k(r-s+1), tau_{k+1})
-//  4. master mu: the prefix holds a extra blocks, the suffix b, the master
-//     W - a - b, so with H_mu[c] = min_{a+b=c} max(F_{mu-1}[a], G_{mu+1}[b])
-//        V_mu = max(tau_mu, tau_{mu+1}, min_c max(H_mu[c], l_mu^head(W - c)))
-//     (F_0 and G_{m+1} are the empty stage: 0 at index 0, +inf after); the
-//     warp fetches l_mu^head asynchronously while it builds H_mu;
-//  5. mu* = smallest mu with the least V_mu; its prefix columns D_k (master at
-//     mu*) are recomputed for the traceback;
-//  6. traceback with the smallest-split rule (n_k = number of n <= r+1 with
-//     l_k(n) <= D, counted with warp ballots); the bottleneck T (the largest
-//     stage or link time of the partition, equal to V) and Lambda (summed in
-//     pipeline order) in float64 from the stage and link tables; meanwhile
-//     warp 1 claims the next item.
-// Every comparison is between ranks of the same stage and link times the
-// oracle compares, so V, mu*, the partition, T and Lambda are bit-identical to
-// Alg. 1.
-template <typename Key, bool SPILL>
-__device__ __forceinline__ void dp_eval_body(const Dims &dm, const Tables &tb, const DevPop &pop, const EvalOut &out,
-                                             const WorkList &wl, const SlotInfo &si, const SplitOut &so, int cls)
+__global__ void __launch_bounds__(256) bins_kernel(Dims dm, SlotInfo si, unsigned *hist, unsigned long long *stats)
 {
-    extern __shared__ __align__(16) unsigned char smem[];
-    __shared__ int s_S0, s_Z, s_mu, s_done;
-    __shared__ uint32_t s_V;
-    __shared__ double s_L, s_T;
-    __shared__ unsigned s_item, s_next;           // s_next: an item claimed during the last traceback
-    // (spilled layout) s_next's item word, replica size and offset, and where its device ids,
-    // capacities and keys wait in shared memory (-1: not fetched)
-    __shared__ unsigned long long s_pre_item;
-    __shared__ int s_pre_m, s_pre_off, s_pre_at, s_pre_use;
-    __shared__ unsigned long long s_bestkey;     // (V << 32) | mu of the best master so far
-    __shared__ uint32_t s_V0, s_V1;
-    __shared__ unsigned s_prb[3];                // probes of a column over 32, 64, 128 threads
-
-    const int K = dm.K, M = dm.M, N = dm.N;
-    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, NW = blockDim.x >> 5;
-    constexpr Key kInf = (Key)~(Key)0;
-    const unsigned n_items = wl.ctrl[kCtrlEnd + cls];         // this class's items end here
-    constexpr bool spill = SPILL;
-    // this CTA's suffix-column scratch (only the first launch's CTAs spill)
-    uint32_t *gsp = spill ? wl.gspill + (size_t)blockIdx.x * wl.spill_stride : nullptr;
-    if (tid == 0) { s_next = ~0u; s_pre_at = -1; }
-  for (;;) {
-    // ---- next work item of the class (heaviest first); warp 1 claims it
-    //      while warp 0 traces the last one back
-    if (tid == 0) {
-        const unsigned nx = s_next;
-        s_next = ~0u;
-        s_item = nx != ~0u ? nx : atomicAdd(&wl.ctrl[kCtrlNext + cls], 1u);
-        s_pre_use = nx != ~0u ? s_pre_at : -1;
-        s_pre_at = -1;
-    }
+    __shared__ unsigned s_bin[kListBins];
+    const int total = dm.P * dm.K, chunk = (total + gridDim.x - 1) / gridDim.x;
+    const int lo = blockIdx.x * chunk, hi = min(total, lo + chunk);
+    for (int b = threadIdx.x; b < kListBins; b += blockDim.x) s_bin[b] = 0;
+    if (blockIdx.x == 0)
+        for (int i = threadIdx.x; i < kNumStats; i += blockDim.x) stats[i] = 0;
     __syncthreads();
-    const unsigned idx = s_item;
-    const int pre_at = SPILL ? s_pre_use : -1;                  // the item's data fetched already
-    __syncthreads();
-    if (idx >= n_items) break;
-    const uint64_t item = pre_at >= 0 ? s_pre_item : wl.items[idx];
-    const int slot = (int)(item >> 8), code = (int)(item & 0x3Fu);
-    if (tid == 0) s_done = *(volatile const int32_t *)&si.best[slot] > code;   // a larger batch won
-    __syncthreads();
-    if (s_done) continue;
-    const int g = slot / K, c = slot - g * K;
-    const size_t gk = (size_t)g * K + c;
-    const int off = pre_at >= 0 ? s_pre_off : si.off[slot], m = pre_at >= 0 ? s_pre_m : pop.sizes[gk];
-    const int role = (int)((item >> 7) & 1u);                   // decode
-    const bool sweep = (item >> 6) & 1u;                        // the result advances the decode sweep
-    uint64_t vmask = 1ull << code;
-    int16_t *lay_out = so.layers + ((size_t)g * dm.V + code) * M + off;
-
-    unsigned long long st_runs = 0, st_cells = 0, st_probes = 0;
-    bool served = false;
-
-    if (m <= N && vmask) {
-        const int W = N - m + 1;
-        int *cnt0 = reinterpret_cast<int *>(smem);              // [m]
-        int *cnt1 = cnt0 + m;                                   // [m]
-        int *nk = cnt1 + m;                                     // [m]
-        Key *leaf0 = reinterpret_cast<Key *>(nk + m);           // [m][W] l_k(n)
-        Key *Fst = leaf0 + (size_t)m * W;                       // [m][W] prefix / traceback columns
-        Key *Gst = Fst + (size_t)m * W;                         // [m][W] suffix columns ([2][W] spilled)
-        Key *Hb = Gst + (size_t)(spill ? 2 : m) * W;            // [NW][W] per-warp convolution
-        Key *Lb = Hb + (size_t)NW * W;                          // [NW][W] per-warp head row
-        Key *Sb = Lb + (size_t)NW * W;                          // [NW][W] per-warp suffix column (spilled)
-        Key *row1s = Sb + (spill ? (size_t)NW * W : 0);         // [W] head row of mu*
-        Key *delta = row1s + W;                                 // [W] the empty stage
-        Key *tauk = delta + W;                                  // [m] tauk[k] = link (k-1) -> k
-        Key *lbm = tauk + m;                                    // [m] l^head_k(1)
-        uint16_t *devs = reinterpret_cast<uint16_t *>(lbm + m);   // [m]
-
-        int p_c0 = 0, p_c1 = 0;                                 // this thread's device's fetched
-        Key p_t = 0, p_l = 0;                                   // capacities and keys (pre_at >= 0)
-        if (pre_at >= 0) {                                      // read them all before any is overwritten
-            const int *q0 = reinterpret_cast<const int *>(smem + pre_at), *q1 = q0 + m;
-            const Key *qt = reinterpret_cast<const Key *>(q1 + m), *ql = qt + m;
-            const uint16_t *qd = reinterpret_cast<const uint16_t *>(ql + m);
-            int d = 0;
-            if (tid < m) { d = qd[tid]; p_c0 = q0[tid]; p_c1 = q1[tid]; p_t = qt[tid]; p_l = ql[tid]; }
-            __syncthreads();
-            if (tid < m) devs[tid] = (uint16_t)d;
-        } else {
-            for (int k = tid; k < m; k += blockDim.x) devs[k] = pop.perm[(size_t)g * M + off + k];
-        }
-        if (tid < 3) s_prb[tid] = c_span_probes[tid][W];
-        for (int r = tid; r < W; r += blockDim.x) delta[r] = r ? kInf : (Key)0;
-        __syncthreads();
-
-        // column accessors (1-based device index k)
-        auto colF = [&](int k) -> const Key * {
-            return k == 0 ? delta : k == 1 ? leaf0 : Fst + (size_t)(k - 1) * W;
-        };
-        // suffix column G_k: in shared memory (two of them, alternating, when spilled;
-        // the others then live in this CTA's global scratch, gsp)
-        auto colG = [&](int k) -> const Key * {
-            return k == m + 1 ? delta : k == m ? leaf0 + (size_t)(m - 1) * W
-                                               : Gst + (size_t)(spill ? (k & 1) : k - 1) * W;
-        };
-
-        const unsigned long long lprobe = 32 - __clz(W);
-        while (vmask && !served) {
-            const int bit = 63 - __clzll((long long)vmask);          // highest batch first
-            vmask &= ~(1ull << bit);
-            const int v = role ? bit + 1 : 0;
-            const size_t vM = (size_t)v * M;
-            // ---- 1. capacities, link ranks and master-free cost rows
-            if (pre_at >= 0) {
-                if (tid < m) { cnt0[tid] = p_c0; cnt1[tid] = p_c1; tauk[tid] = p_t; lbm[tid] = p_l; }
-            } else {
-                for (int k = tid; k < m; k += blockDim.x) {
-                    const size_t vd = vM + devs[k];
-                    const int c0 = tb.cap[vd * 2], c1 = tb.cap[vd * 2 + 1];
-                    cnt0[k] = c0 < W ? c0 : W;
-                    cnt1[k] = c1 < W ? c1 : W;
-                    tauk[k] = k ? (Key)tb.tau_rank[(vM + devs[k - 1]) * M + devs[k]] : (Key)0;
-                    lbm[k] = (Key)tb.leaf_rank[((vM + devs[k]) * 2 + 1) * dm.LS];   // l^head_k(1)
-                }
-            }
-            for (int k = wid; k < m; k += NW)                       // the loads of a row overlap
-                stage_row(leaf0 + (size_t)k * W, tb.leaf_rank + (vM + devs[k]) * 2 * dm.LS, W, lane);
-            if (SPILL && wid == NW - 1)                             // device 1's head row (step 3)
-                stage_row(row1s, tb.leaf_rank + ((vM + devs[0]) * 2 + 1) * dm.LS, W, lane);
-            cp_async_wait_all();
-            __syncthreads();
-            // ---- 2. masters the memory allows (the pre-pass guarantees one)
-            if (wid == 0) {
-                int s = 0, z = 0;
-                for (int k = lane; k < m; k += 32) { s += cnt0[k]; z += cnt0[k] == 0; }
-                s = warp_sum(s); z = warp_sum(z);
-                if (lane == 0) { s_S0 = s; s_Z = z; }
-            }
-            __syncthreads();
-            const int S0 = s_S0, Z = s_Z;
-            auto mu_ok = [&](int mu) {
-                const int k = mu - 1;
-                return (Z - (cnt0[k] == 0)) == 0 && cnt1[k] >= 1 && S0 - cnt0[k] + cnt1[k] >= N;
-            };
-            ++st_runs;
-            // ---- 3. prefix columns (warps 0-1) and suffix columns (warps 2-3).
-            //      With the spilled layout (the largest replicas) the prefix chain
-            //      runs first with the head on device 1: if then V_1 (its last
-            //      cell) equals V0 (the master-free optimum, from the suffix
-            //      side), every V_mu >= V0 = V_1, so mu* = 1 and these are the
-            //      columns step 5 would recompute; steps 4 and 5 are skipped.
-            //      Otherwise the chain runs again without the head.
-            auto prefix_chain = [&](bool head1) {
-                for (int k = 2; k <= m - 1; ++k) {
-                    const Key *prev = (head1 && k == 2) ? row1s : colF(k - 1), *row = leaf0 + (size_t)(k - 1) * W;
-                    const Key t = tauk[k - 1];
-                    Key *cur = Fst + (size_t)(k - 1) * W;
-                    const int per = (W + 63) >> 6;                 // cells per thread
-                    dp_span(prev, row, t, cur, tid * per, min(W, (tid + 1) * per));
-                    bar_named(1, 64);
-                }
-            };
-            // the last cell of a chain, its minimum over every split taken by a warp's lanes
-            auto top_cell = [&](const Key *a, const Key *b, Key t) -> uint32_t {
-                uint32_t x = kInf;
-                for (int q = lane; q < W; q += 32) x = min(x, (uint32_t)max(a[q], b[W - 1 - q]));
-#pragma unroll
-                for (int o = 16; o; o >>= 1) x = min(x, __shfl_xor_sync(0xFFFFFFFFu, x, o));
-                return max(x, (uint32_t)t);
-            };
-            if (wid < 2) {
-                prefix_chain(SPILL);
-                if (wid == 0) {                                   // V0 = F_m[W-1] (V_1 when spilled)
-                    uint32_t v = 0;
-                    if (m >= 2)
-                        v = top_cell((SPILL && m == 2) ? row1s : colF(m - 1), leaf0 + (size_t)(m - 1) * W, tauk[m - 1]);
-                    if (lane == 0) {
-                        if (SPILL) {                              // (V_1, 1) seeds the best master
-                            s_V1 = v;
-                            s_bestkey = (m >= 2 && v != (uint32_t)kInf) ? ((unsigned long long)v << 32) | 1u : ~0ull;
-                        } else {
-                            s_V0 = v;
-                            s_bestkey = ~0ull;
-                        }
-                    }
-                }
-            } else {
-                for (int k = m - 1; k >= 2; --k) {
-                    const Key *prev = colG(k + 1), *row = leaf0 + (size_t)(k - 1) * W;
-                    const Key t = tauk[k];
-                    Key *cur = Gst + (size_t)(spill ? (k & 1) : k - 1) * W;
-                    const int per = (W + 63) >> 6;
-                    const int r0 = (tid - 64) * per, r1 = min(W, (tid - 63) * per);
-                    dp_span(prev, row, t, cur, r0, r1);
-                    if (spill)                                      // the thread's own cells, to the scratch
-                        for (int r = r0; r < r1; ++r) __stcg(gsp + (size_t)(k - 1) * W + r, (uint32_t)cur[r]);
-                    bar_named(2, 64);
-                }
-                if (SPILL && wid == 2) {                          // V0 = G_1[W-1]
-                    const uint32_t v = m >= 2 ? top_cell(leaf0, colG(2), tauk[1]) : 0u;
-                    if (lane == 0) s_V0 = v;
-                }
-            }
-            if (tid == 0 && m >= 3) {
-                st_cells += 2ull * (m - 2) * W;
-                st_probes += 2ull * (m - 2) * s_prb[1];
-            }
-            __syncthreads();
-            // ---- 4. one master per warp at a time, skipping a master whose lower
-            //      bound V_mu >= max(V0, l^head_mu(1)) (V0 the master-free
-            //      optimum F_m[W-1]: the head only adds) exceeds the best V found
-            //      so far, or ties it with a larger index
-            const uint32_t V0 = s_V0;
-            bool spec = false;                                    // mu* = 1 proved (the spilled layout)
-            if (SPILL) {
-                spec = m >= 2 && s_V1 == V0 && V0 != (uint32_t)kInf;
-                if (tid == 0 && m >= 2) { st_cells += 1; st_probes += lprobe; }
-                if (!spec && m >= 3) {                            // the combine needs the master-free columns
-                    if (wid < 2) prefix_chain(false);
-                    if (tid == 0) {
-                        st_cells += (unsigned long long)(m - 2) * W;
-                        st_probes += (unsigned long long)(m - 2) * s_prb[1];
-                    }
-                    __syncthreads();
-                }
-            }
-            auto bound = [&](int k) -> uint32_t { return mu_ok(k + 1) ? max(V0, (uint32_t)lbm[k]) : (uint32_t)kInf; };
-
-            unsigned long long w_cells = 0, w_probes = 0;
-            Key *H = Hb + (size_t)wid * W, *L1 = Lb + (size_t)wid * W;
-            for (int mu = wid + 1; mu <= m && !spec; mu += NW) {
-                if (!mu_ok(mu) || (SPILL && m >= 2 && mu == 1)) continue;   // (V_1 is known when spilled)
-                const uint32_t lb = bound(mu - 1);
-                const unsigned long long bk = *reinterpret_cast<volatile unsigned long long *>(&s_bestkey);
-                const uint32_t bv = (uint32_t)(bk >> 32);
-                if (lb > bv || (lb == bv && (unsigned)mu > (unsigned)(bk & 0xFFFFFFFFu))) continue;
-                const uint32_t *hrow = tb.leaf_rank + ((vM + devs[mu - 1]) * 2 + 1) * dm.LS;
-                const Key *P = colF(mu - 1), *S = colG(mu + 1);
-                HeadRow<Key> hr;
-                hr.start(L1, hrow, W, lane);                          // in flight while H is built
-                if (spill && mu + 1 <= m - 1) {                       // the suffix column from the scratch
-                    Key *sb = Sb + (size_t)wid * W;                   // (L2: written by this CTA's other warps)
-                    for (int r = lane; r < W; r += 32) sb[r] = (Key)__ldcg(gsp + (size_t)mu * W + r);
-                    __syncwarp();
-                    S = sb;
-                }
-                const int per = (W + 31) >> 5;
-                dp_span(P, S, (Key)0, H, lane * per, min(W, (lane + 1) * per));
-                hr.finish(L1, hrow, W, lane);
-                __syncwarp();
-                uint32_t V = dp_cell(H, L1, (Key)0, W - 1);
-                if (mu >= 2) V = max(V, (uint32_t)tauk[mu - 1]);
-                if (mu <= m - 1) V = max(V, (uint32_t)tauk[mu]);
-                __syncwarp();
-                w_cells += W + 1;
-                w_probes += s_prb[0] + lprobe;
-                if (lane == 0) atomicMin(&s_bestkey, ((unsigned long long)V << 32) | (unsigned)mu);
-            }
-            if (lane == 0) { st_cells += w_cells; st_probes += w_probes; }
-            if (tid == 0 && m >= 2) { st_cells += 1; st_probes += lprobe; }
-            __syncthreads();
-            if (tid == 0) {
-                s_V = (uint32_t)(s_bestkey >> 32);
-                s_mu = (int)(s_bestkey & 0xFFFFFFFFu);
-            }
-            __syncthreads();
-            const uint32_t V = s_V;
-            const int mus = s_mu;
-            if (V == kInf) {
-                // the pre-pass tested this variant's memory exactly, unless the
-                // profile's costs do not grow with the batch: then the batches
-                // below the largest that passed run untested, and may have no
-                // partition.  Otherwise this cannot happen.
-                if (tid == 0 && (dm.grows || !role)) atomicAdd(&out.stats[kStDeviceErrors], 1ull);
-                continue;
-            }
-            if (!spec) {
-                for (int r = tid; r < W; r += blockDim.x)
-                    row1s[r] = (Key)tb.leaf_rank[((vM + devs[mus - 1]) * 2 + 1) * dm.LS + r];
-                __syncthreads();
-            }
-            // ---- 5. mu*'s prefix columns, for the traceback (already there when spec)
-            auto rowk = [&](int k) -> const Key * { return k == mus ? row1s : leaf0 + (size_t)(k - 1) * W; };
-            auto colD = [&](int k) -> const Key * {
-                if (k == 1) return mus == 1 ? row1s : leaf0;
-                return Fst + (size_t)(k - 1) * W;
-            };
-            for (int k = (mus > 2 ? mus : 2); k <= m - 1 && !spec; ++k) {
-                const Key *prev = colD(k - 1), *row = rowk(k);
-                const Key t = tauk[k - 1];
-                Key *cur = Fst + (size_t)(k - 1) * W;
-                const int per = (W + 127) >> 7;
-                dp_span(prev, row, t, cur, tid * per, min(W, (tid + 1) * per));
-                __syncthreads();
-                if (tid == 0) { st_cells += W; st_probes += s_prb[2]; }
-            }
-            // ---- 6. traceback (smallest split on ties), T and Lambda
-            if (wid == 0) {
-                int r = W - 1;
-                uint32_t D = V;
-                for (int k = m; k >= 2; --k) {
-                    const Key *row = rowk(k);
-                    int n = 0;                                    // #{n <= r+1 : l_k(n) <= D}
-                    for (int base = 0; base <= r; base += 32) {
-                        const int p = base + lane;
-                        const unsigned b = __ballot_sync(0xFFFFFFFFu, p <= r && row[p] <= D);
-                        n += __popc(b);
-                        if (b != 0xFFFFFFFFu) break;
-                    }
-                    if (lane == 0) nk[k - 1] = n;
-                    r = r + 1 - n;
-                    D = colD(k - 1)[r];
-                }
-                if (lane == 0) nk[0] = r + 1;
-                __syncwarp();
-                // stage and link times of the partition, lane k holds device k
-                const double *lrow = tb.leaf + vM * 2 * dm.LS;
-                const double *trow = tb.tau + vM * M;
-                double lam = 0.0;
-                uint64_t tmax = 0;
-                for (int base = 0; base < m; base += 32) {
-                    const int k = base + lane;               // 0-based device
-                    double lk = 0.0, tk = 0.0;
-                    if (k < m) {
-                        lk = lrow[((size_t)devs[k] * 2 + (k == mus - 1)) * dm.LS + nk[k] - 1];
-                        if (k >= 1) tk = trow[(size_t)devs[k - 1] * M + devs[k]];
-                        tmax = umax64(tmax, umax64(dkey(lk), dkey(tk)));
-                    }
-                    for (int q = 0; q < 32 && base + q < m; ++q) {
-                        const double lq = __shfl_sync(0xFFFFFFFFu, lk, q);
-                        const double tq = __shfl_sync(0xFFFFFFFFu, tk, q);
-                        if (base + q == 0) lam = lq;
-                        else { lam = lam + tq; lam = lam + lq; }
-                    }
-                }
-#pragma unroll
-                for (int o = 16; o; o >>= 1) tmax = umax64(tmax, __shfl_xor_sync(0xFFFFFFFFu, tmax, o));
-                if (lane == 0) {
-                    s_L = lam;
-                    s_T = keyd(tmax);
-                    s_done = (!role) || lam <= dm.lam_max;       // 1.0 / lam >= Min_TPS
-                }
-            } else if (wid == 1) {
-                unsigned nx = 0;
-                if (lane == 0) nx = atomicAdd(&wl.ctrl[kCtrlNext + cls], 1u);
-                nx = __shfl_sync(0xFFFFFFFFu, nx, 0);
-                if (lane == 0) s_next = nx;
-                if (SPILL && nx < n_items) {
-                    // (spilled layout) the next item's header, device ids, capacities
-                    // and keys, into this run's suffix-column and per-warp buffers,
-                    // which nothing reads from here to the next item
-                    const uint64_t it2 = wl.items[nx];
-                    const int slot2 = (int)(it2 >> 8), code2 = (int)(it2 & 0x3Fu);
-                    const int g2 = slot2 / K, c2 = slot2 - g2 * K;
-                    const int off2 = si.off[slot2], m2 = pop.sizes[(size_t)g2 * K + c2];
-                    const int at = (int)(reinterpret_cast<unsigned char *>(Gst) - smem);
-                    const long room = reinterpret_cast<unsigned char *>(row1s) - reinterpret_cast<unsigned char *>(Gst);
-                    if (m2 <= N && m2 <= (int)blockDim.x && 18L * m2 <= room) {
-                        const int W2 = N - m2 + 1;
-                        const size_t vM2 = (size_t)(((it2 >> 7) & 1u) ? code2 + 1 : 0) * M;
-                        int *q0 = reinterpret_cast<int *>(smem + at), *q1 = q0 + m2;
-                        Key *qt = reinterpret_cast<Key *>(q1 + m2), *ql = qt + m2;
-                        uint16_t *qd = reinterpret_cast<uint16_t *>(ql + m2);
-                        for (int k = lane; k < m2; k += 32) {
-                            const int d = pop.perm[(size_t)g2 * M + off2 + k];
-                            qd[k] = (uint16_t)d;
-                            const int a0 = tb.cap[(vM2 + d) * 2], a1 = tb.cap[(vM2 + d) * 2 + 1];
-                            q0[k] = a0 < W2 ? a0 : W2;
-                            q1[k] = a1 < W2 ? a1 : W2;
-                            ql[k] = (Key)tb.leaf_rank[((vM2 + d) * 2 + 1) * dm.LS];
-                        }
-                        __syncwarp();
-                        for (int k = lane; k < m2; k += 32)
-                            qt[k] = k ? (Key)tb.tau_rank[(vM2 + qd[k - 1]) * M + qd[k]] : (Key)0;
-                        if (lane == 0) { s_pre_item = it2; s_pre_m = m2; s_pre_off = off2; s_pre_at = at; }
-                    }
-                }
-            }
-            __syncthreads();
-            if (s_done) {
-                for (int k = tid; k < m; k += blockDim.x) lay_out[k] = (int16_t)nk[k];
-                if (tid == 0) {
-                    const size_t sv = gk * dm.V + code;
-                    so.mu[sv] = (int16_t)(mus - 1);
-                    so.T[sv] = s_T;
-                    so.L[sv] = s_L;
-                    __threadfence();
-                    if (sweep) atomicMax(&si.best[slot], code);
-                }
-                served = true;
-            }
-            __syncthreads();
+    for (int i = lo + threadIdx.x; i < hi; i += blockDim.x) {
+        const uint32_t info = si.info[i];
+        const int n = items_of(info);
+        if (dm.layered) {
+            for (int lv = 0; lv < (int)(info & kSlotDecMask); ++lv) atomicAdd(&s_bin[layered_bin(info, lv)], 1u);
+            if (info & kSlotPrefill) atomicAdd(&s_bin[layered_bin(info, 0)], 1u);
+        } else if (n) {
+            atomicAdd(&s_bin[info >> kSlotBinShift], (unsigned)n);
         }
     }
     __syncthreads();
-    if (lane == 0 && (st_cells | st_probes)) {
-        atomicAdd(&out.stats[kStCells], st_cells);
-        atomicAdd(&out.stats[kStProbes], st_probes);
+    for (int b = threadIdx.x; b < kListBins; b += blockDim.x) hist[(size_t)blockIdx.x * kListBins + b] = s_bin[b];
+}
+
+// Items are (slot << 8) | role << 7 | top: the decode sweep (role 1) from batch
+// top + 1 down (per-layer profiles: that batch), or the prefill run (role 0).  Block 0 also sets the classes'
+// ends and cursors.
+__global__ void __launch_bounds__(256) order_scatter_kernel(Dims dm, SlotInfo si, WorkList wl, const unsigned *hist)
+{
+    __shared__ unsigned s_all[4][kListBins], s_before[4][kListBins], s_at[kListBins];
+    const int total = dm.P * dm.K, chunk = (total + gridDim.x - 1) / gridDim.x;
+    const int lo = blockIdx.x * chunk, hi = min(total, lo + chunk);
+    {
+        const int b = threadIdx.x & (kListBins - 1), part = threadIdx.x / kListBins;
+        unsigned all = 0, before = 0;
+        for (int q = part; q < (int)gridDim.x; q += 4) {
+            const unsigned x = hist[(size_t)q * kListBins + b];
+            all += x;
+            if (q < (int)blockIdx.x) before += x;
+        }
+        s_all[part][b] = all;
+        s_before[part][b] = before;
     }
-    if (tid == 0 && st_runs) atomicAdd(&out.stats[cls ? kStDpRunsSmall : kStDpRuns], st_runs);
-  }
+    __syncthreads();
+    if (threadIdx.x < kListBins) {
+        const int b = threadIdx.x;
+        unsigned start = 0;                                  // all items of the bins before b
+        for (int q = 0; q < b; ++q) start += s_all[0][q] + s_all[1][q] + s_all[2][q] + s_all[3][q];
+        s_at[b] = start + s_before[0][b] + s_before[1][b] + s_before[2][b] + s_before[3][b];
+        if (blockIdx.x == 0) {
+            const unsigned end = start + s_all[0][b] + s_all[1][b] + s_all[2][b] + s_all[3][b];
+            if (b == 0) wl.ctrl[kCtrlNext] = 0;
+            if (b == kListBins - 1) wl.ctrl[kCtrlEnd + 1] = end;
+            if (b == (dm.dp_split ? kListBins / 2 : kListBins) - 1) wl.ctrl[kCtrlEnd] = wl.ctrl[kCtrlNext + 1] = end;
+        }
+    }
+    __syncthreads();
+    for (int i = lo + threadIdx.x; i < hi; i += blockDim.x) {
+        const uint32_t info = si.info[i];
+        const int n = items_of(info);
+        if (!n) continue;
+        const uint64_t slot = (uint64_t)i << 8;
+        if (dm.layered) {
+            const int top = (int)(info & kSlotDecMask) - 1;
+            for (int bit = top; bit >= 0; --bit)
+                wl.items[atomicAdd(&s_at[layered_bin(info, top - bit)], 1u)] = slot | 0x80u | (unsigned)bit;
+            if (info & kSlotPrefill) wl.items[atomicAdd(&s_at[layered_bin(info, 0)], 1u)] = slot;
+            continue;
+        }
+        unsigned at = atomicAdd(&s_at[info >> kSlotBinShift], (unsigned)n);
+        if (info & kSlotDecMask) wl.items[at++] = slot | 0x80u | ((info & kSlotDecMask) - 1u);
+        if (info & kSlotPrefill) wl.items[at] = slot;
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -911,8 +417,13 @@ __device__ __forceinline__ uint64_t crossover(const uint64_t *col, const uint64_
     return umin64(left, right);
 }
 
+__device__ __forceinline__ void bar_named(int id, int nthreads)
+{
+    asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(nthreads) : "memory");
+}
+
 __global__ void __launch_bounds__(32 * kLayeredWarps) dp_layered_kernel(Dims dm, Tables tb, DevPop pop, EvalOut out,
-                                                                        WorkList wl, SlotInfo si, SplitOut so)
+                                                                        WorkList wl, SlotInfo si, VariantOut vo)
 {
     extern __shared__ __align__(16) unsigned char lsm[];
     __shared__ unsigned s_item;
@@ -932,16 +443,14 @@ __global__ void __launch_bounds__(32 * kLayeredWarps) dp_layered_kernel(Dims dm,
         if (idx >= n_items) break;
         const uint64_t item = wl.items[idx];
         const int slot = (int)(item >> 8), code = (int)(item & 0x3Fu);
-        if (tid == 0) s_done = *(volatile const int32_t *)&si.best[slot] > code;   // a larger batch won
+        if (tid == 0) s_done = (item >> 7 & 1u) && *(volatile const int32_t *)&vo.best[slot] > code;
         __syncthreads();
-        if (s_done) continue;
-        const int g = slot / K, c = slot - g * K;
-        const size_t gk = (size_t)g * K + c;
-        const int off = si.off[slot], m = pop.sizes[gk];
+        if (s_done) continue;                                     // a larger batch won
+        const int g = slot / K;
+        const int off = si.off[slot], m = pop.sizes[slot];
         const int role = (int)((item >> 7) & 1u);
-        const bool sweep = (item >> 6) & 1u;
         const int v = role ? code + 1 : 0;
-        const size_t sv = gk * dm.V + code;
+        const size_t sv = (size_t)slot * dm.V + v;
         const int W = N - m + 1;
         const size_t levels = sparse_levels((unsigned)W);
         uint64_t *F = reinterpret_cast<uint64_t *>(lsm);          // [m][W] prefix (then mu*'s) columns
@@ -1062,8 +571,8 @@ __global__ void __launch_bounds__(32 * kLayeredWarps) dp_layered_kernel(Dims dm,
         __syncthreads();                                          // (s_mu and s_V are the next run's)
         if (V == INF) {                                           // no partition (memory)
             if (tid == 0 && !role) {                              // a prefill result that does not exist
-                so.T[sv] = keyd(kInfKey);
-                so.L[sv] = keyd(kInfKey);
+                vo.T[sv] = keyd(kInfKey);
+                vo.L[sv] = keyd(kInfKey);
             }
             {                                                         // every thread's probes
                 unsigned p = (unsigned)probes;
@@ -1147,17 +656,17 @@ __global__ void __launch_bounds__(32 * kLayeredWarps) dp_layered_kernel(Dims dm,
         }
         __syncthreads();
         if (s_done) {
-            int16_t *lay_out = so.layers + ((size_t)g * dm.V + code) * M + off;
+            int16_t *lay_out = vo.layers + ((size_t)g * dm.V + v) * M + off;
             for (int k = tid; k < m; k += blockDim.x) lay_out[k] = (int16_t)nk[k];
             if (tid == 0) {
-                so.mu[sv] = (int16_t)(mus - 1);
-                so.T[sv] = s_T;
-                so.L[sv] = s_L;
+                vo.mu[sv] = (int16_t)(mus - 1);
+                vo.T[sv] = s_T;
+                vo.L[sv] = s_L;
                 __threadfence();
-                if (sweep) atomicMax(&si.best[slot], code);
+                if (role) atomicMax(&vo.best[slot], code);
             }
         } else if (tid == 0 && !role) {
-            so.T[sv] = keyd(kInfKey);
+            vo.T[sv] = keyd(kInfKey);
         }
         {                                                         // every thread's probes
             unsigned p = (unsigned)probes;
@@ -1172,15 +681,38 @@ __global__ void __launch_bounds__(32 * kLayeredWarps) dp_layered_kernel(Dims dm,
     }
 }
 
-// One launch per DP class (cls): the same code over the class's items, with
-// the class's shared-memory allocation.
-// SPILL: the suffix columns live in the global scratch (dm.g_spill), a
-// separate instance so that the other contexts keep their register count.
-template <bool SPILL>
-__global__ void __launch_bounds__(128, SPILL ? 6 : 0) dp_eval_kernel(Dims dm, Tables tb, DevPop pop, EvalOut out, WorkList wl,
-                                                      SlotInfo si, SplitOut so, int cls)
+// The accepted runs' results become the replicas' outputs, a warp per slot: the
+// largest accepted batch of a decode sweep, and the prefill run unless it found
+// no partition.
+__global__ void __launch_bounds__(128) layered_pick_kernel(Dims dm, DevPop pop, SlotInfo si, VariantOut vo, EvalOut out,
+                                                           SplitOut so)
 {
-    dp_eval_body<uint32_t, SPILL>(dm, tb, pop, out, wl, si, so, cls);
+    const int lane = threadIdx.x & 31;
+    const long long slot = (long long)blockIdx.x * 4 + (threadIdx.x >> 5);
+    if (slot >= (long long)dm.P * dm.K) return;
+    const uint32_t info = si.info[slot];
+    const int M = dm.M, g = (int)(slot / dm.K), off = si.off[slot];
+    for (int role = 0; role < 2; ++role) {
+        if (!(role ? info & kSlotDecMask : info & kSlotPrefill)) continue;
+        const int m = pop.sizes[slot];
+        const int best = role ? vo.best[slot] : 0;
+        const size_t sv = (size_t)slot * dm.V + (role ? best + 1 : 0);
+        const bool ok = role ? best >= 0 : vo.T[sv] < keyd(kInfKey);
+        const int16_t *lay = vo.layers + ((size_t)g * dm.V + (role ? best + 1 : 0)) * M + off;
+        int16_t *to = dm.role_search ? so.layers + ((size_t)g * 2 + role) * M + off : out.layers + (size_t)g * M + off;
+        for (int k = lane; k < m; k += 32) to[k] = ok ? lay[k] : (int16_t)-1;
+        if (lane != 0) continue;
+        if (dm.role_search) {
+            const size_t s2 = (size_t)slot * 2 + role;
+            so.code[s2] = (int16_t)(ok ? best : -1);
+            if (ok) { so.mu[s2] = vo.mu[sv]; so.T[s2] = vo.T[sv]; so.L[s2] = vo.L[sv]; }
+        } else {
+            out.master[slot] = ok ? vo.mu[sv] : (int16_t)-1;
+            out.bsel[slot] = (int16_t)(ok ? (role ? best + 1 : 0) : -1);
+            out.T[slot] = ok ? vo.T[sv] : keyd(kInfKey);
+            out.L[slot] = ok ? vo.L[sv] : keyd(kInfKey);
+        }
+    }
 }
 
 // The genome's objective from the role sums (PS, DS; PL, DL the rate-weighted
@@ -1208,20 +740,44 @@ __device__ __forceinline__ void objective(const Dims &dm, double PS, double DS, 
     }
 }
 
-// One warp per genome.  Each replica that had work gets its outputs from its
-// lane: the largest accepted variant is the sweep's answer (Alg. 2 keeps the
-// highest feasible batch), with its master, batch and times, and the serving
-// replica's rate (NP / T for prefill, b / T for decode).  The lanes then copy
-// the partition, position by position, from the accepted variant's split
-// results.  Lane 0 sums PS and DS in ascending replica order and applies
-// Eq. 3 (bottleneck phase), Eq. 4 (backlog) and Eq. 5 (waiting time).  A
-// 64-bit fingerprint of the genome, folded as a tree over the lanes, serves
-// the elites' duplicate test.
-__global__ void __launch_bounds__(128) finalize_score_kernel(Dims dm, DevPop pop, SlotInfo si, SplitOut so,
-                                                             EvalOut out)
+// A replica's pre-pass verdicts as counts: variants that its memory (n_pre)
+// and the latency bound (n_tps) rejected.
+__device__ __forceinline__ void slot_tallies(const Dims &dm, uint32_t info, unsigned &n_pre, unsigned &n_tps)
 {
-    __shared__ int s_off[4][E2_MAX_CLUSTERS + 1];     // replica start in the ordering
-    __shared__ int s_best[4][E2_MAX_CLUSTERS];        // accepted variant bit, -1 none, -2 no work here
+    if (info & kSlotDecTested) {
+        const unsigned mem = (info >> kSlotMemShift) & kSlotDecMask;
+        n_pre += (unsigned)dm.b_max - mem;
+        n_tps += mem - (info & kSlotDecMask);
+    }
+    if ((info & (kSlotPreTested | kSlotPrefill)) == kSlotPreTested) ++n_pre;
+}
+
+// A genome's counts, summed over its warp's lanes into the evaluation's counters.
+__device__ __forceinline__ void genome_tallies(const EvalOut &out, int R, unsigned n_served, unsigned n_pre,
+                                               unsigned n_tps, unsigned long long n_paper, int lane)
+{
+    n_served = __reduce_add_sync(0xFFFFFFFFu, n_served);
+    n_pre = __reduce_add_sync(0xFFFFFFFFu, n_pre);
+    n_tps = __reduce_add_sync(0xFFFFFFFFu, n_tps);
+#pragma unroll
+    for (int o = 16; o; o >>= 1) n_paper += __shfl_xor_sync(0xFFFFFFFFu, n_paper, o);
+    if (lane != 0) return;
+    atomicAdd(&out.stats[kStGenomes], 1ull);
+    atomicAdd(&out.stats[kStReplicas], (unsigned long long)R);
+    if (n_paper) atomicAdd(&out.stats[kStPaper], n_paper);
+    if (n_served) atomicAdd(&out.stats[kStServed], (unsigned long long)n_served);
+    if (n_pre) atomicAdd(&out.stats[kStPrecheck], (unsigned long long)n_pre);
+    if (n_tps) atomicAdd(&out.stats[kStTpsPruned], (unsigned long long)n_tps);
+}
+
+// One warp per genome, after the DP has written every replica's outputs: each
+// lane takes its replicas' rates (NP / T for prefill, b / T for decode), lane
+// 0 sums PS and DS in ascending replica order and applies Eq. 3 (bottleneck
+// phase), Eq. 4 (backlog) and Eq. 5 (waiting time).  A 64-bit fingerprint of
+// the genome, folded as a tree over the lanes, serves the elites' duplicate
+// test.
+__global__ void __launch_bounds__(128) finalize_score_kernel(Dims dm, DevPop pop, SlotInfo si, EvalOut out)
+{
     const int wl = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int g = blockIdx.x * 4 + wl;
     if (g >= dm.P) return;
@@ -1238,7 +794,8 @@ __global__ void __launch_bounds__(128) finalize_score_kernel(Dims dm, DevPop pop
         const uint16_t *pp = pop.perm + (size_t)g * M;
         for (int i = lane; i < M; i += 32) hl = mix(hl, pp[i]);
     }
-    unsigned long long n_rep = 0, n_served = 0, n_paper = 0;
+    unsigned n_served = 0, n_pre = 0, n_tps = 0;
+    unsigned long long n_paper = 0;
     double rate[2], lat[2];
     int kind[2];                                   // -1 none, 0 prefill, 1 decode
 #pragma unroll
@@ -1248,63 +805,22 @@ __global__ void __launch_bounds__(128) finalize_score_kernel(Dims dm, DevPop pop
         rate[h] = 0.0;
         lat[h] = 0.0;
         if (c < R) {
-            const int slot = g * K + c;
-            const uint64_t mask = si.mask[slot];
-            s_off[wl][c] = si.off[slot];
-            int best = -2;                         // no work: outputs written by the pre-pass
-            if (mask) {
-                const int m = h ? sz_hi : sz_lo;
-                const int role = (int)((roles >> c) & 1ull);
-                best = si.best[slot];
-                unsigned long long nrun = role ? (unsigned long long)dm.b_max : 1ull;
-                if (best < 0) {
-                    out.master[slot] = -1; out.bsel[slot] = -1;
-                    out.T[slot] = keyd(kInfKey); out.L[slot] = keyd(kInfKey);
-                } else {
-                    const size_t sv = (size_t)slot * dm.V + best;
-                    const double T = so.T[sv];
-                    out.master[slot] = so.mu[sv];
-                    out.bsel[slot] = (int16_t)(role ? best + 1 : 0);
-                    out.T[slot] = T;
-                    lat[h] = so.L[sv];
-                    out.L[slot] = lat[h];
-                    if (role) nrun = (unsigned long long)(dm.b_max - best);   // variants b_max .. best+1
-                    ++n_served;
-                    kind[h] = role;
-                    rate[h] = role ? (double)(best + 1) / T : (double)dm.NP / T;
-                }
-                ++n_rep;
-                n_paper += nrun * paper_candidates(m, dm.N);
+            const int slot = g * K + c, b = out.bsel[slot], role = (int)((roles >> c) & 1ull);
+            const int m = h ? sz_hi : sz_lo;
+            slot_tallies(dm, si.info[slot], n_pre, n_tps);
+            unsigned long long nrun = role ? (unsigned long long)dm.b_max : 1ull;
+            if (b >= 0) {
+                const double T = out.T[slot];
+                lat[h] = out.L[slot];
+                kind[h] = role;
+                rate[h] = role ? (double)b / T : (double)dm.NP / T;
+                if (role) nrun = (unsigned long long)(dm.b_max - b + 1);   // variants b_max .. b
+                ++n_served;
             }
-            s_best[wl][c] = best;
+            if (m <= dm.N) n_paper += nrun * paper_candidates(m, dm.N);
         }
     }
-    if (lane == 0) s_off[wl][R] = M;
-    __syncwarp();
-    // partition: position i belongs to the last replica c with off_c <= i
-    const int16_t *split = so.layers + (size_t)g * dm.V * M;
-    for (int i = lane; i < M; i += 32) {
-        int lo = 0, hi = R - 1;
-        while (lo < hi) {
-            const int mid = (lo + hi + 1) >> 1;
-            if (s_off[wl][mid] <= i) lo = mid;
-            else hi = mid - 1;
-        }
-        const int best = s_best[wl][lo];
-        if (best >= 0) out.layers[(size_t)g * M + i] = split[(size_t)best * M + i];
-        else if (best == -1) out.layers[(size_t)g * M + i] = -1;
-    }
-#pragma unroll
-    for (int o = 16; o; o >>= 1) {
-        n_rep += __shfl_xor_sync(0xFFFFFFFFu, n_rep, o);
-        n_served += __shfl_xor_sync(0xFFFFFFFFu, n_served, o);
-        n_paper += __shfl_xor_sync(0xFFFFFFFFu, n_paper, o);
-    }
-    if (lane == 0 && n_rep) {
-        atomicAdd(&out.stats[kStReplicas], n_rep);
-        atomicAdd(&out.stats[kStPaper], n_paper);
-        if (n_served) atomicAdd(&out.stats[kStServed], n_served);
-    }
+    genome_tallies(out, R, n_served, n_pre, n_tps, n_paper, lane);
     double PS = 0.0, DS = 0.0, PL = 0.0, DL = 0.0;   // PL, DL: rate-weighted latencies (finishing time)
     for (int c = 0; c < R; ++c) {
         const int h = c >> 5;
@@ -1334,7 +850,6 @@ __global__ void __launch_bounds__(128) finalize_score_kernel(Dims dm, DevPop pop
     h = mix(h, (uint64_t)R << 40);
     h = mix(h, roles);
     out.hash[g] = h;
-    atomicAdd(&out.stats[kStGenomes], 1ull);
 }
 
 // Alg. 2's role search, one warp per genome (or a block, below).  The lead
@@ -1380,7 +895,7 @@ __global__ void __launch_bounds__(128) finalize_roles_kernel(Dims dm, DevPop pop
     const int id = WPG == 1 ? lane : (int)threadIdx.x; // the thread's place in its genome's search
     const bool lead = WPG == 1 || wl == 0;              // the warp that reads and writes the genome
     if (g >= dm.P) return;
-    const int K = dm.K, M = dm.M, V = dm.V, bp = dm.b_max;
+    const int K = dm.K, M = dm.M, bp = dm.b_max;
     const int R = pop.nclus[g];
     const uint64_t roles0 = pop.roles[g];
     // the objective of full assignment r, PS and DS (and, for the finishing
@@ -1413,18 +928,17 @@ __global__ void __launch_bounds__(128) finalize_roles_kernel(Dims dm, DevPop pop
             const int c = lane + 32 * h;
             if (c >= R) continue;
             const int slot = g * K + c;
-            const uint64_t mask = si.mask[slot];
+            const size_t sp = (size_t)slot * 2, sd = sp + 1;      // its prefill run and its decode sweep
             m[h] = pop.sizes[slot];
-            pok[h] = (int)((mask >> bp) & 1ull);
-            if (pok[h] && dm.layered) pok[h] = so.T[(size_t)slot * V + bp] < keyd(kInfKey);   // the run found none
-            best[h] = mask ? si.best[slot] : -1;
+            pok[h] = so.code[sp] >= 0;
+            best[h] = so.code[sd];
             s_off[gw][c] = si.off[slot];
             s_pv[gw][c] = pok[h];
             s_dv[gw][c] = best[h] >= 0;
-            s_ps[gw][c] = pok[h] ? (double)dm.NP / so.T[(size_t)slot * V + bp] : 0.0;
-            s_ds[gw][c] = best[h] >= 0 ? (double)(best[h] + 1) / so.T[(size_t)slot * V + best[h]] : 0.0;
-            s_pl[gw][c] = pok[h] ? s_ps[gw][c] * so.L[(size_t)slot * V + bp] : 0.0;
-            s_dl[gw][c] = best[h] >= 0 ? s_ds[gw][c] * so.L[(size_t)slot * V + best[h]] : 0.0;
+            s_ps[gw][c] = pok[h] ? (double)dm.NP / so.T[sp] : 0.0;
+            s_ds[gw][c] = best[h] >= 0 ? (double)(best[h] + 1) / so.T[sd] : 0.0;
+            s_pl[gw][c] = pok[h] ? s_ps[gw][c] * so.L[sp] : 0.0;
+            s_dl[gw][c] = best[h] >= 0 ? s_ds[gw][c] * so.L[sd] : 0.0;
         }
         // the free replicas: those that can decode, and under the finishing
         // time also those that can only prefill
@@ -1684,34 +1198,34 @@ __global__ void __launch_bounds__(128) finalize_roles_kernel(Dims dm, DevPop pop
     }
     // ---- outputs of the chosen roles (the genome's first warp)
     const uint64_t brf = capped ? (roles0 & freem) : expand(br);
-    unsigned long long n_rep = 0, n_served = 0, n_paper = 0;
+    unsigned n_served = 0, n_pre = 0, n_tps = 0;
+    unsigned long long n_paper = 0;
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
         const int c = lane + 32 * h;
         if (c >= R) continue;
         const int slot = g * K + c;
         const int role = (int)((brf >> c) & 1ull);
-        const int code = role ? best[h] : (pok[h] ? bp : -1);
-        s_code[gw][c] = code;
+        const size_t sv = (size_t)slot * 2 + role;
+        const int code = role ? best[h] : (pok[h] ? 0 : -1);
+        s_code[gw][c] = code < 0 ? -1 : role;
         if (code < 0) {
             out.master[slot] = -1; out.bsel[slot] = -1;
             out.T[slot] = keyd(kInfKey); out.L[slot] = keyd(kInfKey);
         } else {
-            const size_t sv = (size_t)slot * V + code;
+            const double T = so.T[sv], L = so.L[sv];
             out.master[slot] = so.mu[sv];
             out.bsel[slot] = (int16_t)(role ? code + 1 : 0);
-            out.T[slot] = so.T[sv];
-            out.L[slot] = so.L[sv];
+            out.T[slot] = T;
+            out.L[slot] = L;
             ++n_served;
         }
-        if (si.mask[slot]) {                         // replicas with no work were counted by the pre-pass
-            const unsigned long long ndec = best[h] >= 0 ? (unsigned long long)(bp - best[h]) : (unsigned long long)bp;
-            ++n_rep;
-            n_paper += (1 + ndec) * paper_candidates(m[h], dm.N);
-        }
+        slot_tallies(dm, si.info[slot], n_pre, n_tps);
+        const unsigned long long ndec = (unsigned long long)(best[h] >= 0 ? bp - best[h] : bp);
+        if (m[h] <= dm.N) n_paper += (1 + ndec) * paper_candidates(m[h], dm.N);
     }
     __syncwarp();
-    const int16_t *split = so.layers + (size_t)g * V * M;
+    const int16_t *split = so.layers + (size_t)g * 2 * M;
     for (int i = lane; i < M; i += 32) {
         int lo = 0, hi = R - 1;
         while (lo < hi) {
@@ -1722,12 +1236,7 @@ __global__ void __launch_bounds__(128) finalize_roles_kernel(Dims dm, DevPop pop
         const int code = s_code[gw][lo];
         out.layers[(size_t)g * M + i] = code >= 0 ? split[(size_t)code * M + i] : (int16_t)-1;
     }
-#pragma unroll
-    for (int o = 16; o; o >>= 1) {
-        n_rep += __shfl_xor_sync(0xFFFFFFFFu, n_rep, o);
-        n_served += __shfl_xor_sync(0xFFFFFFFFu, n_served, o);
-        n_paper += __shfl_xor_sync(0xFFFFFFFFu, n_paper, o);
-    }
+    genome_tallies(out, R, n_served, n_pre, n_tps, n_paper, lane);
     // fingerprint of the genome with its chosen roles (a tree fold over the lanes)
     uint64_t hl = 0x9E3779B97F4A7C15ull ^ (uint64_t)lane;
     auto mix = [](uint64_t h, uint64_t x) { h = (h ^ x) * 0xBF58476D1CE4E5B9ull; return h ^ (h >> 31); };
@@ -1739,11 +1248,6 @@ __global__ void __launch_bounds__(128) finalize_roles_kernel(Dims dm, DevPop pop
         if (lane < o) hl = mix(hl, other);
     }
     if (lane != 0) return;
-    if (n_rep) {
-        atomicAdd(&out.stats[kStReplicas], n_rep);
-        atomicAdd(&out.stats[kStPaper], n_paper);
-    }
-    if (n_served) atomicAdd(&out.stats[kStServed], n_served);
     if (capped) atomicAdd(&out.stats[kStRoleCapped], 1ull);
     double PS, DS, w, phase;
     score(brf, PS, DS, w, phase);
@@ -1756,7 +1260,6 @@ __global__ void __launch_bounds__(128) finalize_roles_kernel(Dims dm, DevPop pop
     h = mix(h, (uint64_t)R << 40);
     h = mix(h, brf);
     out.hash[g] = h;
-    atomicAdd(&out.stats[kStGenomes], 1ull);
 }
 
 // The adapted-SplitWise rule of the paper's comparison (Sec. 4.2, "Baseline
@@ -1773,11 +1276,11 @@ __global__ void __launch_bounds__(128) finalize_splitwise_kernel(Dims dm, DevPop
                                                                  EvalOut out)
 {
     __shared__ int s_off[4][E2_MAX_CLUSTERS + 1];     // replica start in the ordering
-    __shared__ int s_code[4][E2_MAX_CLUSTERS];        // variant bit of the chosen role's result, -1 none
+    __shared__ int s_code[4][E2_MAX_CLUSTERS];        // the role whose result is taken, -1 none
     const int wl = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int g = blockIdx.x * 4 + wl;
     if (g >= dm.P) return;
-    const int K = dm.K, M = dm.M, V = dm.V, bp = dm.b_max;
+    const int K = dm.K, M = dm.M, bp = dm.b_max;
     const int R = pop.nclus[g];
     double strength[2];
     int pok[2], best[2], m[2];
@@ -1790,13 +1293,12 @@ __global__ void __launch_bounds__(128) finalize_splitwise_kernel(Dims dm, DevPop
         m[h] = 0;
         if (c < R) {
             const int slot = g * K + c;
-            const uint64_t mask = si.mask[slot];
+            const size_t sp = (size_t)slot * 2;
             m[h] = pop.sizes[slot];
-            pok[h] = (int)((mask >> bp) & 1ull);
-            if (pok[h] && dm.layered) pok[h] = so.T[(size_t)slot * V + bp] < keyd(kInfKey);   // the run found none
-            best[h] = mask ? si.best[slot] : -1;
+            pok[h] = so.code[sp] >= 0;
+            best[h] = so.code[sp + 1];
             s_off[wl][c] = si.off[slot];
-            if (pok[h]) strength[h] = (double)dm.NP / so.T[(size_t)slot * V + bp];
+            if (pok[h]) strength[h] = (double)dm.NP / so.T[sp];
         }
     }
     if (lane == 0) s_off[wl][R] = M;
@@ -1821,40 +1323,39 @@ __global__ void __launch_bounds__(128) finalize_splitwise_kernel(Dims dm, DevPop
     const unsigned dec_hi = __ballot_sync(0xFFFFFFFFu, lane + 32 < R && rank[1] >= nP);
     const uint64_t roles = (uint64_t)dec_lo | ((uint64_t)dec_hi << 32);
     // outputs of the chosen roles
-    unsigned long long n_rep = 0, n_served = 0, n_paper = 0;
     double rate[2] = {0.0, 0.0}, lat[2] = {0.0, 0.0};
     int kind[2] = {-1, -1};
+    unsigned n_served = 0, n_pre = 0, n_tps = 0;
+    unsigned long long n_paper = 0;
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
         const int c = lane + 32 * h;
         if (c >= R) continue;
         const int slot = g * K + c;
         const int role = (int)((roles >> c) & 1ull);
-        const int code = role ? best[h] : (pok[h] ? bp : -1);
-        s_code[wl][c] = code;
+        const size_t sv = (size_t)slot * 2 + role;
+        const int code = role ? best[h] : (pok[h] ? 0 : -1);
+        s_code[wl][c] = code < 0 ? -1 : role;
         if (code < 0) {
             out.master[slot] = -1; out.bsel[slot] = -1;
             out.T[slot] = keyd(kInfKey); out.L[slot] = keyd(kInfKey);
         } else {
-            const size_t sv = (size_t)slot * V + code;
-            const double T = so.T[sv];
+            const double T = so.T[sv], L = so.L[sv];
             out.master[slot] = so.mu[sv];
             out.bsel[slot] = (int16_t)(role ? code + 1 : 0);
             out.T[slot] = T;
-            lat[h] = so.L[sv];
-            out.L[slot] = lat[h];
+            out.L[slot] = L;
+            lat[h] = L;
             kind[h] = role;
             rate[h] = role ? (double)(code + 1) / T : (double)dm.NP / T;
             ++n_served;
         }
-        if (si.mask[slot]) {                         // replicas with no work were counted by the pre-pass
-            const unsigned long long ndec = best[h] >= 0 ? (unsigned long long)(bp - best[h]) : (unsigned long long)bp;
-            ++n_rep;
-            n_paper += (1 + ndec) * paper_candidates(m[h], dm.N);
-        }
+        slot_tallies(dm, si.info[slot], n_pre, n_tps);
+        const unsigned long long ndec = (unsigned long long)(best[h] >= 0 ? bp - best[h] : bp);
+        if (m[h] <= dm.N) n_paper += (1 + ndec) * paper_candidates(m[h], dm.N);
     }
     __syncwarp();
-    const int16_t *split = so.layers + (size_t)g * V * M;
+    const int16_t *split = so.layers + (size_t)g * 2 * M;
     for (int i = lane; i < M; i += 32) {
         int lo = 0, hi = R - 1;
         while (lo < hi) {
@@ -1865,12 +1366,7 @@ __global__ void __launch_bounds__(128) finalize_splitwise_kernel(Dims dm, DevPop
         const int code = s_code[wl][lo];
         out.layers[(size_t)g * M + i] = code >= 0 ? split[(size_t)code * M + i] : (int16_t)-1;
     }
-#pragma unroll
-    for (int o = 16; o; o >>= 1) {
-        n_rep += __shfl_xor_sync(0xFFFFFFFFu, n_rep, o);
-        n_served += __shfl_xor_sync(0xFFFFFFFFu, n_served, o);
-        n_paper += __shfl_xor_sync(0xFFFFFFFFu, n_paper, o);
-    }
+    genome_tallies(out, R, n_served, n_pre, n_tps, n_paper, lane);
     double PS = 0.0, DS = 0.0, PL = 0.0, DL = 0.0;
     for (int c = 0; c < R; ++c) {
         const int h = c >> 5;
@@ -1891,11 +1387,6 @@ __global__ void __launch_bounds__(128) finalize_splitwise_kernel(Dims dm, DevPop
         if (lane < o) hl = mix(hl, other);
     }
     if (lane != 0) return;
-    if (n_rep) {
-        atomicAdd(&out.stats[kStReplicas], n_rep);
-        atomicAdd(&out.stats[kStPaper], n_paper);
-    }
-    if (n_served) atomicAdd(&out.stats[kStServed], n_served);
     double w, phase;
     objective(dm, PS, DS, PL, DL, w, phase);
     double *f = out.fit + (size_t)g * 4;
@@ -1907,7 +1398,6 @@ __global__ void __launch_bounds__(128) finalize_splitwise_kernel(Dims dm, DevPop
     h = mix(h, (uint64_t)R << 40);
     h = mix(h, roles);
     out.hash[g] = h;
-    atomicAdd(&out.stats[kStGenomes], 1ull);
 }
 
 // The G--C split of the plans (Sec. 4.3) under GPU-CPU offload, one warp per
@@ -1958,161 +1448,71 @@ __global__ void __launch_bounds__(128) gc_split_kernel(Dims dm, DevPop pop, cons
     }
 }
 
-// Persistent grids of the DP.  Shared memory is what limits CTAs per SM when
-// the largest replica's DP is big (many blocks); the replica sizes whose DP
-// fits in half of it then form class 1, launched with that smaller allocation
-// and a grid of as many CTAs as fit, where this raises the CTAs per SM.
-// The probe counts of c_span_probes (a function of W alone).
-static cudaError_t load_span_probes()
-{
-    static uint16_t t[3][E2_MAX_BLOCKS + 1];
-    for (int i = 0; i < 3; ++i) {
-        const int T = 32 << i;
-        t[i][0] = 0;
-        for (int W = 1; W <= E2_MAX_BLOCKS; ++W) {
-            const int per = (W + T - 1) / T, spans = (W + per - 1) / per;
-            unsigned n = (unsigned)(W - spans);
-            for (int j = 0; j < spans; ++j) {
-                unsigned bits = 0;
-                for (unsigned x = (unsigned)(j * per + 1); x; x >>= 1) ++bits;   // floor(log2(r + 1)) + 1
-                n += bits;
-            }
-            t[i][W] = (uint16_t)n;
-        }
-    }
-    return cudaMemcpyToSymbol(c_span_probes, t, sizeof t);
-}
+// Persistent grids of the DP.  Replicas of up to 32 devices (a device per
+// lane) and larger ones (several per lane, more registers) form two launches
+// where both sizes can occur.  On fleets without the larger sizes,
+// populations of kSplitSlots slots or more launch the replicas of more than 8
+// devices apart.
+constexpr long long kSplitSlots = 32768;
 
 cudaError_t configure_eval(e2_ctx *c)
 {
-    cudaError_t e = load_span_probes();
+    cudaError_t e = cudaSuccess;
+    int sms = 0;
+    e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device);
     if (e != cudaSuccess) return e;
+    if (sms < 1) sms = 1;
+    const int mmax = c->dm.M < c->dm.N ? c->dm.M : c->dm.N;
+    c->dm.dp_mmax = mmax;
+    c->dm.dp_split = 0;
+    c->dp_grid1 = 0;
+    c->dp_smem1 = 0;
     if (c->dm.layered) {                         // the plain-scan path: one launch, one class
         const void *lk = reinterpret_cast<const void *>(dp_layered_kernel);
         e = cudaFuncSetAttribute(lk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)c->dp_smem);
         if (e != cudaSuccess) return e;
-        int per_sm = 0, sms = 0;
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, lk, c->dp_threads, c->dp_smem);
+        int per_sm = 0;
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, lk, 32 * kLayeredWarps, c->dp_smem);
         if (e != cudaSuccess) return e;
-        e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device);
-        if (e != cudaSuccess) return e;
-        c->dp_grid = (per_sm > 0 ? per_sm : 1) * (sms > 0 ? sms : 1);
-        c->dm.dp_warps = c->dp_threads / 32;
-        c->dm.dp_small = 0;
-        c->dp_warp1 = 0;
-        c->dp_grid1 = 0;
-        c->dp_smem1 = 0;
+        c->dp_grid = (per_sm > 0 ? per_sm : 1) * sms;
         return cudaSuccess;
     }
-    // class 0 runs every replica size (spilling its suffix columns where that
-    // raises its occupancy); class 1, where it raises the occupancy of the
-    // sizes it takes, runs the small ones without spilling
-    const void *kernel = c->dm.g_spill ? reinterpret_cast<const void *>(dp_eval_kernel<true>)
-                                       : reinterpret_cast<const void *>(dp_eval_kernel<false>);
-    const void *kernel1 = reinterpret_cast<const void *>(dp_eval_kernel<false>);
-    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)c->dp_smem);
+    const bool off = c->dm.offload != 0;
+    if (mmax > 32) c->dm.dp_split = 32;
+    else if (mmax > 8 && (long long)c->dm.P * c->dm.K >= kSplitSlots) c->dm.dp_split = 8;
+    const int m0 = c->dm.dp_split ? c->dm.dp_split : mmax;   // class 0's largest replica
+    int per_sm = 0;
+    e = dp_order_occupancy(m0, 0, off, &per_sm);
     if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
-    if (e != cudaSuccess) return e;
-    int per_sm = 0, per_sm1 = 0, sms = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, c->dp_threads, c->dp_smem);
-    if (e != cudaSuccess) return e;
-    e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device);
-    if (e != cudaSuccess) return e;
-    if (sms < 1) sms = 1;
     c->dp_grid = (per_sm > 0 ? per_sm : 1) * sms;
-    const int warps = c->dp_threads / 32, mmax = c->dm.M < c->dm.N ? c->dm.M : c->dm.N;
-    size_t small = 0;
-    if (!c->dm.g_spill) {
-        // the sizes whose run fits in half the largest one's shared memory
-        for (int m = 1; m <= mmax; ++m) {
-            const size_t b = dp_item_bytes(m, c->dm.N, warps, 4, false);
-            if (2 * b <= c->dp_smem && b > small) small = b;
-        }
-    } else {
-        // the non-spilling kernel's best occupancy (its registers' limit), and the
-        // largest size that keeps it
-        e = cudaFuncSetAttribute(kernel1, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)c->dp_smem);
+    c->dp_smem = dp_order_smem(m0, 0);
+    if (c->dm.dp_split) {
+        e = dp_order_occupancy(mmax, 1, off, &per_sm);
         if (e != cudaSuccess) return e;
-        e = cudaFuncSetAttribute(kernel1, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                 cudaSharedmemCarveoutMaxShared);
-        if (e != cudaSuccess) return e;
-        int best1 = 0;
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&best1, kernel1, c->dp_threads, 16);
-        if (e != cudaSuccess) return e;
-        for (int m = 1; m <= mmax; ++m) {
-            const size_t b = dp_item_bytes(m, c->dm.N, warps, 4, false);
-            if (b <= small || b > c->dp_smem) continue;
-            int occ = 0;
-            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kernel1, c->dp_threads, b);
-            if (e != cudaSuccess) return e;
-            if (occ >= best1) small = b;
-        }
+        c->dp_grid1 = (per_sm > 0 ? per_sm : 1) * sms;
+        c->dp_smem1 = dp_order_smem(mmax, 1);
     }
-    c->dm.dp_warps = warps;
-    c->dm.dp_small = 0;
-    c->dp_grid1 = 0;
-    c->dp_smem1 = 0;
-    if (small > 0) {
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm1, kernel1, c->dp_threads, small);
-        if (e != cudaSuccess) return e;
-        if (per_sm1 > per_sm) {
-            c->dm.dp_small = (unsigned)small;
-            c->dp_grid1 = per_sm1 * sms;
-            c->dp_smem1 = small;
-        }
-    }
-    // without a four-warp class 1, the small sizes may run one per warp: the
-    // largest per-warp slice whose runs in flight per SM are at least twice
-    // class 0's (its CTAs per SM).  A warp's run takes longer than a CTA's, so
-    // this pays only with many runs per warp: the population's slots at least
-    // eight times the class's runs in flight on the GPU.
-    c->dp_warp1 = 0;
-    if (c->dm.dp_small == 0) {
-        size_t wslice = 0;
-        int wocc = 0;
-        for (int m = 1; m <= mmax; ++m) {
-            const size_t b = dp_item_bytes(m, c->dm.N, 1, 4, false);
-            if (b <= wslice || b > c->dp_smem) continue;
-            int occ = 0;
-            e = dp_warp_occupancy((unsigned)b, &occ);
-            if (e != cudaSuccess) return e;
-            if (occ * kDpWarpRuns >= 2 * per_sm) { wslice = b; wocc = occ; }
-        }
-        const long long slots = (long long)c->dm.P * c->dm.K;
-        if (wslice > 0 && slots < 8LL * kDpWarpRuns * wocc * sms) wslice = 0;
-        if (wslice > 0) {
-            e = dp_warp_occupancy((unsigned)wslice, &wocc);
-            if (e != cudaSuccess) return e;
-            c->dm.dp_small = (unsigned)wslice;
-            c->dm.dp_warps = 1;
-            c->dp_warp1 = 1;
-            c->dp_grid1 = wocc * sms;
-            c->dp_smem1 = wslice;
-        }
-    }
-    if (c->dm.g_spill && c->dp_grid > kSpillCtas) c->dp_grid = kSpillCtas;   // the scratch holds kSpillCtas CTAs
-    c->dm.dp_grid0 = c->dp_grid;
     return cudaSuccess;
 }
 
 cudaError_t launch_eval(const e2_ctx *c, const DevPop &p)
 {
     Tables tb{c->rate, c->bw, c->mem, c->rate_cpu, c->bw_cpu, c->mem_cpu, c->prof, c->leaf, c->tau, c->cap,
-              c->capg, c->cpb, c->tau_lb, c->leaf_rank, c->tau_rank, c->lcost};
+              c->capg, c->cpb, c->tau_lb, c->leaf_rank, c->tau_rank, c->lcost, c->drec, c->fxs};
     EvalOut out{c->fit, c->layers, c->master, c->bsel, c->T, c->L, c->hash, c->stats, c->gpu_layers};
-    SlotInfo si{c->slot_off, c->slot_mask, c->slot_size, c->slot_best};
-    WorkList wl{c->items, c->order_bins, c->gspill, (unsigned)c->spill_stride};
-    SplitOut so{c->split_T, c->split_L, c->split_mu, c->split_layers};
+    SlotInfo si{c->slot_off, c->slot_info};
+    WorkList wl{c->items, c->list_ctrl};
+    SplitOut so{c->split_T, c->split_L, c->split_mu, c->split_code, c->split_layers};
+    VariantOut vo{c->var_T, c->var_L, c->var_mu, c->var_layers, c->var_best};
     const long long slots = (long long)c->dm.P * c->dm.K;
-    cudaError_t e = cudaMemsetAsync(c->order_bins, 0, sizeof(unsigned) * kCtrlWords, c->stream);
-    if (e != cudaSuccess) return e;
-    const unsigned gb = (unsigned)((slots + 255) / 256 < 1024 ? (slots + 255) / 256 : 1024);
     const int mcap = c->dm.M < c->dm.N ? c->dm.M : c->dm.N;
-    slot_kernel<<<(unsigned)((slots + 1) / 2), 64, 2 * variant_stride(mcap), c->stream>>>(c->dm, tb, p, si, out,
-                                                                                      c->order_bins);
-    bins_kernel<<<1, 32, 0, c->stream>>>(c->dm, c->order_bins);
-    order_scatter_kernel<<<gb, 256, 0, c->stream>>>(c->dm, p, si, wl);
+    cudaError_t e = cudaSuccess;
+    slot_kernel<<<(unsigned)((slots + 1) / 2), 64, 2 * variant_stride(mcap), c->stream>>>(c->dm, tb, p, si, out, so, vo);
+    // (about 4,096 slots per block of the count and the scatter)
+    const long long nb = (slots + 4095) / 4096;
+    const unsigned lb = (unsigned)(nb < kListBlocks ? nb : kListBlocks);
+    bins_kernel<<<lb, 256, 0, c->stream>>>(c->dm, si, c->list_hist, c->stats);
+    order_scatter_kernel<<<lb, 256, 0, c->stream>>>(c->dm, si, wl, c->list_hist);
     // while a launch sequence is being recorded, the timing events become
     // event-record nodes of the graph (an ordinary record would only mark a
     // dependency)
@@ -2120,34 +1520,25 @@ cudaError_t launch_eval(const e2_ctx *c, const DevPop &p)
     if (c->ev_dp_start && (e = cudaStreamIsCapturing(c->stream, &cs)) != cudaSuccess) return e;
     const unsigned rec = cs == cudaStreamCaptureStatusActive ? cudaEventRecordExternal : cudaEventRecordDefault;
     if (c->ev_dp_start && (e = cudaEventRecordWithFlags(c->ev_dp_start, c->stream, rec)) != cudaSuccess) return e;
-    // a four-warp class 1 runs beside class 0, on the side stream; the
-    // warp-per-run class runs after it on the context's stream (sharing the
-    // SMs with class 0's CTAs was slower: DP +4.6% at c3, +2.3% at c5)
-    const bool beside = c->dp_grid1 > 0 && !c->dp_warp1;
-    if (beside) {
-        if ((e = cudaEventRecord(c->ev_dp_fork, c->stream)) != cudaSuccess) return e;
-        if ((e = cudaStreamWaitEvent(c->side, c->ev_dp_fork, 0)) != cudaSuccess) return e;
-    }
-    if (c->dm.layered)
-        dp_layered_kernel<<<(unsigned)c->dp_grid, c->dp_threads, c->dp_smem, c->stream>>>(c->dm, tb, p, out, wl, si, so);
-    else if (c->dm.g_spill)
-        dp_eval_kernel<true><<<(unsigned)c->dp_grid, c->dp_threads, c->dp_smem, c->stream>>>(c->dm, tb, p, out, wl, si,
-                                                                                           so, 0);
-    else
-        dp_eval_kernel<false><<<(unsigned)c->dp_grid, c->dp_threads, c->dp_smem, c->stream>>>(c->dm, tb, p, out, wl, si,
-                                                                                            so, 0);
-    if (c->dp_grid1 > 0) {                       // class 1: the small sizes, never spilling
-        if (c->dp_warp1)
-            e = dp_warp_launch(c->dp_grid1, (unsigned)c->dp_smem1, c->stream, c->dm, tb, p, out, wl, si, so);
-        else
-            dp_eval_kernel<false><<<(unsigned)c->dp_grid1, c->dp_threads, c->dp_smem1, c->side>>>(c->dm, tb, p, out,
-                                                                                                wl, si, so, 1);
-        if (e == cudaSuccess) e = cudaGetLastError();
+    if (c->dm.layered) {
+        dp_layered_kernel<<<(unsigned)c->dp_grid, 32 * kLayeredWarps, c->dp_smem, c->stream>>>(c->dm, tb, p, out, wl, si,
+                                                                                            vo);
+        layered_pick_kernel<<<(unsigned)((slots + 3) / 4), 128, 0, c->stream>>>(c->dm, p, si, vo, out, so);
+        ++c->launches;
+    } else {
+        // the larger replicas run beside the others on the side stream (few runs,
+        // each a longer chain)
+        if (c->dp_grid1 > 0) {
+            if ((e = cudaEventRecord(c->ev_fork, c->stream)) != cudaSuccess) return e;
+            if ((e = cudaStreamWaitEvent(c->side, c->ev_fork, 0)) != cudaSuccess) return e;
+            e = dp_order_launch(c->dp_grid1, c->dm.dp_mmax, 1, c->side, c->dm, tb, p, out, wl, c->slot_off, so);
+            if (e != cudaSuccess) return e;
+            if ((e = cudaEventRecord(c->ev_join, c->side)) != cudaSuccess) return e;
+        }
+        e = dp_order_launch(c->dp_grid, c->dm.dp_split ? c->dm.dp_split : c->dm.dp_mmax, 0, c->stream, c->dm, tb, p, out,
+                            wl, c->slot_off, so);
+        if (e == cudaSuccess && c->dp_grid1 > 0) e = cudaStreamWaitEvent(c->stream, c->ev_join, 0);
         if (e != cudaSuccess) return e;
-    }
-    if (beside) {
-        if ((e = cudaEventRecord(c->ev_dp_join, c->side)) != cudaSuccess) return e;
-        if ((e = cudaStreamWaitEvent(c->stream, c->ev_dp_join, 0)) != cudaSuccess) return e;
     }
     if (c->ev_dp_stop && (e = cudaEventRecordWithFlags(c->ev_dp_stop, c->stream, rec)) != cudaSuccess) return e;
     const unsigned fb = (unsigned)(((size_t)c->dm.P * 32 + 127) / 128);
@@ -2160,7 +1551,7 @@ cudaError_t launch_eval(const e2_ctx *c, const DevPop &p)
         if (c->dm.objective == 1) finalize_roles_kernel<1, true><<<fb, 128, 0, c->stream>>>(c->dm, p, si, so, out);
         else finalize_roles_kernel<1, false><<<fb, 128, 0, c->stream>>>(c->dm, p, si, so, out);
     }
-    else finalize_score_kernel<<<fb, 128, 0, c->stream>>>(c->dm, p, si, so, out);
+    else finalize_score_kernel<<<fb, 128, 0, c->stream>>>(c->dm, p, si, out);
     c->launches += c->dp_grid1 > 0 ? 6 : 5;
     if (c->dm.offload) {
         gc_split_kernel<<<fb, 128, 0, c->stream>>>(c->dm, p, c->capg, out);

@@ -21,10 +21,10 @@ size_t align_up(size_t x, size_t a = 256) { return (x + a - 1) / a * a; }
 
 struct Layout {
     size_t rate, bw, mem, rate_cpu, bw_cpu, mem_cpu, link_bw, cong, prof, leaf, tau, tau_lb, cap, capg, cpb,
-        leaf_sorted, beff_sorted, tau_sorted, leaf_rank, tau_rank, gpu_layers, psum, lcost, gspill;
+        leaf_sorted, beff_sorted, tau_sorted, leaf_rank, tau_rank, gpu_layers, psum, lcost, drec, fxs;
     size_t perm[2], sizes[2], nclus[2], roles[2];
-    size_t fit, layers, master, bsel, T, L, hash, dup, dup_key, dup_idx, elite, elite_fit, elite_ctl, elite_cand, stats, err, order_bins, items, slot_off, slot_mask, slot_size, slot_best,
-        split_T, split_L, split_mu, split_layers, total;
+    size_t fit, layers, master, bsel, T, L, hash, dup, dup_key, dup_idx, elite, elite_fit, elite_ctl, elite_cand, stats, err, list_ctrl, list_hist, items, slot_off, slot_info,
+        split_T, split_L, split_mu, split_code, split_layers, var_T, var_L, var_mu, var_layers, var_best, total;
     int LS;
 };
 
@@ -58,6 +58,8 @@ Layout layout(int M, int N, int b_max, int P, int Q, int K, bool layered = false
     l.cap = take(4 * V * M * 2);
     l.capg = take(4 * V * M * 2);
     l.cpb = take(4 * V * M);
+    l.drec = take(16 * V * M);
+    l.fxs = take(4 * V);
     l.tau_lb = take(4 * V * MM);
     l.leaf_sorted = take(8 * V * rank_pow2((size_t)M * 2 * N));
     l.beff_sorted = take(8 * rank_pow2(MM));
@@ -87,21 +89,24 @@ Layout layout(int M, int N, int b_max, int P, int Q, int K, bool layered = false
     l.elite_cand = take(4 * (size_t)P);                       // its candidate list
     l.stats = take(8 * kNumStats);
     l.err = take(4);
-    l.order_bins = take(4 * (size_t)kCtrlWords);
-    l.items = take(8 * (size_t)P * K * V);
+    l.list_ctrl = take(4 * (size_t)kCtrlWords);
+    l.list_hist = take(4 * (size_t)kListBlocks * kListBins);
+    l.items = take(8 * (size_t)P * K * (layered ? V : 2));    // a decode sweep (or its batches) and a prefill run
     l.slot_off = take(4 * (size_t)P * K);
-    l.slot_mask = take(8 * (size_t)P * K);
-    l.slot_size = take((size_t)P * K);
-    l.slot_best = take(4 * (size_t)P * K);
-    l.split_T = take(8 * (size_t)P * K * V);                 // per (slot, variant bit): decode b = bit + 1,
-    l.split_L = take(8 * (size_t)P * K * V);                 // and bit b_max = prefill when roles are searched
-    l.split_mu = take(2 * (size_t)P * K * V);
-    l.split_layers = take(2 * (size_t)P * V * M);
+    l.slot_info = take(4 * (size_t)P * K);
+    l.split_T = take(8 * (size_t)P * K * 2);                 // per (slot, role): used where both roles are
+    l.split_L = take(8 * (size_t)P * K * 2);                 // evaluated (role_search)
+    l.split_mu = take(2 * (size_t)P * K * 2);
+    l.split_code = take(2 * (size_t)P * K * 2);
+    l.split_layers = take(2 * (size_t)P * 2 * M);
     if (layered) {
         l.psum = take(8 * 3 * V * ((size_t)N + 1));
         l.lcost = take(8 * V * M * 2 * (size_t)N * N);
-    } else if (dp_spills(M, N, 4)) {
-        l.gspill = take(4 * (size_t)kSpillCtas * dp_spill_stride(M, N));
+        l.var_T = take(8 * (size_t)P * K * V);
+        l.var_L = take(8 * (size_t)P * K * V);
+        l.var_mu = take(2 * (size_t)P * K * V);
+        l.var_layers = take(2 * (size_t)P * V * M);
+        l.var_best = take(4 * (size_t)P * K);
     }
     l.total = o;
     return l;
@@ -381,9 +386,18 @@ int e2_create(const e2_devices *devs, const e2_links *links, const e2_layer_prof
     e2_ctx *c = new (std::nothrow) e2_ctx();
     if (!c) return E2_ENOMEM;
     c->stream = static_cast<cudaStream_t>(stream);
-    c->dm = Dims{M, N, b_max + 1, b_max, P, Q, K, l.LS, prm->tournament, prof->NP, prof->ND,
-                 prm->min_tps, prm->t_a, latency_ceiling(prm->min_tps), prm->role_search, 0.0f, 0u, 4,
-                 costs_grow_with_batch(prof, b_max), prm->objective};
+    c->dm = Dims{};
+    c->dm.M = M; c->dm.N = N; c->dm.V = b_max + 1; c->dm.b_max = b_max; c->dm.P = P; c->dm.Q = Q; c->dm.K = K;
+    c->dm.LS = l.LS;
+    c->dm.tournament = prm->tournament;
+    c->dm.NP = prof->NP;
+    c->dm.ND = prof->ND;
+    c->dm.min_tps = prm->min_tps;
+    c->dm.t_a = prm->t_a;
+    c->dm.lam_max = latency_ceiling(prm->min_tps);
+    c->dm.role_search = prm->role_search;
+    c->dm.grows = costs_grow_with_batch(prof, b_max);
+    c->dm.objective = prm->objective;
     c->dm.layered = layered ? 1 : 0;
     c->dm.offload = 0;
     if (devs->mem_cpu)
@@ -393,6 +407,8 @@ int e2_create(const e2_devices *devs, const e2_links *links, const e2_layer_prof
         float f = (float)lm;
         if ((double)f < lm) f = nextafterf(f, HUGE_VALF);
         c->dm.lam_max_up = f;
+        // the fixed-point latency test where its float scale is well inside the range
+        c->dm.lam_fx = lm > 1e-20 && lm < 1e20 ? (float)(4194304.0 / lm) : 0.0f;
     }
     c->cong_lo = links->cong_lo;
     c->cong_hi = links->cong_hi;
@@ -408,8 +424,6 @@ int e2_create(const e2_devices *devs, const e2_links *links, const e2_layer_prof
         if (c->side) cudaStreamDestroy(c->side);
         if (c->ev_fork) cudaEventDestroy(c->ev_fork);
         if (c->ev_join) cudaEventDestroy(c->ev_join);
-        if (c->ev_dp_fork) cudaEventDestroy(c->ev_dp_fork);
-        if (c->ev_dp_join) cudaEventDestroy(c->ev_dp_join);
         delete c;
         return reject(code, why);
     };
@@ -417,19 +431,15 @@ int e2_create(const e2_devices *devs, const e2_links *links, const e2_layer_prof
     int smem_optin = 0;
     if (cudaDeviceGetAttribute(&smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, c->device) != cudaSuccess)
         return fail_free(E2_ECUDA, "cudaDeviceGetAttribute failed");
-    c->dp_threads = 128;
-    c->dm.g_spill = !layered && dp_spills(M, N, c->dp_threads / 32);
-    c->dp_smem = layered ? dp_layered_smem_bytes(M, N) : dp_smem_bytes(M, N, c->dp_threads, 4, c->dm.g_spill);
+    c->dp_smem = layered ? dp_layered_smem_bytes(M, N) : 0;
     if ((M < N ? M : N) > kMaxReplicaDevices)
         return fail_free(E2_EINVAL, "replicas could exceed 256 devices (min(M, N) > 256)");
-    if (c->dp_smem + 1024 > (size_t)smem_optin)
+    if ((layered ? c->dp_smem : dp_size_limit_bytes(M, N)) + 1024 > (size_t)smem_optin)
         return fail_free(E2_EINVAL, "the largest replica's DP does not fit in shared memory (N too large)");
     if (configure_eval(c) != cudaSuccess) return fail_free(E2_ECUDA, "configuring the DP kernel failed");
     if (cudaStreamCreateWithFlags(&c->side, cudaStreamNonBlocking) != cudaSuccess ||
         cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming) != cudaSuccess ||
-        cudaEventCreateWithFlags(&c->ev_join, cudaEventDisableTiming) != cudaSuccess ||
-        cudaEventCreateWithFlags(&c->ev_dp_fork, cudaEventDisableTiming) != cudaSuccess ||
-        cudaEventCreateWithFlags(&c->ev_dp_join, cudaEventDisableTiming) != cudaSuccess)
+        cudaEventCreateWithFlags(&c->ev_join, cudaEventDisableTiming) != cudaSuccess)
         return fail_free(E2_ECUDA, "creating the side stream failed");
 
     unsigned char *ws = static_cast<unsigned char *>(workspace);
@@ -444,10 +454,11 @@ int e2_create(const e2_devices *devs, const e2_links *links, const e2_layer_prof
     if (layered) {
         c->psum = reinterpret_cast<uint64_t *>(ws + l.psum);
         c->lcost = reinterpret_cast<double *>(ws + l.lcost);
-    }
-    if (c->dm.g_spill) {
-        c->gspill = reinterpret_cast<uint32_t *>(ws + l.gspill);
-        c->spill_stride = dp_spill_stride(M, N);
+        c->var_T = reinterpret_cast<double *>(ws + l.var_T);
+        c->var_L = reinterpret_cast<double *>(ws + l.var_L);
+        c->var_mu = reinterpret_cast<int16_t *>(ws + l.var_mu);
+        c->var_layers = reinterpret_cast<int16_t *>(ws + l.var_layers);
+        c->var_best = reinterpret_cast<int32_t *>(ws + l.var_best);
     }
     c->link_bw = reinterpret_cast<double *>(ws + l.link_bw);
     c->cong = reinterpret_cast<double *>(ws + l.cong);
@@ -456,6 +467,8 @@ int e2_create(const e2_devices *devs, const e2_links *links, const e2_layer_prof
     c->tau = reinterpret_cast<double *>(ws + l.tau);
     c->cap = reinterpret_cast<int32_t *>(ws + l.cap);
     c->cpb = reinterpret_cast<float *>(ws + l.cpb);
+    c->drec = reinterpret_cast<uint4 *>(ws + l.drec);
+    c->fxs = reinterpret_cast<float *>(ws + l.fxs);
     c->tau_lb = reinterpret_cast<float *>(ws + l.tau_lb);
     c->leaf_sorted = reinterpret_cast<uint64_t *>(ws + l.leaf_sorted);
     c->beff_sorted = reinterpret_cast<uint64_t *>(ws + l.beff_sorted);
@@ -479,20 +492,30 @@ int e2_create(const e2_devices *devs, const e2_links *links, const e2_layer_prof
     c->elite_cand = reinterpret_cast<int32_t *>(ws + l.elite_cand);
     c->stats = reinterpret_cast<unsigned long long *>(ws + l.stats);
     c->err = reinterpret_cast<int32_t *>(ws + l.err);
-    c->order_bins = reinterpret_cast<unsigned *>(ws + l.order_bins);
+    c->list_ctrl = reinterpret_cast<unsigned *>(ws + l.list_ctrl);
+    c->list_hist = reinterpret_cast<unsigned *>(ws + l.list_hist);
     c->items = reinterpret_cast<uint64_t *>(ws + l.items);
-    c->slot_best = reinterpret_cast<int32_t *>(ws + l.slot_best);
     c->split_T = reinterpret_cast<double *>(ws + l.split_T);
     c->split_L = reinterpret_cast<double *>(ws + l.split_L);
     c->split_mu = reinterpret_cast<int16_t *>(ws + l.split_mu);
+    c->split_code = reinterpret_cast<int16_t *>(ws + l.split_code);
     c->split_layers = reinterpret_cast<int16_t *>(ws + l.split_layers);
     c->slot_off = reinterpret_cast<int32_t *>(ws + l.slot_off);
-    c->slot_mask = reinterpret_cast<uint64_t *>(ws + l.slot_mask);
-    c->slot_size = ws + l.slot_size;
+    c->slot_info = reinterpret_cast<uint32_t *>(ws + l.slot_info);
 
     const size_t V = (size_t)b_max + 1, MM = (size_t)M * M;
     uint64_t *prof_h = new (std::nothrow) uint64_t[kNumProf * V];
     if (!prof_h) return fail_free(E2_ENOMEM, "host allocation failed");
+    float fxs_h[E2_MAX_BATCH + 1];                            // fixed-point scales of the DP's estimate
+    for (size_t v = 0; v < V; ++v) {
+        double least = HUGE_VAL;
+        for (int d = 0; d < M; ++d) {
+            const double t = fmax((double)prof->blk_flops[v] / devs->rate[d], (double)prof->blk_bytes[v] / devs->bw[d]);
+            if (t > 0.0 && t < least) least = t;
+        }
+        const double s = isfinite(least) ? 4194304.0 * least : 1.0;
+        fxs_h[v] = (float)(s < 1e30 ? (s > 1e-30 ? s : 1e-30) : 1e30);
+    }
     const uint64_t *arr[kNumProf] = {prof->blk_flops, prof->blk_bytes, prof->blk_mem, prof->head_flops,
                                      prof->head_bytes, prof->head_mem, prof->act_bytes};
     for (int a = 0; a < kNumProf; ++a) memcpy(prof_h + a * V, arr[a], 8 * V);
@@ -510,6 +533,7 @@ int e2_create(const e2_devices *devs, const e2_links *links, const e2_layer_prof
     chk(cudaMemcpyAsync(c->link_bw, links->bw, 8 * MM, cudaMemcpyHostToDevice, c->stream));
     chk(cudaMemcpyAsync(c->cong, links->cong, 8 * MM, cudaMemcpyHostToDevice, c->stream));
     chk(cudaMemcpyAsync(c->prof, prof_h, 8 * kNumProf * V, cudaMemcpyHostToDevice, c->stream));
+    chk(cudaMemcpyAsync(c->fxs, fxs_h, 4 * V, cudaMemcpyHostToDevice, c->stream));
     if (layered) {
         const size_t row = 8 * V * ((size_t)N + 1);
         chk(cudaMemcpyAsync(c->psum, prof->PF, row, cudaMemcpyHostToDevice, c->stream));
@@ -551,8 +575,7 @@ cudaError_t record_generation(e2_ctx *c, int b)
     c->stream = c->cap_stream;
     e = cudaStreamBeginCapture(c->cap_stream, cudaStreamCaptureModeThreadLocal);
     if (e == cudaSuccess) {
-        cudaError_t le = cudaMemsetAsync(c->stats, 0, 8 * kNumStats, c->stream);
-        if (le == cudaSuccess) le = launch_eval(c, c->pop[b]);
+        cudaError_t le = launch_eval(c, c->pop[b]);
         if (le == cudaSuccess) le = launch_step(c, c->pop[b], c->pop[b ^ 1], 0, 0);
         cudaGraph_t g = nullptr;
         e = cudaStreamEndCapture(c->cap_stream, &g);
@@ -589,8 +612,6 @@ int e2_destroy(e2_ctx *c)
     if (c->side) cudaStreamDestroy(c->side);
     if (c->ev_fork) cudaEventDestroy(c->ev_fork);
     if (c->ev_join) cudaEventDestroy(c->ev_join);
-    if (c->ev_dp_fork) cudaEventDestroy(c->ev_dp_fork);
-    if (c->ev_dp_join) cudaEventDestroy(c->ev_dp_join);
     delete c;
     return e == cudaSuccess ? E2_OK : E2_ECUDA;
 }
@@ -622,7 +643,6 @@ int e2_eval_population(e2_ctx *c, const e2_genomes *genomes, double *fitness_out
         int st = set_and_validate(c, genomes);
         if (st) return st;
     }
-    E2_CUDA(c, cudaMemsetAsync(c->stats, 0, 8 * kNumStats, c->stream));
     E2_CUDA(c, launch_eval(c, c->pop[c->cur]));
     c->evaluated = true;
     c->have_results = true;
@@ -775,7 +795,7 @@ int e2_get_stats(e2_ctx *c, e2_stats *out)
     out->dp_smem = c->dp_smem;
     out->dp_ctas_small = (uint64_t)c->dp_grid1;
     out->dp_smem_small = c->dp_smem1;
-    out->dp_runs_per_cta_small = c->dp_grid1 > 0 ? (c->dp_warp1 ? (uint64_t)kDpWarpRuns : 1u) : 0u;
+    out->dp_runs_per_cta_small = c->dp_grid1 > 0 ? (uint64_t)dp_order_warps(1) : 0u;
     out->launches = c->launches;
     if (out->device_errors)
         return fail(c, E2_EDEVICE, "a device-side consistency check of the last evaluation failed");

@@ -37,50 +37,45 @@ struct DevPop {
 // of a replica per warp in shared memory.
 constexpr int kMaxReplicaDevices = 256;
 
-// Buckets of the work ordering of the evaluation: 64 levels (the rank of a
-// variant among its replica's variants, largest batch first) x 16 work sizes,
-// once per shared-memory class of the DP (class 0: every replica size; class
-// 1, where it exists: the sizes whose DP fits in the smaller allocation that
-// lets more CTAs share an SM).
-constexpr int kOrderBins = 1024;
-constexpr int kSizeBins = 16;
-constexpr int kDpClasses = 2;
-constexpr int kAllBins = kDpClasses * kOrderBins;
-// Control words after the ordering bins: where each class's items end (class
-// 1's follow class 0's), each class's DP cursor (starting where its items
-// start), the pre-pass's warp ticket.
-enum CtrlWord { kCtrlEnd = kAllBins, kCtrlNext = kCtrlEnd + kDpClasses, kCtrlTicket = kCtrlNext + kDpClasses,
-                kCtrlWords };
+// The DP's work list: items in kListBins bins of replica sizes (class 0 before
+// class 1, larger first), placed from per-block counts of the slots' items by
+// at most kListBlocks blocks.
+constexpr int kListBins = 64;
+constexpr int kListBlocks = 256;
+// Its control words: where each class's items end (class 1's follow class
+// 0's) and each class's DP cursor (starting where its items start).
+enum CtrlWord { kCtrlEnd = 0, kCtrlNext = 2, kCtrlWords = 4 };
 
-// Shared memory of one DP run on a replica of m devices over N blocks, with
-// `warps` warps per CTA and `key_bytes`-byte order keys: the per-device
-// counters, the cost rows and the prefix and suffix columns ([m][W] each),
-// the per-warp rows, the head row, the empty stage, the link and head keys and
-// the device ids (rounded up to 16 bytes).  No slack: a few bytes more per CTA
-// can cost a CTA per SM (the 80-block model's largest DP, 22,208 B, fits 10
-// per SM; 16 B more fit 9).
-//
-// With `spill` the suffix columns live in a global scratch (L2) and shared
-// memory keeps two of them (the chain's previous and current column) plus a
-// per-warp buffer the master combine stages its suffix column into: about a
-// third less shared memory for the large replicas, and more CTAs per SM.
-__host__ __device__ __forceinline__ unsigned dp_item_bytes(int m, int N, int warps, int key_bytes, bool spill = false)
+// A slot's info word: the largest decode batch to run (0: none), the largest
+// its memory allows, whether the prefill run can matter, which tests were
+// made, and the bin of its size in the work list.
+constexpr uint32_t kSlotDecMask = 0x7F;
+constexpr int kSlotMemShift = 7;
+constexpr uint32_t kSlotPrefill = 1u << 14, kSlotDecTested = 1u << 15, kSlotPreTested = 1u << 16;
+constexpr int kSlotBinShift = 24;
+
+// Shared memory the limits of the ABI are stated in: an input whose largest
+// replica (m devices, W = N - m + 1 block counts) would need more than an SM
+// has in this layout -- per device three counters, two cost rows (three below
+// 40 KB), the link and head keys and the id, and the work rows of four warps
+// -- is refused by e2_create.
+__host__ __forceinline__ size_t dp_table_bytes(int m, int N, bool spill)
 {
-    const unsigned W = (unsigned)(N - m + 1);
-    const unsigned gcols = spill ? 2u : (unsigned)m;
-    const unsigned keys = 2u * (unsigned)m * W + gcols * W + (unsigned)((spill ? 3 : 2) * warps + 2) * W +
-                          2u * (unsigned)m;
-    const unsigned bytes = (unsigned)m * 12u + keys * (unsigned)key_bytes + (unsigned)m * 2u;
-    return (bytes + 15u) & ~15u;
+    const size_t W = (size_t)(N - m + 1), mm = (size_t)m;
+    const size_t keys = 2 * mm * W + (spill ? 2 : mm) * W + (spill ? 14 : 10) * W + 2 * mm;
+    return (mm * 12 + keys * 4 + mm * 2 + 15) & ~(size_t)15;
 }
-
-// Whether the DP spills its suffix columns (see dp_item_bytes): when the
-// largest replica's run would otherwise need more than kSpillAbove bytes of
-// shared memory (fewer than five CTAs per SM), as with the 126-block model.
-// A function of the sizes alone, so that the workspace size can include the
-// scratch: kSpillCtas persistent CTAs at most, each with room for the largest
-// run's suffix columns.
-constexpr unsigned kSpillAbove = 40u * 1024u;
+__host__ __forceinline__ size_t dp_size_limit_bytes(int M, int N)
+{
+    const int mmax = M < N ? M : N;
+    size_t best[2] = {0, 0};
+    for (int m = 1; m <= mmax; ++m)
+        for (int s = 0; s < 2; ++s) {
+            const size_t b = dp_table_bytes(m, N, s != 0);
+            if (b > best[s]) best[s] = b;
+        }
+    return best[0] > 40u * 1024u ? best[1] : best[0];
+}
 // Slots of the duplicate test's fingerprint table: the power of two >= 2P.
 __host__ __device__ __forceinline__ unsigned dup_table_size(int P)
 {
@@ -88,28 +83,6 @@ __host__ __device__ __forceinline__ unsigned dup_table_size(int P)
     while (t < 2u * (unsigned)P) t <<= 1;
     return t;
 }
-constexpr int kSpillCtas = 4096;
-__host__ __forceinline__ bool dp_spills(int M, int N, int warps)
-{
-    const int mmax = M < N ? M : N;
-    unsigned best = 0;
-    for (int m = 1; m <= mmax; ++m) {
-        const unsigned b = dp_item_bytes(m, N, warps, 4, false);
-        if (b > best) best = b;
-    }
-    return best > kSpillAbove;
-}
-__host__ __forceinline__ size_t dp_spill_stride(int M, int N)   // keys per CTA: max over m of m * W
-{
-    const int mmax = M < N ? M : N;
-    size_t best = 0;
-    for (int m = 1; m <= mmax; ++m) {
-        const size_t k = (size_t)m * (size_t)(N - m + 1);
-        if (k > best) best = k;
-    }
-    return (best + 3) & ~(size_t)3;
-}
-
 // Stats slots (unsigned long long, atomically accumulated).
 enum StatSlot { kStGenomes = 0, kStReplicas, kStDpRuns, kStCells, kStProbes, kStPaper, kStPrecheck,
                 kStServed, kStTpsPruned, kStDpRunsSmall, kStRoleCapped, kStDeviceErrors, kNumStats };
@@ -125,16 +98,14 @@ struct Dims {
     int role_search;     // 1: both roles per replica, best assignment per genome (Alg. 2);
                          // 2: both roles per replica, the adapted-SplitWise rule picks the roles
     float lam_max_up;    // lam_max rounded up to float (the float latency bound is compared with it)
-    unsigned dp_small;   // shared-memory bytes of DP class 1 (0: one class); m is in class 1 iff
-                         // dp_item_bytes(m, N, dp_warps, 4, false) <= dp_small (class 1 never spills)
-    int dp_warps;        // warps of a class-1 run's layout: 1 when class 1 runs one run per warp
+    int dp_mmax;         // min(M, N): the largest replica's devices
+    int dp_split;        // DP class 0: the replicas of at most this many devices (0: all of them)
+    float lam_fx;        // 2^22 / lam_max for the fixed-point latency test (0: not used)
     int grows;           // 1: block memory, head memory, block flops and bytes and activation bytes never
                          // shrink from one decode batch to the next (the pre-pass tests are then monotone)
     int objective;       // 0: waiting time w (Eq. 3-5); 1: per-request finishing time FT
     int offload;         // 1: some device has host memory for offloaded blocks
     int layered;         // 1: blocks of several types (per-layer prefix sums): the plain-scan DP path
-    int g_spill;         // 1: the DP keeps its suffix columns in the global scratch (dp_item_bytes)
-    int dp_grid0;        // CTAs of the first DP launch (the ones with a suffix-column scratch)
 };
 
 struct Tables {
@@ -154,29 +125,39 @@ struct Tables {
     const uint32_t *tau_rank;  // [V][M][M]
     const double *lcost;       // [V][M][2][N][N] (per-layer profiles only): lcost[((v*M+d)*2+mf)*N*N + j*N + n-1]
                                // = time of blocks j..j+n-1 on device d (+inf beyond the model or memory)
+    const uint4 *drec;         // [V][M] the DP's view of a device: {cap | cap with head << 16, and as floats
+                               // 1 / block time, the head in blocks, host block rate / device block rate}
+    const float *fxs;          // [V] 2^22 / the largest 1 / block time: its fixed-point scale
 };
 
 // Per (genome, replica slot) results of the evaluation pre-pass.
 struct SlotInfo {
     int32_t *off;              // [P*K] offset of the replica in the ordering chromosome
-    uint64_t *mask;            // [P*K] variants to run (bit i: prefill v=0 / decode v=i+1)
-    uint8_t *size;             // [P*K] log-scale work size of one DP run of the slot | DP class << 4
-    int32_t *best;             // [P*K] largest variant bit accepted so far (-1: none)
+    uint32_t *info;            // [P*K] its verdicts (kSlot*)
 };
 
-// Work items of the DP: (slot << 8) | role << 7 | sweep << 6 | variant bit.
+// Work items of the DP: (slot << 8) | role << 7 | variant bit.
 struct WorkList {
-    uint64_t *items;           // [P*K*(b_max+1)] (slot << 8) | role << 7 | sweep << 6 | variant bit
-    unsigned *ctrl;            // [kAllBins] bins/cursors, then the CtrlWord words
-    uint32_t *gspill;          // [kSpillCtas][spill_stride] suffix columns of each persistent DP CTA
-    unsigned spill_stride;     // keys per CTA
+    uint64_t *items;           // [2*P*K] (per-layer profiles: [V*P*K])
+    unsigned *ctrl;            // [kCtrlWords]
 };
 
-// Results of the DP runs, per (slot, variant bit).
+// Results per (slot, role) where both roles are evaluated (role_search); with
+// roles in the genome the DP writes the replica's outputs directly.
 struct SplitOut {
-    double *T, *L;             // [P*K*b_max]
-    int16_t *mu;               // [P*K*b_max]
-    int16_t *layers;           // [P*b_max][M]
+    double *T, *L;             // [P*K][2]
+    int16_t *mu;               // [P*K][2]
+    int16_t *code;             // [P*K][2] the accepted variant's bit (prefill: 0), -1: none
+    int16_t *layers;           // [P][2][M]
+};
+
+// Results per (slot, variant) of per-layer profiles, whose batches run as
+// separate items (prefill: variant 0, decode batch b: variant b).
+struct VariantOut {
+    double *T, *L;             // [P*K][V]
+    int16_t *mu;               // [P*K][V]
+    int16_t *layers;           // [P][V][M]
+    int32_t *best;             // [P*K] largest batch accepted so far - 1 (-1: none)
 };
 
 struct EvalOut {
@@ -283,24 +264,24 @@ struct e2_ctx {
     int32_t *elite_cand = nullptr;             // [P] its candidates
     unsigned long long *stats = nullptr;
     int32_t *err = nullptr;
-    unsigned *order_bins = nullptr;   // [kCtrlWords]
-    uint64_t *items = nullptr;        // [P*K*b_max] DP work items, heaviest first
-    uint32_t *gspill = nullptr;       // suffix-column scratch of the DP CTAs (dm.g_spill only)
-    size_t spill_stride = 0;          // its keys per CTA
+    unsigned *list_ctrl = nullptr;    // [kCtrlWords]
+    unsigned *list_hist = nullptr;    // [kListBlocks][kListBins]
+    uint64_t *items = nullptr;        // [2*P*K] DP work items, largest replicas first
     int32_t *slot_off = nullptr;      // [P*K]
-    uint64_t *slot_mask = nullptr;    // [P*K]
-    uint8_t *slot_size = nullptr;     // [P*K]
-    int32_t *slot_best = nullptr;     // [P*K]
-    double *split_T = nullptr, *split_L = nullptr;   // [P*K*b_max]
-    int16_t *split_mu = nullptr;                     // [P*K*b_max]
-    int16_t *split_layers = nullptr;                 // [P*b_max*M]
+    uint32_t *slot_info = nullptr;    // [P*K]
+    uint4 *drec = nullptr;            // [V][M]
+    float *fxs = nullptr;             // [V]
+    double *split_T = nullptr, *split_L = nullptr;   // [P*K][2]
+    int16_t *split_mu = nullptr, *split_code = nullptr;   // [P*K][2]
+    int16_t *split_layers = nullptr;                 // [P][2][M]
+    double *var_T = nullptr, *var_L = nullptr;       // [P*K][V] (layered)
+    int16_t *var_mu = nullptr, *var_layers = nullptr;   // [P*K][V], [P][V][M] (layered)
+    int32_t *var_best = nullptr;                     // [P*K] (layered)
     mutable unsigned long long launches = 0;   // kernels launched (a graph replay adds its kernel nodes)
     unsigned long long gen_kernels[2] = {0, 0}; // kernel nodes of each recorded generation
     int dp_grid = 0;                  // persistent DP CTAs of class 0
     int dp_grid1 = 0;                 // persistent DP CTAs of class 1 (0: one class)
-    size_t dp_smem1 = 0;              // their shared memory (per warp with dp_warp1)
-    int dp_warp1 = 0;                 // 1: class 1 runs one DP run per warp (dp_warp.cu)
-    cudaEvent_t ev_dp_fork = nullptr, ev_dp_join = nullptr;   // class 1 runs on the side stream
+    size_t dp_smem1 = 0;              // their shared memory
     cudaEvent_t ev_dp_start = nullptr, ev_dp_stop = nullptr;   // optional timing hook
     // recorded generation (e2_run_generation), one per population buffer
     cudaStream_t cap_stream = nullptr;                          // private stream the graphs are recorded on
@@ -309,9 +290,7 @@ struct e2_ctx {
     cudaGraphNode_t gen_ga_node[2] = {nullptr, nullptr};        // the generation kernel's node
     cudaEvent_t gen_ev[2][2] = {{nullptr, nullptr}, {nullptr, nullptr}};   // timing events recorded in it
     bool gen_eager = false;                                     // recording failed: eager launches
-    // launch shapes
-    int dp_threads = 128;
-    size_t dp_smem = 0;
+    size_t dp_smem = 0;               // shared memory of class 0's CTAs
     bool evaluated = false;
     bool have_elites = false;
     bool have_results = false;           // an evaluation has filled the result buffers
@@ -335,15 +314,15 @@ cudaError_t launch_step(const e2_ctx *c, const DevPop &src, const DevPop &dst, u
 cudaError_t find_ga_node(cudaGraph_t graph, cudaGraphNode_t *node);
 cudaError_t set_ga_node(const e2_ctx *c, cudaGraphExec_t exec, cudaGraphNode_t node, const DevPop &src,
                         const DevPop &dst, uint64_t seed, uint32_t gen);
-size_t dp_smem_bytes(int M, int N, int threads, int key_bytes, bool spill = false);
-// The warp-per-run DP kernel of the small replica sizes (dp_warp.cu): its CTA
-// size, its CTAs per SM with `slice` bytes of shared memory per warp, and its
-// launch on `stream` over class 1 of the work list.
-constexpr int kDpWarpRuns = 4;
-cudaError_t dp_warp_occupancy(unsigned slice, int *per_sm);
-cudaError_t dp_warp_launch(int grid, unsigned slice, cudaStream_t stream, const Dims &dm, const Tables &tb,
-                           const DevPop &pop, const EvalOut &out, const WorkList &wl, const SlotInfo &si,
-                           const SplitOut &so);
+// The DP of identical blocks (dp_order.cu) over class cls of the work list,
+// for replicas of up to mmax devices, a run per warp: warps per CTA, shared
+// memory per CTA, CTAs per SM and the launch.
+__host__ __device__ constexpr int dp_order_warps(int cls) { return cls ? 4 : 12; }
+size_t dp_order_smem(int mmax, int cls);
+cudaError_t dp_order_occupancy(int mmax, int cls, bool off, int *per_sm);
+cudaError_t dp_order_launch(int grid, int mmax, int cls, cudaStream_t stream, const Dims &dm, const Tables &tb,
+                            const DevPop &pop, const EvalOut &out, const WorkList &wl, const int32_t *slot_off,
+                            const SplitOut &so);
 size_t dp_layered_smem_bytes(int M, int N);   // the plain-scan DP's shared memory for the largest replica
 cudaError_t configure_eval(e2_ctx *c);   // shared memory limit and persistent grid size
 size_t rank_pow2(size_t n);

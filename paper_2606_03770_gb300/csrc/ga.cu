@@ -107,10 +107,13 @@ __global__ void layered_tables_kernel(Dims dm, const double *rate, const double 
 // the G--C split; -1 where the head does not fit), and the per-block time
 // rounded down to float, used by the latency bound: max(blk_flops/rate,
 // blk_bytes/bw), or the host's per-block time where that is smaller and the
-// device offloads (a lower bound on every block's time either way).
+// device offloads (a lower bound on every block's time either way).  drec
+// gathers what the DP's estimate needs of a device in 16 bytes (Tables); the
+// head in blocks is how much later its row reaches a count of a few blocks.
 __global__ void captab_kernel(Dims dm, const double *rate, const double *bw, const uint64_t *mem,
                               const double *rate_cpu, const double *bw_cpu, const uint64_t *mem_cpu,
-                              const uint64_t *prof, int32_t *cap, int32_t *capg, float *cpb)
+                              const uint64_t *prof, const double *leaf, int32_t *cap, int32_t *capg, float *cpb,
+                              uint4 *drec)
 {
     const size_t total = (size_t)dm.V * dm.M;
     for (size_t idx = blockIdx.x * (size_t)blockDim.x + threadIdx.x; idx < total;
@@ -131,13 +134,28 @@ __global__ void captab_kernel(Dims dm, const double *rate, const double *bw, con
         const double tc = __ull2double_rn(prof[kBlkFlops * V + v]) / rate[d];
         const double tm = __ull2double_rn(prof[kBlkBytes * V + v]) / bw[d];
         double t = tc >= tm ? tc : tm;
+        const double tdev = t;
+        float ratio = 0.0f;                                          // host block rate / device block rate
         if (dm.offload && hc > 0) {
             const double hc_ = __ull2double_rn(prof[kBlkFlops * V + v]) / rate_cpu[d];
             const double hb = __ull2double_rn(prof[kBlkBytes * V + v]) / bw_cpu[d];
             const double th = hc_ >= hb ? hc_ : hb;
+            ratio = th > 0.0 ? (float)fmin(tdev / th, 1e6) : 1e6f;
             t = th < t ? th : t;
         }
         cpb[idx] = __double2float_rd(t);
+        const float cinv = tdev > 1e-30 ? (float)(1.0 / tdev) : 1e30f;
+        float head = 1e6f;
+        const int nr = c1 < 4 ? (int)c1 : N < 4 ? (int)N : 4;
+        if (nr >= 1 && tdev > 0.0) {
+            const double *row = leaf + (size_t)idx * 2 * dm.LS;
+            const double x = (row[dm.LS + nr - 1] - row[nr - 1]) / tdev;
+            if (x >= 0.0 && x < 1e6) head = (float)x;
+        } else if (nr >= 1) {
+            head = 0.0f;
+        }
+        drec[idx] = make_uint4((uint32_t)cap[idx * 2] | (uint32_t)cap[idx * 2 + 1] << 16, __float_as_uint(cinv),
+                               __float_as_uint(head), __float_as_uint(ratio));
     }
 }
 
@@ -803,7 +821,8 @@ cudaError_t launch_tables(const e2_ctx *c)
                                                                 c->mem_cpu, c->prof, c->leaf);
     const size_t vm = (size_t)c->dm.V * c->dm.M;
     captab_kernel<<<grid_for(vm, 256), 256, 0, c->stream>>>(c->dm, c->rate, c->bw, c->mem, c->rate_cpu, c->bw_cpu,
-                                                             c->mem_cpu, c->prof, c->cap, c->capg, c->cpb);
+                                                             c->mem_cpu, c->prof, c->leaf, c->cap, c->capg, c->cpb,
+                                                             c->drec);
     c->launches += 2;
     if (c->dm.layered) {
         const size_t lt = (size_t)c->dm.V * c->dm.M * 2 * c->dm.N * c->dm.N;
