@@ -30,10 +30,6 @@ __device__ __forceinline__ int warp_sum(int x) { return __reduce_add_sync(0xFFFF
 
 }  // namespace
 
-// Shared-memory bytes per warp of the pre-pass (18 bytes per device, rounded
-// up to 16 so that every warp's arrays start aligned).
-__host__ __device__ __forceinline__ size_t variant_stride(int mcap) { return ((size_t)mcap * 18 + 15) & ~(size_t)15; }
-
 // Bin of a replica of m devices in the work list: with two DP classes, the
 // sizes up to dp_split (class 0) take bins 0..31 and the larger ones bins
 // 32..63; larger first within a class.
@@ -45,191 +41,260 @@ __device__ __forceinline__ uint32_t size_bin(const Dims &dm, int m)
     return (uint32_t)(kListBins - 1 - (m - dm.dp_split - 1) * half / (dm.dp_mmax - dm.dp_split));
 }
 
-// Pre-pass, one warp per (genome, replica slot).  For each
+// Pre-pass, one block per genome, a warp per replica at a time.  For each
 // variant of the replica (prefill: v = 0; decode: v = 1..b_max, bit v-1) the
 // warp decides whether a DP run can matter:
 //  * memory: with identical blocks a partition with master mu exists iff every
 //    device holds >= 1 block and the capacities, capped at W = N - m + 1, add
 //    up to N (exact);
 //  * decode latency: Lambda >= sum of link times + sum_k n_k c_k (c_k the
-//    per-block time, the head only adds), whose least value puts one block on
-//    each device and the other N - m on the cheapest devices up to their
-//    capacity.  It is summed in float from times rounded down, every operation
-//    rounded toward -inf, so it never exceeds the exact bound; a variant whose
-//    bound is above Lambda_max (rounded up to float) fails whatever partition
-//    the DP returns.
+//    per-block time; the head only adds), at least, for any price x >= 0,
+//        x (N - m) + sum_k c_k + sum_{c_k < x} (cap_k - 1) (c_k - x)
+//    (the linear program's dual: one block on each device, the other N - m
+//    bought at x, less what devices cheaper than x save).  The block time of
+//    the marginal device, up to which the cheaper devices just hold N - m more
+//    blocks, gives the program's own optimum; it is found by bisection at the
+//    first batch tested and kept for the others.  All in float from times rounded down, every operation rounded toward -inf, so
+//    the bound never exceeds the exact value; a variant whose bound is above
+//    Lambda_max (rounded up to float) fails whatever partition the DP returns.
 // Both tests are monotone in the batch: the capacities shrink as b grows (more
-// KV memory per block), and the bound is the least of a linear cost whose
-// coefficients (per-block and link times) grow with b over a feasible set that
-// shrinks with b, when the profile's costs grow with the batch (physical
-// profiles do; checked at e2_create).  So the largest batch the memory allows
-// is found by a search (the largest batch first, then the smallest, then
-// bisection), and the largest the bound keeps by a second search below it;
-// every smaller batch is kept.  A failed test is exact (memory) or a proof
-// (the bound never exceeds the exact value), so every batch above it fails
-// too; rounding can only keep a variant the exact bound would drop, which
-// costs a DP run and changes no result.  Other profiles test every batch from
-// the largest down, and the first that passes keeps the smaller ones.
+// KV memory per block), and the program's optimum is the least of a linear
+// cost whose coefficients (per-block and link times) grow with b over a
+// feasible set that shrinks with b, when the profile's costs grow with the
+// batch (physical profiles do; checked at e2_create).  So the largest batch the
+// memory allows is found by a search (the largest batch first, then the
+// smallest, then bisection), and the largest the bound keeps by a second
+// search below it; every smaller batch is kept.  A failed test is exact
+// (memory) or a proof (the bound never exceeds the optimum, and the optimum
+// of every larger batch is no smaller), so every batch above it fails too;
+// rounding and the price can only keep a variant the optimum would drop,
+// which costs a DP run and changes no result.  Other profiles test every
+// batch from the largest down, and the first that passes keeps the smaller
+// ones.
 // The verdicts go into the slot's info word (SlotBits), with the bin of its
 // size in the work list's order.  A replica with nothing to run (more devices
-// than blocks, no variant left) gets its outputs here, and the genome's last
-// replica writes those of its empty slots.
-__global__ void __launch_bounds__(64, 20) slot_kernel(Dims dm, Tables tb, DevPop pop, SlotInfo si, EvalOut out,
-                                                       SplitOut so, VariantOut vo)
+// than blocks, no variant left) gets its outputs here, and so do the empty
+// slots.
+//
+// Bound by the chain of dependent reads per replica (device, its record and
+// link, the verdicts).  Per device one 16-byte record serves every variant
+// (1 / rate, 1 / bandwidth, the capacities of the smallest and the largest
+// batch), and one 1 / bandwidth per link every batch's link time, so a second
+// variant reads nothing.
+constexpr int kPreWarps = 8;
+
+// A replica's devices for the pre-pass: lane k holds device k (SMALL: at most
+// 32 devices) or visits devices k, k + 32, ...
+template <bool SMALL, typename F>
+__device__ __forceinline__ void each_device(int m, int lane, F f)
 {
-    // per warp: device ids, capacities and per-block times of up to mcap devices
-    extern __shared__ __align__(16) unsigned char vsm[];
-    const int mcap = dm.M < dm.N ? dm.M : dm.N;
-    const int lane = threadIdx.x & 31, wl = threadIdx.x >> 5;
-    const int K = dm.K, M = dm.M, N = dm.N;
-    const long long slot = (long long)blockIdx.x * (blockDim.x >> 5) + wl;
-    if (slot < (long long)dm.P * K) {
-        const int g = (int)(slot / K), c = (int)(slot - (long long)g * K);
-        // the genome's replica count, sizes and roles, loaded together (all in bounds)
-        const uint16_t *sz = pop.sizes + (size_t)g * K;
-        const int R = pop.nclus[g];
-        const int m_c = sz[c];
-        const uint64_t roles = pop.roles[g];
-        const int s_lo = lane < c ? sz[lane] : 0, s_hi = lane + 32 < c ? sz[lane + 32] : 0;
-        uint32_t info = 0;
-        int m = 0, off = 0, role = 0;
-        if (c < R) {
-            m = m_c;
-            role = (int)((roles >> c) & 1ull);
-            off = warp_sum(s_lo) + warp_sum(s_hi);
-            if (lane == 0) si.off[slot] = off;
-        }
-        if (c < R && m <= N) {
-            const int W = N - m + 1;
-            unsigned char *wbase = vsm + (size_t)wl * variant_stride(mcap);
-            uint32_t *scb = reinterpret_cast<uint32_t *>(wbase);          // per-block times (float bits)
-            float *stau = reinterpret_cast<float *>(scb + mcap);          // link (k-1) -> k
-            int *sc0 = reinterpret_cast<int *>(stau + mcap), *sc1 = sc0 + mcap;
-            uint16_t *sdev = reinterpret_cast<uint16_t *>(sc1 + mcap);
-            for (int k = lane; k < m; k += 32) sdev[k] = pop.perm[(size_t)g * M + off + k];
-            __syncwarp();
-            // with the role search, the decode sweep and then the prefill variant
-            // (its result goes to bit b_max); otherwise the genome's role only
-            const int npass = dm.role_search ? 2 : 1;
-            // Stage variant i (capacities, and the per-block and link times
-            // when the latency bound applies) and return its memory verdict.
-            auto stage = [&](int prole, int i, bool bound) -> bool {
-                const int v = prole ? i + 1 : 0;
-                const int32_t *cap = tb.cap + (size_t)v * M * 2;
-                const float *cpb = tb.cpb + (size_t)v * M;
-                const float *tau = tb.tau_lb + (size_t)v * M * M;
-                int s0 = 0, z = 0;
-                __syncwarp();
-                for (int k = lane; k < m; k += 32) {                   // every load of the variant at once
-                    const int d = sdev[k];
-                    const int c0 = min(cap[d * 2], W), c1 = min(cap[d * 2 + 1], W);
-                    if (bound) {
-                        scb[k] = __float_as_uint(cpb[d]);               // non-negative: bits order as values
-                        stau[k] = k ? tau[(size_t)sdev[k - 1] * M + d] : 0.0f;
-                    }
-                    sc0[k] = c0;
-                    sc1[k] = c1;
-                    s0 += c0;
-                    z += c0 == 0;
-                }
-                s0 = warp_sum(s0);
-                z = warp_sum(z);
-                __syncwarp();
-                bool ok = false;
-                for (int k = lane; k < m && !ok; k += 32)
-                    ok = (z - (sc0[k] == 0)) == 0 && sc1[k] >= 1 && s0 - sc0[k] + sc1[k] >= N;
-                return __any_sync(0xFFFFFFFFu, ok);
-            };
-            // The latency bound of the staged variant, against Lambda_max.
-            auto fast_enough = [&]() -> bool {
-                float part = 0.0f;
-                for (int k = lane; k < m; k += 32) {
-                    const uint32_t ck = scb[k];
-                    int before = 0;                  // capacity of the cheaper devices
-                    for (int j = 0; j < m; ++j) {
-                        const uint32_t cj = scb[j];
-                        if (cj < ck || (cj == ck && j < k)) before += sc0[j] - 1;
-                    }
-                    const int ek = sc0[k] - 1;
-                    const int room = (N - m) - before;
-                    const int take = room <= 0 ? 0 : (room < ek ? room : ek);
-                    part = __fadd_rd(part, __fmul_rd(__uint_as_float(ck), (float)(1 + take)));
-                    if (k >= 1) part = __fadd_rd(part, stau[k]);
-                }
+    if (SMALL) {
+        if (lane < m) f(lane);
+    } else {
+        for (int k = lane; k < m; k += 32) f(k);
+    }
+}
+
+// Whether the capacities (without | with the head << 16 of each device) admit
+// a partition of N blocks.
+template <bool SMALL, typename Caps>
+__device__ __forceinline__ bool memory_ok(int m, int N, int lane, Caps caps)
+{
+    const int W = N - m + 1;
+    int s = 0;
+    uint32_t own = 0;
+    each_device<SMALL>(m, lane, [&](int k) {
+        const uint32_t x = caps(k);
+        own = x;
+        const int c0 = min((int)(x & 0xFFFFu), W);
+        s += c0 + (c0 == 0 ? 1 << 20 : 0);
+    });
+    s = warp_sum(s);
+    const int zero = s >> 20, S = s & 0xFFFFF;
+    bool ok = false;
+    each_device<SMALL>(m, lane, [&](int k) {
+        const uint32_t x = SMALL ? own : caps(k);
+        const int c0 = min((int)(x & 0xFFFFu), W), c1 = min((int)(x >> 16), W);
+        ok |= zero - (c0 == 0) == 0 && c1 >= 1 && S - c0 + c1 >= N;
+    });
+    return __any_sync(0xFFFFFFFFu, ok);
+}
+
+__device__ __forceinline__ float warp_sum_rd(float x)
+{
 #pragma unroll
-                for (int o = 16; o; o >>= 1) part = __fadd_rd(part, __shfl_xor_sync(0xFFFFFFFFu, part, o));
-                return !(part > dm.lam_max_up);                         // 1.0 / Lambda >= Min_TPS possible
-            };
-            for (int pass = 0; pass < npass; ++pass) {
-                const int prole = dm.role_search ? (pass == 0) : role;
-                const int nvar = prole ? dm.b_max : 1;
-                if (dm.layered) {                           // per-layer profiles: every variant runs (the
-                    if (prole) info |= (uint32_t)nvar | (uint32_t)nvar << kSlotMemShift;   // tests assume
-                    else info |= kSlotPrefill;                                          // identical blocks)
-                    continue;
-                }
-                const bool bound = prole && dm.min_tps > 0.0;
-                // When the costs grow with the batch both verdicts are monotone,
-                // so each is found by a search over the variants: the largest
-                // first (it usually decides), then the smallest, then bisection
-                // between the largest known pass (lo) and the smallest known
-                // failure (hi).  The memory search comes first; the bound then
-                // searches the variants the memory allows.  Otherwise each
-                // variant is tested from the largest down, and the first that
-                // passes both keeps the smaller ones.
-                int lo = -1, hi = nvar, next = nvar - 1, staged = -1, bm = -1;
-                bool tps = false;
-                while (hi - lo > 1) {
-                    bool pass = true;
-                    if (staged != next) {
-                        pass = stage(prole, next, bound);
-                        staged = next;
-                    }
-                    if (tps && pass) pass = fast_enough();
-                    if (pass) lo = next;
-                    else hi = next;
-                    if (!tps && hi - lo <= 1) {                 // the memory search is done
-                        bm = lo;
-                        if (!bound || bm < 0) break;
-                        tps = true;
-                        lo = -1;
-                        hi = bm + 1;
-                        next = bm;
-                        continue;
-                    }
-                    next = !dm.grows ? hi - 1 : lo < 0 ? 0 : (lo + hi) >> 1;
-                }
-                const int bs = tps ? lo : bm;               // largest variant both tests keep
-                if (prole) info |= kSlotDecTested | (uint32_t)(bs + 1) | (uint32_t)(bm + 1) << kSlotMemShift;
-                else info |= kSlotPreTested | (bs >= 0 ? kSlotPrefill : 0u);
+    for (int o = 16; o; o >>= 1) x = __fadd_rd(x, __shfl_xor_sync(0xFFFFFFFFu, x, o));
+    return x;
+}
+
+// The decode verdicts of a replica on devices dev[0..m-1]: the largest batch
+// its memory allows and, of those, the largest the latency bound keeps.
+template <bool SMALL>
+__device__ __forceinline__ uint32_t decode_verdict(const Dims &dm, const Tables &tb, const uint16_t *dev, int m, int lane)
+{
+    const int M = dm.M, N = dm.N, W = N - m + 1, need = N - m;
+    const bool timed = dm.min_tps > 0.0;                   // the latency bound applies
+    // lane k's device and its link, kept; the devices beyond 32 are read again
+    const uint4 mine = lane < m ? tb.prec[dev[lane]] : make_uint4(0, 0, 0, 0);
+    float X = 0.0f;                                        // sum of the links' 1 / bandwidth
+    if (timed) each_device<SMALL>(m, lane, [&](int k) {
+        if (k >= 1) X = __fadd_rd(X, tb.ibw[(size_t)dev[k - 1] * M + dev[k]]);
+    });
+    auto rec = [&](int k) -> uint4 { return SMALL || k == lane ? mine : tb.prec[dev[k]]; };
+    auto caps = [&](int k, int v) -> uint32_t {
+        if (v == 1) return rec(k).z;
+        if (v == dm.b_max) return rec(k).w;
+        return tb.capv[(size_t)dev[k] * dm.V + v];
+    };
+    if (timed) X = warp_sum_rd(X);
+    auto mem_of = [&](int v) { return memory_ok<SMALL>(m, N, lane, [&](int k) { return caps(k, v); }); };
+    // the marginal device: the price is its block time (found once, at the first
+    // batch tested: which devices are cheap hardly depends on the batch)
+    int marginal = -1;
+    auto fast_enough = [&](int v) -> bool {
+        const float4 q = tb.fpr[v];                        // block flops and bytes, activation bytes, rounded down
+        auto cost = [&](int k) -> float {                  // a block's time, rounded down
+            const uint4 r = rec(k);
+            float t = fmaxf(__fmul_rd(q.x, __uint_as_float(r.x)), __fmul_rd(q.y, __uint_as_float(r.y)));
+            if (dm.offload) {
+                const float2 h = tb.prech[dev[k]];
+                if (h.x > 0.0f) t = fminf(t, fmaxf(__fmul_rd(q.x, h.x), __fmul_rd(q.y, h.y)));
             }
+            return t;
+        };
+        float c_own = 0.0f;
+        int e_own = 0;
+        if (lane < m) {
+            c_own = cost(lane);
+            e_own = min((int)(caps(lane, v) & 0xFFFFu), W) - 1;
+        }
+        auto c_of = [&](int k) -> float { return SMALL || k == lane ? c_own : cost(k); };
+        auto e_of = [&](int k) -> int { return SMALL || k == lane ? e_own : min((int)(caps(k, v) & 0xFFFFu), W) - 1; };
+        float price = 0.0f;
+        if (need > 0) {
+            if (marginal < 0) {
+                uint32_t lo = 0x7F800000u, hi = 0;         // (bits order as the non-negative values)
+                each_device<SMALL>(m, lane, [&](int k) {
+                    const uint32_t x = __float_as_uint(c_of(k));
+                    lo = min(lo, x);
+                    hi = max(hi, x);
+                });
+                lo = __reduce_min_sync(0xFFFFFFFFu, lo);
+                hi = __reduce_max_sync(0xFFFFFFFFu, hi);
+                for (int it = 0; it < 7 && lo < hi; ++it) {
+                    const uint32_t mid = lo + ((hi - lo) >> 1);
+                    int s = 0;
+                    each_device<SMALL>(m, lane, [&](int k) { if (__float_as_uint(c_of(k)) <= mid) s += e_of(k); });
+                    if (warp_sum(s) >= need) hi = mid;
+                    else lo = mid + 1;
+                }
+                // the dearest device at or below the price found (there is one: the cheapest)
+                unsigned best = 0;
+                int at = 0;
+                each_device<SMALL>(m, lane, [&](int k) {
+                    const uint32_t x = __float_as_uint(c_of(k));
+                    if (x <= hi && x >= best) { best = x; at = k; }
+                });
+                const unsigned top = __reduce_max_sync(0xFFFFFFFFu, best);
+                marginal = (int)__reduce_max_sync(0xFFFFFFFFu, best == top && lane < m ? (unsigned)at : 0u);
+            }
+            price = SMALL ? __shfl_sync(0xFFFFFFFFu, c_own, marginal) : cost(marginal);
+        }
+        float sum = 0.0f;
+        each_device<SMALL>(m, lane, [&](int k) {
+            const float ck = c_of(k);
+            sum = __fadd_rd(sum, ck);
+            if (ck < price) sum = __fadd_rd(sum, __fmul_rd((float)e_of(k), __fsub_rd(ck, price)));
+        });
+        sum = warp_sum_rd(sum);
+        sum = __fadd_rd(sum, __fmul_rd(price, (float)need));
+        sum = __fadd_rd(sum, __fmul_rd(q.z, X));
+        return !(sum > dm.lam_max_up);                     // 1.0 / Lambda >= Min_TPS possible
+    };
+    // the largest batch (variant v = 1..b_max; 0: none) that a test passes, from top down
+    auto search = [&](int top, auto pass) -> int {
+        int lo = 0, hi = top + 1, next = top;
+        while (hi - lo > 1) {
+            if (pass(next)) lo = next;
+            else hi = next;
+            next = !dm.grows ? hi - 1 : lo < 1 ? 1 : (lo + hi) >> 1;
+        }
+        return lo;
+    };
+    const int bm = search(dm.b_max, mem_of);
+    int bs = bm;
+    if (timed && bm > 0) bs = search(bm, [&](int v) { return (dm.grows || mem_of(v)) && fast_enough(v); });
+    return kSlotDecTested | (uint32_t)bs | (uint32_t)bm << kSlotMemShift;
+}
+
+__global__ void __launch_bounds__(32 * kPreWarps) slot_kernel(Dims dm, Tables tb, DevPop pop, SlotInfo si, EvalOut out,
+                                                              SplitOut so, VariantOut vo)
+{
+    extern __shared__ uint16_t s_perm[];                   // the genome's ordering
+    __shared__ int s_off[E2_MAX_CLUSTERS], s_size[E2_MAX_CLUSTERS];
+    const int g = blockIdx.x;
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, NW = blockDim.x >> 5;
+    const int K = dm.K, M = dm.M, N = dm.N;
+    const int R = pop.nclus[g];
+    const uint64_t roles = pop.roles[g];
+    const size_t base = (size_t)g * K;
+    if (wid == 0) {                                        // replica offsets: a scan of the sizes
+        const int lo = lane < R ? pop.sizes[base + lane] : 0;
+        const int hi = lane + 32 < R ? pop.sizes[base + lane + 32] : 0;
+        int a = lo, b = hi;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int x = __shfl_up_sync(0xFFFFFFFFu, a, o), y = __shfl_up_sync(0xFFFFFFFFu, b, o);
+            if (lane >= o) { a += x; b += y; }
+        }
+        b += __shfl_sync(0xFFFFFFFFu, a, 31);
+        if (lane < R) { s_off[lane] = a - lo; s_size[lane] = lo; si.off[base + lane] = a - lo; }
+        if (lane + 32 < R) { s_off[lane + 32] = b - hi; s_size[lane + 32] = hi; si.off[base + lane + 32] = b - hi; }
+    }
+    for (int i = tid; i < M; i += blockDim.x) s_perm[i] = pop.perm[(size_t)g * M + i];
+    for (int c = R + tid; c < K; c += blockDim.x) {        // the empty slots
+        si.info[base + c] = 0;
+        out.master[base + c] = -1; out.bsel[base + c] = -1;
+        out.T[base + c] = keyd(kInfKey); out.L[base + c] = keyd(kInfKey);
+    }
+    __syncthreads();
+    for (int c = wid; c < R; c += NW) {
+        const int off = s_off[c], m = s_size[c], role = (int)((roles >> c) & 1ull);
+        const size_t slot = base + c;
+        uint32_t info = 0;
+        if (m <= N && dm.layered) {                        // per-layer profiles: every variant runs (the
+            if (dm.role_search || role) info |= (uint32_t)dm.b_max | (uint32_t)dm.b_max << kSlotMemShift;   // tests
+            if (dm.role_search || !role) info |= kSlotPrefill;                      // assume identical blocks)
+            info |= size_bin(dm, m) << kSlotBinShift;
+        } else if (m <= N) {
+            const uint16_t *dev = s_perm + off;
+            if (dm.role_search || !role) {
+                auto caps = [&](int k) { return tb.drec[dev[k]].x; };
+                const bool ok = m <= 32 ? memory_ok<true>(m, N, lane, caps) : memory_ok<false>(m, N, lane, caps);
+                info |= kSlotPreTested | (ok ? kSlotPrefill : 0u);
+            }
+            if (dm.role_search || role)
+                info |= m <= 32 ? decode_verdict<true>(dm, tb, dev, m, lane) : decode_verdict<false>(dm, tb, dev, m, lane);
             info |= size_bin(dm, m) << kSlotBinShift;
         }
-        // ---- the slot's verdicts, and the outputs of a replica that cannot serve (the
-        //      genome's last replica also writes those of its slots past R)
+        // ---- the slot's verdicts, and the outputs of a replica that cannot serve
+        const bool dec = (info & kSlotDecMask) != 0, pre = (info & kSlotPrefill) != 0;
         if (lane == 0) {
             si.info[slot] = info;
             if (dm.layered) vo.best[slot] = -1;
         }
-        const bool dec = (info & kSlotDecMask) != 0, pre = (info & kSlotPrefill) != 0;
         if (dm.role_search) {
-            if (lane == 0 && c < R) {
+            if (lane == 0) {
                 if (!pre) so.code[slot * 2] = -1;
                 if (!dec) so.code[slot * 2 + 1] = -1;
             }
-        } else if (c < R && !dec && !pre) {
-            for (int k = lane; k < m_c; k += 32) out.layers[(size_t)g * M + off + k] = -1;
+        } else if (!dec && !pre) {
+            for (int k = lane; k < m; k += 32) out.layers[(size_t)g * M + off + k] = -1;
             if (lane == 0) {
                 out.master[slot] = -1; out.bsel[slot] = -1;
                 out.T[slot] = keyd(kInfKey); out.L[slot] = keyd(kInfKey);
             }
         }
-        if (c == R - 1)
-            for (int e = R + lane; e < K; e += 32) {
-                const size_t es = (size_t)g * K + e;
-                out.master[es] = -1; out.bsel[es] = -1;
-                out.T[es] = keyd(kInfKey); out.L[es] = keyd(kInfKey);
-            }
     }
 }
 
@@ -1497,17 +1562,18 @@ cudaError_t configure_eval(e2_ctx *c)
 
 cudaError_t launch_eval(const e2_ctx *c, const DevPop &p)
 {
-    Tables tb{c->rate, c->bw, c->mem, c->rate_cpu, c->bw_cpu, c->mem_cpu, c->prof, c->leaf, c->tau, c->cap,
-              c->capg, c->cpb, c->tau_lb, c->leaf_rank, c->tau_rank, c->lcost, c->drec, c->fxs};
+    Tables tb{c->rate, c->bw, c->mem, c->rate_cpu, c->bw_cpu, c->mem_cpu, c->prof, c->leaf, c->tau,
+              c->capg, c->tau_lb, c->leaf_rank, c->tau_rank, c->lcost, c->drec, c->fxs, c->prec, c->prech, c->capv,
+              c->ibw, c->fpr};
     EvalOut out{c->fit, c->layers, c->master, c->bsel, c->T, c->L, c->hash, c->stats, c->gpu_layers};
     SlotInfo si{c->slot_off, c->slot_info};
     WorkList wl{c->items, c->list_ctrl};
     SplitOut so{c->split_T, c->split_L, c->split_mu, c->split_code, c->split_layers};
     VariantOut vo{c->var_T, c->var_L, c->var_mu, c->var_layers, c->var_best};
     const long long slots = (long long)c->dm.P * c->dm.K;
-    const int mcap = c->dm.M < c->dm.N ? c->dm.M : c->dm.N;
     cudaError_t e = cudaSuccess;
-    slot_kernel<<<(unsigned)((slots + 1) / 2), 64, 2 * variant_stride(mcap), c->stream>>>(c->dm, tb, p, si, out, so, vo);
+    slot_kernel<<<(unsigned)c->dm.P, 32 * (c->dm.K < kPreWarps ? c->dm.K : kPreWarps), 2 * (size_t)c->dm.M, c->stream>>>(
+        c->dm, tb, p, si, out, so, vo);
     // (about 4,096 slots per block of the count and the scatter)
     const long long nb = (slots + 4095) / 4096;
     const unsigned lb = (unsigned)(nb < kListBlocks ? nb : kListBlocks);

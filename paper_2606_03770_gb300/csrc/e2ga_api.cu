@@ -20,7 +20,7 @@ thread_local char g_create_error[256] = "";
 size_t align_up(size_t x, size_t a = 256) { return (x + a - 1) / a * a; }
 
 struct Layout {
-    size_t rate, bw, mem, rate_cpu, bw_cpu, mem_cpu, link_bw, cong, prof, leaf, tau, tau_lb, cap, capg, cpb,
+    size_t rate, bw, mem, rate_cpu, bw_cpu, mem_cpu, link_bw, cong, prof, leaf, tau, tau_lb, capg, prec, prech, capv, ibw, fpr,
         leaf_sorted, beff_sorted, tau_sorted, leaf_rank, tau_rank, gpu_layers, psum, lcost, drec, fxs;
     size_t perm[2], sizes[2], nclus[2], roles[2];
     size_t fit, layers, master, bsel, T, L, hash, dup, dup_key, dup_idx, elite, elite_fit, elite_ctl, elite_cand, stats, err, list_ctrl, list_hist, items, slot_off, slot_info,
@@ -55,9 +55,12 @@ Layout layout(int M, int N, int b_max, int P, int Q, int K, bool layered = false
     l.prof = take(8 * kNumProf * V);
     l.leaf = take(8 * V * M * 2 * (size_t)l.LS);
     l.tau = take(8 * V * MM);
-    l.cap = take(4 * V * M * 2);
     l.capg = take(4 * V * M * 2);
-    l.cpb = take(4 * V * M);
+    l.prec = take(16 * (size_t)M);
+    l.prech = take(8 * (size_t)M);
+    l.capv = take(4 * V * M);
+    l.ibw = take(4 * MM);
+    l.fpr = take(16 * V);
     l.drec = take(16 * V * M);
     l.fxs = take(4 * V);
     l.tau_lb = take(4 * V * MM);
@@ -465,8 +468,11 @@ int e2_create(const e2_devices *devs, const e2_links *links, const e2_layer_prof
     c->prof = reinterpret_cast<uint64_t *>(ws + l.prof);
     c->leaf = reinterpret_cast<double *>(ws + l.leaf);
     c->tau = reinterpret_cast<double *>(ws + l.tau);
-    c->cap = reinterpret_cast<int32_t *>(ws + l.cap);
-    c->cpb = reinterpret_cast<float *>(ws + l.cpb);
+    c->prec = reinterpret_cast<uint4 *>(ws + l.prec);
+    c->prech = reinterpret_cast<float2 *>(ws + l.prech);
+    c->capv = reinterpret_cast<uint32_t *>(ws + l.capv);
+    c->ibw = reinterpret_cast<float *>(ws + l.ibw);
+    c->fpr = reinterpret_cast<float4 *>(ws + l.fpr);
     c->drec = reinterpret_cast<uint4 *>(ws + l.drec);
     c->fxs = reinterpret_cast<float *>(ws + l.fxs);
     c->tau_lb = reinterpret_cast<float *>(ws + l.tau_lb);

@@ -116,10 +116,8 @@ struct Tables {
     const uint64_t *prof;      // [kNumProf][V]
     const double *leaf;        // [V][M][2][LS]: leaf[((v*M+d)*2+mf)*LS + n-1] = l_d(n blocks, master mf)
     const double *tau;         // [V][M][M]
-    const int32_t *cap;        // [V][M][2]: most blocks device d holds (device + host memory), without / with
-                               // the head
-    const int32_t *capg;       // [V][M][2]: of those, the most in device memory (-1: the head does not fit)
-    const float *cpb;          // [V][M]: per-block time max(blk_flops/rate, blk_bytes/bw), rounded down
+    const int32_t *capg;       // [V][M][2]: most blocks in device memory, without / with the head (-1: the head
+                               // does not fit)
     const float *tau_lb;       // [V][M][M]: tau rounded down
     const uint32_t *leaf_rank; // [V][M][2][LS]: order key of leaf within its variant's value set
     const uint32_t *tau_rank;  // [V][M][M]
@@ -128,6 +126,12 @@ struct Tables {
     const uint4 *drec;         // [V][M] the DP's view of a device: {cap | cap with head << 16, and as floats
                                // 1 / block time, the head in blocks, host block rate / device block rate}
     const float *fxs;          // [V] 2^22 / the largest 1 / block time: its fixed-point scale
+    const uint4 *prec;         // [M] the pre-pass's view of a device: 1 / rate and 1 / bandwidth rounded down
+                               // (float bits), its capacities (| with the head << 16) at batch 1 and b_max
+    const float2 *prech;       // [M] 1 / rate and 1 / bandwidth of its host, rounded down (0: no host memory)
+    const uint32_t *capv;      // [M][V] its capacities (| with the head << 16)
+    const float *ibw;          // [M][M] 1 / effective link bandwidth, rounded down
+    const float4 *fpr;         // [V] block flops, block bytes, activation bytes, rounded down
 };
 
 // Per (genome, replica slot) results of the evaluation pre-pass.
@@ -242,8 +246,11 @@ struct e2_ctx {
     double *link_bw = nullptr, *cong = nullptr;
     uint64_t *prof = nullptr;
     double *leaf = nullptr, *tau = nullptr;
-    int32_t *cap = nullptr;
-    float *cpb = nullptr;
+    uint4 *prec = nullptr;            // [M]
+    float2 *prech = nullptr;          // [M]
+    uint32_t *capv = nullptr;         // [M][V]
+    float *ibw = nullptr;             // [M][M]
+    float4 *fpr = nullptr;            // [V]
     float *tau_lb = nullptr;
     uint64_t *leaf_sorted = nullptr;  // [V][pow2(2 M N)] sorted stage-time keys
     uint64_t *beff_sorted = nullptr;  // [pow2(M M)] sorted effective link bandwidths
@@ -299,7 +306,7 @@ struct e2_ctx {
 
 namespace e2 {
 // launchers (defined in the .cu files); return cudaGetLastError()
-cudaError_t launch_tables(const e2_ctx *c);   // leaf, cap and cpb tables (and lcost for per-layer profiles)
+cudaError_t launch_tables(const e2_ctx *c);   // stage times and device tables (and lcost for per-layer profiles)
 cudaError_t launch_tau(const e2_ctx *c);
 cudaError_t launch_redraw(const e2_ctx *c, uint64_t seed, uint32_t gen);
 cudaError_t launch_validate(const e2_ctx *c, const DevPop &p);

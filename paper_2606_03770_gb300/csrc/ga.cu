@@ -103,17 +103,15 @@ __global__ void layered_tables_kernel(Dims dm, const double *rate, const double 
 
 // Per (variant, device): the most blocks the device can hold in device and
 // host memory together, without and with the LM head (the number of finite
-// entries of its two cost rows), the most of them in device memory (the G of
-// the G--C split; -1 where the head does not fit), and the per-block time
-// rounded down to float, used by the latency bound: max(blk_flops/rate,
-// blk_bytes/bw), or the host's per-block time where that is smaller and the
-// device offloads (a lower bound on every block's time either way).  drec
-// gathers what the DP's estimate needs of a device in 16 bytes (Tables); the
-// head in blocks is how much later its row reaches a count of a few blocks.
+// entries of its two cost rows), and the most of them in device memory (the G
+// of the G--C split; -1 where the head does not fit).  drec gathers what the
+// DP's estimate needs of a device in 16 bytes (Tables); the head in blocks is
+// how much later its row reaches a count of a few blocks.  prec, prech, capv
+// and fpr are the pre-pass's view (Tables).
 __global__ void captab_kernel(Dims dm, const double *rate, const double *bw, const uint64_t *mem,
                               const double *rate_cpu, const double *bw_cpu, const uint64_t *mem_cpu,
-                              const uint64_t *prof, const double *leaf, int32_t *cap, int32_t *capg, float *cpb,
-                              uint4 *drec)
+                              const uint64_t *prof, const double *leaf, int32_t *capg,
+                              uint4 *drec, uint4 *prec, float2 *prech, uint32_t *capv, float4 *fpr)
 {
     const size_t total = (size_t)dm.V * dm.M;
     for (size_t idx = blockIdx.x * (size_t)blockDim.x + threadIdx.x; idx < total;
@@ -127,23 +125,33 @@ __global__ void captab_kernel(Dims dm, const double *rate, const double *bw, con
         const uint64_t c0 = g0 + hc;
         const uint64_t g1 = mm < hm ? 0ull : (bm ? (mm - hm) / bm : N);
         const uint64_t c1 = mm < hm ? 0ull : g1 + hc;
-        cap[idx * 2] = (int32_t)(c0 < N ? c0 : N);
-        cap[idx * 2 + 1] = (int32_t)(c1 < N ? c1 : N);
         capg[idx * 2] = (int32_t)(g0 < N ? g0 : N);
         capg[idx * 2 + 1] = mm < hm ? -1 : (int32_t)(g1 < N ? g1 : N);
         const double tc = __ull2double_rn(prof[kBlkFlops * V + v]) / rate[d];
         const double tm = __ull2double_rn(prof[kBlkBytes * V + v]) / bw[d];
-        double t = tc >= tm ? tc : tm;
-        const double tdev = t;
+        const double tdev = tc >= tm ? tc : tm;
         float ratio = 0.0f;                                          // host block rate / device block rate
         if (dm.offload && hc > 0) {
-            const double hc_ = __ull2double_rn(prof[kBlkFlops * V + v]) / rate_cpu[d];
+            const double hf = __ull2double_rn(prof[kBlkFlops * V + v]) / rate_cpu[d];
             const double hb = __ull2double_rn(prof[kBlkBytes * V + v]) / bw_cpu[d];
-            const double th = hc_ >= hb ? hc_ : hb;
+            const double th = hf >= hb ? hf : hb;
             ratio = th > 0.0 ? (float)fmin(tdev / th, 1e6) : 1e6f;
-            t = th < t ? th : t;
         }
-        cpb[idx] = __double2float_rd(t);
+        const uint32_t caps = (uint32_t)(c0 < N ? c0 : N) | (uint32_t)(c1 < N ? c1 : N) << 16;
+        capv[(size_t)d * V + v] = caps;
+        if (d == 0)
+            fpr[v] = make_float4(__ull2float_rd(prof[kBlkFlops * V + v]), __ull2float_rd(prof[kBlkBytes * V + v]),
+                                 __ull2float_rd(prof[kAct * V + v]), 0.0f);
+        if (v == 1) prec[d].z = caps;
+        if (v == dm.b_max) prec[d].w = caps;
+        if (v == 0) {
+            prec[d].x = __float_as_uint(__double2float_rd(__ddiv_rd(1.0, rate[d])));
+            prec[d].y = __float_as_uint(__double2float_rd(__ddiv_rd(1.0, bw[d])));
+            const bool host = dm.offload && mem_cpu[d] > 0;
+            prech[d] = host ? make_float2(__double2float_rd(__ddiv_rd(1.0, rate_cpu[d])),
+                                          __double2float_rd(__ddiv_rd(1.0, bw_cpu[d])))
+                            : make_float2(0.0f, 0.0f);
+        }
         const float cinv = tdev > 1e-30 ? (float)(1.0 / tdev) : 1e30f;
         float head = 1e6f;
         const int nr = c1 < 4 ? (int)c1 : N < 4 ? (int)N : 4;
@@ -154,15 +162,15 @@ __global__ void captab_kernel(Dims dm, const double *rate, const double *bw, con
         } else if (nr >= 1) {
             head = 0.0f;
         }
-        drec[idx] = make_uint4((uint32_t)cap[idx * 2] | (uint32_t)cap[idx * 2 + 1] << 16, __float_as_uint(cinv),
-                               __float_as_uint(head), __float_as_uint(ratio));
+        drec[idx] = make_uint4(caps, __float_as_uint(cinv), __float_as_uint(head), __float_as_uint(ratio));
     }
 }
 
-// tau_v(a, b) = A_v / (B(a,b) * congestion(a,b)) (Sec. 3.2), and the same
-// rounded down to float for the latency bound.
+// tau_v(a, b) = A_v / (B(a,b) * congestion(a,b)) (Sec. 3.2), the same rounded
+// down to float for the DP's estimate, and 1 / (B * congestion) rounded down
+// for the latency bound.
 __global__ void tau_kernel(Dims dm, const double *link_bw, const double *cong, const uint64_t *prof,
-                           double *tau, float *tau_lb)
+                           double *tau, float *tau_lb, float *ibw)
 {
     const size_t MM = (size_t)dm.M * dm.M, total = (size_t)dm.V * MM;
     for (size_t idx = blockIdx.x * (size_t)blockDim.x + threadIdx.x; idx < total;
@@ -173,6 +181,7 @@ __global__ void tau_kernel(Dims dm, const double *link_bw, const double *cong, c
         const double t = __ull2double_rn(prof[kAct * dm.V + v]) / beff;
         tau[idx] = t;
         tau_lb[idx] = __double2float_rd(t);
+        if (v == 0) ibw[ab] = __double2float_rd(__ddiv_rd(1.0, beff));
     }
 }
 
@@ -821,8 +830,8 @@ cudaError_t launch_tables(const e2_ctx *c)
                                                                 c->mem_cpu, c->prof, c->leaf);
     const size_t vm = (size_t)c->dm.V * c->dm.M;
     captab_kernel<<<grid_for(vm, 256), 256, 0, c->stream>>>(c->dm, c->rate, c->bw, c->mem, c->rate_cpu, c->bw_cpu,
-                                                             c->mem_cpu, c->prof, c->leaf, c->cap, c->capg, c->cpb,
-                                                             c->drec);
+                                                             c->mem_cpu, c->prof, c->leaf, c->capg, c->drec,
+                                                             c->prec, c->prech, c->capv, c->fpr);
     c->launches += 2;
     if (c->dm.layered) {
         const size_t lt = (size_t)c->dm.V * c->dm.M * 2 * c->dm.N * c->dm.N;
@@ -836,7 +845,7 @@ cudaError_t launch_tables(const e2_ctx *c)
 cudaError_t launch_tau(const e2_ctx *c)
 {
     const size_t total = (size_t)c->dm.V * c->dm.M * c->dm.M;
-    tau_kernel<<<grid_for(total, 256), 256, 0, c->stream>>>(c->dm, c->link_bw, c->cong, c->prof, c->tau, c->tau_lb);
+    tau_kernel<<<grid_for(total, 256), 256, 0, c->stream>>>(c->dm, c->link_bw, c->cong, c->prof, c->tau, c->tau_lb, c->ibw);
     ++c->launches;
     return cudaGetLastError();
 }
