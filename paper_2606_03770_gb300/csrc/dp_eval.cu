@@ -817,8 +817,10 @@ __device__ __forceinline__ void slot_tallies(const Dims &dm, uint32_t info, unsi
     if ((info & (kSlotPreTested | kSlotPrefill)) == kSlotPreTested) ++n_pre;
 }
 
-// A genome's counts, summed over its warp's lanes into the evaluation's counters.
-__device__ __forceinline__ void genome_tallies(const EvalOut &out, int R, unsigned n_served, unsigned n_pre,
+// A genome's counts, summed over its warp's lanes into `sum` (genomes,
+// replicas, served, memory rejections, latency rejections, paper candidates).
+constexpr int kTallies = 6;
+__device__ __forceinline__ void genome_tallies(unsigned long long *sum, int R, unsigned n_served, unsigned n_pre,
                                                unsigned n_tps, unsigned long long n_paper, int lane)
 {
     n_served = __reduce_add_sync(0xFFFFFFFFu, n_served);
@@ -826,95 +828,120 @@ __device__ __forceinline__ void genome_tallies(const EvalOut &out, int R, unsign
     n_tps = __reduce_add_sync(0xFFFFFFFFu, n_tps);
 #pragma unroll
     for (int o = 16; o; o >>= 1) n_paper += __shfl_xor_sync(0xFFFFFFFFu, n_paper, o);
-    if (lane != 0) return;
-    atomicAdd(&out.stats[kStGenomes], 1ull);
-    atomicAdd(&out.stats[kStReplicas], (unsigned long long)R);
-    if (n_paper) atomicAdd(&out.stats[kStPaper], n_paper);
-    if (n_served) atomicAdd(&out.stats[kStServed], (unsigned long long)n_served);
-    if (n_pre) atomicAdd(&out.stats[kStPrecheck], (unsigned long long)n_pre);
-    if (n_tps) atomicAdd(&out.stats[kStTpsPruned], (unsigned long long)n_tps);
+    const unsigned long long x = lane == 0 ? 1ull : lane == 1 ? (unsigned long long)R : lane == 2 ? n_served
+                               : lane == 3 ? n_pre : lane == 4 ? n_tps : n_paper;
+    if (lane < kTallies && x) atomicAdd(&sum[lane], x);
 }
 
-// One warp per genome, after the DP has written every replica's outputs: each
-// lane takes its replicas' rates (NP / T for prefill, b / T for decode), lane
-// 0 sums PS and DS in ascending replica order and applies Eq. 3 (bottleneck
-// phase), Eq. 4 (backlog) and Eq. 5 (waiting time).  A 64-bit fingerprint of
-// the genome, folded as a tree over the lanes, serves the elites' duplicate
-// test.
-__global__ void __launch_bounds__(128) finalize_score_kernel(Dims dm, DevPop pop, SlotInfo si, EvalOut out)
+// ... and into the evaluation's counters (threads 0..kTallies-1).
+__device__ __forceinline__ void add_tallies(const EvalOut &out, const unsigned long long *sum, int i)
 {
-    const int wl = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int g = blockIdx.x * 4 + wl;
-    if (g >= dm.P) return;
-    const int K = dm.K, M = dm.M;
-    const int R = pop.nclus[g];
-    const uint64_t roles = pop.roles[g];
-    // the fingerprint's inputs, loaded up front: replica sizes (lane c holds
-    // sizes[c] and sizes[c + 32]) and the ordering folded by the lanes
+    constexpr int to[kTallies] = {kStGenomes, kStReplicas, kStServed, kStPrecheck, kStTpsPruned, kStPaper};
+    if (i < kTallies && sum[i]) atomicAdd(&out.stats[to[i]], sum[i]);
+}
+
+// 64-bit fingerprint of a genome (ordering, replica sizes and count, roles) for
+// the elites' duplicate test, by a warp: the lanes mix interleaved slices, then
+// fold as a tree.  Valid in lane 0.
+__device__ __forceinline__ uint64_t fingerprint(const uint16_t *perm, int M, int sz_lo, int sz_hi, int R, uint64_t roles,
+                                                int lane)
+{
     auto mix = [](uint64_t h, uint64_t x) { h = (h ^ x) * 0xBF58476D1CE4E5B9ull; return h ^ (h >> 31); };
-    const int sz_lo = lane < K ? pop.sizes[(size_t)g * K + lane] : 0;
-    const int sz_hi = lane + 32 < K ? pop.sizes[(size_t)g * K + lane + 32] : 0;
-    uint64_t hl = 0x9E3779B97F4A7C15ull ^ (uint64_t)lane;
-    {
-        const uint16_t *pp = pop.perm + (size_t)g * M;
-        for (int i = lane; i < M; i += 32) hl = mix(hl, pp[i]);
+    uint64_t h = 0x9E3779B97F4A7C15ull ^ (uint64_t)lane;
+    if ((M & 1) == 0) {                                    // rows start on 4 bytes: two positions per load
+        const uint32_t *p2 = reinterpret_cast<const uint32_t *>(perm);
+        for (int i = lane; i < M / 2; i += 32) h = mix(h, p2[i]);
+    } else {
+        for (int i = lane; i < M; i += 32) h = mix(h, perm[i]);
     }
-    unsigned n_served = 0, n_pre = 0, n_tps = 0;
-    unsigned long long n_paper = 0;
-    double rate[2], lat[2];
-    int kind[2];                                   // -1 none, 0 prefill, 1 decode
+    if (lane < R) h = mix(h, (uint64_t)sz_lo << 16);
+    if (lane + 32 < R) h = mix(h, (uint64_t)sz_hi << 16);
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
-        const int c = lane + 32 * h;
-        kind[h] = -1;
-        rate[h] = 0.0;
-        lat[h] = 0.0;
-        if (c < R) {
+    for (int o = 16; o; o >>= 1) {
+        const uint64_t other = __shfl_down_sync(0xFFFFFFFFu, h, o);
+        if (lane < o) h = mix(h, other);
+    }
+    return mix(mix(h, (uint64_t)R << 40), roles);
+}
+
+// Scores the genomes after the DP has written every replica's outputs, eight
+// per block, a warp each: the lanes take their replicas' rates (NP / T for
+// prefill, b / T for decode) into shared memory, and one warp then sums PS and
+// DS of all eight in ascending replica order, a lane per sum (a replica of the
+// other role adds 0.0, which changes no sum), and applies Eq. 3 (bottleneck
+// phase), Eq. 4 (backlog) and Eq. 5 (waiting time).
+//
+// Bound by the float64 pipe (two lanes per SM: a warp instruction takes 16
+// cycles whatever its lanes) when a warp per genome summed alone: 70 us for
+// 16,384 genomes of 32 replicas on average, 32 with eight genomes' sums per
+// instruction, the latency sums only where the objective needs them and the
+// counters added once per block.
+constexpr int kScoreGenomes = 8;
+
+template <bool FT>
+__global__ void __launch_bounds__(32 * kScoreGenomes) finalize_score_kernel(Dims dm, DevPop pop, SlotInfo si, EvalOut out)
+{
+    constexpr int S = FT ? 4 : 2;                          // PS, DS (and the rate-weighted latencies PL, DL)
+    __shared__ double s_x[S][kScoreGenomes][E2_MAX_CLUSTERS + 1];
+    __shared__ int s_R[kScoreGenomes];
+    __shared__ unsigned long long s_tally[kTallies];
+    const int wl = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int g0 = blockIdx.x * kScoreGenomes, g = g0 + wl;
+    if (threadIdx.x < kTallies) s_tally[threadIdx.x] = 0;
+    __syncthreads();
+    int R = 0;
+    if (g < dm.P) {
+        const int K = dm.K, M = dm.M;
+        R = pop.nclus[g];
+        const uint64_t roles = pop.roles[g];
+        const int sz_lo = lane < R ? pop.sizes[(size_t)g * K + lane] : 0;
+        const int sz_hi = lane + 32 < R ? pop.sizes[(size_t)g * K + lane + 32] : 0;
+        unsigned n_served = 0, n_pre = 0, n_tps = 0;
+        unsigned long long n_paper = 0;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int c = lane + 32 * h;
+            if (c >= R) continue;
             const int slot = g * K + c, b = out.bsel[slot], role = (int)((roles >> c) & 1ull);
             const int m = h ? sz_hi : sz_lo;
             slot_tallies(dm, si.info[slot], n_pre, n_tps);
             unsigned long long nrun = role ? (unsigned long long)dm.b_max : 1ull;
+            double rate = 0.0, weighted = 0.0;
             if (b >= 0) {
-                const double T = out.T[slot];
-                lat[h] = out.L[slot];
-                kind[h] = role;
-                rate[h] = role ? (double)b / T : (double)dm.NP / T;
+                rate = (role ? (double)b : (double)dm.NP) / out.T[slot];
+                if (FT) weighted = rate * out.L[slot];
                 if (role) nrun = (unsigned long long)(dm.b_max - b + 1);   // variants b_max .. b
                 ++n_served;
             }
+            s_x[0][wl][c] = role ? 0.0 : rate;
+            s_x[1][wl][c] = role ? rate : 0.0;
+            if (FT) {
+                s_x[S - 2][wl][c] = role ? 0.0 : weighted;
+                s_x[S - 1][wl][c] = role ? weighted : 0.0;
+            }
             if (m <= dm.N) n_paper += nrun * paper_candidates(m, dm.N);
         }
+        genome_tallies(s_tally, R, n_served, n_pre, n_tps, n_paper, lane);
+        const uint64_t h = fingerprint(pop.perm + (size_t)g * M, M, sz_lo, sz_hi, R, roles, lane);
+        if (lane == 0) out.hash[g] = h;
     }
-    genome_tallies(out, R, n_served, n_pre, n_tps, n_paper, lane);
-    double PS = 0.0, DS = 0.0, PL = 0.0, DL = 0.0;   // PL, DL: rate-weighted latencies (finishing time)
-    for (int c = 0; c < R; ++c) {
-        const int h = c >> 5;
-        const double x = __shfl_sync(0xFFFFFFFFu, h ? rate[1] : rate[0], c & 31);
-        const double l = __shfl_sync(0xFFFFFFFFu, h ? lat[1] : lat[0], c & 31);
-        const int k = __shfl_sync(0xFFFFFFFFu, h ? kind[1] : kind[0], c & 31);
-        if (k == 0) { PS = PS + x; PL = PL + x * l; }
-        else if (k == 1) { DS = DS + x; DL = DL + x * l; }
-    }
-    // fingerprint: lanes mixed interleaved slices of the ordering; a tree fold,
-    // then the sizes in replica order (from the lanes that hold them)
-#pragma unroll
-    for (int o = 16; o; o >>= 1) {
-        const uint64_t other = __shfl_down_sync(0xFFFFFFFFu, hl, o);
-        if (lane < o) hl = mix(hl, other);
-    }
-    uint64_t h = hl;
-    for (int i = 0; i < R; ++i) {
-        const int si_ = __shfl_sync(0xFFFFFFFFu, i < 32 ? sz_lo : sz_hi, i & 31);
-        h = mix(h, (uint64_t)si_ << 16);
-    }
-    if (lane != 0) return;
+    if (lane == 0) s_R[wl] = R;
+    __syncthreads();
+    if (wl == 1) add_tallies(out, s_tally, lane);
+    if (wl != 0) return;
+    // lane: sum lane / 8 (PS, DS, PL, DL) of genome lane % 8
+    const int q = lane & (kScoreGenomes - 1), which = lane / kScoreGenomes;
+    double x = 0.0;
+    if (which < S)
+        for (int c = 0; c < s_R[q]; ++c) x = x + s_x[which < S ? which : 0][q][c];
+    const double DS = __shfl_sync(0xFFFFFFFFu, x, q + kScoreGenomes);
+    const double PL = FT ? __shfl_sync(0xFFFFFFFFu, x, q + 2 * kScoreGenomes) : 0.0;
+    const double DL = FT ? __shfl_sync(0xFFFFFFFFu, x, q + 3 * kScoreGenomes) : 0.0;
+    if (lane >= kScoreGenomes || g0 + q >= dm.P) return;
     double w, phase;
-    objective(dm, PS, DS, PL, DL, w, phase);
-    double *f = out.fit + (size_t)g * 4;
-    f[0] = w; f[1] = phase; f[2] = PS; f[3] = DS;
-    h = mix(h, (uint64_t)R << 40);
-    h = mix(h, roles);
-    out.hash[g] = h;
+    objective(dm, x, DS, PL, DL, w, phase);
+    double *f = out.fit + (size_t)(g0 + q) * 4;
+    f[0] = w; f[1] = phase; f[2] = x; f[3] = DS;
 }
 
 // Alg. 2's role search, one warp per genome (or a block, below).  The lead
@@ -952,6 +979,7 @@ __global__ void __launch_bounds__(128) finalize_roles_kernel(Dims dm, DevPop pop
     __shared__ double s_bw[4], s_bph[4];
     __shared__ unsigned long long s_wmin[4];           // the least w a warp of the genome has scored (bits)
     __shared__ uint64_t s_br[4];
+    __shared__ unsigned long long s_tally[4][kTallies];    // (a row per warp)
     const int wl = threadIdx.x >> 5, lane = threadIdx.x & 31;
     // WPG warps per genome: 1 (four genomes per block), or 4 (one genome per
     // block, its assignments split over the block's 128 threads)
@@ -1301,17 +1329,12 @@ __global__ void __launch_bounds__(128) finalize_roles_kernel(Dims dm, DevPop pop
         const int code = s_code[gw][lo];
         out.layers[(size_t)g * M + i] = code >= 0 ? split[(size_t)code * M + i] : (int16_t)-1;
     }
-    genome_tallies(out, R, n_served, n_pre, n_tps, n_paper, lane);
-    // fingerprint of the genome with its chosen roles (a tree fold over the lanes)
-    uint64_t hl = 0x9E3779B97F4A7C15ull ^ (uint64_t)lane;
-    auto mix = [](uint64_t h, uint64_t x) { h = (h ^ x) * 0xBF58476D1CE4E5B9ull; return h ^ (h >> 31); };
-    const uint16_t *pp = pop.perm + (size_t)g * M;
-    for (int i = lane; i < M; i += 32) hl = mix(hl, pp[i]);
-#pragma unroll
-    for (int o = 16; o; o >>= 1) {
-        const uint64_t other = __shfl_down_sync(0xFFFFFFFFu, hl, o);
-        if (lane < o) hl = mix(hl, other);
-    }
+    if (lane < kTallies) s_tally[wl][lane] = 0;
+    __syncwarp();
+    genome_tallies(s_tally[wl], R, n_served, n_pre, n_tps, n_paper, lane);
+    __syncwarp();
+    add_tallies(out, s_tally[wl], lane);
+    const uint64_t h = fingerprint(pop.perm + (size_t)g * M, M, m[0], m[1], R, brf, lane);
     if (lane != 0) return;
     if (capped) atomicAdd(&out.stats[kStRoleCapped], 1ull);
     double PS, DS, w, phase;
@@ -1319,11 +1342,6 @@ __global__ void __launch_bounds__(128) finalize_roles_kernel(Dims dm, DevPop pop
     double *f = out.fit + (size_t)g * 4;
     f[0] = w; f[1] = phase; f[2] = PS; f[3] = DS;
     pop.roles[g] = brf;
-    uint64_t h = hl;
-    const uint16_t *ss = pop.sizes + (size_t)g * K;
-    for (int i = 0; i < R; ++i) h = mix(h, (uint64_t)ss[i] << 16);
-    h = mix(h, (uint64_t)R << 40);
-    h = mix(h, brf);
     out.hash[g] = h;
 }
 
@@ -1342,6 +1360,7 @@ __global__ void __launch_bounds__(128) finalize_splitwise_kernel(Dims dm, DevPop
 {
     __shared__ int s_off[4][E2_MAX_CLUSTERS + 1];     // replica start in the ordering
     __shared__ int s_code[4][E2_MAX_CLUSTERS];        // the role whose result is taken, -1 none
+    __shared__ unsigned long long s_tally[4][kTallies];   // (a row per warp)
     const int wl = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int g = blockIdx.x * 4 + wl;
     if (g >= dm.P) return;
@@ -1431,7 +1450,11 @@ __global__ void __launch_bounds__(128) finalize_splitwise_kernel(Dims dm, DevPop
         const int code = s_code[wl][lo];
         out.layers[(size_t)g * M + i] = code >= 0 ? split[(size_t)code * M + i] : (int16_t)-1;
     }
-    genome_tallies(out, R, n_served, n_pre, n_tps, n_paper, lane);
+    if (lane < kTallies) s_tally[wl][lane] = 0;
+    __syncwarp();
+    genome_tallies(s_tally[wl], R, n_served, n_pre, n_tps, n_paper, lane);
+    __syncwarp();
+    add_tallies(out, s_tally[wl], lane);
     double PS = 0.0, DS = 0.0, PL = 0.0, DL = 0.0;
     for (int c = 0; c < R; ++c) {
         const int h = c >> 5;
@@ -1441,27 +1464,13 @@ __global__ void __launch_bounds__(128) finalize_splitwise_kernel(Dims dm, DevPop
         if (k == 0) { PS = PS + x; PL = PL + x * l; }
         else if (k == 1) { DS = DS + x; DL = DL + x * l; }
     }
-    // fingerprint of the genome with its roles (a tree fold over the lanes)
-    auto mix = [](uint64_t h, uint64_t x) { h = (h ^ x) * 0xBF58476D1CE4E5B9ull; return h ^ (h >> 31); };
-    uint64_t hl = 0x9E3779B97F4A7C15ull ^ (uint64_t)lane;
-    const uint16_t *pp = pop.perm + (size_t)g * M;
-    for (int i = lane; i < M; i += 32) hl = mix(hl, pp[i]);
-#pragma unroll
-    for (int o = 16; o; o >>= 1) {
-        const uint64_t other = __shfl_down_sync(0xFFFFFFFFu, hl, o);
-        if (lane < o) hl = mix(hl, other);
-    }
+    const uint64_t h = fingerprint(pop.perm + (size_t)g * M, M, m[0], m[1], R, roles, lane);
     if (lane != 0) return;
     double w, phase;
     objective(dm, PS, DS, PL, DL, w, phase);
     double *f = out.fit + (size_t)g * 4;
     f[0] = w; f[1] = phase; f[2] = PS; f[3] = DS;
     pop.roles[g] = roles;
-    uint64_t h = hl;
-    const uint16_t *ss = pop.sizes + (size_t)g * K;
-    for (int i = 0; i < R; ++i) h = mix(h, (uint64_t)ss[i] << 16);
-    h = mix(h, (uint64_t)R << 40);
-    h = mix(h, roles);
     out.hash[g] = h;
 }
 
@@ -1617,7 +1626,11 @@ cudaError_t launch_eval(const e2_ctx *c, const DevPop &p)
         if (c->dm.objective == 1) finalize_roles_kernel<1, true><<<fb, 128, 0, c->stream>>>(c->dm, p, si, so, out);
         else finalize_roles_kernel<1, false><<<fb, 128, 0, c->stream>>>(c->dm, p, si, so, out);
     }
-    else finalize_score_kernel<<<fb, 128, 0, c->stream>>>(c->dm, p, si, out);
+    else {
+        const unsigned sb = (unsigned)((c->dm.P + kScoreGenomes - 1) / kScoreGenomes);
+        if (c->dm.objective == 1) finalize_score_kernel<true><<<sb, 32 * kScoreGenomes, 0, c->stream>>>(c->dm, p, si, out);
+        else finalize_score_kernel<false><<<sb, 32 * kScoreGenomes, 0, c->stream>>>(c->dm, p, si, out);
+    }
     c->launches += c->dp_grid1 > 0 ? 6 : 5;
     if (c->dm.offload) {
         gc_split_kernel<<<fb, 128, 0, c->stream>>>(c->dm, p, c->capg, out);
