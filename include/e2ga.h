@@ -391,7 +391,7 @@ int e2_set_timing_events(e2_ctx *ctx, void *dp_start, void *dp_stop);
  * pay cudaMalloc's implicit synchronisation.  It computes what e2_ga_step's
  * elite step computes (the Q best distinct genomes of an evaluated
  * population by (w, phase, index)) without a context or workspace: its
- * scratch is a file-scope device array sized for E2_NOALLOC_MAX_POP genomes (1 MiB,
+ * scratch is a file-scope device array sized for E2_NOALLOC_MAX_POP genomes (1.6 MiB,
  * held by every GPU that loads the library until the process exits).
  *   pop       population [P] in the genome layout, DEVICE pointers
  *   fitness   [P][4] {w, phase, PS, DS} from e2_eval_population, DEVICE
@@ -406,8 +406,9 @@ int e2_set_timing_events(e2_ctx *ctx, void *dp_start, void *dp_stop);
  * device current; make that first call before any stream capture.  All calls
  * share the one scratch array and overwrite it; calls that overlap on the GPU
  * (other streams, other host threads) race and must be serialised by the
- * caller.  Cost: two O(P^2) passes over shared-memory tiles of the fitness
- * keys, one warp per genome (the same shape as e2_ga_step's elites). */
+ * caller.  Cost: one read of the population for its fingerprints, and the
+ * selection e2_ga_step uses; with fewer than Q distinct genomes, one O(P^2)
+ * pass over the fitness keys. */
 #define E2_NOALLOC_MAX_POP 65536
 int e2_select_elites_noalloc(const e2_genomes *pop, const double *fitness, int32_t P, int32_t M,
                              int32_t K_max, int32_t Q, int32_t *elite_idx, void *stream);

@@ -10,6 +10,7 @@
 // CTAs over the list; and a warp per genome (a block per genome for a wide
 // role search) that scores the genome.
 #include "e2ga_internal.cuh"
+#include "elites.cuh"
 
 namespace e2 {
 
@@ -838,30 +839,6 @@ __device__ __forceinline__ void add_tallies(const EvalOut &out, const unsigned l
 {
     constexpr int to[kTallies] = {kStGenomes, kStReplicas, kStServed, kStPrecheck, kStTpsPruned, kStPaper};
     if (i < kTallies && sum[i]) atomicAdd(&out.stats[to[i]], sum[i]);
-}
-
-// 64-bit fingerprint of a genome (ordering, replica sizes and count, roles) for
-// the elites' duplicate test, by a warp: the lanes mix interleaved slices, then
-// fold as a tree.  Valid in lane 0.
-__device__ __forceinline__ uint64_t fingerprint(const uint16_t *perm, int M, int sz_lo, int sz_hi, int R, uint64_t roles,
-                                                int lane)
-{
-    auto mix = [](uint64_t h, uint64_t x) { h = (h ^ x) * 0xBF58476D1CE4E5B9ull; return h ^ (h >> 31); };
-    uint64_t h = 0x9E3779B97F4A7C15ull ^ (uint64_t)lane;
-    if ((M & 1) == 0) {                                    // rows start on 4 bytes: two positions per load
-        const uint32_t *p2 = reinterpret_cast<const uint32_t *>(perm);
-        for (int i = lane; i < M / 2; i += 32) h = mix(h, p2[i]);
-    } else {
-        for (int i = lane; i < M; i += 32) h = mix(h, perm[i]);
-    }
-    if (lane < R) h = mix(h, (uint64_t)sz_lo << 16);
-    if (lane + 32 < R) h = mix(h, (uint64_t)sz_hi << 16);
-#pragma unroll
-    for (int o = 16; o; o >>= 1) {
-        const uint64_t other = __shfl_down_sync(0xFFFFFFFFu, h, o);
-        if (lane < o) h = mix(h, other);
-    }
-    return mix(mix(h, (uint64_t)R << 40), roles);
 }
 
 // Scores the genomes after the DP has written every replica's outputs, eight

@@ -264,8 +264,7 @@ struct e2_ctx {
     double *T = nullptr, *L = nullptr;
     uint64_t *hash = nullptr;
     int32_t *dup = nullptr, *elite = nullptr;
-    uint64_t *dup_key = nullptr;      // [dup_table_size(P)] fingerprint table of the duplicate test
-    int32_t *dup_idx = nullptr;       //   and the smallest genome index of each fingerprint
+    unsigned long long *dup_tab = nullptr;   // [dup_table_size(P)] fingerprint table of the duplicate test
     double *elite_fit = nullptr;
     unsigned long long *elite_ctl = nullptr;   // [8]: threshold key of the elite selection, counts, path flag
     int32_t *elite_cand = nullptr;             // [P] its candidates

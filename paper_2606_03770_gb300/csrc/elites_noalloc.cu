@@ -18,32 +18,43 @@
 // calls that overlap on the GPU -- on different streams, or from different
 // host threads -- race on it and must be serialised by the caller.
 //
-// The duplicate test and the ranks follow the same order as e2_ga_step's
-// elites: fitness keys compared as the bit patterns of w and phase (the order
-// of the values for the non-negative and +inf results an evaluation produces,
-// and a total order for any other input), staged tile by tile in shared
-// memory with one warp per genome.
+// The duplicate test and the selection are e2_ga_step's (elites.cuh), in the
+// same order: fitness keys compared as the bit patterns of w and phase (the
+// order of the values for the non-negative and +inf results an evaluation
+// produces, and a total order for any other input).
+//
+// Bound by the read of the population for the fingerprints and by the
+// selection's passes on one SM: 62 us for 16,384 genomes of 512 devices (two
+// O(P^2) passes over the keys and a thread per genome for its fingerprint took
+// 562).
 #include <mutex>
 
 #include "e2ga_internal.cuh"
+#include "elites.cuh"
 
 namespace {
 
 constexpr int kNoallocMaxPop = E2_NOALLOC_MAX_POP;
 constexpr int kMaxDeviceIds = 64;
-constexpr int kTile = 1024;
 constexpr int kWarps = 8;
 
-// Scratch: [0, P) fingerprints (u64), then [P, 2P) duplicate flags (stored in
-// the low word of a u64 slot so that the array stays one type).
-static __device__ __align__(256) unsigned long long g_noalloc_scratch[2 * kNoallocMaxPop];
+// Scratch: the fingerprints, the fingerprint table (reused for the candidate
+// list once the duplicates are known), the duplicate flags and the selection's
+// control words.
+struct Scratch {
+    uint64_t hash[kNoallocMaxPop];
+    unsigned long long table[2 * kNoallocMaxPop];
+    uint8_t dup[kNoallocMaxPop];
+    unsigned long long ctl[8];
+};
+static __device__ __align__(256) Scratch g_noalloc_scratch;
 
 // Device address of g_noalloc_scratch per device id, with the CUDA context
 // that was current when it was looked up (a reset device gets a new context,
 // and the address is looked up again).
 struct ScratchSlot {
     void *ctx = nullptr;
-    unsigned long long *addr = nullptr;
+    Scratch *addr = nullptr;
 };
 ScratchSlot g_scratch[kMaxDeviceIds];
 std::mutex g_scratch_mutex;
@@ -71,101 +82,62 @@ void *current_context()
     return ctx;
 }
 
-__device__ __forceinline__ uint64_t key_bits(const double *fit, size_t i, int q)
+// A warp per genome; the blocks also clear the fingerprint table.  The
+// fitness here is the caller's, so w and phase are part of what makes a
+// duplicate (an evaluation gives equal genomes equal ones).
+__global__ void __launch_bounds__(32 * kWarps) fingerprint_noalloc(e2::DevPop p, const uint64_t *fk, int P, int M, int K,
+                                                                   Scratch *sc, unsigned slots)
 {
-    return (uint64_t)__double_as_longlong(fit[i * 4 + q]);
+    const int lane = threadIdx.x & 31, g = blockIdx.x * kWarps + (threadIdx.x >> 5);
+    for (unsigned s = blockIdx.x * blockDim.x + threadIdx.x; s < slots; s += gridDim.x * blockDim.x)
+        sc->table[s] = e2::kFreeSlot;
+    if (g >= P) return;
+    const int R = min((int)p.nclus[g], K);
+    const int lo = lane < R ? p.sizes[(size_t)g * K + lane] : 0, hi = lane + 32 < R ? p.sizes[(size_t)g * K + lane + 32] : 0;
+    const uint64_t h = e2::fingerprint(p.perm + (size_t)g * M, M, lo, hi, R, p.roles[g], lane,
+                                       0x9E3779B97F4A7C15ull ^ fk[(size_t)g * 4] ^ (fk[(size_t)g * 4 + 1] << 1));
+    if (lane == 0) sc->hash[g] = h;
 }
 
-__global__ void fingerprint_noalloc(e2::DevPop p, int P, int M, int K, unsigned long long *hash)
+__global__ void __launch_bounds__(256) insert_noalloc(int P, Scratch *sc, unsigned mask)
 {
     const int g = blockIdx.x * blockDim.x + threadIdx.x;
+    if (g < P) e2::table_insert(sc->table, mask, sc->hash[g], g);
+}
+
+__global__ void __launch_bounds__(32 * kWarps) dup_noalloc(e2::DevPop p, const uint64_t *fk, int P, int M, int K, Scratch *sc,
+                                                           unsigned mask)
+{
+    const int lane = threadIdx.x & 31, g = blockIdx.x * kWarps + (threadIdx.x >> 5);
     if (g >= P) return;
-    uint64_t h = 0x9E3779B97F4A7C15ull;
-    auto mix = [&](uint64_t x) { h = (h ^ x) * 0xBF58476D1CE4E5B9ull; h ^= h >> 31; };
-    const int R = p.nclus[g];
-    for (int i = 0; i < M; ++i) mix(p.perm[(size_t)g * M + i]);
-    for (int i = 0; i < R && i < K; ++i) mix((uint64_t)p.sizes[(size_t)g * K + i] << 16);
-    mix((uint64_t)R << 40);
-    mix(p.roles[g]);
-    hash[g] = h;
+    const bool d = e2::is_duplicate(p, sc->table, mask, sc->hash, g, M, K, lane, fk);
+    if (lane == 0) sc->dup[g] = d;
 }
 
-// Duplicate flag, one warp per genome: equal to a lower-indexed genome
-// (compared in full only where the fitness keys and the fingerprint agree).
-__global__ void __launch_bounds__(32 * kWarps) dup_noalloc(e2::DevPop p, int P, int M, int K, const double *fit,
-                                                           const unsigned long long *hash, unsigned long long *dup)
+// The listed genomes' ranks; with fewer than Q distinct genomes, the ranks of
+// all of them in the order (duplicate, w, phase, index), a warp each.
+__global__ void __launch_bounds__(32 * kWarps) rank_noalloc(int P, int Q, const double *fit, const Scratch *sc, int32_t *elite)
 {
-    __shared__ uint64_t s_w[kTile], s_p[kTile], s_h[kTile];
-    const int lane = threadIdx.x & 31, wl = threadIdx.x >> 5;
-    const int g = blockIdx.x * kWarps + wl;
-    const bool live = g < P;
-    const uint64_t w = live ? key_bits(fit, g, 0) : 0, ph = live ? key_bits(fit, g, 1) : 0;
-    const uint64_t h = live ? hash[g] : 0;
-    const int gmax = min(P, (int)(blockIdx.x + 1) * kWarps);
-    int d = 0;
-    for (int base = 0; base < gmax - 1; base += kTile) {
-        __syncthreads();
-        for (int t = threadIdx.x; t < kTile && base + t < P; t += blockDim.x) {
-            s_w[t] = key_bits(fit, base + t, 0);
-            s_p[t] = key_bits(fit, base + t, 1);
-            s_h[t] = hash[base + t];
-        }
-        __syncthreads();
-        if (!live || d) continue;
-        const int lim = min(kTile, g - base);
-        for (int t0 = 0; t0 < lim && !d; t0 += 32) {
-            const int t = t0 + lane;
-            const bool cand = t < lim && s_h[t] == h && s_w[t] == w && s_p[t] == ph;
-            unsigned b = __ballot_sync(0xFFFFFFFFu, cand);
-            while (b && !d) {
-                const int o = base + t0 + __ffs(b) - 1;
-                b &= b - 1;
-                bool diff = p.nclus[o] != p.nclus[g] || p.roles[o] != p.roles[g];
-                for (int i = lane; i < M && !diff; i += 32) diff = p.perm[(size_t)o * M + i] != p.perm[(size_t)g * M + i];
-                for (int i = lane; i < K && !diff; i += 32) diff = p.sizes[(size_t)o * K + i] != p.sizes[(size_t)g * K + i];
-                d = __ballot_sync(0xFFFFFFFFu, diff) == 0u;
-            }
-        }
+    if (sc->ctl[2] != 0) {
+        e2::rank_listed(Q, fit, sc->ctl, reinterpret_cast<const int32_t *>(sc->table), [&](int rank, int g, int lane) {
+            if (lane == 0) elite[rank] = g;
+        });
+        return;
     }
-    if (live && lane == 0) dup[g] = (unsigned long long)d;
-}
-
-// rank(g) in the order (duplicate, w bits, phase bits, index), one warp per
-// genome over shared-memory tiles of the keys; ranks below Q are the elites.
-__global__ void __launch_bounds__(32 * kWarps) rank_noalloc(int P, int Q, const double *fit,
-                                                            const unsigned long long *dup, int32_t *elite)
-{
-    __shared__ uint64_t s_w[kTile], s_p[kTile];
-    __shared__ int s_d[kTile];
-    const int lane = threadIdx.x & 31, wl = threadIdx.x >> 5;
-    const int g = blockIdx.x * kWarps + wl;
-    const bool live = g < P;
-    const uint64_t w = live ? key_bits(fit, g, 0) : 0, ph = live ? key_bits(fit, g, 1) : 0;
-    const int dg = live ? (int)dup[g] : 0;
-    int rank = 0;
-    for (int base = 0; base < P; base += kTile) {
-        __syncthreads();
-        for (int t = threadIdx.x; t < kTile && base + t < P; t += blockDim.x) {
-            s_w[t] = key_bits(fit, base + t, 0);
-            s_p[t] = key_bits(fit, base + t, 1);
-            s_d[t] = (int)dup[base + t];
+    const uint64_t *fk = reinterpret_cast<const uint64_t *>(fit);
+    const int lane = threadIdx.x & 31;
+    for (int g = blockIdx.x * kWarps + (threadIdx.x >> 5); g < P; g += gridDim.x * kWarps) {
+        const uint64_t w = fk[(size_t)g * 4], ph = fk[(size_t)g * 4 + 1];
+        const int dg = sc->dup[g];
+        unsigned rank = 0;
+        for (int o = lane; o < P; o += 32) {
+            const uint64_t wo = fk[(size_t)o * 4], po = fk[(size_t)o * 4 + 1];
+            const int d = sc->dup[o];
+            rank += d != dg ? d < dg : wo != w ? wo < w : po != ph ? po < ph : o < g;
         }
-        __syncthreads();
-        const int lim = min(kTile, P - base);
-        if (live)
-            for (int t = lane; t < lim; t += 32) {
-                const int o = base + t;
-                bool before;
-                if (s_d[t] != dg) before = s_d[t] < dg;
-                else if (s_w[t] != w) before = s_w[t] < w;
-                else if (s_p[t] != ph) before = s_p[t] < ph;
-                else before = o < g;
-                rank += before;
-            }
+        rank = __reduce_add_sync(0xFFFFFFFFu, rank);
+        if (lane == 0 && rank < (unsigned)Q) elite[rank] = g;
     }
-#pragma unroll
-    for (int x = 16; x; x >>= 1) rank += __shfl_xor_sync(0xFFFFFFFFu, rank, x);
-    if (live && lane == 0 && rank < Q) elite[rank] = g;
 }
 
 // Device memory of device `dev` (or managed memory).
@@ -200,7 +172,7 @@ extern "C" int e2_select_elites_noalloc(const e2_genomes *pop, const double *fit
     if (!on_device(pop->perm, dev) || !on_device(pop->sizes, dev) || !on_device(pop->nclus, dev) ||
         !on_device(pop->roles, dev) || !on_device(fitness, dev) || (Q > 0 && !on_device(elite_idx, dev)))
         return reject(E2_EINVAL, "inputs and output must be device memory of the current device");
-    unsigned long long *hash = nullptr;
+    Scratch *sc = nullptr;
     {
         // set-up, once per device and context: the scratch array's device
         // address, looked up with that device current
@@ -214,19 +186,24 @@ extern "C" int e2_select_elites_noalloc(const e2_genomes *pop, const double *fit
                 cudaGetLastError();
                 return reject(E2_ECUDA, "cudaGetSymbolAddress of the scratch array failed");
             }
-            sl.addr = static_cast<unsigned long long *>(addr);
+            sl.addr = static_cast<Scratch *>(addr);
             sl.ctx = ctx;
         }
-        hash = sl.addr;
+        sc = sl.addr;
     }
-    unsigned long long *dup = hash + P;
     const e2::DevPop p{pop->perm, pop->sizes, pop->nclus, pop->roles};
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    const unsigned blocks = (unsigned)((P + 255) / 256);
+    const uint64_t *fk = reinterpret_cast<const uint64_t *>(fitness);
+    const unsigned slots = e2::dup_table_size(P);
     const unsigned wblocks = (unsigned)((P + kWarps - 1) / kWarps);
-    fingerprint_noalloc<<<blocks, 256, 0, s>>>(p, P, M, K_max, hash);
-    dup_noalloc<<<wblocks, 32 * kWarps, 0, s>>>(p, P, M, K_max, fitness, hash, dup);
-    if (Q > 0) rank_noalloc<<<wblocks, 32 * kWarps, 0, s>>>(P, Q, fitness, dup, elite_idx);
+    fingerprint_noalloc<<<wblocks, 32 * kWarps, 0, s>>>(p, fk, P, M, K_max, sc, slots);
+    insert_noalloc<<<(unsigned)((P + 255) / 256), 256, 0, s>>>(P, sc, slots - 1);
+    dup_noalloc<<<wblocks, 32 * kWarps, 0, s>>>(p, fk, P, M, K_max, sc, slots - 1);
+    if (Q > 0) {
+        e2::elite_select_kernel<<<1, e2::kSelThreads, 0, s>>>(P, Q, fitness, sc->dup, sc->ctl,
+                                                                reinterpret_cast<int32_t *>(sc->table));
+        rank_noalloc<<<wblocks < 608 ? wblocks : 608, 32 * kWarps, 0, s>>>(P, Q, fitness, sc, elite_idx);
+    }
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return reject(E2_ECUDA, cudaGetErrorString(e));
     return E2_OK;

@@ -4,6 +4,7 @@
 // Philox-4x32-10 streams keyed by (seed, generation, slot, purpose), so a
 // generation replays bit for bit whatever the thread mapping.
 #include "e2ga_internal.cuh"
+#include "elites.cuh"
 
 namespace e2 {
 
@@ -304,6 +305,50 @@ __global__ void init_kernel(Dims dm, DevPop p, uint64_t seed)
     p.roles[s] = roles;
 }
 
+// Duplicate test: dup_insert_kernel fills the fingerprint table (elites.cuh) in
+// global memory and dup_lookup_kernel looks each genome up, a warp each.
+// Below kDupTableFrom genomes one kernel does both: every block fills a table
+// of its own in shared memory and looks up its share of the genomes, which
+// saves the fill, a launch and the global atomics.
+constexpr int kDupTableFrom = 4096;
+
+// (the table is filled with kFreeSlot beforehand)
+__global__ void __launch_bounds__(256) dup_insert_kernel(int P, const uint64_t *hash, unsigned long long *tab,
+                                                         unsigned mask)
+{
+    const int g = blockIdx.x * blockDim.x + threadIdx.x;
+    if (g < P) table_insert(tab, mask, hash[g], g);
+}
+
+__global__ void __launch_bounds__(256) dup_lookup_kernel(Dims dm, DevPop p, const uint64_t *hash,
+                                                         const unsigned long long *tab, unsigned mask, int32_t *dup)
+{
+    const int lane = threadIdx.x & 31;
+    const int g = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    if (g >= dm.P) return;
+    const bool d = is_duplicate(p, tab, mask, hash, g, dm.M, dm.K, lane);
+    if (lane == 0) dup[g] = d;
+}
+
+// (comparing each genome's keys with every lower-indexed one's took 8 us at
+// 1,024 genomes and 28 at 2,048)
+constexpr int kDupThreads = 512;
+
+__global__ void __launch_bounds__(kDupThreads) dup_kernel(Dims dm, DevPop p, const uint64_t *hash, int32_t *dup,
+                                                          unsigned mask)
+{
+    extern __shared__ unsigned long long tab[];
+    const int lane = threadIdx.x & 31;
+    for (unsigned s = threadIdx.x; s <= mask; s += kDupThreads) tab[s] = kFreeSlot;
+    __syncthreads();
+    for (int g = threadIdx.x; g < dm.P; g += kDupThreads) table_insert(tab, mask, hash[g], g);
+    __syncthreads();
+    for (int g = blockIdx.x * (kDupThreads / 32) + (threadIdx.x >> 5); g < dm.P; g += gridDim.x * (kDupThreads / 32)) {
+        const bool d = is_duplicate(p, tab, mask, hash, g, dm.M, dm.K, lane);
+        if (lane == 0) dup[g] = d;
+    }
+}
+
 // Total order of the elites: distinct genomes before duplicates, then lower w,
 // lower bottleneck phase, lower index.  w and phase are non-negative or +inf,
 // so they are compared as their bit patterns (same order, integer pipe).
@@ -316,127 +361,6 @@ __device__ __forceinline__ bool elite_before(int da, uint64_t wa, uint64_t pa, i
     return a < b;
 }
 
-// Fitness keys of the elites' comparisons are staged in shared memory, tile
-// by tile, and shared by the block's warps (one warp per genome).
-constexpr int kEliteTile = 1024;
-
-// A genome equal to a lower-indexed one is a duplicate.  Equal genomes have
-// equal fingerprints (the finaliser's hash of the ordering, the replica sizes,
-// their count and the roles), so a genome is compared in full only with
-// genomes of its fingerprint: first with the lowest-indexed one, found in an
-// open-addressing table (dup_table_size(P) >= 2P slots, linear probing, so
-// never full; a slot keeps its fingerprint and the smallest index that carries
-// it); if the two differ -- a 64-bit collision, or genomes that differ only
-// in sizes or role bits past their replica count, which the fingerprint does
-// not cover -- with every lower-indexed genome of its fingerprint.
-// From kDupTableFrom genomes on (below, the table's fill and extra launch cost
-// more than the quadratic test: 1,024 genomes +2% per generation, 4,096 -1.8%).
-constexpr int kDupTableFrom = 4096;
-constexpr uint64_t kNoKey = ~0ull;                       // an empty slot
-__device__ __forceinline__ uint64_t table_key(uint64_t h) { return h == kNoKey ? kNoKey - 1 : h; }
-__device__ __forceinline__ unsigned table_start(uint64_t k, unsigned mask) { return (unsigned)(k ^ (k >> 32)) & mask; }
-
-// (the table is filled with kNoKey and INT32_MAX beforehand)
-__global__ void __launch_bounds__(256) dup_insert_kernel(int P, const uint64_t *hash, unsigned long long *tkey,
-                                                         int32_t *tidx, unsigned mask)
-{
-    for (int g = blockIdx.x * blockDim.x + threadIdx.x; g < P; g += gridDim.x * blockDim.x) {
-        const uint64_t k = table_key(hash[g]);
-        unsigned s = table_start(k, mask);
-        for (unsigned i = 0; i <= mask; ++i, s = (s + 1) & mask) {   // (a free slot is always found)
-            const unsigned long long prev = atomicCAS(&tkey[s], (unsigned long long)kNoKey, (unsigned long long)k);
-            if (prev == kNoKey || prev == k) {
-                atomicMin(&tidx[s], g);
-                break;
-            }
-        }
-    }
-}
-
-// Whether genomes a and b are equal (ordering, sizes, replica count, roles); a warp.
-__device__ __forceinline__ bool same_genome(const DevPop &p, int a, int b, int M, int K, int lane)
-{
-    bool diff = p.nclus[a] != p.nclus[b] || p.roles[a] != p.roles[b];
-    for (int i = lane; i < M && !diff; i += 32) diff = p.perm[(size_t)a * M + i] != p.perm[(size_t)b * M + i];
-    for (int i = lane; i < K && !diff; i += 32) diff = p.sizes[(size_t)a * K + i] != p.sizes[(size_t)b * K + i];
-    return __ballot_sync(0xFFFFFFFFu, diff) == 0u;
-}
-
-// One warp per genome.
-__global__ void __launch_bounds__(256) dup_lookup_kernel(Dims dm, DevPop p, const uint64_t *hash,
-                                                         const unsigned long long *tkey, const int32_t *tidx,
-                                                         unsigned mask, int32_t *dup)
-{
-    const int lane = threadIdx.x & 31;
-    const int g = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    if (g >= dm.P) return;
-    const uint64_t hr = hash[g], k = table_key(hr);
-    int first = g;
-    if (lane == 0) {                                              // (present: g itself was inserted)
-        unsigned s = table_start(k, mask);
-        for (unsigned i = 0; i < mask && tkey[s] != k; ++i) s = (s + 1) & mask;
-        if (tkey[s] == k) first = tidx[s];
-    }
-    first = __shfl_sync(0xFFFFFFFFu, first, 0);
-    bool d = false;
-    if (first < g) {
-        d = same_genome(p, first, g, dm.M, dm.K, lane);
-        for (int base = first + 1; base < g && !d; base += 32) {  // a fingerprint shared by different genomes
-            const int o = base + lane;
-            unsigned b = __ballot_sync(0xFFFFFFFFu, o < g && hash[o] == hr);
-            while (b && !d) {
-                const int oo = base + __ffs(b) - 1;
-                b &= b - 1;
-                d = same_genome(p, oo, g, dm.M, dm.K, lane);
-            }
-        }
-    }
-    if (lane == 0) dup[g] = d;
-}
-
-// Below kDupTableFrom genomes, the duplicate test compares each genome with
-// every lower-indexed one: equal genomes have equal fitness (the evaluation is
-// deterministic) and equal fingerprints, so only those pairs are compared in
-// full.
-__global__ void __launch_bounds__(256) dup_kernel(Dims dm, DevPop p, const double *fit,
-                                                  const uint64_t *hash, int32_t *dup)
-{
-    __shared__ uint64_t s_w[kEliteTile], s_p[kEliteTile], s_h[kEliteTile];
-    const int lane = threadIdx.x & 31, wl = threadIdx.x >> 5;
-    const int g = blockIdx.x * (blockDim.x >> 5) + wl;
-    const bool live = g < dm.P;
-    const uint64_t *fk = reinterpret_cast<const uint64_t *>(fit);
-    const uint64_t w = live ? fk[(size_t)g * 4] : 0, ph = live ? fk[(size_t)g * 4 + 1] : 0, h = live ? hash[g] : 0;
-    const int M = dm.M, K = dm.K;
-    const int gmax = min(dm.P, (int)((blockIdx.x + 1) * (blockDim.x >> 5)));   // highest genome of the block
-    int d = 0;
-    for (int base = 0; base < gmax - 1; base += kEliteTile) {
-        __syncthreads();
-        for (int t = threadIdx.x; t < kEliteTile && base + t < dm.P; t += blockDim.x) {
-            s_w[t] = fk[(size_t)(base + t) * 4];
-            s_p[t] = fk[(size_t)(base + t) * 4 + 1];
-            s_h[t] = hash[base + t];
-        }
-        __syncthreads();
-        if (!live || d) continue;
-        const int lim = min(kEliteTile, g - base);
-        for (int t0 = 0; t0 < lim && !d; t0 += 32) {
-            const int t = t0 + lane;
-            const bool cand = t < lim && s_h[t] == h && s_w[t] == w && s_p[t] == ph;
-            unsigned b = __ballot_sync(0xFFFFFFFFu, cand);
-            while (b && !d) {
-                const int oo = base + t0 + __ffs(b) - 1;
-                b &= b - 1;
-                bool diff = p.nclus[oo] != p.nclus[g] || p.roles[oo] != p.roles[g];
-                for (int i = lane; i < M && !diff; i += 32) diff = p.perm[(size_t)oo * M + i] != p.perm[(size_t)g * M + i];
-                for (int i = lane; i < K && !diff; i += 32) diff = p.sizes[(size_t)oo * K + i] != p.sizes[(size_t)g * K + i];
-                d = __ballot_sync(0xFFFFFFFFu, diff) == 0u;
-            }
-        }
-    }
-    if (live && lane == 0) dup[g] = d;
-}
-
 // rank(g) = number of genomes before g in the elite order (duplicate flag,
 // w, phase, index); the first Q ranks are the elites, and the warp of an elite
 // copies it into slot rank(g) of the next population.
@@ -446,7 +370,7 @@ __global__ void __launch_bounds__(256) rank_kernel(Dims dm, const double *fit, c
 {
     __shared__ uint64_t s_w[kEliteTile], s_p[kEliteTile];
     __shared__ int s_d[kEliteTile];
-    if (ctl[2] != 0) return;                       // the candidate ranking took the elites
+    if (ctl[2] != 0) return;                       // elite_cand_rank_kernel took the elites
     const int lane = threadIdx.x & 31, wl = threadIdx.x >> 5;
     const int g = blockIdx.x * (blockDim.x >> 5) + wl;
     const bool live = g < dm.P;
@@ -481,182 +405,23 @@ __global__ void __launch_bounds__(256) rank_kernel(Dims dm, const double *fit, c
     }
 }
 
-// Elite selection without ranking every genome.  When at least Q genomes are
-// distinct, the elites are the Q first distinct genomes in the order (w,
-// phase, index), and each has w <= w_Q, the Q-th smallest w among the
-// distinct genomes (a genome with a larger w has at least Q distinct genomes
-// before it).  One CTA finds w_Q exactly by a radix select over the bit
-// patterns of w (8 passes of 8 bits, highest first) and lists the distinct
-// genomes with w <= w_Q; only they are ranked against the population.  When
-// w_Q is +inf (fewer than Q genomes have a finite w, as early in a search on
-// a large fleet) the finite ones are ranked and the rest of the elites are
-// the first distinct genomes of the (+inf, +inf) group in index order.  With
-// fewer than Q distinct genomes (duplicates then fill the elite slots) the
-// full ranking runs instead.  ctl: [0] w_Q bits, [1] candidates to rank,
-// [2] 1 = the selection applies (0: full ranking), [3] elites listed after
-// the candidates whose rank is their place in the list.
-constexpr int kSelThreads = 1024;
-
-__global__ void __launch_bounds__(kSelThreads) elite_select_kernel(int P, int Q, const double *fit, const int32_t *dup,
-                                                                   unsigned long long *ctl, int32_t *cand)
-{
-    __shared__ unsigned hist[256];
-    __shared__ unsigned long long s_prefix;
-    __shared__ unsigned s_need, s_distinct, s_ncand;
-    const uint64_t *fk = reinterpret_cast<const uint64_t *>(fit);
-    const int tid = threadIdx.x;
-    if (tid == 0) { s_prefix = 0; s_need = (unsigned)Q; s_distinct = 0; s_ncand = 0; }
-    __syncthreads();
-    unsigned nd = 0;
-    for (int g = tid; g < P; g += kSelThreads) nd += dup[g] == 0;
-    atomicAdd(&s_distinct, nd);
-    __syncthreads();
-    const bool apply = Q > 0 && s_distinct >= (unsigned)Q;
-    for (int pass = 0; apply && pass < 8; ++pass) {
-        const int shift = 56 - 8 * pass;
-        const uint64_t hi_mask = pass ? ~0ull << (shift + 8) : 0ull;
-        for (int b = tid; b < 256; b += kSelThreads) hist[b] = 0;
-        __syncthreads();
-        const uint64_t prefix = s_prefix;
-        for (int g = tid; g < P; g += kSelThreads) {
-            if (dup[g]) continue;
-            const uint64_t w = fk[(size_t)g * 4];
-            if ((w & hi_mask) == prefix) atomicAdd(&hist[(w >> shift) & 0xFFu], 1u);
-        }
-        __syncthreads();
-        if (tid < 32) {                                   // the bucket holding the need-th smallest:
-            const unsigned need = s_need;                 // a warp scan of eight-bin sums, then the
-            unsigned c = 0;                               // lane whose sums cross need scans its bins
-#pragma unroll
-            for (int j = 0; j < 8; ++j) c += hist[tid * 8 + j];
-            unsigned incl = c;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const unsigned y = __shfl_up_sync(0xFFFFFFFFu, incl, o);
-                if (tid >= o) incl += y;
-            }
-            const unsigned crossed = __ballot_sync(0xFFFFFFFFu, incl >= need);
-            if (tid == __ffs(crossed) - 1) {
-                unsigned left = need - (incl - c), b = (unsigned)tid * 8;
-                while (hist[b] < left) { left -= hist[b]; ++b; }
-                s_need = left;
-                s_prefix = prefix | ((uint64_t)b << shift);
-            }
-        }
-        __syncthreads();
-    }
-    __shared__ unsigned s_bad, s_wsum[kSelThreads / 32], s_run;
-    unsigned direct = 0;                                  // elites whose rank is their place in the list
-    bool use = apply;
-    if (apply) {
-        const uint64_t wq = s_prefix;
-        if (wq != kInfKey) {                              // rank every distinct genome with w <= w_Q
-            for (int g = tid; g < P; g += kSelThreads)
-                if (!dup[g] && fk[(size_t)g * 4] <= wq) cand[atomicAdd(&s_ncand, 1u)] = g;
-            __syncthreads();
-        } else {
-            // fewer than Q distinct genomes with a finite w: those are ranked; the
-            // rest of the elites are the first distinct genomes of the (+inf, +inf)
-            // group, in index order (an infinite w comes with an infinite phase;
-            // anything else takes the full ranking)
-            if (tid == 0) s_bad = 0;
-            __syncthreads();
-            for (int g = tid; g < P; g += kSelThreads) {
-                if (dup[g]) continue;
-                if (fk[(size_t)g * 4] != kInfKey) cand[atomicAdd(&s_ncand, 1u)] = g;
-                else if (fk[(size_t)g * 4 + 1] != kInfKey) s_bad = 1;
-            }
-            __syncthreads();
-            use = s_bad == 0;
-            const unsigned F = s_ncand, need = (unsigned)Q - F;
-            if (use) {
-                const int lane = tid & 31, wl = tid >> 5;
-                if (tid == 0) s_run = 0;
-                __syncthreads();
-                for (int base = 0; base < P && s_run < need; base += kSelThreads) {
-                    const int g = base + tid;
-                    const bool f = g < P && !dup[g] && fk[(size_t)g * 4] == kInfKey;
-                    const unsigned bal = __ballot_sync(0xFFFFFFFFu, f);
-                    if (lane == 0) s_wsum[wl] = __popc(bal);
-                    __syncthreads();
-                    unsigned before = 0;
-                    for (int w2 = 0; w2 < wl; ++w2) before += s_wsum[w2];
-                    const unsigned ord = s_run + before + __popc(bal & ((1u << lane) - 1u));
-                    if (f && ord < need) cand[F + ord] = g;
-                    __syncthreads();
-                    if (tid == 0) {
-                        unsigned t = 0;
-                        for (int w2 = 0; w2 < kSelThreads / 32; ++w2) t += s_wsum[w2];
-                        s_run += t;
-                    }
-                    __syncthreads();
-                }
-                direct = need;
-            }
-        }
-    }
-    if (tid == 0) {
-        ctl[0] = s_prefix;
-        ctl[1] = use ? s_ncand : 0;
-        ctl[2] = use ? 1ull : 0ull;
-        ctl[3] = use ? direct : 0;
-    }
-}
-
-// rank(g) for the candidates, one warp each.  Every genome before a candidate
-// in the elite order is distinct with a w no larger, so it is a candidate
-// itself: a candidate's rank is its count of candidates before it, taken
-// over tiles of the candidate list staged in shared memory.  An elite (rank
-// < Q) is copied into slot rank of the next population.
+// The listed genomes' ranks, a warp each; the elites are copied into slots
+// [0, Q) of the next population.
 __global__ void __launch_bounds__(256) elite_cand_rank_kernel(Dims dm, const double *fit,
                                                               const unsigned long long *ctl, const int32_t *cand,
                                                               int32_t *elite, double *elite_fit, DevPop src, DevPop dst)
 {
-    __shared__ uint64_t s_w[kEliteTile], s_p[kEliteTile];
-    __shared__ int s_g[kEliteTile];
-    if (ctl[2] == 0) return;
-    const unsigned ncand = (unsigned)ctl[1], total = ncand + (unsigned)ctl[3];
-    const int lane = threadIdx.x & 31, NWB = blockDim.x >> 5;
-    const uint64_t *fk = reinterpret_cast<const uint64_t *>(fit);
-    for (unsigned i0 = blockIdx.x * NWB; i0 < total; i0 += gridDim.x * NWB) {   // uniform over the block
-        const unsigned i = i0 + (threadIdx.x >> 5);
-        const bool live = i < total, ranked = i < ncand;
-        const int g = live ? cand[i] : 0;
-        const uint64_t w = ranked ? fk[(size_t)g * 4] : 0, ph = ranked ? fk[(size_t)g * 4 + 1] : 0;
-        int rank = (int)i;                               // entries past ncand: rank = place in the list
-        if (i0 < ncand) {
-            int cnt = 0;
-            for (unsigned base = 0; base < ncand; base += kEliteTile) {
-                __syncthreads();
-                for (unsigned t = threadIdx.x; t < kEliteTile && base + t < ncand; t += blockDim.x) {
-                    const int h = cand[base + t];
-                    s_g[t] = h;
-                    s_w[t] = fk[(size_t)h * 4];
-                    s_p[t] = fk[(size_t)h * 4 + 1];
-                }
-                __syncthreads();
-                if (ranked) {
-                    const unsigned lim = min((unsigned)kEliteTile, ncand - base);
-                    for (unsigned t = lane; t < lim; t += 32)
-                        cnt += elite_before(0, s_w[t], s_p[t], s_g[t], 0, w, ph, g);
-                }
-            }
-#pragma unroll
-            for (int x = 16; x; x >>= 1) cnt += __shfl_xor_sync(0xFFFFFFFFu, cnt, x);
-            if (ranked) rank = cnt;
+    rank_listed(dm.Q, fit, ctl, cand, [&](int rank, int g, int lane) {
+        const int M = dm.M, K = dm.K;
+        for (int j = lane; j < M; j += 32) dst.perm[(size_t)rank * M + j] = src.perm[(size_t)g * M + j];
+        for (int j = lane; j < K; j += 32) dst.sizes[(size_t)rank * K + j] = src.sizes[(size_t)g * K + j];
+        if (lane < 4) elite_fit[(size_t)rank * 4 + lane] = fit[(size_t)g * 4 + lane];
+        if (lane == 0) {
+            dst.nclus[rank] = src.nclus[g];
+            dst.roles[rank] = src.roles[g];
+            elite[rank] = g;
         }
-        if (live && rank < dm.Q) {
-            const int M = dm.M, K = dm.K;
-            for (int j = lane; j < M; j += 32) dst.perm[(size_t)rank * M + j] = src.perm[(size_t)g * M + j];
-            for (int j = lane; j < K; j += 32) dst.sizes[(size_t)rank * K + j] = src.sizes[(size_t)g * K + j];
-            if (lane == 0) {
-                dst.nclus[rank] = src.nclus[g];
-                dst.roles[rank] = src.roles[g];
-                elite[rank] = g;
-                for (int q = 0; q < 4; ++q) elite_fit[(size_t)rank * 4 + q] = fit[(size_t)g * 4 + q];
-            }
-        }
-    }
+    });
 }
 
 struct GaThr {
@@ -884,33 +649,37 @@ cudaError_t launch_init(const e2_ctx *c, const DevPop &p, uint64_t seed)
     return cudaGetLastError();
 }
 
-// Duplicate flags, then ranks; the elites go to slots [0, Q) of dst.
+// Duplicate flags, then the selection; the elites go to slots [0, Q) of dst.
 cudaError_t launch_elites(const e2_ctx *c, const DevPop &p, const DevPop &dst)
 {
-    const unsigned blocks = (unsigned)(((size_t)c->dm.P * 32 + 255) / 256);
-    const bool table = c->dm.P >= kDupTableFrom;
+    const int P = c->dm.P, Q = c->dm.Q;
+    const unsigned blocks = (unsigned)(((size_t)P * 32 + 255) / 256);
+    const bool table = P >= kDupTableFrom;
+    const unsigned tsize = dup_table_size(P);
     if (table) {
-        const unsigned tsize = dup_table_size(c->dm.P);
-        cudaError_t e = cudaMemsetAsync(c->dup_key, 0xFF, sizeof(uint64_t) * tsize, c->stream);
-        if (e == cudaSuccess) e = cudaMemsetAsync(c->dup_idx, 0x7F, sizeof(int32_t) * tsize, c->stream);
+        const cudaError_t e = cudaMemsetAsync(c->dup_tab, 0x7F, sizeof(*c->dup_tab) * tsize, c->stream);
         if (e != cudaSuccess) return e;
-        dup_insert_kernel<<<(unsigned)((c->dm.P + 255) / 256), 256, 0, c->stream>>>(
-            c->dm.P, c->hash, reinterpret_cast<unsigned long long *>(c->dup_key), c->dup_idx, tsize - 1);
-        dup_lookup_kernel<<<blocks, 256, 0, c->stream>>>(c->dm, p, c->hash,
-                                                         reinterpret_cast<const unsigned long long *>(c->dup_key),
-                                                         c->dup_idx, tsize - 1, c->dup);
+        dup_insert_kernel<<<(unsigned)((P + 255) / 256), 256, 0, c->stream>>>(P, c->hash, c->dup_tab, tsize - 1);
+        dup_lookup_kernel<<<blocks, 256, 0, c->stream>>>(c->dm, p, c->hash, c->dup_tab, tsize - 1, c->dup);
     } else {
-        dup_kernel<<<blocks, 256, 0, c->stream>>>(c->dm, p, c->fit, c->hash, c->dup);
+        // (four genomes per warp and block: more blocks would fill more tables than they look up in)
+        const int per = 4 * kDupThreads / 32;
+        const size_t smem = sizeof(unsigned long long) * tsize;
+        if (smem > 48 * 1024) {
+            const cudaError_t e = cudaFuncSetAttribute(dup_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            if (e != cudaSuccess) return e;
+        }
+        dup_kernel<<<(unsigned)((P + per - 1) / per), kDupThreads, smem, c->stream>>>(c->dm, p, c->hash, c->dup, tsize - 1);
     }
-    if (c->dm.Q > 0) {
-        elite_select_kernel<<<1, kSelThreads, 0, c->stream>>>(c->dm.P, c->dm.Q, c->fit, c->dup, c->elite_ctl,
-                                                              c->elite_cand);
-        elite_cand_rank_kernel<<<152 * 4, 256, 0, c->stream>>>(c->dm, c->fit, c->elite_ctl, c->elite_cand,
-                                                               c->elite, c->elite_fit, p, dst);
+    if (Q > 0) {
+        elite_select_kernel<<<1, kSelThreads, 0, c->stream>>>(P, Q, c->fit, c->dup, c->elite_ctl, c->elite_cand);
+        const unsigned rb = (unsigned)((Q + 7) / 8 < 152 * 4 ? (Q + 7) / 8 : 152 * 4);
+        elite_cand_rank_kernel<<<rb, 256, 0, c->stream>>>(c->dm, c->fit, c->elite_ctl, c->elite_cand, c->elite,
+                                                          c->elite_fit, p, dst);
         rank_kernel<<<blocks, 256, 0, c->stream>>>(c->dm, c->fit, c->dup, c->elite, c->elite_fit, p, dst,
                                                    c->elite_ctl);
     }
-    c->launches += (table ? 2 : 1) + (c->dm.Q > 0 ? 3 : 0);
+    c->launches += (table ? 2 : 1) + (Q > 0 ? 3 : 0);
     return cudaGetLastError();
 }
 
