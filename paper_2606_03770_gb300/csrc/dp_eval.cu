@@ -531,7 +531,7 @@ __global__ void __launch_bounds__(32 * kLayeredWarps) dp_layered_kernel(Dims dm,
         for (int k = tid; k < m; k += blockDim.x) devs[k] = pop.perm[(size_t)g * M + off + k];
         __syncthreads();
         for (int k = tid; k < m; k += blockDim.x)
-            tk[k] = k ? dkey(tb.tau[((size_t)v * M + devs[k - 1]) * M + devs[k]]) : 0ull;
+            tk[k] = k ? dkey(tb.tau[((size_t)v * M + devs[k - 1]) * M + devs[k]].t) : 0ull;
         // device k's (0-based) times: entry [j][n - 1] of blocks j .. j+n-1, with the head when mf
         auto rows = [&](int k, int mf) -> const double * { return lc + ((size_t)devs[k] * 2 + mf) * NN; };
         unsigned long long probes = 0;
@@ -1549,7 +1549,7 @@ cudaError_t configure_eval(e2_ctx *c)
 cudaError_t launch_eval(const e2_ctx *c, const DevPop &p)
 {
     Tables tb{c->rate, c->bw, c->mem, c->rate_cpu, c->bw_cpu, c->mem_cpu, c->prof, c->leaf, c->tau,
-              c->capg, c->tau_lb, c->leaf_rank, c->tau_rank, c->lcost, c->drec, c->fxs, c->prec, c->prech, c->capv,
+              c->capg, c->leaf_rank, c->lcost, c->drec, c->fxs, c->prec, c->prech, c->capv,
               c->ibw, c->fpr};
     EvalOut out{c->fit, c->layers, c->master, c->bsel, c->T, c->L, c->hash, c->stats, c->gpu_layers};
     SlotInfo si{c->slot_off, c->slot_info};

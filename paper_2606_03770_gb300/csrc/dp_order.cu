@@ -68,6 +68,17 @@ __device__ __forceinline__ float trunc_float(double x)
     return __uint_as_float(((hi - 0x38000000u) << 3) | (lo >> 29));
 }
 
+// A link's record in one 16-byte load.
+__device__ __forceinline__ LinkRec load_link(const Tables &tb, size_t i)
+{
+    const uint4 x = reinterpret_cast<const uint4 *>(tb.tau)[i];
+    LinkRec r;
+    r.t = __hiloint2double((int)x.y, (int)x.x);
+    r.key = x.z;
+    r.lb = __uint_as_float(x.w);
+    return r;
+}
+
 // Exclusive prefix sums over devices 0..32 D - 1 (lane l holds l, l + 32, ...).
 template <int D>
 __device__ __forceinline__ void exclusive_sums(const int (&x)[D], int (&ex)[D], int lane)
@@ -177,12 +188,13 @@ __global__ void __launch_bounds__(32 * dp_order_warps(D == 1 ? 0 : 1), order_cta
                 int c0[D], c1[D];
                 float cinv[D], hb[D], hr[D], gcap[D];
                 uint32_t tr[D];
+                double tk[D];                              // link times (D > 1: read at the end)
                 uint32_t floor_l = 0;
                 float tf_l = 0.0f, hmin_l = 3e38f;
 #pragma unroll
                 for (int j = 0; j < D; ++j) {
                     const int k = lane + 32 * j;
-                    ro[j] = 0; c0[j] = c1[j] = 0; cinv[j] = hb[j] = hr[j] = gcap[j] = 0.0f; tr[j] = 0;
+                    ro[j] = 0; c0[j] = c1[j] = 0; cinv[j] = hb[j] = hr[j] = gcap[j] = 0.0f; tr[j] = 0; tk[j] = 0.0;
                     if (k < m) {
                         const uint4 rec = tb.drec[vM + d[j]];
                         c0[j] = min((int)(rec.x & 0xFFFFu), W);
@@ -195,9 +207,10 @@ __global__ void __launch_bounds__(32 * dp_order_warps(D == 1 ? 0 : 1), order_cta
                         }
                         ro[j] = (uint32_t)(vM + d[j]) * 2u * LS;
                         if (k > 0) {
-                            const size_t e = (vM + dp[j]) * M + d[j];
-                            tr[j] = tb.tau_rank[e];
-                            tf_l = fmaxf(tf_l, tb.tau_lb[e]);
+                            const LinkRec link = load_link(tb, (vM + dp[j]) * M + d[j]);
+                            tr[j] = link.key;
+                            tf_l = fmaxf(tf_l, link.lb);
+                            if (D == 1) tk[j] = link.t;
                         }
                         if (c1[j] >= 1) hmin_l = fminf(hmin_l, hb[j]);
                         if (c0[j] >= 1) tf_l = fmaxf(tf_l, __frcp_rn(cinv[j]));
@@ -590,16 +603,16 @@ __global__ void __launch_bounds__(32 * dp_order_warps(D == 1 ? 0 : 1), order_cta
                 }
                 // ---- T: the largest stage or link time of the partition (equal to V*); the
                 //      decode test on Lambda, in fixed point where that decides it
-                double lk[D], tk[D];
+                double lk[D];
                 uint64_t tmax = 0;
                 float lam_f = 0.0f;
 #pragma unroll
                 for (int j = 0; j < D; ++j) {
                     const int k = lane + 32 * j;
-                    lk[j] = tk[j] = 0.0;
+                    lk[j] = 0.0;
                     if (k < m) {
                         lk[j] = tb.leaf[ro[j] + nk[j] - 1];
-                        if (k > 0) tk[j] = tb.tau[(vM + dp[j]) * M + d[j]];
+                        if (D > 1 && k > 0) tk[j] = tb.tau[(vM + dp[j]) * M + d[j]].t;
                     }
                     tmax = umax64(tmax, umax64(dkey(lk[j]), dkey(tk[j])));
                     lam_f += trunc_float(lk[j]) + trunc_float(tk[j]);
@@ -688,7 +701,7 @@ __global__ void __launch_bounds__(32 * dp_order_warps(D == 1 ? 0 : 1), order_cta
                             nb_ = lay[k];
                         }
                         l[q] = tb.leaf[((vM + dk) * 2 + (k == acc_mu)) * LS + nb_ - 1];
-                        if (k > 0) t[q] = tb.tau[(vM + dprev) * M + dk];
+                        if (k > 0) t[q] = tb.tau[(vM + dprev) * M + dk].t;
                         dprev = dk;
                     }
                 }

@@ -20,8 +20,8 @@ thread_local char g_create_error[256] = "";
 size_t align_up(size_t x, size_t a = 256) { return (x + a - 1) / a * a; }
 
 struct Layout {
-    size_t rate, bw, mem, rate_cpu, bw_cpu, mem_cpu, link_bw, cong, prof, leaf, tau, tau_lb, capg, prec, prech, capv, ibw, fpr,
-        leaf_sorted, beff_sorted, tau_sorted, leaf_rank, tau_rank, gpu_layers, psum, lcost, drec, fxs;
+    size_t rate, bw, mem, rate_cpu, bw_cpu, mem_cpu, link_bw, cong, prof, leaf, tau, capg, prec, prech, capv, ibw, fpr,
+        leaf_sorted, leaf_rank, gpu_layers, psum, lcost, drec, fxs;
     size_t perm[2], sizes[2], nclus[2], roles[2];
     size_t fit, layers, master, bsel, T, L, hash, dup, dup_tab, elite, elite_fit, elite_ctl, elite_cand, stats, err, list_ctrl, list_hist, items, slot_off, slot_info,
         split_T, split_L, split_mu, split_code, split_layers, var_T, var_L, var_mu, var_layers, var_best, total;
@@ -54,7 +54,7 @@ Layout layout(int M, int N, int b_max, int P, int Q, int K, bool layered = false
     l.cong = take(8 * MM);
     l.prof = take(8 * kNumProf * V);
     l.leaf = take(8 * V * M * 2 * (size_t)l.LS);
-    l.tau = take(8 * V * MM);
+    l.tau = take(sizeof(LinkRec) * V * MM);
     l.capg = take(4 * V * M * 2);
     l.prec = take(16 * (size_t)M);
     l.prech = take(8 * (size_t)M);
@@ -63,12 +63,8 @@ Layout layout(int M, int N, int b_max, int P, int Q, int K, bool layered = false
     l.fpr = take(16 * V);
     l.drec = take(16 * V * M);
     l.fxs = take(4 * V);
-    l.tau_lb = take(4 * V * MM);
     l.leaf_sorted = take(8 * V * rank_pow2((size_t)M * 2 * N));
-    l.beff_sorted = take(8 * rank_pow2(MM));
-    l.tau_sorted = take(8 * V * MM);
     l.leaf_rank = take(4 * V * M * 2 * (size_t)l.LS);
-    l.tau_rank = take(4 * V * MM);
     for (int b = 0; b < 2; ++b) {
         l.perm[b] = take(2 * (size_t)P * M);
         l.sizes[b] = take(2 * (size_t)P * K);
@@ -466,7 +462,7 @@ int e2_create(const e2_devices *devs, const e2_links *links, const e2_layer_prof
     c->cong = reinterpret_cast<double *>(ws + l.cong);
     c->prof = reinterpret_cast<uint64_t *>(ws + l.prof);
     c->leaf = reinterpret_cast<double *>(ws + l.leaf);
-    c->tau = reinterpret_cast<double *>(ws + l.tau);
+    c->tau = reinterpret_cast<LinkRec *>(ws + l.tau);
     c->prec = reinterpret_cast<uint4 *>(ws + l.prec);
     c->prech = reinterpret_cast<float2 *>(ws + l.prech);
     c->capv = reinterpret_cast<uint32_t *>(ws + l.capv);
@@ -474,12 +470,8 @@ int e2_create(const e2_devices *devs, const e2_links *links, const e2_layer_prof
     c->fpr = reinterpret_cast<float4 *>(ws + l.fpr);
     c->drec = reinterpret_cast<uint4 *>(ws + l.drec);
     c->fxs = reinterpret_cast<float *>(ws + l.fxs);
-    c->tau_lb = reinterpret_cast<float *>(ws + l.tau_lb);
     c->leaf_sorted = reinterpret_cast<uint64_t *>(ws + l.leaf_sorted);
-    c->beff_sorted = reinterpret_cast<uint64_t *>(ws + l.beff_sorted);
-    c->tau_sorted = reinterpret_cast<double *>(ws + l.tau_sorted);
     c->leaf_rank = reinterpret_cast<uint32_t *>(ws + l.leaf_rank);
-    c->tau_rank = reinterpret_cast<uint32_t *>(ws + l.tau_rank);
     for (int b = 0; b < 2; ++b) c->pop[b] = pop_at(ws, l, b);
     c->fit = reinterpret_cast<double *>(ws + l.fit);
     c->layers = reinterpret_cast<int16_t *>(ws + l.layers);
@@ -545,9 +537,8 @@ int e2_create(const e2_devices *devs, const e2_links *links, const e2_layer_prof
         chk(cudaMemcpyAsync(c->psum + 2 * V * ((size_t)N + 1), prof->PM, row, cudaMemcpyHostToDevice, c->stream));
     }
     if (e == cudaSuccess) e = launch_tables(c);
+    if (e == cudaSuccess) e = build_stage_keys(c);
     if (e == cudaSuccess) e = launch_tau(c);
-    if (e == cudaSuccess) e = build_leaf_sorted(c);
-    if (e == cudaSuccess) e = build_ranks(c);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
     delete[] prof_h;
     if (e != cudaSuccess) return fail_free(E2_ECUDA, cudaGetErrorString(e));
@@ -745,7 +736,6 @@ int e2_redraw_congestion(e2_ctx *c, uint64_t seed, uint32_t generation)
     if (!c) return E2_EINVAL;
     E2_CUDA(c, launch_redraw(c, seed, generation));
     E2_CUDA(c, launch_tau(c));
-    E2_CUDA(c, build_ranks(c));
     c->evaluated = false;
     return E2_OK;
 }

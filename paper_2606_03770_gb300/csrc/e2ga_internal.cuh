@@ -108,6 +108,14 @@ struct Dims {
     int layered;         // 1: blocks of several types (per-layer prefix sums): the plain-scan DP path
 };
 
+// A link of a variant: its time, its order key against the stage times
+// (ranks.cu) and the time rounded down.
+struct __align__(16) LinkRec {
+    double t;
+    uint32_t key;
+    float lb;
+};
+
 struct Tables {
     const double *rate, *bw;
     const uint64_t *mem;
@@ -115,12 +123,10 @@ struct Tables {
     const uint64_t *mem_cpu;           // [M] host memory for blocks, bytes (offload only)
     const uint64_t *prof;      // [kNumProf][V]
     const double *leaf;        // [V][M][2][LS]: leaf[((v*M+d)*2+mf)*LS + n-1] = l_d(n blocks, master mf)
-    const double *tau;         // [V][M][M]
+    const LinkRec *tau;        // [V][M][M]
     const int32_t *capg;       // [V][M][2]: most blocks in device memory, without / with the head (-1: the head
                                // does not fit)
-    const float *tau_lb;       // [V][M][M]: tau rounded down
     const uint32_t *leaf_rank; // [V][M][2][LS]: order key of leaf within its variant's value set
-    const uint32_t *tau_rank;  // [V][M][M]
     const double *lcost;       // [V][M][2][N][N] (per-layer profiles only): lcost[((v*M+d)*2+mf)*N*N + j*N + n-1]
                                // = time of blocks j..j+n-1 on device d (+inf beyond the model or memory)
     const uint4 *drec;         // [V][M] the DP's view of a device: {cap | cap with head << 16, and as floats
@@ -218,6 +224,18 @@ __device__ __forceinline__ uint32_t below(uint32_t x, uint32_t n)
     return (uint32_t)(((uint64_t)x * n) >> 32);
 }
 
+// Entries of the ascending list a[0, n) below x.
+__device__ __forceinline__ size_t count_below(const uint64_t *a, size_t n, uint64_t x)
+{
+    size_t lo = 0, hi = n;
+    while (lo < hi) {
+        const size_t mid = (lo + hi) >> 1;
+        if (a[mid] < x) lo = mid + 1;
+        else hi = mid;
+    }
+    return lo;
+}
+
 __device__ __forceinline__ uint64_t dkey(double x) { return (uint64_t)__double_as_longlong(x); }
 __device__ __forceinline__ double keyd(uint64_t k) { return __longlong_as_double((long long)k); }
 __device__ __forceinline__ uint64_t umin64(uint64_t a, uint64_t b) { return a < b ? a : b; }
@@ -245,18 +263,15 @@ struct e2_ctx {
     int16_t *gpu_layers = nullptr;                    // [P][M] G of the G--C split (offload only)
     double *link_bw = nullptr, *cong = nullptr;
     uint64_t *prof = nullptr;
-    double *leaf = nullptr, *tau = nullptr;
+    double *leaf = nullptr;
+    e2::LinkRec *tau = nullptr;
     uint4 *prec = nullptr;            // [M]
     float2 *prech = nullptr;          // [M]
     uint32_t *capv = nullptr;         // [M][V]
     float *ibw = nullptr;             // [M][M]
     float4 *fpr = nullptr;            // [V]
-    float *tau_lb = nullptr;
     uint64_t *leaf_sorted = nullptr;  // [V][pow2(2 M N)] sorted stage-time keys
-    uint64_t *beff_sorted = nullptr;  // [pow2(M M)] sorted effective link bandwidths
-    double *tau_sorted = nullptr;     // [V][M M] sorted link times
     uint32_t *leaf_rank = nullptr;    // [V][M][2][LS]
-    uint32_t *tau_rank = nullptr;     // [V][M][M]
     e2::DevPop pop[2]{};
     int cur = 0;
     double *fit = nullptr;
@@ -332,6 +347,5 @@ cudaError_t dp_order_launch(int grid, int mmax, int cls, cudaStream_t stream, co
 size_t dp_layered_smem_bytes(int M, int N);   // the plain-scan DP's shared memory for the largest replica
 cudaError_t configure_eval(e2_ctx *c);   // shared memory limit and persistent grid size
 size_t rank_pow2(size_t n);
-cudaError_t build_leaf_sorted(const e2_ctx *c);   // once per context
-cudaError_t build_ranks(const e2_ctx *c);         // after every change of the link table
+cudaError_t build_stage_keys(const e2_ctx *c);    // once per context, before launch_tau
 }  // namespace e2

@@ -167,21 +167,25 @@ __global__ void captab_kernel(Dims dm, const double *rate, const double *bw, con
     }
 }
 
-// tau_v(a, b) = A_v / (B(a,b) * congestion(a,b)) (Sec. 3.2), the same rounded
-// down to float for the DP's estimate, and 1 / (B * congestion) rounded down
-// for the latency bound.
+// tau_v(a, b) = A_v / (B(a,b) * congestion(a,b)) (Sec. 3.2), its order key (the
+// stage times of the variant that are no larger, ranks.cu) and itself rounded
+// down to float for the DP's estimate, one 16-byte record per link and variant;
+// and 1 / (B * congestion) rounded down for the latency bound.
 __global__ void tau_kernel(Dims dm, const double *link_bw, const double *cong, const uint64_t *prof,
-                           double *tau, float *tau_lb, float *ibw)
+                           const uint64_t *sorted, size_t cap, LinkRec *tau, float *ibw)
 {
-    const size_t MM = (size_t)dm.M * dm.M, total = (size_t)dm.V * MM;
+    const size_t MM = (size_t)dm.M * dm.M, total = (size_t)dm.V * MM, n = (size_t)dm.M * 2 * dm.N;
     for (size_t idx = blockIdx.x * (size_t)blockDim.x + threadIdx.x; idx < total;
          idx += (size_t)gridDim.x * blockDim.x) {
         const int v = (int)(idx / MM);
         const size_t ab = idx - (size_t)v * MM;
         const double beff = link_bw[ab] * cong[ab];
-        const double t = __ull2double_rn(prof[kAct * dm.V + v]) / beff;
-        tau[idx] = t;
-        tau_lb[idx] = __double2float_rd(t);
+        LinkRec r;
+        r.t = __ull2double_rn(prof[kAct * dm.V + v]) / beff;
+        const uint64_t x = dkey(r.t);
+        r.key = x >= kInfKey ? 0xFFFFFFFFu : (uint32_t)count_below(sorted + v * cap, n, x + 1);
+        r.lb = __double2float_rd(r.t);
+        tau[idx] = r;
         if (v == 0) ibw[ab] = __double2float_rd(__ddiv_rd(1.0, beff));
     }
 }
@@ -621,7 +625,9 @@ cudaError_t launch_tables(const e2_ctx *c)
 cudaError_t launch_tau(const e2_ctx *c)
 {
     const size_t total = (size_t)c->dm.V * c->dm.M * c->dm.M;
-    tau_kernel<<<grid_for(total, 256), 256, 0, c->stream>>>(c->dm, c->link_bw, c->cong, c->prof, c->tau, c->tau_lb, c->ibw);
+    tau_kernel<<<grid_for(total, 256), 256, 0, c->stream>>>(c->dm, c->link_bw, c->cong, c->prof,
+                                                            c->leaf_sorted, rank_pow2((size_t)c->dm.M * 2 * c->dm.N), c->tau,
+                                                            c->ibw);
     ++c->launches;
     return cudaGetLastError();
 }

