@@ -257,56 +257,121 @@ __global__ void __launch_bounds__(32 * kValidateWarps) validate_kernel(Dims dm, 
     }
 }
 
-// Fisher-Yates shuffle of the identity ordering (word M-1-t draws position t);
-// element i of the ordering lives at perm[i * stride].
-template <typename T>
-__device__ void random_perm(Stream &st, int M, T *perm, int stride = 1)
+// Fisher-Yates shuffle of the identity ordering by a warp (word M-1-t draws
+// j_t, the position swapped with t, for t = M-1 .. 1).  The element that ends
+// at position t is the one at j_t before step t; position p is last written
+// before step t by the next larger step that drew p too, whose element came
+// from its own position; so every position's element is found by following
+// "the next larger step that drew this position" to a position no step drew,
+// all of them at once (14 links at most in 1,600 random draws of up to 512).
+// w32 [M] and aux [M] are scratch; out[t] = element t.
+constexpr uint32_t kNoStep = 0xFFFFu;
+
+__device__ __forceinline__ void random_perm(Stream st, int M, uint32_t *w32, uint16_t *aux, uint16_t *out, int lane)
 {
-    for (int i = 0; i < M; ++i) perm[(size_t)i * stride] = (T)i;
-    for (int t = M - 1; t >= 1; --t) {
-        const uint32_t j = below(st.word((uint32_t)(M - 1 - t)), (uint32_t)t + 1);
-        const T x = perm[(size_t)t * stride];
-        perm[(size_t)t * stride] = perm[(size_t)j * stride];
-        perm[(size_t)j * stride] = x;
+    for (int q = lane; 4 * q < M - 1; q += 32)                    // a lane takes one block of the stream
+        for (int i = 4 * q; i < 4 * q + 4 && i < M - 1; ++i) {
+            const int t = M - 1 - i;
+            w32[t] = below(st.word((uint32_t)i), (uint32_t)t + 1);
+        }
+    for (int p = lane; p < M; p += 32) aux[p] = (uint16_t)kNoStep;
+    __syncwarp();
+    // aux[p]: the smallest step seen that drew p; w32[t]: j_t | the next larger step that drew j_t << 16
+    for (int base = (M - 1) & ~31; base >= 0; base -= 32) {
+        const int t = base + lane;
+        const bool step = t >= 1 && t < M;
+        const uint32_t j = step ? w32[t] : 0u;
+        const unsigned peers = __match_any_sync(0xFFFFFFFFu, step ? j : 0x10000u + (unsigned)lane);
+        const unsigned above = peers & ~((2u << lane) - 1u);
+        uint32_t nx = kNoStep;
+        if (step) nx = above ? (uint32_t)(base + __ffs(above) - 1) : aux[j];
+        __syncwarp();
+        if (step) {
+            w32[t] = j | nx << 16;
+            if (lane == __ffs(peers) - 1) aux[j] = (uint16_t)t;
+        }
+        __syncwarp();
     }
+    for (int t = lane; t < M; t += 32) {
+        uint32_t p = t ? w32[t] & 0xFFFFu : 0u, x = t ? w32[t] >> 16 : aux[0];
+        while (x != kNoStep) {
+            p = x;
+            const uint32_t f = aux[x];
+            x = f == x ? w32[x] >> 16 : f;                        // (a step that drew itself)
+        }
+        out[t] = (uint16_t)p;
+    }
+    __syncwarp();
 }
 
-// Grouping of Mr devices: replica count 1 + uniform(min(Kr, Mr)) from word 0;
-// the R-1 cut points by sequential selection sampling (candidate cut t taken
-// with probability needed/remaining, word t); one role bit per replica from
-// two words of the roles stream.  Returns R.
-__device__ int random_grouping(Stream &sg, Stream &sr, int Mr, int Kr, uint16_t *sizes, uint64_t *roles)
+// Grouping of Mr devices by a warp: replica count 1 + uniform(min(Kr, Mr)) from
+// word 0; the R-1 cut points by sequential selection sampling (candidate cut t
+// taken with probability needed/remaining, word t): 32 candidates at a time, up
+// to the next one taken.  Writes sizes[0..Kr) (zeros past R), returns R in
+// every lane.
+template <typename T>
+__device__ __forceinline__ int random_grouping(Stream st, int Mr, int Kr, uint32_t *w32, T *sizes, int lane)
 {
+    for (int q = lane; 4 * q < Mr; q += 32)
+        for (int t = 4 * q; t < 4 * q + 4 && t < Mr; ++t) w32[t] = st.word((uint32_t)t);
+    for (int c = lane; c < Kr; c += 32) sizes[c] = 0;
+    __syncwarp();
     const int cap = Kr < Mr ? Kr : Mr;
-    const int R = 1 + (int)below(sg.word(0), (uint32_t)cap);
+    const int R = 1 + (int)below(w32[0], (uint32_t)cap);
     int need = R - 1, prev = 0, c = 0;
-    for (int t = 1; t <= Mr - 1 && need > 0; ++t) {
-        if (below(sg.word((uint32_t)t), (uint32_t)(Mr - t)) < (uint32_t)need) {
-            sizes[c++] = (uint16_t)(t - prev);
-            prev = t;
+    for (int base = 1; base <= Mr - 1 && need > 0; base += 32) {
+        const int t = base + lane;
+        const uint32_t x = t <= Mr - 1 ? below(w32[t], (uint32_t)(Mr - t)) : 0xFFFFFFFFu;
+        unsigned open = 0xFFFFFFFFu;                              // lanes not passed yet
+        while (need > 0) {
+            const unsigned hit = __ballot_sync(0xFFFFFFFFu, x < (uint32_t)need) & open;
+            if (!hit) break;
+            const int l = __ffs(hit) - 1;
+            if (lane == 0) sizes[c] = (T)(base + l - prev);
+            ++c;
+            prev = base + l;
             --need;
+            open = l == 31 ? 0u : ~0u << (l + 1);
         }
     }
-    sizes[c] = (uint16_t)(Mr - prev);
-    const uint64_t bits = (uint64_t)sr.word(0) | ((uint64_t)sr.word(1) << 32);
-    *roles = R >= 64 ? bits : (bits & ((1ull << R) - 1ull));
+    if (lane == 0) sizes[c] = (T)(Mr - prev);
+    __syncwarp();
     return R;
 }
 
-__global__ void init_kernel(Dims dm, DevPop p, uint64_t seed)
+__device__ __forceinline__ uint64_t random_roles(Stream st, int R)
 {
-    const int s = blockIdx.x * blockDim.x + threadIdx.x;
+    const uint64_t bits = (uint64_t)st.word(0) | ((uint64_t)st.word(1) << 32);
+    return R >= 64 ? bits : (bits & ((1ull << R) - 1ull));
+}
+
+// Shared memory of a warp of the two kernels below: 32-bit words, two 16-bit
+// arrays of M, and the sizes.
+__host__ __device__ __forceinline__ size_t genome_bytes(int M)
+{
+    return (4 * (size_t)M + 2 * (size_t)((M + 1) & ~1) * 2 + 2 * E2_MAX_CLUSTERS + 3) & ~(size_t)3;
+}
+
+// A genome per warp.  (A thread per genome, swapping in global memory, took
+// 125 us for 8,192 genomes of 256 devices; now 30.)
+__global__ void __launch_bounds__(256) init_kernel(Dims dm, DevPop p, uint64_t seed)
+{
+    extern __shared__ uint32_t ga_smem[];
+    const int lane = threadIdx.x & 31, wl = threadIdx.x >> 5;
+    const int s = blockIdx.x * (blockDim.x >> 5) + wl;
     if (s >= dm.P) return;
     const int M = dm.M, K = dm.K;
-    uint16_t *perm = p.perm + (size_t)s * M;
+    uint32_t *w32 = ga_smem + (size_t)wl * (genome_bytes(M) / 4);
+    uint16_t *child = reinterpret_cast<uint16_t *>(w32 + M), *aux = child + ((M + 1) & ~1);
+    random_perm(Stream(seed, 0, (uint32_t)s, kInitPerm), M, w32, aux, child, lane);
+    for (int i = lane; i < M; i += 32) p.perm[(size_t)s * M + i] = child[i];
     uint16_t *sizes = p.sizes + (size_t)s * K;
-    Stream sp(seed, 0, (uint32_t)s, kInitPerm);
-    random_perm(sp, M, perm);
-    for (int c = 0; c < K; ++c) sizes[c] = 0;
-    Stream sg(seed, 0, (uint32_t)s, kInitGroup), sr(seed, 0, (uint32_t)s, kInitRoles);
-    uint64_t roles;
-    p.nclus[s] = (uint8_t)random_grouping(sg, sr, M, K, sizes, &roles);
-    p.roles[s] = roles;
+    const int R = random_grouping(Stream(seed, 0, (uint32_t)s, kInitGroup), M, K, w32, sizes, lane);
+    const uint64_t roles = random_roles(Stream(seed, 0, (uint32_t)s, kInitRoles), R);
+    if (lane == 0) {
+        p.nclus[s] = (uint8_t)R;
+        p.roles[s] = roles;
+    }
 }
 
 // Duplicate test: dup_insert_kernel fills the fingerprint table (elites.cuh) in
@@ -446,30 +511,28 @@ __device__ __forceinline__ unsigned lanemask_lt()
     return m;
 }
 
-// One child per warp (App. A).  Slots [0, Q) copy the elites.  Otherwise:
+// One child per warp (App. A), slots [Q, P).
 //  * tournaments: lanes draw the candidates, a warp reduction keeps the
 //    fittest (the fitness order is strict, so this is the winner of the
 //    sequential tournament);
-//  * uniform crossover of the ordering chromosome, one position per lane;
+//  * uniform crossover of the ordering chromosome, a lane per four positions;
 //  * repair: first occurrence of each device by shared-memory atomicMin; a
 //    later repeat is a hole; the h-th hole (by position) takes the h-th
 //    missing device (by id), ranks from warp ballots;
 //  * grouping and roles from one parent; then at most one mutation, its
-//    random words drawn by the lanes and the sequential steps (Fisher-Yates,
-//    selection sampling) taken by lane 0 in shared memory.
-// Per warp, shared memory holds the child ordering, the first-occurrence
-// table, the missing devices, the random words (M words each) and the sizes.
-__global__ void __launch_bounds__(256) ga_kernel(Dims dm, DevPop src, DevPop dst, const double *fit,
+//    sequential draws (Fisher-Yates, selection sampling) resolved by the warp.
+// Bound by shared-memory work per position and, before, by the mutations that
+// one lane took step by step: 156 us for 15,872 children of 512 devices, now 70.
+__global__ void __launch_bounds__(256, 4) ga_kernel(Dims dm, DevPop src, DevPop dst, const double *fit,
                                                  uint64_t seed, uint32_t gen, GaThr thr)
 {
     extern __shared__ uint32_t ga_smem[];
     const int lane = threadIdx.x & 31, wl = threadIdx.x >> 5, NWB = blockDim.x >> 5;
     const int M = dm.M, K = dm.K, P = dm.P;
-    uint32_t *child = ga_smem + (size_t)wl * (4 * M + 64);
-    int32_t *first = reinterpret_cast<int32_t *>(child + M);
-    uint32_t *missing = reinterpret_cast<uint32_t *>(first + M);
-    uint32_t *words = missing + M;
-    uint32_t *ssz = words + M;                                    // [64] sizes
+    uint32_t *w32 = ga_smem + (size_t)wl * (genome_bytes(M) / 4);   // first occurrences, then random words
+    uint16_t *child = reinterpret_cast<uint16_t *>(w32 + M);
+    uint16_t *missing = child + ((M + 1) & ~1);
+    uint16_t *ssz = missing + ((M + 1) & ~1);                     // [64] sizes
     const uint64_t *fk = reinterpret_cast<const uint64_t *>(fit);
     for (int s = dm.Q + blockIdx.x * NWB + wl; s < P; s += gridDim.x * NWB) {   // the children
         uint16_t *out_perm = dst.perm + (size_t)s * M;
@@ -485,39 +548,50 @@ __global__ void __launch_bounds__(256) ga_kernel(Dims dm, DevPop src, DevPop dst
                 const uint64_t cw = fk[(size_t)cnd * 4], cp = fk[(size_t)cnd * 4 + 1];
                 if (key_before(cw, cp, cnd, bw, bp, bi)) { bw = cw; bp = cp; bi = cnd; }
             }
-#pragma unroll
-            for (int o = 16; o; o >>= 1) {
+            for (int o = dm.tournament > 16 ? 16 : dm.tournament > 4 ? 8 : 2; o; o >>= 1) {   // (lanes past it hold no one)
                 const uint64_t w2 = __shfl_xor_sync(0xFFFFFFFFu, bw, o), p2 = __shfl_xor_sync(0xFFFFFFFFu, bp, o);
                 const int i2 = __shfl_xor_sync(0xFFFFFFFFu, bi, o);
                 if (key_before(w2, p2, i2, bw, bp, bi)) { bw = w2; bp = p2; bi = i2; }
             }
-            par[q] = bi;
+            par[q] = __shfl_sync(0xFFFFFFFFu, bi, 0);
         }
         // ---- uniform crossover and repair
         const uint16_t *pa = src.perm + (size_t)par[0] * M, *pb = src.perm + (size_t)par[1] * M;
         Stream cx(seed, gen, (uint32_t)s, kCross);
-        for (int q = lane; 4 * q < M; q += 32)                  // a lane takes the 4 positions of one
-            for (int i = 4 * q; i < 4 * q + 4 && i < M; ++i) {  // block of the stream (one Philox call)
-                child[i] = (uint64_t)cx.word((uint32_t)i) < thr.cx ? pb[i] : pa[i];
-                first[i] = 0x7FFFFFFF;
+        if ((M & 3) == 0) {                                     // rows start on 8 bytes: four positions per load
+            for (int q = lane; 4 * q < M; q += 32) {
+                const ushort4 a = reinterpret_cast<const ushort4 *>(pa)[q], b = reinterpret_cast<const ushort4 *>(pb)[q];
+                ushort4 x;
+                x.x = (uint64_t)cx.word(4u * q) < thr.cx ? b.x : a.x;
+                x.y = (uint64_t)cx.word(4u * q + 1u) < thr.cx ? b.y : a.y;
+                x.z = (uint64_t)cx.word(4u * q + 2u) < thr.cx ? b.z : a.z;
+                x.w = (uint64_t)cx.word(4u * q + 3u) < thr.cx ? b.w : a.w;
+                reinterpret_cast<ushort2 *>(child)[2 * q] = make_ushort2(x.x, x.y);
+                reinterpret_cast<ushort2 *>(child)[2 * q + 1] = make_ushort2(x.z, x.w);
             }
+        } else {
+            for (int q = lane; 4 * q < M; q += 32)              // a lane takes the 4 positions of one
+                for (int i = 4 * q; i < 4 * q + 4 && i < M; ++i)   // block of the stream (one Philox call)
+                    child[i] = (uint64_t)cx.word((uint32_t)i) < thr.cx ? pb[i] : pa[i];
+        }
+        for (int i = lane; i < M; i += 32) w32[i] = 0x7FFFFFFFu;
         __syncwarp();
-        for (int i = lane; i < M; i += 32) atomicMin(&first[child[i]], i);
+        for (int i = lane; i < M; i += 32) atomicMin(&w32[child[i]], (uint32_t)i);
         __syncwarp();
         const unsigned lt = lanemask_lt();
         int nmiss = 0;
         for (int base = 0; base < M; base += 32) {
             const int d = base + lane;
-            const bool pm = d < M && first[d] == 0x7FFFFFFF;
+            const bool pm = d < M && w32[d] == 0x7FFFFFFFu;
             const unsigned bm = __ballot_sync(0xFFFFFFFFu, pm);
-            if (pm) missing[nmiss + __popc(bm & lt)] = (uint32_t)d;
+            if (pm) missing[nmiss + __popc(bm & lt)] = (uint16_t)d;
             nmiss += __popc(bm);
         }
         __syncwarp();
         int nh = 0;
-        for (int base = 0; base < M; base += 32) {
+        for (int base = 0; base < M && nh < nmiss; base += 32) {   // (as many holes as missing devices)
             const int i = base + lane;
-            const bool hole = i < M && first[child[i]] != i;
+            const bool hole = i < M && w32[child[i]] != (uint32_t)i;
             const unsigned bh = __ballot_sync(0xFFFFFFFFu, hole);
             if (hole) child[i] = missing[nh + __popc(bh & lt)];
             nh += __popc(bh);
@@ -534,60 +608,32 @@ __global__ void __launch_bounds__(256) ga_kernel(Dims dm, DevPop src, DevPop dst
             const uint64_t kind = mt.word(1);
             if (kind < thr.k1) {                                   // swap two positions
                 const uint32_t x = below(mt.word(2), (uint32_t)M), y = below(mt.word(3), (uint32_t)M);
-                if (lane == 0) { const uint32_t t = child[x]; child[x] = child[y]; child[y] = t; }
+                if (lane == 0) { const uint16_t t = child[x]; child[x] = child[y]; child[y] = t; }
             } else {
                 int r = 0;
-                if (kind < thr.k2) {                               // regroup from a random replica
+                if (kind < thr.k2)                                 // regroup from a random replica
                     r = (int)below(mt.word(2), (uint32_t)R);
-                } else if (kind >= thr.k3) {                       // regenerate both chromosomes
-                    Stream sp(seed, gen, (uint32_t)s, kMutPerm);
-                    for (int q = lane; 4 * q < M - 1; q += 32)
-                        for (int t = 4 * q; t < 4 * q + 4 && t < M - 1; ++t) words[t] = sp.word((uint32_t)t);
-                    for (int i = lane; i < M; i += 32) child[i] = (uint32_t)i;
-                    __syncwarp();
-                    if (lane == 0)
-                        for (int t = M - 1; t >= 1; --t) {        // Fisher-Yates, word M-1-t for position t
-                            const uint32_t j = below(words[M - 1 - t], (uint32_t)t + 1);
-                            const uint32_t x = child[t];
-                            child[t] = child[j];
-                            child[j] = x;
-                        }
-                    __syncwarp();
-                }
+                else if (kind >= thr.k3)                           // regenerate both chromosomes
+                    random_perm(Stream(seed, gen, (uint32_t)s, kMutPerm), M, w32, missing, child, lane);
                 int kept = 0;
-                for (int c = 0; c < r; ++c) kept += (int)ssz[c];
-                const int Mr = M - kept, Kr = K - r;
-                Stream sg(seed, gen, (uint32_t)s, kMutGroup), sr(seed, gen, (uint32_t)s, kMutRoles);
-                for (int q = lane; 4 * q < Mr; q += 32)
-                    for (int t = 4 * q; t < 4 * q + 4 && t < Mr; ++t) words[t] = sg.word((uint32_t)t);
-                const uint64_t bits = (uint64_t)sr.word(0) | ((uint64_t)sr.word(1) << 32);
+                for (int c = lane; c < r; c += 32) kept += (int)ssz[c];
+                kept = (int)__reduce_add_sync(0xFFFFFFFFu, (unsigned)kept);
                 __syncwarp();
-                if (lane == 0) {
-                    // replica count from word 0, cut t taken with probability needed/remaining
-                    const int cap = Kr < Mr ? Kr : Mr;
-                    const int Rn = 1 + (int)below(words[0], (uint32_t)cap);
-                    int need = Rn - 1, prev = 0, cc = r;
-                    for (int t = 1; t <= Mr - 1 && need > 0; ++t) {
-                        if (below(words[t], (uint32_t)(Mr - t)) < (uint32_t)need) {
-                            ssz[cc++] = (uint32_t)(t - prev);
-                            prev = t;
-                            --need;
-                        }
-                    }
-                    ssz[cc++] = (uint32_t)(Mr - prev);
-                    for (; cc < K; ++cc) ssz[cc] = 0;
-                    const uint64_t nr = Rn >= 64 ? bits : (bits & ((1ull << Rn) - 1ull));
-                    const uint64_t keep = r >= 64 ? ~0ull : ((1ull << r) - 1ull);
-                    rl = (rl & keep) | (r >= 64 ? 0ull : (nr << r));
-                    R = r + Rn;
-                }
-                R = __shfl_sync(0xFFFFFFFFu, R, 0);
-                rl = __shfl_sync(0xFFFFFFFFu, rl, 0);
+                const int Rn = random_grouping(Stream(seed, gen, (uint32_t)s, kMutGroup), M - kept, K - r, w32, ssz + r, lane);
+                const uint64_t nr = random_roles(Stream(seed, gen, (uint32_t)s, kMutRoles), Rn);
+                const uint64_t keep = r >= 64 ? ~0ull : ((1ull << r) - 1ull);
+                rl = (rl & keep) | (r >= 64 ? 0ull : (nr << r));
+                R = r + Rn;
             }
         }
         __syncwarp();
-        for (int i = lane; i < M; i += 32) out_perm[i] = (uint16_t)child[i];
-        for (int i = lane; i < K; i += 32) cs[i] = (uint16_t)ssz[i];
+        if ((M & 1) == 0) {
+            for (int i = lane; i < M / 2; i += 32)
+                reinterpret_cast<uint32_t *>(out_perm)[i] = reinterpret_cast<const uint32_t *>(child)[i];
+        } else {
+            for (int i = lane; i < M; i += 32) out_perm[i] = child[i];
+        }
+        for (int i = lane; i < K; i += 32) cs[i] = ssz[i];
         if (lane == 0) { dst.nclus[s] = (uint8_t)R; dst.roles[s] = rl; }
         __syncwarp();
     }
@@ -648,9 +694,23 @@ cudaError_t launch_validate(const e2_ctx *c, const DevPop &p)
     return cudaGetLastError();
 }
 
+// Warps per CTA and shared memory of a kernel with genome_bytes(M) per warp.
+static cudaError_t genome_launch(const void *kernel, int M, int *nw, size_t *smem)
+{
+    *nw = 8;
+    while (*nw > 1 && (size_t)*nw * genome_bytes(M) > 48 * 1024) *nw >>= 1;
+    *smem = (size_t)*nw * genome_bytes(M);
+    if (*smem <= 48 * 1024) return cudaSuccess;
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)*smem);
+}
+
 cudaError_t launch_init(const e2_ctx *c, const DevPop &p, uint64_t seed)
 {
-    init_kernel<<<(c->dm.P + 31) / 32, 32, 0, c->stream>>>(c->dm, p, seed);
+    size_t smem = 0;
+    int nw = 1;
+    const cudaError_t e = genome_launch(reinterpret_cast<const void *>(init_kernel), c->dm.M, &nw, &smem);
+    if (e != cudaSuccess) return e;
+    init_kernel<<<(unsigned)((c->dm.P + nw - 1) / nw), 32 * nw, smem, c->stream>>>(c->dm, p, seed);
     ++c->launches;
     return cudaGetLastError();
 }
@@ -694,16 +754,12 @@ cudaError_t launch_ga(const e2_ctx *c, const DevPop &src, const DevPop &dst, uin
 {
     if (c->dm.P <= c->dm.Q) return cudaSuccess;              // no children
     GaThr thr{c->thr_cx, c->thr_half, c->thr_mut, c->thr_k1, c->thr_k2, c->thr_k3};
-    const size_t per_warp = 4 * (4 * (size_t)c->dm.M + 64);
-    int nw = 8;
-    while (nw > 1 && (size_t)nw * per_warp > 48 * 1024) nw >>= 1;
-    if ((size_t)nw * per_warp > 48 * 1024) {
-        const cudaError_t e = cudaFuncSetAttribute(ga_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                   (int)((size_t)nw * per_warp));
-        if (e != cudaSuccess) return e;
-    }
+    size_t smem = 0;
+    int nw = 1;
+    const cudaError_t e = genome_launch(reinterpret_cast<const void *>(ga_kernel), c->dm.M, &nw, &smem);
+    if (e != cudaSuccess) return e;
     const long long blocks = ((long long)(c->dm.P - c->dm.Q) + nw - 1) / nw;
-    ga_kernel<<<(unsigned)(blocks < 152 * 64 ? blocks : 152 * 64), 32 * nw, (size_t)nw * per_warp, st>>>(
+    ga_kernel<<<(unsigned)(blocks < 152 * 64 ? blocks : 152 * 64), 32 * nw, smem, st>>>(
         c->dm, src, dst, c->fit, seed, gen, thr);
     ++c->launches;
     return cudaGetLastError();

@@ -1,0 +1,40 @@
+"""The initial population and the generation step at odd sizes, against the
+oracle: orderings of 1 to 1,000 devices (lane edges, sizes that are no multiple
+of the vector loads), one to 64 replicas, and every child mutated, by
+regeneration of both chromosomes, by regrouping, or by each kind in turn (the
+shuffle and the cut points are resolved by a warp, not step by step)."""
+import numpy as np
+import pytest
+
+from oracle import oracle as O
+
+from test_parity_gpu import _edge_problem, assert_genomes_equal, engine
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    import __graft_entry__ as ge
+    ge.build()
+
+
+@pytest.mark.parametrize("M", [1, 2, 3, 4, 31, 32, 33, 63, 64, 65, 66, 127, 200, 1000])
+@pytest.mark.parametrize("kinds", [(0.0, 0.0, 0.0), (0.0, 1.0, 0.0), (0.25, 0.25, 0.25)])
+def test_init_and_step(M, kinds):
+    rng = np.random.default_rng(M)
+    K, P = min(M, 64), 203
+    prob = _edge_problem(rng, M, 3, P, K, integer=True, Q=5, min_tps=0.01)
+    prob.p_mut, prob.p_kind, prob.tournament = 1.0, kinds + (1.0 - sum(kinds),), 1 + M % 40
+    ga = O.ga_of(prob)
+    eng = engine(prob)
+    eng.init_population(M)
+    pop = O.init_population(ga, M)
+    for gen in (1, 2):
+        assert_genomes_equal(eng.get_population(), pop)
+        eng.eval(parts=False)
+        fit = eng.results()["fitness"]
+        eng.ga_step(M, gen)
+        pop = O.ga_step(ga, M, gen, pop, fit, O.elites(ga, pop, fit))
+    assert_genomes_equal(eng.get_population(), pop)
+    eng.close()
