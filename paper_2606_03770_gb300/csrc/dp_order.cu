@@ -213,7 +213,7 @@ __global__ void __launch_bounds__(32 * dp_order_warps(D == 1 ? 0 : 1), order_cta
                             if (D == 1) tk[j] = link.t;
                         }
                         if (c1[j] >= 1) hmin_l = fminf(hmin_l, hb[j]);
-                        if (c0[j] >= 1) tf_l = fmaxf(tf_l, __frcp_rn(cinv[j]));
+                        if (c0[j] >= 1) tf_l = fmaxf(tf_l, __fdividef(1.0f, cinv[j]));
                     }
                     floor_l = max(floor_l, tr[j]);
                 }
@@ -456,6 +456,17 @@ __global__ void __launch_bounds__(32 * dp_order_warps(D == 1 ? 0 : 1), order_cta
                 }
                 head_at = mus;
                 int e = (int)__reduce_add_sync(kFull, s_l) - N;
+                // ---- a decode batch too slow whatever the traceback does: the partition takes the
+                //      counts C less e blocks in all, so Lambda is at least the links and
+                //      sum C_k c_k - e max c_k (the head only adds); in fixed point as below.
+                //      About three quarters of the batches that fail the test end here.
+                if (D == 1 && !OFF && role && dm.lam_fx > 0.0f) {
+                    const float x = (float)C[0] * __fdividef(1.0f, cinv[0]) + trunc_float(tk[0]);
+                    const unsigned s = __reduce_add_sync(
+                        kFull, lane < m ? (unsigned)fminf(x * (1.0f - 3e-6f) * dm.lam_fx, 8388608.0f) : 0u);
+                    const float back = fminf((float)e * t_min * (1.0f + 3e-6f) * dm.lam_fx, 1e9f);
+                    if (s > (1u << 22) + 64u + (unsigned)back) continue;
+                }
                 // ---- traceback
                 if (e > 0) {
                     // fl[k]: the largest link or first-block key of devices 0..k
