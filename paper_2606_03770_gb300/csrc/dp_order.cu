@@ -493,10 +493,11 @@ __global__ void __launch_bounds__(32 * dp_order_warps(D == 1 ? 0 : 1), order_cta
                             if (j == (lim - 1) >> 5) f = y;
                         }
                         // drop the e largest entries of the prefix, down to f: many of them by a
-                        // new estimate (and up again from there if it dropped too many) ...
+                        // new estimate (and up again from there if it dropped too many; the whole
+                        // pipeline's threshold is V*, with nothing to drop) ...
                         uint32_t x = 0;
                         int C2[D];
-                        if (e > kMaxDrop) {
+                        if (e > kMaxDrop && lim < m) {
                             int total = 0;
 #pragma unroll
                             for (int j = 0; j < D; ++j) total += lane + 32 * j < lim ? C[j] : 0;
