@@ -1560,8 +1560,9 @@ cudaError_t launch_eval(const e2_ctx *c, const DevPop &p)
     cudaError_t e = cudaSuccess;
     slot_kernel<<<(unsigned)c->dm.P, 32 * (c->dm.K < kPreWarps ? c->dm.K : kPreWarps), 2 * (size_t)c->dm.M, c->stream>>>(
         c->dm, tb, p, si, out, so, vo);
-    // (about 4,096 slots per block of the count and the scatter)
-    const long long nb = (slots + 4095) / 4096;
+    // (1,024 slots per block of the count and the scatter, more on large populations:
+    // 8.7 us a generation for both at 32,768 slots, 14 with 4,096 per block)
+    const long long nb = (slots + 1023) / 1024;
     const unsigned lb = (unsigned)(nb < kListBlocks ? nb : kListBlocks);
     bins_kernel<<<lb, 256, 0, c->stream>>>(c->dm, si, c->list_hist, c->stats);
     order_scatter_kernel<<<lb, 256, 0, c->stream>>>(c->dm, si, wl, c->list_hist);
