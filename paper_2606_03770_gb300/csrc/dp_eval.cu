@@ -55,17 +55,18 @@ __device__ __forceinline__ uint32_t size_bin(const Dims &dm, int m)
 //    bought at x, less what devices cheaper than x save).  The block time of
 //    the marginal device, up to which the cheaper devices just hold N - m more
 //    blocks, gives the program's own optimum; it is found by bisection at the
-//    first batch tested and kept for the others.  All in float from times rounded down, every operation rounded toward -inf, so
+//    smallest and the largest batch and kept for those between.  All in float from times rounded down, every operation rounded toward -inf, so
 //    the bound never exceeds the exact value; a variant whose bound is above
 //    Lambda_max (rounded up to float) fails whatever partition the DP returns.
 // Both tests are monotone in the batch: the capacities shrink as b grows (more
 // KV memory per block), and the program's optimum is the least of a linear
 // cost whose coefficients (per-block and link times) grow with b over a
 // feasible set that shrinks with b, when the profile's costs grow with the
-// batch (physical profiles do; checked at e2_create).  So the largest batch the
-// memory allows is found by a search (the largest batch first, then the
-// smallest, then bisection), and the largest the bound keeps by a second
-// search below it; every smaller batch is kept.  A failed test is exact
+// batch (physical profiles do; checked at e2_create).  So both are tested on
+// the smallest batch first; if it passes, the largest batch the memory allows
+// is found by a search (the largest batch first, then bisection), and the
+// largest the bound keeps by a second search below it; every smaller batch is
+// kept.  A failed test is exact
 // (memory) or a proof (the bound never exceeds the optimum, and the optimum
 // of every larger batch is no smaller), so every batch above it fails too;
 // rounding and the price can only keep a variant the optimum would drop,
@@ -149,8 +150,9 @@ __device__ __forceinline__ uint32_t decode_verdict(const Dims &dm, const Tables 
     };
     if (timed) X = warp_sum_rd(X);
     auto mem_of = [&](int v) { return memory_ok<SMALL>(m, N, lane, [&](int k) { return caps(k, v); }); };
-    // the marginal device: the price is its block time (found once, at the first
-    // batch tested: which devices are cheap hardly depends on the batch)
+    // the marginal device: the price is its block time (found at the smallest batch
+    // and again at the largest, and kept: which devices are cheap hardly depends on
+    // the batch, but how much they hold does)
     int marginal = -1;
     auto fast_enough = [&](int v) -> bool {
         const float4 q = tb.fpr[v];                        // block flops and bytes, activation bytes, rounded down
@@ -212,23 +214,40 @@ __device__ __forceinline__ uint32_t decode_verdict(const Dims &dm, const Tables 
         sum = __fadd_rd(sum, __fmul_rd(q.z, X));
         return !(sum > dm.lam_max_up);                     // 1.0 / Lambda >= Min_TPS possible
     };
-    // the largest batch (variant v = 1..b_max; 0: none) that a test passes, from top down
-    auto search = [&](int top, auto pass) -> int {
-        int lo = 0, hi = top + 1, next = top;
+    // the largest batch above lo, from top down, that a test passes (lo: none does)
+    auto search = [&](int lo, int top, auto pass) -> int {
+        int hi = top + 1, next = top;
         while (hi - lo > 1) {
             if (pass(next)) lo = next;
             else hi = next;
-            next = !dm.grows ? hi - 1 : lo < 1 ? 1 : (lo + hi) >> 1;
+            next = dm.grows ? (lo + hi) >> 1 : hi - 1;
         }
         return lo;
     };
-    const int bm = search(dm.b_max, mem_of);
-    int bs = bm;
-    if (timed && bm > 0) bs = search(bm, [&](int v) { return (dm.grows || mem_of(v)) && fast_enough(v); });
+    int bm = 0, bs = 0;
+    if (dm.grows) {
+        // the smallest batch first: its capacities are at hand, and a replica that
+        // cannot hold it (72% of a 512-device population), or is too slow with it,
+        // fails at every other (512 devices: 273-320 us with the largest batch first,
+        // 260 so; 256 devices, where most serve the largest: 125-130 and 147, and the
+        // price found here saves DP runs, so the evaluation is no slower)
+        if (mem_of(1)) {
+            bm = search(1, dm.b_max, mem_of);
+            if (!timed) {
+                bs = bm;
+            } else if (fast_enough(1)) {
+                marginal = -1;                             // (found again at the largest batch's capacities)
+                bs = search(1, bm, fast_enough);
+            }
+        }
+    } else {
+        bm = search(0, dm.b_max, mem_of);
+        bs = timed ? search(0, bm, [&](int v) { return mem_of(v) && fast_enough(v); }) : bm;
+    }
     return kSlotDecTested | (uint32_t)bs | (uint32_t)bm << kSlotMemShift;
 }
 
-__global__ void __launch_bounds__(32 * kPreWarps) slot_kernel(Dims dm, Tables tb, DevPop pop, SlotInfo si, EvalOut out,
+__global__ void __launch_bounds__(32 * kPreWarps, 5) slot_kernel(Dims dm, Tables tb, DevPop pop, SlotInfo si, EvalOut out,
                                                               SplitOut so, VariantOut vo)
 {
     extern __shared__ uint16_t s_perm[];                   // the genome's ordering
