@@ -319,7 +319,22 @@ struct e2_ctx {
 };
 
 namespace e2 {
+// Arrays of one device copied by one kernel (copy_kernel): blocks
+// first[i]..first[i+1]-1 copy piece i, kCopyChunk bytes each.
+constexpr int kCopyPieces = 7;
+constexpr size_t kCopyChunk = 16 * 1024;
+struct CopyList {
+    const unsigned char *src[kCopyPieces];
+    unsigned char *dst[kCopyPieces];
+    unsigned long long bytes[kCopyPieces];
+    unsigned first[kCopyPieces + 1];
+    int n;
+    int32_t *word;           // a word to set to `value` besides (nullptr: none)
+    int32_t value;
+};
+
 // launchers (defined in the .cu files); return cudaGetLastError()
+cudaError_t launch_copies(const CopyList &l, cudaStream_t st);
 cudaError_t launch_tables(const e2_ctx *c);   // stage times and device tables (and lcost for per-layer profiles)
 cudaError_t launch_tau(const e2_ctx *c);
 cudaError_t launch_redraw(const e2_ctx *c, uint64_t seed, uint32_t gen);
