@@ -250,6 +250,7 @@ __device__ __forceinline__ uint32_t decode_verdict(const Dims &dm, const Tables 
 __global__ void __launch_bounds__(32 * kPreWarps, 5) slot_kernel(Dims dm, Tables tb, DevPop pop, SlotInfo si, EvalOut out,
                                                               SplitOut so, VariantOut vo)
 {
+    after_previous();
     extern __shared__ uint16_t s_perm[];                   // the genome's ordering
     __shared__ int s_off[E2_MAX_CLUSTERS], s_size[E2_MAX_CLUSTERS];
     const int g = blockIdx.x;
@@ -338,6 +339,7 @@ __device__ __forceinline__ uint32_t layered_bin(uint32_t info, int level)
 
 __global__ void __launch_bounds__(256) bins_kernel(Dims dm, SlotInfo si, unsigned *hist, unsigned long long *stats)
 {
+    after_previous();
     __shared__ unsigned s_bin[kListBins];
     const int total = dm.P * dm.K, chunk = (total + gridDim.x - 1) / gridDim.x;
     const int lo = blockIdx.x * chunk, hi = min(total, lo + chunk);
@@ -364,6 +366,7 @@ __global__ void __launch_bounds__(256) bins_kernel(Dims dm, SlotInfo si, unsigne
 // ends and cursors.
 __global__ void __launch_bounds__(256) order_scatter_kernel(Dims dm, SlotInfo si, WorkList wl, const unsigned *hist)
 {
+    after_previous();
     __shared__ unsigned s_all[4][kListBins], s_before[4][kListBins], s_at[kListBins];
     const int total = dm.P * dm.K, chunk = (total + gridDim.x - 1) / gridDim.x;
     const int lo = blockIdx.x * chunk, hi = min(total, lo + chunk);
@@ -510,6 +513,7 @@ __device__ __forceinline__ void bar_named(int id, int nthreads)
 __global__ void __launch_bounds__(32 * kLayeredWarps) dp_layered_kernel(Dims dm, Tables tb, DevPop pop, EvalOut out,
                                                                         WorkList wl, SlotInfo si, VariantOut vo)
 {
+    after_previous();
     extern __shared__ __align__(16) unsigned char lsm[];
     __shared__ unsigned s_item;
     __shared__ int s_done, s_mu;
@@ -772,6 +776,7 @@ __global__ void __launch_bounds__(32 * kLayeredWarps) dp_layered_kernel(Dims dm,
 __global__ void __launch_bounds__(128) layered_pick_kernel(Dims dm, DevPop pop, SlotInfo si, VariantOut vo, EvalOut out,
                                                            SplitOut so)
 {
+    after_previous();
     const int lane = threadIdx.x & 31;
     const long long slot = (long long)blockIdx.x * 4 + (threadIdx.x >> 5);
     if (slot >= (long long)dm.P * dm.K) return;
@@ -877,6 +882,7 @@ constexpr int kScoreGenomes = 8;
 template <bool FT>
 __global__ void __launch_bounds__(32 * kScoreGenomes) finalize_score_kernel(Dims dm, DevPop pop, SlotInfo si, EvalOut out)
 {
+    after_previous();
     constexpr int S = FT ? 4 : 2;                          // PS, DS (and the rate-weighted latencies PL, DL)
     __shared__ double s_x[S][kScoreGenomes][E2_MAX_CLUSTERS + 1];
     __shared__ int s_R[kScoreGenomes];
@@ -964,6 +970,7 @@ template <int WPG, bool FT>
 __global__ void __launch_bounds__(128) finalize_roles_kernel(Dims dm, DevPop pop, SlotInfo si, SplitOut so,
                                                              EvalOut out)
 {
+    after_previous();
     constexpr int KC = E2_MAX_CLUSTERS, KF = E2_MAX_ROLE_SEARCH;
     __shared__ double s_ps[4][KC], s_ds[4][KC];
     __shared__ double s_pl[4][KC], s_dl[4][KC];        // rate x Lambda (finishing time)
@@ -1354,6 +1361,7 @@ __global__ void __launch_bounds__(128) finalize_roles_kernel(Dims dm, DevPop pop
 __global__ void __launch_bounds__(128) finalize_splitwise_kernel(Dims dm, DevPop pop, SlotInfo si, SplitOut so,
                                                                  EvalOut out)
 {
+    after_previous();
     __shared__ int s_off[4][E2_MAX_CLUSTERS + 1];     // replica start in the ordering
     __shared__ int s_code[4][E2_MAX_CLUSTERS];        // the role whose result is taken, -1 none
     __shared__ unsigned long long s_tally[4][kTallies];   // (a row per warp)
@@ -1477,6 +1485,7 @@ __global__ void __launch_bounds__(128) finalize_splitwise_kernel(Dims dm, DevPop
 // replica cannot serve.  Runs after the replicas' outputs are final.
 __global__ void __launch_bounds__(128) gc_split_kernel(Dims dm, DevPop pop, const int32_t *capg, EvalOut out)
 {
+    after_previous();
     __shared__ int s_off[4][E2_MAX_CLUSTERS + 1];
     const int wl = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int g = blockIdx.x * 4 + wl;
@@ -1583,8 +1592,9 @@ cudaError_t launch_eval(const e2_ctx *c, const DevPop &p)
     // 8.7 us a generation for both at 32,768 slots, 14 with 4,096 per block)
     const long long nb = (slots + 1023) / 1024;
     const unsigned lb = (unsigned)(nb < kListBlocks ? nb : kListBlocks);
-    bins_kernel<<<lb, 256, 0, c->stream>>>(c->dm, si, c->list_hist, c->stats);
-    order_scatter_kernel<<<lb, 256, 0, c->stream>>>(c->dm, si, wl, c->list_hist);
+    if ((e = launch_kernel(bins_kernel, lb, 256, 0, c->stream, true, c->dm, si, c->list_hist, c->stats)) != cudaSuccess) return e;
+    if ((e = launch_kernel(order_scatter_kernel, lb, 256, 0, c->stream, true, c->dm, si, wl, c->list_hist)) != cudaSuccess)
+        return e;
     // while a launch sequence is being recorded, the timing events become
     // event-record nodes of the graph (an ordinary record would only mark a
     // dependency)
@@ -1593,9 +1603,11 @@ cudaError_t launch_eval(const e2_ctx *c, const DevPop &p)
     const unsigned rec = cs == cudaStreamCaptureStatusActive ? cudaEventRecordExternal : cudaEventRecordDefault;
     if (c->ev_dp_start && (e = cudaEventRecordWithFlags(c->ev_dp_start, c->stream, rec)) != cudaSuccess) return e;
     if (c->dm.layered) {
-        dp_layered_kernel<<<(unsigned)c->dp_grid, 32 * kLayeredWarps, c->dp_smem, c->stream>>>(c->dm, tb, p, out, wl, si,
-                                                                                            vo);
-        layered_pick_kernel<<<(unsigned)((slots + 3) / 4), 128, 0, c->stream>>>(c->dm, p, si, vo, out, so);
+        e = launch_kernel(dp_layered_kernel, (unsigned)c->dp_grid, 32 * kLayeredWarps, c->dp_smem, c->stream, !c->ev_dp_start,
+                          c->dm, tb, p, out, wl, si, vo);
+        if (e == cudaSuccess)
+            e = launch_kernel(layered_pick_kernel, (unsigned)((slots + 3) / 4), 128, 0, c->stream, true, c->dm, p, si, vo, out, so);
+        if (e != cudaSuccess) return e;
         ++c->launches;
     } else {
         // the larger replicas run beside the others on the side stream (few runs,
@@ -1603,34 +1615,37 @@ cudaError_t launch_eval(const e2_ctx *c, const DevPop &p)
         if (c->dp_grid1 > 0) {
             if ((e = cudaEventRecord(c->ev_fork, c->stream)) != cudaSuccess) return e;
             if ((e = cudaStreamWaitEvent(c->side, c->ev_fork, 0)) != cudaSuccess) return e;
-            e = dp_order_launch(c->dp_grid1, c->dm.dp_mmax, 1, c->side, c->dm, tb, p, out, wl, c->slot_off, so);
+            e = dp_order_launch(c->dp_grid1, c->dm.dp_mmax, 1, c->side, c->dm, tb, p, out, wl, c->slot_off, so, false);
             if (e != cudaSuccess) return e;
             if ((e = cudaEventRecord(c->ev_join, c->side)) != cudaSuccess) return e;
         }
+        // (an early class 0 would fill the SMs before class 1, which has the longer chains:
+        // 1,057 us instead of 978 for four generations of 4,096 genomes of 128 devices)
         e = dp_order_launch(c->dp_grid, c->dm.dp_split ? c->dm.dp_split : c->dm.dp_mmax, 0, c->stream, c->dm, tb, p, out,
-                            wl, c->slot_off, so);
+                            wl, c->slot_off, so, !c->ev_dp_start && c->dp_grid1 == 0);
         if (e == cudaSuccess && c->dp_grid1 > 0) e = cudaStreamWaitEvent(c->stream, c->ev_join, 0);
         if (e != cudaSuccess) return e;
     }
     if (c->ev_dp_stop && (e = cudaEventRecordWithFlags(c->ev_dp_stop, c->stream, rec)) != cudaSuccess) return e;
-    const unsigned fb = (unsigned)(((size_t)c->dm.P * 32 + 127) / 128);
+    const unsigned fb = (unsigned)(((size_t)c->dm.P * 32 + 127) / 128), fg = (unsigned)c->dm.P;
+    const bool early = !c->ev_dp_stop && (c->dm.layered || c->dp_grid1 == 0);   // (a kernel comes right before)
+    const bool ft = c->dm.objective == 1;
     if (c->dm.role_search == 2)
-        finalize_splitwise_kernel<<<fb, 128, 0, c->stream>>>(c->dm, p, si, so, out);
-    else if (c->dm.role_search && c->dm.K >= 12) {    // up to 2^K_max assignments: a block per genome
-        if (c->dm.objective == 1) finalize_roles_kernel<4, true><<<(unsigned)c->dm.P, 128, 0, c->stream>>>(c->dm, p, si, so, out);
-        else finalize_roles_kernel<4, false><<<(unsigned)c->dm.P, 128, 0, c->stream>>>(c->dm, p, si, so, out);
-    } else if (c->dm.role_search) {
-        if (c->dm.objective == 1) finalize_roles_kernel<1, true><<<fb, 128, 0, c->stream>>>(c->dm, p, si, so, out);
-        else finalize_roles_kernel<1, false><<<fb, 128, 0, c->stream>>>(c->dm, p, si, so, out);
-    }
-    else {
-        const unsigned sb = (unsigned)((c->dm.P + kScoreGenomes - 1) / kScoreGenomes);
-        if (c->dm.objective == 1) finalize_score_kernel<true><<<sb, 32 * kScoreGenomes, 0, c->stream>>>(c->dm, p, si, out);
-        else finalize_score_kernel<false><<<sb, 32 * kScoreGenomes, 0, c->stream>>>(c->dm, p, si, out);
-    }
+        e = launch_kernel(finalize_splitwise_kernel, fb, 128, 0, c->stream, early, c->dm, p, si, so, out);
+    else if (c->dm.role_search && c->dm.K >= 12)      // up to 2^K_max assignments: a block per genome
+        e = launch_kernel(ft ? finalize_roles_kernel<4, true> : finalize_roles_kernel<4, false>, fg, 128, 0, c->stream, early,
+                          c->dm, p, si, so, out);
+    else if (c->dm.role_search)
+        e = launch_kernel(ft ? finalize_roles_kernel<1, true> : finalize_roles_kernel<1, false>, fb, 128, 0, c->stream, early,
+                          c->dm, p, si, so, out);
+    else
+        e = launch_kernel(ft ? finalize_score_kernel<true> : finalize_score_kernel<false>,
+                          (unsigned)((c->dm.P + kScoreGenomes - 1) / kScoreGenomes), 32 * kScoreGenomes, 0, c->stream, early,
+                          c->dm, p, si, out);
+    if (e != cudaSuccess) return e;
     c->launches += c->dp_grid1 > 0 ? 6 : 5;
     if (c->dm.offload) {
-        gc_split_kernel<<<fb, 128, 0, c->stream>>>(c->dm, p, c->capg, out);
+        if ((e = launch_kernel(gc_split_kernel, fb, 128, 0, c->stream, true, c->dm, p, c->capg, out)) != cudaSuccess) return e;
         ++c->launches;
     }
     return cudaGetLastError();

@@ -120,6 +120,7 @@ template <int D, bool OFF>
 __global__ void __launch_bounds__(32 * dp_order_warps(D == 1 ? 0 : 1), order_ctas(D)) dp_order_kernel(Dims dm, Tables tb, DevPop pop, EvalOut out, WorkList wl,
                                                        const int32_t *slot_off, SplitOut so, int cls)
 {
+    after_previous();
     extern __shared__ uint32_t s_dyn[];                    // D == 1: the claim's partitions, per warp
                                                            // D > 1: the run's device ids, per warp
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -784,13 +785,12 @@ cudaError_t dp_order_occupancy(int mmax, int cls, bool off, int *per_sm)
 
 cudaError_t dp_order_launch(int grid, int mmax, int cls, cudaStream_t stream, const Dims &dm, const Tables &tb,
                             const DevPop &pop, const EvalOut &out, const WorkList &wl, const int32_t *slot_off,
-                            const SplitOut &so)
+                            const SplitOut &so, bool early)
 {
     int per_lane = 1;
     const OrderKernel k = order_kernel(mmax, dm.offload != 0, &per_lane);
-    k<<<(unsigned)grid, 32 * dp_order_warps(cls), dp_order_smem(mmax, cls), stream>>>(dm, tb, pop, out, wl, slot_off,
-                                                                                    so, cls);
-    return cudaGetLastError();
+    return launch_kernel(k, (unsigned)grid, 32 * dp_order_warps(cls), dp_order_smem(mmax, cls), stream, early, dm, tb, pop,
+                         out, wl, slot_off, so, cls);
 }
 
 }  // namespace e2

@@ -210,6 +210,7 @@ public:
         l_.value = value;
         return launch_copies(l_, c_->stream);
     }
+    bool launched() const { return l_.n > 0; }             // go() ended in a kernel
     bool any_host() const { return host_; }
 
 private:
@@ -343,7 +344,7 @@ int upload_and_validate(e2_ctx *c, const e2_genomes *g)
     E2_CUDA(c, in.add(p.nclus, g->nclus, P, g->nclus));
     E2_CUDA(c, in.add(p.roles, g->roles, 8 * P, g->roles));
     E2_CUDA(c, in.go(c->err, kNoBadGenome));
-    E2_CUDA(c, launch_validate(c, c->pop[c->cur]));
+    E2_CUDA(c, launch_validate(c, c->pop[c->cur], in.launched()));
     c->evaluated = false;
     return E2_OK;
 }
@@ -635,7 +636,7 @@ cudaError_t record_generation(e2_ctx *c, int b)
     e = cudaStreamBeginCapture(c->cap_stream, cudaStreamCaptureModeThreadLocal);
     if (e == cudaSuccess) {
         cudaError_t le = launch_eval(c, c->pop[b]);
-        if (le == cudaSuccess) le = launch_step(c, c->pop[b], c->pop[b ^ 1], 0, 0);
+        if (le == cudaSuccess) le = launch_step(c, c->pop[b], c->pop[b ^ 1], 0, 0, true);
         cudaGraph_t g = nullptr;
         e = cudaStreamEndCapture(c->cap_stream, &g);
         if (le != cudaSuccess) e = le;
@@ -744,7 +745,7 @@ int e2_ga_step(e2_ctx *c, uint64_t seed, uint32_t generation)
 {
     if (!c) return E2_EINVAL;
     if (!c->evaluated) return fail(c, E2_ESTATE, "the current population has not been evaluated");
-    E2_CUDA(c, launch_step(c, c->pop[c->cur], c->pop[c->cur ^ 1], seed, generation));
+    E2_CUDA(c, launch_step(c, c->pop[c->cur], c->pop[c->cur ^ 1], seed, generation, false));
     c->cur ^= 1;
     c->evaluated = false;
     c->have_elites = true;

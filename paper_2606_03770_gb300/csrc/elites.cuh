@@ -151,6 +151,7 @@ template <typename Dup>
 __global__ void __launch_bounds__(kSelThreads) elite_select_kernel(int P, int Q, const double *fit, const Dup *dup,
                                                                    unsigned long long *ctl, int32_t *cand)
 {
+    after_previous();
     __shared__ unsigned hist[256];
     __shared__ unsigned long long s_prefix, s_and, s_or;
     __shared__ unsigned s_need, s_count, s_minima, s_n, s_run, s_wsum[kSelThreads / 32];

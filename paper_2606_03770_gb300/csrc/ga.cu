@@ -220,6 +220,7 @@ constexpr int kValidateWarps = 4;
 
 __global__ void __launch_bounds__(32 * kValidateWarps) validate_kernel(Dims dm, DevPop p, int32_t *err)
 {
+    after_previous();
     __shared__ uint32_t s_seen[kValidateWarps][kBitmapWords];
     const int lane = threadIdx.x & 31, wl = threadIdx.x >> 5;
     const int g = blockIdx.x * kValidateWarps + wl;
@@ -392,6 +393,7 @@ __global__ void __launch_bounds__(256) dup_insert_kernel(int P, const uint64_t *
 __global__ void __launch_bounds__(256) dup_lookup_kernel(Dims dm, DevPop p, const uint64_t *hash,
                                                          const unsigned long long *tab, unsigned mask, int32_t *dup)
 {
+    after_previous();
     const int lane = threadIdx.x & 31;
     const int g = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     if (g >= dm.P) return;
@@ -406,6 +408,7 @@ constexpr int kDupThreads = 512;
 __global__ void __launch_bounds__(kDupThreads) dup_kernel(Dims dm, DevPop p, const uint64_t *hash, int32_t *dup,
                                                           unsigned mask)
 {
+    after_previous();
     extern __shared__ unsigned long long tab[];
     const int lane = threadIdx.x & 31;
     for (unsigned s = threadIdx.x; s <= mask; s += kDupThreads) tab[s] = kFreeSlot;
@@ -437,6 +440,7 @@ __global__ void __launch_bounds__(256) rank_kernel(Dims dm, const double *fit, c
                                                    int32_t *elite, double *elite_fit, DevPop src, DevPop dst,
                                                    const unsigned long long *ctl)
 {
+    after_previous();
     __shared__ uint64_t s_w[kEliteTile], s_p[kEliteTile];
     __shared__ int s_d[kEliteTile];
     if (ctl[2] != 0) return;                       // elite_cand_rank_kernel took the elites
@@ -480,6 +484,7 @@ __global__ void __launch_bounds__(256) elite_cand_rank_kernel(Dims dm, const dou
                                                               const unsigned long long *ctl, const int32_t *cand,
                                                               int32_t *elite, double *elite_fit, DevPop src, DevPop dst)
 {
+    after_previous();
     rank_listed(dm.Q, fit, ctl, cand, [&](int rank, int g, int lane) {
         const int M = dm.M, K = dm.K;
         for (int j = lane; j < M; j += 32) dst.perm[(size_t)rank * M + j] = src.perm[(size_t)g * M + j];
@@ -732,12 +737,11 @@ cudaError_t launch_copies(const CopyList &l, cudaStream_t st)
     return cudaGetLastError();
 }
 
-cudaError_t launch_validate(const e2_ctx *c, const DevPop &p)
+cudaError_t launch_validate(const e2_ctx *c, const DevPop &p, bool early)
 {
-    validate_kernel<<<(c->dm.P + kValidateWarps - 1) / kValidateWarps, 32 * kValidateWarps, 0, c->stream>>>(c->dm, p,
-                                                                                                          c->err);
     ++c->launches;
-    return cudaGetLastError();
+    return launch_kernel(validate_kernel, (c->dm.P + kValidateWarps - 1) / kValidateWarps, 32 * kValidateWarps, 0, c->stream,
+                         early, c->dm, p, c->err);
 }
 
 // Warps per CTA and shared memory of a kernel with genome_bytes(M) per warp.
@@ -762,37 +766,43 @@ cudaError_t launch_init(const e2_ctx *c, const DevPop &p, uint64_t seed)
 }
 
 // Duplicate flags, then the selection; the elites go to slots [0, Q) of dst.
-cudaError_t launch_elites(const e2_ctx *c, const DevPop &p, const DevPop &dst)
+cudaError_t launch_elites(const e2_ctx *c, const DevPop &p, const DevPop &dst, bool early)
 {
+    cudaError_t e = cudaSuccess;
     const int P = c->dm.P, Q = c->dm.Q;
     const unsigned blocks = (unsigned)(((size_t)P * 32 + 255) / 256);
     const bool table = P >= kDupTableFrom;
     const unsigned tsize = dup_table_size(P);
     if (table) {
-        const cudaError_t e = cudaMemsetAsync(c->dup_tab, 0x7F, sizeof(*c->dup_tab) * tsize, c->stream);
+        e = cudaMemsetAsync(c->dup_tab, 0x7F, sizeof(*c->dup_tab) * tsize, c->stream);
         if (e != cudaSuccess) return e;
         dup_insert_kernel<<<(unsigned)((P + 255) / 256), 256, 0, c->stream>>>(P, c->hash, c->dup_tab, tsize - 1);
-        dup_lookup_kernel<<<blocks, 256, 0, c->stream>>>(c->dm, p, c->hash, c->dup_tab, tsize - 1, c->dup);
+        e = launch_kernel(dup_lookup_kernel, blocks, 256, 0, c->stream, true, c->dm, p, c->hash, c->dup_tab, tsize - 1, c->dup);
     } else {
         // (four genomes per warp and block: more blocks would fill more tables than they look up in)
         const int per = 4 * kDupThreads / 32;
         const size_t smem = sizeof(unsigned long long) * tsize;
         if (smem > 48 * 1024) {
-            const cudaError_t e = cudaFuncSetAttribute(dup_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            e = cudaFuncSetAttribute(dup_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
             if (e != cudaSuccess) return e;
         }
-        dup_kernel<<<(unsigned)((P + per - 1) / per), kDupThreads, smem, c->stream>>>(c->dm, p, c->hash, c->dup, tsize - 1);
+        e = launch_kernel(dup_kernel, (unsigned)((P + per - 1) / per), kDupThreads, smem, c->stream, early, c->dm, p, c->hash,
+                          c->dup, tsize - 1);
     }
     if (Q > 0) {
-        elite_select_kernel<<<1, kSelThreads, 0, c->stream>>>(P, Q, c->fit, c->dup, c->elite_ctl, c->elite_cand);
+        if (e == cudaSuccess)
+            e = launch_kernel(elite_select_kernel<int32_t>, 1, kSelThreads, 0, c->stream, true, P, Q, c->fit, c->dup,
+                              c->elite_ctl, c->elite_cand);
         const unsigned rb = (unsigned)((Q + 7) / 8 < 152 * 4 ? (Q + 7) / 8 : 152 * 4);
-        elite_cand_rank_kernel<<<rb, 256, 0, c->stream>>>(c->dm, c->fit, c->elite_ctl, c->elite_cand, c->elite,
-                                                          c->elite_fit, p, dst);
-        rank_kernel<<<blocks, 256, 0, c->stream>>>(c->dm, c->fit, c->dup, c->elite, c->elite_fit, p, dst,
-                                                   c->elite_ctl);
+        if (e == cudaSuccess)
+            e = launch_kernel(elite_cand_rank_kernel, rb, 256, 0, c->stream, true, c->dm, c->fit, c->elite_ctl, c->elite_cand,
+                              c->elite, c->elite_fit, p, dst);
+        if (e == cudaSuccess)
+            e = launch_kernel(rank_kernel, blocks, 256, 0, c->stream, true, c->dm, c->fit, c->dup, c->elite, c->elite_fit, p,
+                              dst, c->elite_ctl);
     }
     c->launches += (table ? 2 : 1) + (Q > 0 ? 3 : 0);
-    return cudaGetLastError();
+    return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 cudaError_t launch_ga(const e2_ctx *c, const DevPop &src, const DevPop &dst, uint64_t seed, uint32_t gen,
@@ -815,13 +825,14 @@ cudaError_t launch_ga(const e2_ctx *c, const DevPop &src, const DevPop &dst, uin
 // stream, concurrently with the duplicate test and the ranks (which copy the
 // elites) on the context's stream; the context's stream then waits for the
 // children.
-cudaError_t launch_step(const e2_ctx *c, const DevPop &src, const DevPop &dst, uint64_t seed, uint32_t gen)
+cudaError_t launch_step(const e2_ctx *c, const DevPop &src, const DevPop &dst, uint64_t seed, uint32_t gen,
+                        bool after_eval)
 {
     cudaError_t e = cudaEventRecord(c->ev_fork, c->stream);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(c->side, c->ev_fork, 0);
     if (e == cudaSuccess) e = launch_ga(c, src, dst, seed, gen, c->side);
     if (e == cudaSuccess) e = cudaEventRecord(c->ev_join, c->side);
-    if (e == cudaSuccess) e = launch_elites(c, src, dst);
+    if (e == cudaSuccess) e = launch_elites(c, src, dst, after_eval);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(c->stream, c->ev_join, 0);
     return e;
 }
