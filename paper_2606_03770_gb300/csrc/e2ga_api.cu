@@ -397,6 +397,15 @@ static int costs_grow_with_batch(const e2_layer_profile *prof, int b_max)
     for (const uint64_t *r : rows)
         for (int v = 1; v < b_max; ++v)
             if (r[v + 1] < r[v]) return 0;
+    if (!prof->PF) return 1;
+    const uint64_t *sums[] = {prof->PF, prof->PB, prof->PM};  // per-layer profiles: every block
+    const size_t row = (size_t)prof->N + 1;
+    for (const uint64_t *s : sums)
+        for (int v = 1; v < b_max; ++v)
+            for (size_t j = 0; j + 1 < row; ++j) {
+                const uint64_t *a = s + (size_t)v * row + j, *b = a + row;
+                if (b[1] - b[0] < a[1] - a[0]) return 0;
+            }
     return 1;
 }
 

@@ -111,7 +111,7 @@ __global__ void layered_tables_kernel(Dims dm, const double *rate, const double 
 // and fpr are the pre-pass's view (Tables).
 __global__ void captab_kernel(Dims dm, const double *rate, const double *bw, const uint64_t *mem,
                               const double *rate_cpu, const double *bw_cpu, const uint64_t *mem_cpu,
-                              const uint64_t *prof, const double *leaf, int32_t *capg,
+                              const uint64_t *prof, const uint64_t *psum, const double *leaf, int32_t *capg,
                               uint4 *drec, uint4 *prec, float2 *prech, uint32_t *capv, float4 *fpr)
 {
     const size_t total = (size_t)dm.V * dm.M;
@@ -138,11 +138,33 @@ __global__ void captab_kernel(Dims dm, const double *rate, const double *bw, con
             const double th = hf >= hb ? hf : hb;
             ratio = th > 0.0 ? (float)fmin(tdev / th, 1e6) : 1e6f;
         }
-        const uint32_t caps = (uint32_t)(c0 < N ? c0 : N) | (uint32_t)(c1 < N ? c1 : N) << 16;
+        uint32_t caps = (uint32_t)(c0 < N ? c0 : N) | (uint32_t)(c1 < N ? c1 : N) << 16;
+        uint64_t bf = prof[kBlkFlops * V + v], bb = prof[kBlkBytes * V + v];
+        if (dm.layered) {
+            // per-layer profiles: the longest run of blocks the device holds, without and
+            // with the head, and the least block's flops and bytes, so that the pre-pass's
+            // tests stay necessary conditions
+            const size_t row = (size_t)dm.N + 1, plane = (size_t)V * row;
+            const uint64_t *pf = psum + (size_t)v * row, *pb = pf + plane, *pm = pb + plane;
+            int n0 = 0, n1 = 0;
+            for (int j = 0; j < dm.N; ++j) {
+                while (j + n0 < dm.N && pm[j + n0 + 1] - pm[j] <= mm) ++n0;
+                while (mm >= hm && j + n1 < dm.N && pm[j + n1 + 1] - pm[j] <= mm - hm) ++n1;
+            }
+            caps = (uint32_t)n0 | (uint32_t)n1 << 16;
+            if (d == 0) {
+                bf = pf[1] - pf[0];
+                bb = pb[1] - pb[0];
+                for (int j = 1; j < dm.N; ++j) {
+                    const uint64_t f = pf[j + 1] - pf[j], b = pb[j + 1] - pb[j];
+                    bf = f < bf ? f : bf;
+                    bb = b < bb ? b : bb;
+                }
+            }
+        }
         capv[(size_t)d * V + v] = caps;
         if (d == 0)
-            fpr[v] = make_float4(__ull2float_rd(prof[kBlkFlops * V + v]), __ull2float_rd(prof[kBlkBytes * V + v]),
-                                 __ull2float_rd(prof[kAct * V + v]), 0.0f);
+            fpr[v] = make_float4(__ull2float_rd(bf), __ull2float_rd(bb), __ull2float_rd(prof[kAct * V + v]), 0.0f);
         if (v == 1) prec[d].z = caps;
         if (v == dm.b_max) prec[d].w = caps;
         if (v == 0) {
@@ -661,7 +683,7 @@ cudaError_t launch_tables(const e2_ctx *c)
                                                                 c->mem_cpu, c->prof, c->leaf);
     const size_t vm = (size_t)c->dm.V * c->dm.M;
     captab_kernel<<<grid_for(vm, 256), 256, 0, c->stream>>>(c->dm, c->rate, c->bw, c->mem, c->rate_cpu, c->bw_cpu,
-                                                             c->mem_cpu, c->prof, c->leaf, c->capg, c->drec,
+                                                             c->mem_cpu, c->prof, c->psum, c->leaf, c->capg, c->drec,
                                                              c->prec, c->prech, c->capv, c->fpr);
     c->launches += 2;
     if (c->dm.layered) {
