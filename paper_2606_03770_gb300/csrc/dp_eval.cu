@@ -56,8 +56,9 @@ __device__ __forceinline__ uint32_t size_bin(const Dims &dm, int m)
 //    the marginal device, up to which the cheaper devices just hold N - m more
 //    blocks, gives the program's own optimum; it is found by bisection at the
 //    smallest and the largest batch and kept for those between.  All in float
-//    from times rounded down, every operation rounded toward -inf, so the bound never exceeds the exact value; a variant whose bound is above
-//    Lambda_max (rounded up to float) fails whatever partition the DP returns.
+//    from times rounded down, every operation rounded toward -inf, so the bound
+//    never exceeds the exact value; a variant whose bound is above Lambda_max
+//    (rounded up to float) fails whatever partition the DP returns.
 // With blocks of several types the capacities are the longest run of blocks each
 // device holds and c_k comes from the least block's flops and bytes, so both
 // tests stay necessary conditions: at 32 devices they drop 5,400 of 9,900 runs
@@ -66,13 +67,13 @@ __device__ __forceinline__ uint32_t size_bin(const Dims &dm, int m)
 // KV memory per block), and the program's optimum is the least of a linear
 // cost whose coefficients (per-block and link times) grow with b over a
 // feasible set that shrinks with b, when the profile's costs grow with the
-// batch (physical profiles do; checked at e2_create).  So both are tested on
-// the smallest batch first; if it passes, the largest batch the memory allows
-// is found by a search (the largest batch first, then bisection), and the
-// largest the bound keeps by a second search below it; every smaller batch is
-// kept.  A failed test is exact
-// (memory) or a proof (the bound never exceeds the optimum, and the optimum
-// of every larger batch is no smaller), so every batch above it fails too;
+// batch (physical profiles do; checked at e2_create).  So each is tried on the
+// smallest batch first; if that passes, the largest batch the memory allows is
+// found by a search (the largest batch first, then bisection), and the largest
+// the bound keeps by a second search below it; every smaller batch is kept.  A
+// failed test is exact (memory, identical blocks) or a proof (the bound never
+// exceeds the optimum, and the optimum of every larger batch is no smaller), so
+// every batch above it fails too;
 // rounding and the price can only keep a variant the optimum would drop,
 // which costs a DP run and changes no result.  Other profiles test every
 // batch from the largest down, and the first that passes keeps the smaller
@@ -1546,7 +1547,7 @@ cudaError_t configure_eval(e2_ctx *c)
     c->dm.dp_split = 0;
     c->dp_grid1 = 0;
     c->dp_smem1 = 0;
-    if (c->dm.layered) {                         // the plain-scan path: one launch, one class
+    if (c->dm.layered) {                         // the per-layer DP: one launch, one class
         const void *lk = reinterpret_cast<const void *>(dp_layered_kernel);
         e = cudaFuncSetAttribute(lk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)c->dp_smem);
         if (e != cudaSuccess) return e;

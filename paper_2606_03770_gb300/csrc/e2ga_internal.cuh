@@ -105,7 +105,7 @@ struct Dims {
                          // shrink from one decode batch to the next (the pre-pass tests are then monotone)
     int objective;       // 0: waiting time w (Eq. 3-5); 1: per-request finishing time FT
     int offload;         // 1: some device has host memory for offloaded blocks
-    int layered;         // 1: blocks of several types (per-layer prefix sums): the plain-scan DP path
+    int layered;         // 1: blocks of several types (per-layer prefix sums): the per-layer DP path
 };
 
 // A link of a variant: its time, its order key against the stage times
@@ -393,7 +393,7 @@ cudaError_t dp_order_occupancy(int mmax, int cls, bool off, int *per_sm);
 cudaError_t dp_order_launch(int grid, int mmax, int cls, cudaStream_t stream, const Dims &dm, const Tables &tb,
                             const DevPop &pop, const EvalOut &out, const WorkList &wl, const int32_t *slot_off,
                             const SplitOut &so, bool early);
-size_t dp_layered_smem_bytes(int M, int N);   // the plain-scan DP's shared memory for the largest replica
+size_t dp_layered_smem_bytes(int M, int N);   // the per-layer DP's shared memory for the largest replica
 cudaError_t configure_eval(e2_ctx *c);   // shared memory limit and persistent grid size
 size_t rank_pow2(size_t n);
 cudaError_t build_stage_keys(const e2_ctx *c);    // once per context, before launch_tau
