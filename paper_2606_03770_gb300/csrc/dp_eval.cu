@@ -98,6 +98,7 @@ __device__ __forceinline__ void each_device(int m, int lane, F f)
     if (SMALL) {
         if (lane < m) f(lane);
     } else {
+#pragma unroll 1
         for (int k = lane; k < m; k += 32) f(k);
     }
 }
@@ -189,6 +190,7 @@ __device__ __forceinline__ uint32_t decode_verdict(const Dims &dm, const Tables 
                 });
                 lo = __reduce_min_sync(0xFFFFFFFFu, lo);
                 hi = __reduce_max_sync(0xFFFFFFFFu, hi);
+#pragma unroll 1
                 for (int it = 0; it < 7 && lo < hi; ++it) {
                     const uint32_t mid = lo + ((hi - lo) >> 1);
                     int s = 0;
@@ -222,6 +224,7 @@ __device__ __forceinline__ uint32_t decode_verdict(const Dims &dm, const Tables 
     // the largest batch above lo, from top down, that a test passes (lo: none does)
     auto search = [&](int lo, int top, auto pass) -> int {
         int hi = top + 1, next = top;
+#pragma unroll 1
         while (hi - lo > 1) {
             if (pass(next)) lo = next;
             else hi = next;
