@@ -121,13 +121,16 @@ __global__ void captab_kernel(Dims dm, const double *rate, const double *bw, con
         const int V = dm.V;
         const uint64_t N = (uint64_t)dm.N;
         const uint64_t bm = prof[kBlkMem * V + v], hm = prof[kHeadMem * V + v], mm = mem[d];
-        const uint64_t hc = bm ? mem_cpu[d] / bm : N;                 // blocks host memory holds
-        const uint64_t g0 = bm ? mm / bm : N;
+        // (each count is capped at the model's blocks before the two are added: an unlimited
+        // memory, 2^64 - 1 bytes, holds 2^64 - 1 blocks of a byte)
+        auto holds = [&](uint64_t bytes) { return bm && bytes / bm < N ? bytes / bm : N; };
+        const uint64_t hc = holds(mem_cpu[d]);                        // blocks host memory holds
+        const uint64_t g0 = holds(mm);
         const uint64_t c0 = g0 + hc;
-        const uint64_t g1 = mm < hm ? 0ull : (bm ? (mm - hm) / bm : N);
+        const uint64_t g1 = mm < hm ? 0ull : holds(mm - hm);
         const uint64_t c1 = mm < hm ? 0ull : g1 + hc;
-        capg[idx * 2] = (int32_t)(g0 < N ? g0 : N);
-        capg[idx * 2 + 1] = mm < hm ? -1 : (int32_t)(g1 < N ? g1 : N);
+        capg[idx * 2] = (int32_t)g0;
+        capg[idx * 2 + 1] = mm < hm ? -1 : (int32_t)g1;
         const double tc = __ull2double_rn(prof[kBlkFlops * V + v]) / rate[d];
         const double tm = __ull2double_rn(prof[kBlkBytes * V + v]) / bw[d];
         const double tdev = tc >= tm ? tc : tm;

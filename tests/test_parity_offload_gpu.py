@@ -113,3 +113,25 @@ def test_offload_generations():
         pop = O.ga_step(ga, 5, gen, pop, ora["fitness"], O.elites(ga, pop, ora["fitness"]))
         assert_genomes_equal(eng.get_population(), pop)
     eng.close()
+
+
+@pytest.mark.parametrize("mem,host", [(2**64 - 1, 2), (2**64 - 1, 2**64 - 1), (2**63, 2**63), (3, 2**64 - 1)])
+def test_unlimited_memories(mem, host):
+    """Device and host memories whose counts of one-byte blocks add up past 2^64."""
+    from test_parity_gpu import _edge_problem
+    rng = np.random.default_rng(5)
+    M, N, K, P = 6, 9, 2, 20
+    prob = _edge_problem(rng, M, N, P, K, integer=True, Q=1)
+    one = np.ones_like(prob.blk_mem)
+    prob = dataclasses.replace(prob, blk_mem=one, head_mem=one, mem=np.full(M, mem, np.uint64), rate_cpu=np.ones(M),
+                               bw_cpu=np.ones(M), mem_cpu=np.full(M, host, np.uint64))
+    eng = engine(prob)
+    g = W.random_genomes(M, K, P, seed=1)
+    eng.eval(g)
+    gpu = eng.results()
+    op = O.OracleProblem(prob)
+    ora = op.eval_population(g, K, nthreads=O.num_threads())
+    assert (ora["bsel"] >= 0).any()
+    assert_eval_equal(gpu, ora)
+    assert np.array_equal(gpu["gpu_layers"], expected_gpu_layers(op, g, ora, K))
+    eng.close()
