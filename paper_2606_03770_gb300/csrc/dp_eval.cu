@@ -1551,8 +1551,16 @@ cudaError_t configure_eval(e2_ctx *c)
     c->dp_grid1 = 0;
     c->dp_smem1 = 0;
     if (c->dm.layered) {                         // the per-layer DP: one launch, one class
+        // the limit on its shared memory belongs to the kernel on this device, not to a
+        // context: every context sets the same one, all that a CTA may have beside the
+        // kernel's own arrays, so none lowers what another one launches with
         const void *lk = reinterpret_cast<const void *>(dp_layered_kernel);
-        e = cudaFuncSetAttribute(lk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)c->dp_smem);
+        cudaFuncAttributes own;
+        int optin = 0;
+        if ((e = cudaFuncGetAttributes(&own, lk)) != cudaSuccess) return e;
+        e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, c->device);
+        if (e != cudaSuccess) return e;
+        e = cudaFuncSetAttribute(lk, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - (int)own.sharedSizeBytes);
         if (e != cudaSuccess) return e;
         int per_sm = 0;
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, lk, 32 * kLayeredWarps, c->dp_smem);

@@ -118,6 +118,33 @@ def test_layered_generations():
     eng.close()
 
 
+def test_a_smaller_context_beside_a_larger_one():
+    """The shared memory that the per-layer DP may ask for is the device's, not
+    the last context's: a context of a small model, created and used after one of
+    a large model (77 KB per CTA), leaves the large one's launches and recordings
+    as they were."""
+    rng = np.random.default_rng(17)
+    from test_oracle_pins import _layered
+    M, N, K, P = 64, 126, 4, 8
+    large = _layered(_edge_problem(rng, M, N, P, K, integer=True, Q=1, min_tps=0.01), rng, integer=True)
+    g = W.random_genomes(M, K, P, seed=6)
+    ora = O.OracleProblem(large).eval_population(g, K, nthreads=O.num_threads())
+    eng = engine(large)
+    eng.eval(g)
+    assert eng.stats()["dp_smem"] > 64 * 1024
+    small = engine(W.make_config("c1_tiny", P=64, layered="alternate"))
+    assert small.stats()["dp_smem"] < 16 * 1024
+    small.init_population(4)
+    small.eval()
+    eng.eval(g)
+    assert_eval_equal(eng.results(), ora)
+    eng.run_generation(2, 1)                              # recorded, with the small context alive
+    assert_eval_equal(eng.results(), ora)
+    small.run_generation(2, 1)
+    small.close()
+    eng.close()
+
+
 def test_layered_inputs_refused():
     """Per-layer sums with GPU-CPU offload, too many blocks, decreasing sums, or
     a workspace sized without the per-layer table: statuses, no launch."""
