@@ -6,6 +6,7 @@
 
 #include <new>
 
+#include "copy_route.cuh"
 #include "e2ga_internal.cuh"
 
 using namespace e2;
@@ -166,8 +167,8 @@ AddressRangeFn address_range_fn()
 }
 
 // Copies between the context's arrays and the caller's, on the context's
-// stream.  Pieces whose caller's side is this device's memory, all of it inside
-// one allocation, are gathered and copied by one kernel: a copy of its own for
+// stream.  Pieces whose caller's side is memory of the context's device, current,
+// all of it inside one allocation, are gathered and copied by one kernel: a copy of its own for
 // each costs about 2 us of host and device time, more than the bytes of a small
 // population (a search of 64 genomes of 8 devices, 11 copies: 149 us, in two
 // launches 122; at 16,384 genomes of 512 devices 38 us of copies, now 22).  Every
@@ -175,16 +176,16 @@ AddressRangeFn address_range_fn()
 // over its allocation) is a copy of its own, which refuses what it always did.
 class Copies {
 public:
-    explicit Copies(e2_ctx *c) : c_(c) { cudaGetDevice(&device_); }
+    explicit Copies(e2_ctx *c) : c_(c) { cudaGetDevice(&current_); }
 
     // `user` is the caller's side of the copy: dst or src.  A null dst is skipped.
     cudaError_t add(void *dst, const void *src, size_t bytes, const void *user)
     {
         if (!dst || !bytes) return cudaSuccess;
-        cudaPointerAttributes a;
-        a.type = cudaMemoryTypeUnregistered;
+        cudaPointerAttributes a{};
         if (cudaPointerGetAttributes(&a, user) != cudaSuccess) {
             cudaGetLastError();
+            a = cudaPointerAttributes{};
             a.type = cudaMemoryTypeUnregistered;
         }
         host_ = host_ || a.type == cudaMemoryTypeHost || a.type == cudaMemoryTypeUnregistered;
@@ -192,7 +193,7 @@ public:
         size_t size = 0;
         const unsigned long long at = (unsigned long long)reinterpret_cast<uintptr_t>(user);
         const AddressRangeFn range = address_range_fn();
-        if (a.type != cudaMemoryTypeDevice || a.device != device_ || l_.n == kCopyPieces || !range ||
+        if (!copied_by_kernel(a.type == cudaMemoryTypeDevice, a.device, c_->device, current_) || l_.n == kCopyPieces || !range ||
             range(&base, &size, at) != 0 || at - base > size || bytes > size - (at - base))
             return cudaMemcpyAsync(dst, src, bytes, cudaMemcpyDefault, c_->stream);
         l_.src[l_.n] = static_cast<const unsigned char *>(src);
@@ -216,7 +217,7 @@ public:
 private:
     e2_ctx *c_;
     CopyList l_{};
-    int device_ = -1;
+    int current_ = -1;
     bool host_ = false;
 };
 
