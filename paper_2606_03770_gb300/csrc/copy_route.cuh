@@ -2,6 +2,8 @@
 // caller's may be made by one kernel.  Plain C++, so that it is tested on the host.
 #pragma once
 
+#include <stddef.h>
+
 namespace e2 {
 
 // A kernel on the context's stream may read or write an array of the caller's
@@ -13,6 +15,13 @@ namespace e2 {
 constexpr bool copied_by_kernel(bool device_memory, int owner, int context, int current)
 {
     return device_memory && owner == context && current == context;
+}
+
+// Whether two arrays share a byte.  The blocks of one kernel write in no order,
+// so outputs that do must not be written by the same one.
+inline bool overlap(const unsigned char *a, size_t na, const unsigned char *b, size_t nb)
+{
+    return a < b + nb && b < a + na;
 }
 
 }  // namespace e2

@@ -189,6 +189,13 @@ public:
             a.type = cudaMemoryTypeUnregistered;
         }
         host_ = host_ || a.type == cudaMemoryTypeHost || a.type == cudaMemoryTypeUnregistered;
+        // an output that shares memory with one gathered before it is written after it
+        for (int i = 0; i < l_.n; ++i)
+            if (overlap(l_.dst[i], l_.bytes[i], static_cast<const unsigned char *>(dst), bytes)) {
+                const cudaError_t e = launch_copies(l_, c_->stream);
+                l_.n = 0;
+                if (e != cudaSuccess) return e;
+            }
         unsigned long long base = 0;
         size_t size = 0;
         const unsigned long long at = (unsigned long long)reinterpret_cast<uintptr_t>(user);

@@ -89,3 +89,35 @@ def test_first_bad_genome():
     with pytest.raises(e2ga.E2Error, match="genome 4 "):
         eng.set_population(pop)
     eng.close()
+
+
+def test_outputs_that_share_memory():
+    """Outputs of one call that share memory are written in the call's order: with
+    one array for layers and gpu_layers, or one that starts inside the other, the
+    later output stands where they meet."""
+    import dataclasses
+    import torch
+    rng = np.random.default_rng(3)
+    P, M, K, N = 4096, 24, 3, 30
+    prob = _edge_problem(rng, M, N, P, K, integer=True, Q=1, min_tps=0.0)
+    one = np.ones_like(prob.blk_mem)
+    prob = dataclasses.replace(prob, blk_mem=one, mem=rng.integers(2, 5, M).astype(np.uint64), rate_cpu=np.ones(M),
+                               bw_cpu=np.ones(M), mem_cpu=np.full(M, N, np.uint64))
+    eng = engine(prob)
+    eng.init_population(3)
+    eng.eval()
+    want = eng.results()
+    layers, split = want["layers"].reshape(-1), want["gpu_layers"].reshape(-1)
+    assert (layers != split).mean() > 0.1
+    n = P * M
+    for shift in (0, 8, n - 8):                                 # gpu_layers starts `shift` entries into layers
+        buf = torch.full((2 * n,), -7, dtype=torch.int16, device="cuda")
+        parts = e2ga.e2_partitions(buf.data_ptr(), None, None, None, None, buf.data_ptr() + 2 * shift)
+        for _ in range(5):
+            assert e2ga.e2_get_results(eng.ctx, None, parts) == e2ga.E2_OK
+            torch.cuda.synchronize()
+            got = buf.cpu().numpy()
+            np.testing.assert_array_equal(got[shift:shift + n], split)
+            np.testing.assert_array_equal(got[:shift], layers[:shift])
+            assert (got[shift + n:] == -7).all()
+    eng.close()
