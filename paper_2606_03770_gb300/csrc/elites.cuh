@@ -320,20 +320,22 @@ __global__ void __launch_bounds__(kSelThreads) elite_select_kernel(int P, int Q,
     }
 }
 
+// Keys staged in shared memory for the ranks, shared by the block's warps.
+constexpr int kEliteTile = 1024;
+struct EliteTile {
+    uint64_t w[kEliteTile], p[kEliteTile];
+    int x[kEliteTile];                             // the genome's index, or its duplicate flag
+};
+
 // Ranks of the listed genomes, a warp each: every genome before a listed one
 // in the elite order is distinct and listed too, so its rank is its count of
 // listed genomes before it, taken over tiles of the list staged in shared
 // memory; entries from ctl[1] on have their place in the list as rank.
 // elite(rank, g, lane) takes a genome of rank < Q (by the whole warp).
-constexpr int kEliteTile = 1024;
-
 template <typename Take>
-__device__ __forceinline__ void rank_listed(int Q, const double *fit, const unsigned long long *ctl, const int32_t *cand,
-                                            Take elite)
+__device__ __forceinline__ void rank_listed(EliteTile &t, int Q, const double *fit, const unsigned long long *ctl,
+                                            const int32_t *cand, Take elite)
 {
-    __shared__ uint64_t s_w[kEliteTile], s_p[kEliteTile];
-    __shared__ int s_g[kEliteTile];
-    if (ctl[2] == 0) return;
     const unsigned ncand = (unsigned)ctl[1], total = ncand + (unsigned)ctl[3];
     const int lane = threadIdx.x & 31, NWB = blockDim.x >> 5;
     const uint64_t *fk = reinterpret_cast<const uint64_t *>(fit);
@@ -347,23 +349,54 @@ __device__ __forceinline__ void rank_listed(int Q, const double *fit, const unsi
             unsigned cnt = 0;
             for (unsigned base = 0; base < ncand; base += kEliteTile) {
                 __syncthreads();
-                for (unsigned t = threadIdx.x; t < kEliteTile && base + t < ncand; t += blockDim.x) {
-                    const int h = cand[base + t];
-                    s_g[t] = h;
-                    s_w[t] = fk[(size_t)h * 4];
-                    s_p[t] = fk[(size_t)h * 4 + 1];
+                for (unsigned j = threadIdx.x; j < kEliteTile && base + j < ncand; j += blockDim.x) {
+                    const int h = cand[base + j];
+                    t.x[j] = h;
+                    t.w[j] = fk[(size_t)h * 4];
+                    t.p[j] = fk[(size_t)h * 4 + 1];
                 }
                 __syncthreads();
                 if (ranked) {
                     const unsigned lim = min((unsigned)kEliteTile, ncand - base);
-                    for (unsigned t = lane; t < lim; t += 32)
-                        cnt += s_w[t] != w ? s_w[t] < w : s_p[t] != ph ? s_p[t] < ph : s_g[t] < g;
+                    for (unsigned j = lane; j < lim; j += 32)
+                        cnt += t.w[j] != w ? t.w[j] < w : t.p[j] != ph ? t.p[j] < ph : t.x[j] < g;
                 }
             }
             cnt = __reduce_add_sync(0xFFFFFFFFu, cnt);
             if (ranked) rank = (int)cnt;
         }
         if (live && rank < Q) elite(rank, g, lane);
+    }
+}
+
+// Ranks of all genomes, a warp each, in the order (duplicate, w, phase, index),
+// over tiles of the keys: where fewer than Q are distinct, so that duplicates
+// fill elite slots.
+template <typename Dup, typename Take>
+__device__ __forceinline__ void rank_all(EliteTile &t, int P, int Q, const double *fit, const Dup *dup, Take elite)
+{
+    const int lane = threadIdx.x & 31, NWB = blockDim.x >> 5;
+    const uint64_t *fk = reinterpret_cast<const uint64_t *>(fit);
+    for (int g0 = blockIdx.x * NWB; g0 < P; g0 += gridDim.x * NWB) {            // uniform over the block
+        const int g = g0 + (threadIdx.x >> 5);
+        const bool live = g < P;
+        const uint64_t w = live ? fk[(size_t)g * 4] : 0, ph = live ? fk[(size_t)g * 4 + 1] : 0;
+        const int dg = live ? dup[g] : 0;
+        unsigned rank = 0;
+        for (int base = 0; base < P; base += kEliteTile) {
+            __syncthreads();
+            for (int j = threadIdx.x; j < kEliteTile && base + j < P; j += blockDim.x) {
+                t.w[j] = fk[(size_t)(base + j) * 4];
+                t.p[j] = fk[(size_t)(base + j) * 4 + 1];
+                t.x[j] = dup[base + j];
+            }
+            __syncthreads();
+            const int lim = live ? min(kEliteTile, P - base) : 0;
+            for (int j = lane; j < lim; j += 32)
+                rank += t.x[j] != dg ? t.x[j] < dg : t.w[j] != w ? t.w[j] < w : t.p[j] != ph ? t.p[j] < ph : base + j < g;
+        }
+        rank = __reduce_add_sync(0xFFFFFFFFu, rank);
+        if (live && rank < (unsigned)Q) elite((int)rank, g, lane);
     }
 }
 

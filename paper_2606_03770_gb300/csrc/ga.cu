@@ -446,80 +446,44 @@ __global__ void __launch_bounds__(kDupThreads) dup_kernel(Dims dm, DevPop p, con
     }
 }
 
-// Total order of the elites: distinct genomes before duplicates, then lower w,
-// lower bottleneck phase, lower index.  w and phase are non-negative or +inf,
-// so they are compared as their bit patterns (same order, integer pipe).
-__device__ __forceinline__ bool elite_before(int da, uint64_t wa, uint64_t pa, int a, int db, uint64_t wb,
-                                             uint64_t pb, int b)
+// An elite goes to slot `rank` of the next population, by the warp that ranked it.
+__device__ __forceinline__ void take_elite(const Dims &dm, const double *fit, const DevPop &src, const DevPop &dst,
+                                           int32_t *elite, double *elite_fit, int rank, int g, int lane)
 {
-    if (da != db) return da < db;
-    if (wa != wb) return wa < wb;
-    if (pa != pb) return pa < pb;
-    return a < b;
+    const int M = dm.M, K = dm.K;
+    for (int j = lane; j < M; j += 32) dst.perm[(size_t)rank * M + j] = src.perm[(size_t)g * M + j];
+    for (int j = lane; j < K; j += 32) dst.sizes[(size_t)rank * K + j] = src.sizes[(size_t)g * K + j];
+    if (lane < 4) elite_fit[(size_t)rank * 4 + lane] = fit[(size_t)g * 4 + lane];
+    if (lane == 0) {
+        dst.nclus[rank] = src.nclus[g];
+        dst.roles[rank] = src.roles[g];
+        elite[rank] = g;
+    }
 }
 
-// rank(g) = number of genomes before g in the elite order (duplicate flag,
-// w, phase, index); the first Q ranks are the elites, and the warp of an elite
-// copies it into slot rank(g) of the next population.
+// The full ranking, a warp per genome, where the selection does not apply.
 __global__ void __launch_bounds__(256) rank_kernel(Dims dm, const double *fit, const int32_t *dup,
                                                    int32_t *elite, double *elite_fit, DevPop src, DevPop dst,
                                                    const unsigned long long *ctl)
 {
     after_previous();
-    __shared__ uint64_t s_w[kEliteTile], s_p[kEliteTile];
-    __shared__ int s_d[kEliteTile];
+    __shared__ EliteTile tile;
     if (ctl[2] != 0) return;                       // elite_cand_rank_kernel took the elites
-    const int lane = threadIdx.x & 31, wl = threadIdx.x >> 5;
-    const int g = blockIdx.x * (blockDim.x >> 5) + wl;
-    const bool live = g < dm.P;
-    const uint64_t *fk = reinterpret_cast<const uint64_t *>(fit);
-    const uint64_t w = live ? fk[(size_t)g * 4] : 0, ph = live ? fk[(size_t)g * 4 + 1] : 0;
-    const int dg = live ? dup[g] : 0;
-    int rank = 0;
-    for (int base = 0; base < dm.P; base += kEliteTile) {
-        __syncthreads();
-        for (int t = threadIdx.x; t < kEliteTile && base + t < dm.P; t += blockDim.x) {
-            s_w[t] = fk[(size_t)(base + t) * 4];
-            s_p[t] = fk[(size_t)(base + t) * 4 + 1];
-            s_d[t] = dup[base + t];
-        }
-        __syncthreads();
-        const int lim = min(kEliteTile, dm.P - base);
-        if (live)
-            for (int t = lane; t < lim; t += 32) rank += elite_before(s_d[t], s_w[t], s_p[t], base + t, dg, w, ph, g);
-    }
-#pragma unroll
-    for (int x = 16; x; x >>= 1) rank += __shfl_xor_sync(0xFFFFFFFFu, rank, x);
-    if (live && rank < dm.Q) {
-        const int M = dm.M, K = dm.K;
-        for (int i = lane; i < M; i += 32) dst.perm[(size_t)rank * M + i] = src.perm[(size_t)g * M + i];
-        for (int i = lane; i < K; i += 32) dst.sizes[(size_t)rank * K + i] = src.sizes[(size_t)g * K + i];
-        if (lane == 0) {
-            dst.nclus[rank] = src.nclus[g];
-            dst.roles[rank] = src.roles[g];
-            elite[rank] = g;
-            for (int q = 0; q < 4; ++q) elite_fit[(size_t)rank * 4 + q] = fit[(size_t)g * 4 + q];
-        }
-    }
+    rank_all(tile, dm.P, dm.Q, fit, dup, [&](int rank, int g, int lane) {
+        take_elite(dm, fit, src, dst, elite, elite_fit, rank, g, lane);
+    });
 }
 
-// The listed genomes' ranks, a warp each; the elites are copied into slots
-// [0, Q) of the next population.
+// The listed genomes' ranks, a warp each.
 __global__ void __launch_bounds__(256) elite_cand_rank_kernel(Dims dm, const double *fit,
                                                               const unsigned long long *ctl, const int32_t *cand,
                                                               int32_t *elite, double *elite_fit, DevPop src, DevPop dst)
 {
     after_previous();
-    rank_listed(dm.Q, fit, ctl, cand, [&](int rank, int g, int lane) {
-        const int M = dm.M, K = dm.K;
-        for (int j = lane; j < M; j += 32) dst.perm[(size_t)rank * M + j] = src.perm[(size_t)g * M + j];
-        for (int j = lane; j < K; j += 32) dst.sizes[(size_t)rank * K + j] = src.sizes[(size_t)g * K + j];
-        if (lane < 4) elite_fit[(size_t)rank * 4 + lane] = fit[(size_t)g * 4 + lane];
-        if (lane == 0) {
-            dst.nclus[rank] = src.nclus[g];
-            dst.roles[rank] = src.roles[g];
-            elite[rank] = g;
-        }
+    __shared__ EliteTile tile;
+    if (ctl[2] == 0) return;
+    rank_listed(tile, dm.Q, fit, ctl, cand, [&](int rank, int g, int lane) {
+        take_elite(dm, fit, src, dst, elite, elite_fit, rank, g, lane);
     });
 }
 
