@@ -407,8 +407,8 @@ int e2_set_timing_events(e2_ctx *ctx, void *dp_start, void *dp_stop);
  * share the one scratch array and overwrite it; calls that overlap on the GPU
  * (other streams, other host threads) race and must be serialised by the
  * caller.  Cost: one read of the population for its fingerprints, and the
- * selection e2_ga_step uses; with fewer than Q distinct genomes, one O(P^2)
- * pass over the fitness keys. */
+ * selection e2_ga_step uses; up to 2,048 genomes, and with fewer than Q distinct
+ * ones, one O(P^2) pass over the fitness keys instead. */
 #define E2_NOALLOC_MAX_POP 65536
 int e2_select_elites_noalloc(const e2_genomes *pop, const double *fitness, int32_t P, int32_t M,
                              int32_t K_max, int32_t Q, int32_t *elite_idx, void *stream);

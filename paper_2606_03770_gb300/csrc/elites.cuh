@@ -123,6 +123,26 @@ __device__ __forceinline__ bool is_duplicate(const DevPop &p, const unsigned lon
     return d;
 }
 
+// Duplicate flags of small populations, by every block of a grid: each fills a
+// table of its own in shared memory (mask + 1 slots) and looks up its share of
+// the genomes, which saves a fill in global memory, a launch and its atomics.
+constexpr int kDupThreads = 512;
+
+template <typename Dup>
+__device__ __forceinline__ void flag_duplicates(unsigned long long *tab, unsigned mask, const DevPop &p, const uint64_t *hash,
+                                                Dup *dup, int P, int M, int K, const uint64_t *fk = nullptr)
+{
+    const int lane = threadIdx.x & 31;
+    for (unsigned s = threadIdx.x; s <= mask; s += kDupThreads) tab[s] = kFreeSlot;
+    __syncthreads();
+    for (int g = threadIdx.x; g < P; g += kDupThreads) table_insert(tab, mask, hash[g], g);
+    __syncthreads();
+    for (int g = blockIdx.x * (kDupThreads / 32) + (threadIdx.x >> 5); g < P; g += gridDim.x * (kDupThreads / 32)) {
+        const bool d = is_duplicate(p, tab, mask, hash, g, M, K, lane, fk);
+        if (lane == 0) dup[g] = d;
+    }
+}
+
 // A list that holds the Q first distinct genomes in the order (w, phase,
 // index), made by one CTA without ranking every genome.  Each thread takes the
 // least key of its share of the genomes; the Q-th least of these minima has at

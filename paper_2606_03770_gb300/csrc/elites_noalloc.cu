@@ -37,6 +37,10 @@ namespace {
 constexpr int kNoallocMaxPop = E2_NOALLOC_MAX_POP;
 constexpr int kMaxDeviceIds = 64;
 constexpr int kWarps = 8;
+// Populations up to this size skip the selection (dup_small_noalloc).  At 4,096
+// genomes the quadratic ranking loses (53 us with Q = P against 31 for a
+// selection), and the table no longer fits the 48 KB that any block may use.
+constexpr int kSmallPop = 2048;
 
 // Scratch: the fingerprints, the fingerprint table (reused for the candidate
 // list once the duplicates are known), the duplicate flags and the selection's
@@ -114,6 +118,28 @@ __global__ void __launch_bounds__(32 * kWarps) dup_noalloc(e2::DevPop p, const u
     if (lane == 0) sc->dup[g] = d;
 }
 
+// Small populations: the duplicates through a table per block, and the ranks of
+// all genomes without a selection.  Three short kernels, the last two placed
+// early: 8 us for 64 genomes of 32 devices, 14 for 1,024, 25 for 2,048; the five
+// kernels below, bound by their chain, take 25, 28 and 29.
+__global__ void __launch_bounds__(e2::kDupThreads) dup_small_noalloc(e2::DevPop p, const uint64_t *fk, int P, int M, int K,
+                                                                     Scratch *sc, unsigned mask)
+{
+    e2::after_previous();
+    extern __shared__ unsigned long long tab[];
+    e2::flag_duplicates(tab, mask, p, sc->hash, sc->dup, P, M, K, fk);
+}
+
+__global__ void __launch_bounds__(32 * kWarps) rank_small_noalloc(int P, int Q, const double *fit, const Scratch *sc,
+                                                                  int32_t *elite)
+{
+    e2::after_previous();
+    __shared__ e2::EliteTile tile;
+    e2::rank_all(tile, P, Q, fit, sc->dup, [&](int rank, int g, int lane) {
+        if (lane == 0) elite[rank] = g;
+    });
+}
+
 // The listed genomes' ranks; with fewer than Q distinct genomes, the ranks of
 // all of them.  Bound by the comparisons of every pair: 312 us for 16,384
 // genomes of 32 devices and 3.9 ms for 65,536; by strided reads of the caller's
@@ -184,6 +210,21 @@ extern "C" int e2_select_elites_noalloc(const e2_genomes *pop, const double *fit
     const uint64_t *fk = reinterpret_cast<const uint64_t *>(fitness);
     const unsigned slots = e2::dup_table_size(P);
     const unsigned wblocks = (unsigned)((P + kWarps - 1) / kWarps);
+    if (P <= kSmallPop) {
+        fingerprint_noalloc<<<wblocks, 32 * kWarps, 0, s>>>(p, fk, P, M, K_max, sc, 0);
+        // (a genome per warp: the blocks are one wave whatever P)
+        const unsigned per = e2::kDupThreads / 32;
+        cudaError_t e = cudaGetLastError();
+        if (e == cudaSuccess)
+            e = e2::launch_kernel(dup_small_noalloc, ((unsigned)P + per - 1) / per, e2::kDupThreads,
+                                  sizeof(unsigned long long) * slots, s, true, p, fk, P, M, K_max, sc, slots - 1);
+        if (e == cudaSuccess && Q > 0)
+            // (early only up to a block per SM: placed while the kernel before it runs, more of
+            // them crowd on the SMs that it leaves free, 31 us instead of 24 at 2,048 genomes)
+            e = e2::launch_kernel(rank_small_noalloc, wblocks, 32 * kWarps, 0, s, wblocks <= 152, P, Q, fitness, sc,
+                                  elite_idx);
+        return e == cudaSuccess ? E2_OK : reject(E2_ECUDA, cudaGetErrorString(e));
+    }
     fingerprint_noalloc<<<wblocks, 32 * kWarps, 0, s>>>(p, fk, P, M, K_max, sc, slots);
     insert_noalloc<<<(unsigned)((P + 255) / 256), 256, 0, s>>>(P, sc, slots - 1);
     dup_noalloc<<<wblocks, 32 * kWarps, 0, s>>>(p, fk, P, M, K_max, sc, slots - 1);

@@ -402,9 +402,7 @@ __global__ void __launch_bounds__(256) init_kernel(Dims dm, DevPop p, uint64_t s
 
 // Duplicate test: dup_insert_kernel fills the fingerprint table (elites.cuh) in
 // global memory and dup_lookup_kernel looks each genome up, a warp each.
-// Below kDupTableFrom genomes one kernel does both: every block fills a table
-// of its own in shared memory and looks up its share of the genomes, which
-// saves the fill, a launch and the global atomics.
+// Below kDupTableFrom genomes one kernel does both (flag_duplicates).
 constexpr int kDupTableFrom = 4096;
 
 // (the table is filled with kFreeSlot beforehand)
@@ -428,22 +426,12 @@ __global__ void __launch_bounds__(256) dup_lookup_kernel(Dims dm, DevPop p, cons
 
 // (comparing each genome's keys with every lower-indexed one's took 8 us at
 // 1,024 genomes and 28 at 2,048)
-constexpr int kDupThreads = 512;
-
 __global__ void __launch_bounds__(kDupThreads) dup_kernel(Dims dm, DevPop p, const uint64_t *hash, int32_t *dup,
                                                           unsigned mask)
 {
     after_previous();
     extern __shared__ unsigned long long tab[];
-    const int lane = threadIdx.x & 31;
-    for (unsigned s = threadIdx.x; s <= mask; s += kDupThreads) tab[s] = kFreeSlot;
-    __syncthreads();
-    for (int g = threadIdx.x; g < dm.P; g += kDupThreads) table_insert(tab, mask, hash[g], g);
-    __syncthreads();
-    for (int g = blockIdx.x * (kDupThreads / 32) + (threadIdx.x >> 5); g < dm.P; g += gridDim.x * (kDupThreads / 32)) {
-        const bool d = is_duplicate(p, tab, mask, hash, g, dm.M, dm.K, lane);
-        if (lane == 0) dup[g] = d;
-    }
+    flag_duplicates(tab, mask, p, hash, dup, dm.P, dm.M, dm.K);
 }
 
 // An elite goes to slot `rank` of the next population, by the warp that ranked it.

@@ -86,3 +86,10 @@ def test_generation_step_on_copies(P, distinct):
     for k in ref:
         assert np.array_equal(nxt[k], ref[k]), k
     eng.close()
+
+
+@pytest.mark.parametrize("P", [2048, 2049])
+@pytest.mark.parametrize("what", ["plateau", "ties", "inf"])
+def test_selection_beside_the_small_populations(P, what):
+    """The largest population ranked without a selection, and the smallest with one."""
+    test_selection(P, what)
