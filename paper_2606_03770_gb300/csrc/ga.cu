@@ -378,6 +378,44 @@ __host__ __device__ __forceinline__ size_t genome_bytes(int M)
     return (4 * (size_t)M + 2 * (size_t)((M + 1) & ~1) * 2 + 2 * E2_MAX_CLUSTERS + 3) & ~(size_t)3;
 }
 
+// Large populations of small fleets: a genome per thread, which takes the draws
+// one after the other; a warp per genome leaves most lanes idle there (65,536
+// genomes of 16 devices 55 us against 24, 262,144 of 8 197 against 18).
+__global__ void __launch_bounds__(32) init_small_kernel(Dims dm, DevPop p, uint64_t seed)
+{
+    const int s = blockIdx.x * blockDim.x + threadIdx.x;
+    if (s >= dm.P) return;
+    const int M = dm.M, K = dm.K;
+    uint16_t *perm = p.perm + (size_t)s * M, *sizes = p.sizes + (size_t)s * K;
+    for (int i = 0; i < M; ++i) perm[i] = (uint16_t)i;
+    Stream order(seed, 0, (uint32_t)s, kInitPerm);
+    for (int t = M - 1; t >= 1; --t) {
+        const uint32_t j = below(order.word((uint32_t)(M - 1 - t)), (uint32_t)t + 1);
+        const uint16_t x = perm[t];
+        perm[t] = perm[j];
+        perm[j] = x;
+    }
+    for (int c = 0; c < K; ++c) sizes[c] = 0;
+    Stream group(seed, 0, (uint32_t)s, kInitGroup);
+    const int R = 1 + (int)below(group.word(0), (uint32_t)min(K, M));
+    int c = 0, prev = 0;
+    for (int t = 1; t < M && c < R - 1; ++t)
+        if (below(group.word((uint32_t)t), (uint32_t)(M - t)) < (uint32_t)(R - 1 - c)) {
+            sizes[c++] = (uint16_t)(t - prev);
+            prev = t;
+        }
+    sizes[c] = (uint16_t)(M - prev);
+    p.nclus[s] = (uint8_t)R;
+    p.roles[s] = random_roles(Stream(seed, 0, (uint32_t)s, kInitRoles), R);
+}
+
+// Whether a thread per genome is about as fast or faster: up to 8 devices always
+// (64 genomes 4 us, a warp each 6), then from 4,096 genomes at up to 16 devices (6
+// against 8), 16,384 at up to 24 (16 to 20 against 18) and 65,536 at up to 32 (54
+// against 57); with a quarter of those genomes it takes 6, 10 and 27 against 6, 8
+// and 19.
+bool init_by_threads(int M, int P) { return M <= 8 || (M <= 32 && P >= 256 << 2 * ((M + 7) / 8)); }
+
 // A genome per warp.  (A thread per genome, swapping in global memory, took
 // 125 us for 8,192 genomes of 256 devices; now 30.)
 __global__ void __launch_bounds__(256) init_kernel(Dims dm, DevPop p, uint64_t seed)
@@ -733,6 +771,11 @@ static cudaError_t genome_launch(const void *kernel, int M, int *nw, size_t *sme
 
 cudaError_t launch_init(const e2_ctx *c, const DevPop &p, uint64_t seed)
 {
+    if (init_by_threads(c->dm.M, c->dm.P)) {
+        init_small_kernel<<<(unsigned)((c->dm.P + 31) / 32), 32, 0, c->stream>>>(c->dm, p, seed);
+        ++c->launches;
+        return cudaGetLastError();
+    }
     size_t smem = 0;
     int nw = 1;
     const cudaError_t e = genome_launch(reinterpret_cast<const void *>(init_kernel), c->dm.M, &nw, &smem);

@@ -38,3 +38,15 @@ def test_init_and_step(M, kinds):
         pop = O.ga_step(ga, M, gen, pop, fit, O.elites(ga, pop, fit))
     assert_genomes_equal(eng.get_population(), pop)
     eng.close()
+
+
+@pytest.mark.parametrize("M,P,K", [(1, 1, 1), (2, 33, 2), (8, 64, 3), (8, 5000, 8), (9, 4095, 9), (9, 4096, 9), (16, 4097, 1),
+                                   (17, 16384, 17), (24, 16390, 5), (25, 16384, 25), (32, 65536, 32), (33, 65536, 4)])
+def test_init_on_both_sides_of_the_thread_per_genome(M, P, K):
+    """Small fleets and large populations, where a thread takes a genome's draws, and the sizes next to them."""
+    prob = _edge_problem(np.random.default_rng(M), M, 3, P, K, integer=True, Q=1, min_tps=0.01)
+    eng = engine(prob)
+    for seed in (1, 2**40 + 7):
+        eng.init_population(seed)
+        assert_genomes_equal(eng.get_population(), O.init_population(O.ga_of(prob), seed))
+    eng.close()
