@@ -237,6 +237,20 @@ __global__ void redraw_kernel(int M, uint64_t seed, uint32_t gen, double lo, dou
     }
 }
 
+// An invalid genome (`lane` of `lanes` threads) is replaced by a valid one, the
+// identity ordering as one prefill replica, so that no later kernel reads it.
+__device__ __forceinline__ void replace_genome(const Dims &dm, const DevPop &p, int g, int32_t *err, int lane, int lanes)
+{
+    const int M = dm.M, K = dm.K;
+    if (lane == 0) atomicMin(err, g);
+    for (int i = lane; i < M; i += lanes) p.perm[(size_t)g * M + i] = (uint16_t)i;
+    for (int c = lane; c < K; c += lanes) p.sizes[(size_t)g * K + c] = (uint16_t)(c ? 0 : M);
+    if (lane == 0) {
+        p.nclus[g] = 1;
+        p.roles[g] = 0;
+    }
+}
+
 // A warp per genome: the lanes check the sizes and mark the devices of the
 // ordering in a shared bitmap (a device marked before is a repeat).  11 us for
 // 16,384 genomes of 512 devices; a thread per genome, with its bitmap in local
@@ -271,16 +285,41 @@ __global__ void __launch_bounds__(32 * kValidateWarps) validate_kernel(Dims dm, 
         if (d >= M) ok = false;
         else if (atomicOr(&seen[d >> 5], 1u << (d & 31)) >> (d & 31) & 1u) ok = false;
     }
-    if (__all_sync(0xFFFFFFFFu, ok)) return;
-    if (lane == 0) atomicMin(err, g);
-    // replaced by a valid genome (the identity ordering as one prefill
-    // replica), so that no later kernel reads an invalid one
-    for (int i = lane; i < M; i += 32) p.perm[(size_t)g * M + i] = (uint16_t)i;
-    for (int c = lane; c < K; c += 32) p.sizes[(size_t)g * K + c] = (uint16_t)(c ? 0 : M);
-    if (lane == 0) {
-        p.nclus[g] = 1;
-        p.roles[g] = 0;
+    if (!__all_sync(0xFFFFFFFFu, ok)) replace_genome(dm, p, g, err, lane, 32);
+}
+
+// Large populations of fleets below 64 devices: a thread per genome, its bitmap one
+// word.  A warp each is bound by its chain of loads and barriers and leaves lanes
+// idle: an upload of 16,384 genomes of 16 devices 29 us, of 262,144 91, by threads
+// 21 and 30; up to 4,096 genomes both take 20.  (At 64 devices, rows of 128 bytes,
+// threads take 28 from 64 genomes on.)
+constexpr int kValidateThreads = 128;
+bool validate_by_threads(int M, int P) { return M < 64 && P >= 8192; }
+
+__global__ void __launch_bounds__(kValidateThreads) validate_small_kernel(Dims dm, DevPop p, int32_t *err)
+{
+    after_previous();
+    const int g = blockIdx.x * kValidateThreads + threadIdx.x;
+    if (g >= dm.P) return;
+    const int M = dm.M, K = dm.K, R = p.nclus[g];
+    const uint64_t roles = p.roles[g];
+    bool ok = R >= 1 && R <= K && R <= M;
+    if (R < 64) ok = ok && (roles >> R) == 0ull;
+    int sum = 0;
+    for (int c = 0; c < K; ++c) {
+        const int s = p.sizes[(size_t)g * K + c];
+        ok = ok && (c < R ? s >= 1 : s == 0);
+        sum += s;
     }
+    ok = ok && sum == M;
+    uint64_t seen = 0;                             // (M distinct devices below M fill the first M bits)
+    for (int i = 0; i < M; ++i) {
+        const int d = p.perm[(size_t)g * M + i];
+        ok = ok && d < M;
+        seen |= d < 64 ? 1ull << d : 0ull;
+    }
+    ok = ok && seen == (1ull << M) - 1ull;
+    if (!ok) replace_genome(dm, p, g, err, 0, 1);
 }
 
 // Fisher-Yates shuffle of the identity ordering by a warp (word M-1-t draws
@@ -755,8 +794,10 @@ cudaError_t launch_copies(const CopyList &l, cudaStream_t st)
 cudaError_t launch_validate(const e2_ctx *c, const DevPop &p, bool early)
 {
     ++c->launches;
-    return launch_kernel(validate_kernel, (c->dm.P + kValidateWarps - 1) / kValidateWarps, 32 * kValidateWarps, 0, c->stream,
-                         early, c->dm, p, c->err);
+    const bool small = validate_by_threads(c->dm.M, c->dm.P);
+    const int threads = small ? kValidateThreads : 32 * kValidateWarps, per = small ? kValidateThreads : kValidateWarps;
+    return launch_kernel(small ? validate_small_kernel : validate_kernel, (unsigned)((c->dm.P + per - 1) / per), threads, 0,
+                         c->stream, early, c->dm, p, c->err);
 }
 
 // Warps per CTA and shared memory of a kernel with genome_bytes(M) per warp.

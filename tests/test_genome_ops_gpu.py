@@ -50,3 +50,40 @@ def test_init_on_both_sides_of_the_thread_per_genome(M, P, K):
         eng.init_population(seed)
         assert_genomes_equal(eng.get_population(), O.init_population(O.ga_of(prob), seed))
     eng.close()
+
+
+@pytest.mark.parametrize("M", [2, 33, 63, 64])
+@pytest.mark.parametrize("P", [8191, 8192])
+def test_validation_on_both_sides_of_the_thread_per_genome(M, P):
+    """Every kind of invalid genome, found and replaced, whether a warp or a thread takes a genome."""
+    from paper_2606_03770_gb300 import e2ga
+    prob = _edge_problem(np.random.default_rng(M), M, 3, P, 2, integer=True, Q=1, min_tps=0.01)
+    eng = engine(prob)
+    eng.init_population(3)
+    pop = eng.get_population()
+    eng.set_population(pop)                                  # all valid
+    assert_genomes_equal(eng.get_population(), pop)
+    bad = {k: v.copy() for k, v in pop.items()}
+    two = np.flatnonzero(pop["nclus"] == 2)
+    rng = np.random.default_rng(P)
+    at = np.sort(rng.choice(two[two > 10], 9, replace=False))
+    rng.shuffle(at)
+    repeat, beyond, far, none, many, empty, total, extra, role = at
+    bad["perm"][repeat, -1] = bad["perm"][repeat, 0]
+    bad["perm"][beyond, 0] = M
+    bad["perm"][far, M // 2] = 65535
+    bad["nclus"][none] = 0
+    bad["nclus"][many] = 3
+    bad["sizes"][empty] = (M, 0)
+    bad["sizes"][total, 1] += 1
+    bad["nclus"][extra] = 1                                  # its second size is beyond
+    bad["roles"][role] |= np.uint64(4)
+    with pytest.raises(e2ga.E2Error, match=f"genome {at.min()} "):
+        eng.set_population(bad)
+    want = {k: v.copy() for k, v in pop.items()}
+    want["perm"][at] = np.arange(M)
+    want["sizes"][at] = (M, 0)
+    want["nclus"][at] = 1
+    want["roles"][at] = 0
+    assert_genomes_equal(eng.get_population(), want)
+    eng.close()
