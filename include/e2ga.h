@@ -225,8 +225,7 @@ typedef struct {
                                    to miss Min_TPS (their DP is skipped)        */
     uint64_t dp_runs_small;     /* of dp_runs, those of the second DP launch: the
                                    replicas with several devices per lane (more
-                                   than 32), or on large populations of smaller
-                                   fleets those of more than 8 devices          */
+                                   than 32)                                     */
     uint64_t dp_launches;       /* DP kernel launches per evaluation (1 or 2;
                                    fixed at e2_create)                          */
     uint64_t dp_ctas;           /* persistent CTAs of the first DP launch       */

@@ -1533,11 +1533,10 @@ __global__ void __launch_bounds__(128) gc_split_kernel(Dims dm, DevPop pop, cons
 
 // Persistent grids of the DP.  Replicas of up to 32 devices (a device per
 // lane) and larger ones (several per lane, more registers) form two launches
-// where both sizes can occur.  On fleets without the larger sizes,
-// populations of kSplitSlots slots or more launch the replicas of more than 8
-// devices apart.
-constexpr long long kSplitSlots = 32768;
-
+// where both sizes can occur.  (A second launch for the replicas of more than 8
+// devices on smaller fleets with 32,768 slots or more was slower at every size
+// measured: 8,192 genomes of 32 devices 172 us a generation against 167, 16,384
+// 280 against 262, 65,536 891 against 870.)
 cudaError_t configure_eval(e2_ctx *c)
 {
     cudaError_t e = cudaSuccess;
@@ -1570,7 +1569,6 @@ cudaError_t configure_eval(e2_ctx *c)
     }
     const bool off = c->dm.offload != 0;
     if (mmax > 32) c->dm.dp_split = 32;
-    else if (mmax > 8 && (long long)c->dm.P * c->dm.K >= kSplitSlots) c->dm.dp_split = 8;
     const int m0 = c->dm.dp_split ? c->dm.dp_split : mmax;   // class 0's largest replica
     int per_sm = 0;
     e = dp_order_occupancy(m0, 0, off, &per_sm);

@@ -28,9 +28,9 @@ def _built():
     ge.build()
 
 
-def _warp_launch(st):
-    assert st["dp_launches"] == 2 and st["dp_runs_per_cta_small"] == 4, st
-    assert st["dp_runs_small"] > 0 and st["device_errors"] == 0, st
+def _launches(st, n):
+    assert st["dp_launches"] == n and st["dp_runs_per_cta_small"] == (4 if n == 2 else 0), st
+    assert (st["dp_runs_small"] > 0) == (n == 2) and st["device_errors"] == 0, st
 
 
 @pytest.mark.parametrize("name,P,role_search", [("c3", 4096, 0), ("c3", 2048, 1), ("c5", 1024, 0)])
@@ -45,7 +45,7 @@ def test_warp_launch_full_population(name, P, role_search):
     if role_search:
         assert np.array_equal(eng.get_population()["roles"], ora["roles"])
     st = eng.stats()
-    _warp_launch(st)
+    _launches(st, 2)
     assert st["paper_candidates"] == ora["cand"]
     assert st["served"] == int((ora["bsel"] >= 0).sum())
     eng.close()
@@ -65,7 +65,7 @@ def test_warp_launch_ties_and_memory_walls(min_tps):
     gpu = eng.results()
     ora = O.OracleProblem(prob).eval_population(g, K, nthreads=O.num_threads())
     assert_eval_equal(gpu, ora)
-    _warp_launch(eng.stats())
+    _launches(eng.stats(), 1)                               # no replica of more than 32 devices
     assert np.isfinite(ora["T"]).sum() > 1000
     ga = O.ga_of(prob)
     eidx = O.elites(ga, g, gpu["fitness"])
