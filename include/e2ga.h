@@ -234,7 +234,9 @@ typedef struct {
     uint64_t dp_smem_small;
     uint64_t launches;          /* kernels this context has launched since
                                    e2_create, cumulative (a recorded generation
-                                   counts its kernel nodes per replay)          */
+                                   counts its kernel nodes per replay; copies to
+                                   and from the caller's arrays do not count,
+                                   whether a kernel or copy calls make them)    */
     uint64_t role_search_capped;/* genomes of the last evaluation whose role
                                    search was not run (more than
                                    E2_MAX_ROLE_SEARCH replicas to enumerate)    */
@@ -279,8 +281,9 @@ size_t e2_workspace_bytes_ex(int32_t M, int32_t N, int32_t b_max, int32_t P, int
  * and to the current device.  The caller keeps ownership of every input and
  * of the workspace.  Synchronises the stream.  Errors: E2_EINVAL for any
  * invalid value, for min(M, N) > 256 (a replica's DP holds at most 256
- * devices) or when the largest replica's DP exceeds shared memory;
- * E2_ENOMEM for a short workspace; E2_ECUDA. */
+ * devices) or, with identical blocks, for more blocks than the fleet's size
+ * admits (up to 16 devices any N within E2_MAX_BLOCKS, 32 devices 752 blocks,
+ * 64 462, 128 337, 256 328); E2_ENOMEM for a short workspace; E2_ECUDA. */
 int e2_create(const e2_devices *devs, const e2_links *links, const e2_layer_profile *prof,
               const e2_params *prm, void *workspace, size_t workspace_bytes, void *stream,
               e2_ctx **out);

@@ -78,7 +78,7 @@ __device__ __forceinline__ uint32_t size_bin(const Dims &dm, int m)
 // which costs a DP run and changes no result.  Other profiles test every
 // batch from the largest down, and the first that passes keeps the smaller
 // ones.
-// The verdicts go into the slot's info word (SlotBits), with the bin of its
+// The verdicts go into the slot's info word (kSlot*), with the bin of its
 // size in the work list's order.  A replica with nothing to run (more devices
 // than blocks, no variant left) gets its outputs here, and so do the empty
 // slots.
@@ -1586,9 +1586,7 @@ cudaError_t configure_eval(e2_ctx *c)
 
 cudaError_t launch_eval(const e2_ctx *c, const DevPop &p)
 {
-    Tables tb{c->rate, c->bw, c->mem, c->rate_cpu, c->bw_cpu, c->mem_cpu, c->prof, c->leaf, c->tau,
-              c->capg, c->leaf_rank, c->lcost, c->drec, c->fxs, c->prec, c->prech, c->capv,
-              c->ibw, c->fpr};
+    Tables tb{c->leaf, c->tau, c->capg, c->leaf_rank, c->lcost, c->drec, c->fxs, c->prec, c->prech, c->capv, c->ibw, c->fpr};
     EvalOut out{c->fit, c->layers, c->master, c->bsel, c->T, c->L, c->hash, c->stats, c->gpu_layers};
     SlotInfo si{c->slot_off, c->slot_info};
     WorkList wl{c->items, c->list_ctrl};

@@ -210,12 +210,12 @@ public:
         ++l_.n;
         return cudaSuccess;
     }
-    // the gathered pieces, and *word = value (every byte of it `value`'s lowest) on the way
-    cudaError_t go(int32_t *word = nullptr, int32_t value = 0)
+    // the gathered pieces, and *word = kNoBadGenome (bytes all 0x7F) on the way
+    cudaError_t go(int32_t *word = nullptr)
     {
-        if (!l_.n) return word ? cudaMemsetAsync(word, value & 0xFF, sizeof *word, c_->stream) : cudaSuccess;
+        static_assert(kNoBadGenome == 0x01010101 * 0x7F, "the memset writes one byte value");
+        if (!l_.n) return word ? cudaMemsetAsync(word, 0x7F, sizeof *word, c_->stream) : cudaSuccess;
         l_.word = word;
-        l_.value = value;
         return launch_copies(l_, c_->stream);
     }
     bool launched() const { return l_.n > 0; }             // go() ended in a kernel
@@ -338,8 +338,6 @@ int check_genomes(e2_ctx *c, const e2_genomes *g)
 // Copy a population into the current buffer and validate it on the device
 // (invalid genomes are replaced there by a valid one); the smallest invalid
 // index lands in the error word, read back by check_validated.
-constexpr int32_t kNoBadGenome = 0x7F7F7F7F;   // the error word's bytes all 0x7F
-
 int upload_and_validate(e2_ctx *c, const e2_genomes *g)
 {
     const int st = check_genomes(c, g);
@@ -351,7 +349,7 @@ int upload_and_validate(e2_ctx *c, const e2_genomes *g)
     E2_CUDA(c, in.add(p.sizes, g->sizes, 2 * P * K, g->sizes));
     E2_CUDA(c, in.add(p.nclus, g->nclus, P, g->nclus));
     E2_CUDA(c, in.add(p.roles, g->roles, 8 * P, g->roles));
-    E2_CUDA(c, in.go(c->err, kNoBadGenome));
+    E2_CUDA(c, in.go(c->err));
     E2_CUDA(c, launch_validate(c, c->pop[c->cur], in.launched()));
     c->evaluated = false;
     return E2_OK;
@@ -515,7 +513,7 @@ int e2_create(const e2_devices *devs, const e2_links *links, const e2_layer_prof
     if ((M < N ? M : N) > kMaxReplicaDevices)
         return fail_free(E2_EINVAL, "replicas could exceed 256 devices (min(M, N) > 256)");
     if ((layered ? c->dp_smem : dp_size_limit_bytes(M, N)) + 1024 > (size_t)smem_optin)
-        return fail_free(E2_EINVAL, "the largest replica's DP does not fit in shared memory (N too large)");
+        return fail_free(E2_EINVAL, "too many blocks for this many devices (N too large)");
     if (configure_eval(c) != cudaSuccess) return fail_free(E2_ECUDA, "configuring the DP kernel failed");
     if (cudaStreamCreateWithFlags(&c->side, cudaStreamNonBlocking) != cudaSuccess ||
         cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming) != cudaSuccess ||

@@ -33,8 +33,7 @@ struct DevPop {
 };
 
 // Largest replica (devices) a DP can receive: replicas with more devices than
-// blocks are infeasible, and the evaluation pre-pass stages up to 256 devices
-// of a replica per warp in shared memory.
+// blocks are infeasible, and the DP's warps hold up to 8 devices per lane.
 constexpr int kMaxReplicaDevices = 256;
 
 // The DP's work list: items in kListBins bins of replica sizes (class 0 before
@@ -54,11 +53,12 @@ constexpr int kSlotMemShift = 7;
 constexpr uint32_t kSlotPrefill = 1u << 14, kSlotDecTested = 1u << 15, kSlotPreTested = 1u << 16;
 constexpr int kSlotBinShift = 24;
 
-// Shared memory the limits of the ABI are stated in: an input whose largest
-// replica (m devices, W = N - m + 1 block counts) would need more than an SM
-// has in this layout -- per device three counters, two cost rows (three below
-// 40 KB), the link and head keys and the id, and the work rows of four warps
-// -- is refused by e2_create.
+// The bound of the ABI on the blocks of a fleet, for models of identical blocks:
+// inputs are refused for which some replica of m devices and its W = N - m + 1
+// block counts come to more bytes, as counted here, than a CTA may have of shared
+// memory (up to 16 devices any N, 32 devices 752 blocks, 64 462, 128 337, 256
+// 328).  No kernel lays this out; the bound is kept so that the sizes accepted stay
+// the same.
 __host__ __forceinline__ size_t dp_table_bytes(int m, int N, bool spill)
 {
     const size_t W = (size_t)(N - m + 1), mm = (size_t)m;
@@ -117,11 +117,6 @@ struct __align__(16) LinkRec {
 };
 
 struct Tables {
-    const double *rate, *bw;
-    const uint64_t *mem;
-    const double *rate_cpu, *bw_cpu;   // [M] host side of offloaded blocks (offload only)
-    const uint64_t *mem_cpu;           // [M] host memory for blocks, bytes (offload only)
-    const uint64_t *prof;      // [kNumProf][V]
     const double *leaf;        // [V][M][2][LS]: leaf[((v*M+d)*2+mf)*LS + n-1] = l_d(n blocks, master mf)
     const LinkRec *tau;        // [V][M][M]
     const int32_t *capg;       // [V][M][2]: most blocks in device memory, without / with the head (-1: the head
@@ -361,9 +356,11 @@ struct CopyList {
     unsigned long long bytes[kCopyPieces];
     unsigned first[kCopyPieces + 1];
     int n;
-    int32_t *word;           // a word to set to `value` besides (nullptr: none)
-    int32_t value;
+    int32_t *word;           // a word to set to kNoBadGenome besides (nullptr: none)
 };
+
+// The error word of an upload without an invalid genome (above every index).
+constexpr int32_t kNoBadGenome = 0x7F7F7F7F;
 
 // launchers (defined in the .cu files); return cudaGetLastError()
 cudaError_t launch_copies(const CopyList &l, cudaStream_t st);

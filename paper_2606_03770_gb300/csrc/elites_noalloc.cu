@@ -11,7 +11,7 @@
 // only its inputs (population and fitness) and its output (elite indices);
 // the scratch lives in the file-scope array below, sized for at most
 // E2_NOALLOC_MAX_POP genomes.  The array is part of the library's device image:
-// every GPU that loads the library holds it (1 MiB) until the process exits.
+// every GPU that loads the library holds it (1.6 MiB) until the process exits.
 //
 // Every call shares that one array and leaves its contents behind.  Nothing in
 // it has to start at zero (each call writes every entry it reads), but two

@@ -782,7 +782,7 @@ __global__ void __launch_bounds__(256) copy_kernel(const __grid_constant__ CopyL
     if (!(bits & 15)) copy_chunk<uint4>(dst, src, n);
     else if (!(bits & 3)) copy_chunk<uint32_t>(dst, src, n);
     else copy_chunk<unsigned char>(dst, src, n);
-    if (blockIdx.x == 0 && threadIdx.x == 0 && l.word) *l.word = l.value;
+    if (blockIdx.x == 0 && threadIdx.x == 0 && l.word) *l.word = kNoBadGenome;
 }
 
 cudaError_t launch_copies(const CopyList &l, cudaStream_t st)
@@ -800,14 +800,13 @@ cudaError_t launch_validate(const e2_ctx *c, const DevPop &p, bool early)
                          c->stream, early, c->dm, p, c->err);
 }
 
-// Warps per CTA and shared memory of a kernel with genome_bytes(M) per warp.
-static cudaError_t genome_launch(const void *kernel, int M, int *nw, size_t *smem)
+// Warps per CTA of a kernel with genome_bytes(M) of shared memory per warp: up to
+// eight within the 48 KB that any block may use (one at 4,096 devices takes 33).
+static int genome_warps(int M)
 {
-    *nw = 8;
-    while (*nw > 1 && (size_t)*nw * genome_bytes(M) > 48 * 1024) *nw >>= 1;
-    *smem = (size_t)*nw * genome_bytes(M);
-    if (*smem <= 48 * 1024) return cudaSuccess;
-    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)*smem);
+    int nw = 8;
+    while (nw > 1 && (size_t)nw * genome_bytes(M) > 48 * 1024) nw >>= 1;
+    return nw;
 }
 
 cudaError_t launch_init(const e2_ctx *c, const DevPop &p, uint64_t seed)
@@ -817,11 +816,8 @@ cudaError_t launch_init(const e2_ctx *c, const DevPop &p, uint64_t seed)
         ++c->launches;
         return cudaGetLastError();
     }
-    size_t smem = 0;
-    int nw = 1;
-    const cudaError_t e = genome_launch(reinterpret_cast<const void *>(init_kernel), c->dm.M, &nw, &smem);
-    if (e != cudaSuccess) return e;
-    init_kernel<<<(unsigned)((c->dm.P + nw - 1) / nw), 32 * nw, smem, c->stream>>>(c->dm, p, seed);
+    const int nw = genome_warps(c->dm.M);
+    init_kernel<<<(unsigned)((c->dm.P + nw - 1) / nw), 32 * nw, nw * genome_bytes(c->dm.M), c->stream>>>(c->dm, p, seed);
     ++c->launches;
     return cudaGetLastError();
 }
@@ -871,12 +867,9 @@ cudaError_t launch_ga(const e2_ctx *c, const DevPop &src, const DevPop &dst, uin
 {
     if (c->dm.P <= c->dm.Q) return cudaSuccess;              // no children
     GaThr thr{c->thr_cx, c->thr_half, c->thr_mut, c->thr_k1, c->thr_k2, c->thr_k3};
-    size_t smem = 0;
-    int nw = 1;
-    const cudaError_t e = genome_launch(reinterpret_cast<const void *>(ga_kernel), c->dm.M, &nw, &smem);
-    if (e != cudaSuccess) return e;
+    const int nw = genome_warps(c->dm.M);
     const long long blocks = ((long long)(c->dm.P - c->dm.Q) + nw - 1) / nw;
-    ga_kernel<<<(unsigned)(blocks < 152 * 64 ? blocks : 152 * 64), 32 * nw, smem, st>>>(
+    ga_kernel<<<(unsigned)(blocks < 152 * 64 ? blocks : 152 * 64), 32 * nw, nw * genome_bytes(c->dm.M), st>>>(
         c->dm, src, dst, c->fit, seed, gen, thr);
     ++c->launches;
     return cudaGetLastError();
