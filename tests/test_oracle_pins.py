@@ -193,11 +193,12 @@ def test_dp_matches_brute_force(seed):
 
 
 def test_head_only_adds_and_a_free_head_on_device_1_decides_the_master():
-    """The facts the spilled DP layout's speculation rests on (Sec. 3.2, Alg. 1),
-    by enumeration: every master's optimum V_mu is at least the master-free
-    optimum V0 (the head only adds cost); so when the head on device 1 leaves
-    the optimum unchanged (V_1 == V0), the first-wins argmin over masters is
-    device 1 and the DP's value is V0.  Small-integer costs make both cases
+    """What lets a search over masters end at the first one that reaches the
+    master-free optimum (Sec. 3.2, Alg. 1; the per-layer DP does), by enumeration:
+    every master's optimum V_mu is at least the master-free optimum V0 (the head
+    only adds cost); so when the head on device 1 leaves the optimum unchanged
+    (V_1 == V0), the first-wins argmin over masters is device 1 and the DP's value
+    is V0.  Small-integer costs make both cases
     (V_1 == V0 and V_1 > V0) frequent."""
     rng = np.random.default_rng(2718)
     hits = misses = 0

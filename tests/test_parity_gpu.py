@@ -74,15 +74,11 @@ def test_eval_parity_full_size_sampled(name, P, sample):
     idx = np.sort(np.random.default_rng(5).choice(P, sample, replace=False))
     ora = O.OracleProblem(prob).eval_population(take(g, idx), prob.K_max, nthreads=O.num_threads())
     assert_eval_equal(gpu, ora, rows=idx)
-    # the 126-block model's largest DP spills its suffix columns to a global
-    # scratch (6 CTAs per SM instead of 4); the small replica sizes run in a
-    # second launch that does not spill, at that kernel's best occupancy
+    # replicas of more than 32 devices have a launch of their own; every workload here holds some
     st = eng.stats()
-    assert st["dp_launches"] == (2 if st["dp_ctas_small"] else 1)
-    assert (st["dp_runs_small"] > 0) == (st["dp_launches"] == 2), st
-    if name == "c4":
-        assert st["dp_launches"] == 2 and st["dp_ctas_small"] > st["dp_ctas"], st
-        assert st["dp_smem_small"] < st["dp_smem"] <= 40 * 1024, st
+    large = int((g["sizes"] > 32).sum())
+    assert st["dp_launches"] == 2 and st["dp_ctas_small"] > 0, st
+    assert large > 0 and 0 < st["dp_runs_small"] < st["dp_runs"], st
     eng.close()
 
 
@@ -190,12 +186,11 @@ def test_eval_parity_edge_cases(case):
 
 
 @pytest.mark.parametrize("min_tps", [0.0, 0.02])
-def test_spilled_layout_tie_heavy(min_tps):
-    """Replicas of ~20 devices over a 126-block model run in the spilled layout,
-    where the prefix chain speculates on the head on device 1: small-integer
-    costs make the master-free optimum, V_1 and the other masters tie often, so
-    both the proof of mu* = 1 and its fallback (the chain again without the
-    head, the combine seeded with master 1) meet exact ties."""
+def test_masters_that_tie_on_a_long_model(min_tps):
+    """Replicas of about 20 devices over a 126-block model with small-integer
+    costs: the optimum without a head, the head on the first device and the other
+    masters tie often, so the smallest master at the least threshold is decided
+    among exact ties."""
     rng = np.random.default_rng(606)
     M, N, K, P = 64, 126, 3, 64
     prob = _edge_problem(rng, M, N, P, K, integer=True, Q=4, min_tps=min_tps)
@@ -206,7 +201,7 @@ def test_spilled_layout_tie_heavy(min_tps):
     ora = O.OracleProblem(prob).eval_population(g, K, nthreads=O.num_threads())
     assert_eval_equal(gpu, ora)
     st = eng.stats()
-    assert st["dp_smem"] <= 40 * 1024 and st["device_errors"] == 0, st   # the spilled layout
+    assert st["device_errors"] == 0, st
     assert st["served"] == int((ora["bsel"] >= 0).sum()) > 20
     eng.close()
 
@@ -410,7 +405,7 @@ def test_recorded_generation_matches_separate_calls(name, P, gens):
         assert np.array_equal(fa, fb), gen
         assert_genomes_equal(a.get_population(), b.get_population())
         # a replay counts the recorded kernel nodes: as many as the separate calls launch
-        # (pre-pass, bin scan, scatter, DP launches, finaliser, duplicates -- from 4,096
+        # (pre-pass, count, scatter, DP launches, finaliser, duplicates -- from 4,096
         # genomes a fingerprint table and a lookup --, elite selection, candidate ranks,
         # full ranks, children)
         sa, sb = a.stats(), b.stats()
@@ -543,8 +538,8 @@ def test_role_search_twenty_replicas(integer, kw):
 
 
 def test_role_search_with_two_dp_launches():
-    """The role search on a fleet whose DP runs in two shared-memory classes
-    (220-block rows): both roles of every replica through both launches."""
+    """The role search on a fleet with replicas on both sides of 32 devices:
+    both roles of every replica through both DP launches."""
     rng = np.random.default_rng(41)
     M, N, K, P = 48, 220, 8, 24
     prob = _edge_problem(rng, M, N, P, K, integer=True, Q=2, min_tps=0.01, role_search=1)
@@ -601,9 +596,9 @@ def _genomes_from(M, K, groups, rng):
 
 @pytest.mark.parametrize("case", ["wide rows", "largest replica"])
 def test_eval_parity_maximum_sizes(case):
-    """The largest shapes the ABI takes: cost rows of ~300 blocks (W > 256,
-    ~190 KB of DP shared memory), and a replica of 256 devices (the limit) next
-    to mixed ones; then a generation step on them."""
+    """The largest shapes the ABI takes: cost rows of ~300 blocks (W > 256), and a
+    replica of 256 devices (the limit) next to mixed ones; then a generation step
+    on them."""
     rng = np.random.default_rng(77)
     if case == "wide rows":
         M, N, K = 64, 300, 6
@@ -621,9 +616,7 @@ def test_eval_parity_maximum_sizes(case):
     st = eng.stats()
     assert st["paper_candidates"] == ora["cand"]
     if case != "wide rows":
-        # replicas of 6, 250 and 256 devices (W <= 255 with few devices, or a
-        # short row) need less than half the shared memory of the 56- and
-        # 200-device ones: they run in the second DP launch
+        # all but the replica of 6 devices run in the second DP launch (more than 32 devices)
         assert st["dp_launches"] == 2 and 0 < st["dp_runs_small"] <= st["dp_runs"], st
     assert np.isfinite(ora["T"]).any()
     ga = O.ga_of(prob)

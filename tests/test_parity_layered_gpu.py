@@ -4,8 +4,8 @@ oracle, through the C ABI.
 Models whose blocks alternate sliding-window and full attention (or end in
 a run of full-attention blocks), given as per-variant prefix sums PF, PB,
 PM: every stage then costs what its own blocks cost, and these contexts run
-the plain-scan DP (every split of every cell, the masters factored through
-prefix and suffix tables).  Fitness, partitions, T and Lambda bit-exact,
+the per-layer DP (columns by bisection on range minima, the masters factored
+through prefix and suffix tables).  Fitness, partitions, T and Lambda bit-exact,
 with role bits, the role search and the adapted-SplitWise rule, and over
 generations; plus the uniform-sum case against the identical-block kernel
 and the inputs e2_create refuses.
@@ -81,7 +81,7 @@ def test_layered_full_size_sampled():
 
 
 def test_uniform_sums_equal_the_identical_block_kernel():
-    """Prefix sums of identical blocks through the plain-scan path give what
+    """Prefix sums of identical blocks through the per-layer DP give what
     the identical-block kernel gives (and what the oracle gives)."""
     prob = W.make_config("c2", P=512)
     ramp = np.arange(prob.N + 1, dtype=np.uint64)[None, :]

@@ -81,3 +81,37 @@ def test_costs_off_the_estimate(what, role_search):
         prob.bw = 2.0 ** rng.integers(-40, 40, M).astype(np.float64)
     ora = _check(prob, M, K, genomes, rng)
     assert np.isfinite(ora["T"]).any()
+
+
+@pytest.mark.parametrize("M,N", [(32, 120), (40, 90), (60, 100)])
+def test_bisection_over_the_keys(M, N):
+    """A head worth more than all blocks: the threshold is far from the estimate,
+    more than the walk's steps, and the bisection takes over.  A walk reads an
+    entry of the two rows at most twice, and four per lane before it; a bisection
+    of 31 rounds reads more than that."""
+    for seed in range(4):
+        rng = np.random.default_rng(seed)
+        prob = _edge_problem(rng, M, N, 1, 1, integer=True, Q=1, min_tps=0.0)
+        prob.mem = np.full(M, 2**40, np.uint64)
+        prob.head_flops = np.full_like(prob.head_flops, 3000)
+        prob.rate = rng.uniform(0.1, 3, M)
+        g = _genomes_from(M, 1, [[M]], rng)
+        g["roles"][:] = 0
+        eng = engine(prob)
+        eng.eval(g)
+        assert_eval_equal(eng.results(), O.OracleProblem(prob).eval_population(g, 1))
+        st = eng.stats()
+        walk = 2 * 2 * M * (N - M + 1) + 4 * 32 * -(-M // 32)
+        assert st["dp_runs"] == 1 and st["dp_probes"] > walk, (st["dp_probes"], walk)
+        eng.close()
+
+
+@pytest.mark.parametrize("M,N", [(8, 700), (16, 1024)])
+def test_long_models_on_small_fleets(M, N):
+    """Up to 16 devices any number of blocks is accepted."""
+    rng = np.random.default_rng(N)
+    genomes = [[M], [1] * 4 + [M - 4], [M - 3, 3]] * 2
+    prob = _edge_problem(rng, M, N, len(genomes), 5, integer=True, Q=1, min_tps=0.0)
+    prob.mem = np.full(M, 2**20, np.uint64)
+    ora = _check(prob, M, 5, genomes, rng)
+    assert np.isfinite(ora["T"]).any()

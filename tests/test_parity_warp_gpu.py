@@ -1,13 +1,10 @@
-"""Parity of the warp-per-run DP launch (the small replica sizes of a large
-population, one DP run per warp) with the oracle, through the C ABI.
+"""Parity of the DP's launches over large populations with the oracle, through
+the C ABI: two launches where replicas of more than 32 devices can occur (the
+larger ones in the second, several devices per lane), one otherwise.
 
-The second DP launch runs one run per warp when the population is large
-enough (its slots at least eight times that launch's runs in flight) and no
-four-warp launch of the small sizes raises the occupancy: the 80-block
-workloads at full size.  Full populations (and role search, where each
-replica runs in both roles) bit for bit, and a large population of
-small-integer costs (many exact ties, memory walls, a Min_TPS floor) on which
-every DP tie rule is exercised by the warp kernel.
+Full populations (and role search, where each replica runs in both roles) bit
+for bit, and a large population of small-integer costs (many exact ties,
+memory walls, a Min_TPS floor) on which every DP tie rule is exercised.
 """
 import dataclasses
 
@@ -34,7 +31,7 @@ def _launches(st, n):
 
 
 @pytest.mark.parametrize("name,P,role_search", [("c3", 4096, 0), ("c3", 2048, 1), ("c5", 1024, 0)])
-def test_warp_launch_full_population(name, P, role_search):
+def test_two_launches_full_population(name, P, role_search):
     prob = dataclasses.replace(W.make_config(name, P=P), role_search=role_search)
     eng = engine(prob)
     g = W.random_genomes(prob.M, prob.K_max, P, seed=41)
@@ -52,7 +49,7 @@ def test_warp_launch_full_population(name, P, role_search):
 
 
 @pytest.mark.parametrize("min_tps", [0.0, 0.1])
-def test_warp_launch_ties_and_memory_walls(min_tps):
+def test_one_launch_ties_and_memory_walls(min_tps):
     """Small-integer costs on 24 devices and 12 blocks (exact ties between
     splits, masters and batches; devices that cannot hold a block), 8,192
     genomes of up to six replicas: the whole population, then a generation."""
@@ -74,13 +71,10 @@ def test_warp_launch_ties_and_memory_walls(min_tps):
     eng.close()
 
 
-def test_small_population_keeps_one_launch():
-    """At 1,024 genomes of the 32-device workload the runs per warp would be
-    few: the small sizes stay in the four-warp launch."""
-    prob = W.make_config("c2")
-    eng = engine(prob)
+def test_small_fleet_has_one_launch():
+    """No replica of the 32-device workload has more than a device per lane."""
+    eng = engine(W.make_config("c2"))
     eng.init_population(3)
     eng.eval()
-    st = eng.stats()
-    assert st["dp_runs_per_cta_small"] in (0, 1), st
+    _launches(eng.stats(), 1)
     eng.close()
