@@ -56,12 +56,12 @@ L2_FLUSH_BYTES = 256 << 20
 OPS_PER_PROBE = 5
 OPS_PER_CELL = 5
 INT32_LANES_PER_SM = 128
-# dram__bytes_read.sum + dram__bytes_write.sum of the two DP launches of one
-# evaluation at the default workload, from the ncu capture in profiles/; cold
-# (ncu flushes the caches before each launch), so it counts the L2-resident
-# tables again
-DP_TRAFFIC_BYTES = 49_037_312
-DP_TRAFFIC_SOURCE = "profiles/dp_order_c4.md (dram read+write, both DP launches of one evaluation, cold)"
+# dram__bytes_read.sum + dram__bytes_write.sum of the two DP launches of this
+# program's second timed generation at the default workload, by ncu; cold (ncu
+# flushes the caches before each launch), so it counts the L2-resident tables
+# again
+DP_TRAFFIC_BYTES = 49_877_504
+DP_TRAFFIC_SOURCE = "profiles/dp_order_c4.md (dram read+write, both DP launches of one generation of this bench, cold)"
 
 
 def parse():
