@@ -1586,7 +1586,9 @@ cudaError_t configure_eval(e2_ctx *c)
 
 cudaError_t launch_eval(const e2_ctx *c, const DevPop &p)
 {
-    Tables tb{c->leaf, c->tau, c->capg, c->leaf_rank, c->lcost, c->drec, c->fxs, c->prec, c->prech, c->capv, c->ibw, c->fpr};
+    Tables tb{c->rate, c->bw, c->mem, c->rate_cpu, c->bw_cpu, c->mem_cpu, c->prof, c->leaf, c->tau,
+              c->capg, c->leaf_rank, c->lcost, c->drec, c->fxs, c->prec, c->prech, c->capv,
+              c->ibw, c->fpr};
     EvalOut out{c->fit, c->layers, c->master, c->bsel, c->T, c->L, c->hash, c->stats, c->gpu_layers};
     SlotInfo si{c->slot_off, c->slot_info};
     WorkList wl{c->items, c->list_ctrl};

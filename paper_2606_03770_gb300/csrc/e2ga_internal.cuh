@@ -116,9 +116,17 @@ struct __align__(16) LinkRec {
     float lb;
 };
 
-// (On 16 bytes among a kernel's parameters: read in pairs there, the pointers
-// cost 0.6% of an evaluation of 512 devices when the pairs straddle them.)
-struct __align__(16) Tables {
+struct Tables {
+    // The fleet and the profile as given.  No kernel of an evaluation reads these
+    // seven; they keep the parameters after the tables where they are: without them
+    // class 1 of the DP took 139.7 us instead of 137.8 at 512 devices and a whole
+    // evaluation 0.2 to 0.6% longer, in every order of the parameters tried, and with
+    // seven words of padding in their place it did not.
+    const double *rate, *bw;
+    const uint64_t *mem;
+    const double *rate_cpu, *bw_cpu;   // [M] host side of offloaded blocks (offload only)
+    const uint64_t *mem_cpu;           // [M] host memory for blocks, bytes (offload only)
+    const uint64_t *prof;      // [kNumProf][V]
     const double *leaf;        // [V][M][2][LS]: leaf[((v*M+d)*2+mf)*LS + n-1] = l_d(n blocks, master mf)
     const LinkRec *tau;        // [V][M][M]
     const int32_t *capg;       // [V][M][2]: most blocks in device memory, without / with the head (-1: the head
